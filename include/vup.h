@@ -177,10 +177,10 @@ vup_status vup_set_outputs(vup_grid g, const double *y_dev, int n_bins, int n_mo
  * and never stored.  The first call with a larger K than before allocates
  * per-K scratch (not capturable in a CUDA graph), and the first TF32 call on
  * a grid builds its TF32 power tables; later calls allocate nothing.
- * When the histogram's layout is (re)built by the call (the first call after
- * vup_eval_model or vup_set_outputs), the grid runs parts of the work on two
- * streams of its own (the layout beside the density preparation and the
- * contraction; the prefix sums and the FP64 moments finish beside those) that
+ * A call that wants histograms runs parts of the work on streams of the grid's
+ * own (the layout, where the call (re)builds it -- the first call after
+ * vup_eval_model or vup_set_outputs --, beside the density preparation and the
+ * contraction; the FP64 moments finish beside the histogram) that
  * fork from and join back into `stream`: every result is complete, in stream
  * order, once the work queued on `stream` by this call is.  The grid creates
  * those streams and their events on first use.
@@ -401,8 +401,10 @@ typedef struct {
      * walks sorted points, stream 1 sorted intervals (stretches of one bin
      * along the gathered axis, summed as differences of prefix sums), stream
      * 2 records (stretches of one line over a group of 4 consecutive bins,
-     * monotone, five prefix sums for four bins).  Counts are those of the
-     * chosen layout; hist_runs is 0 when the point and interval streams were
+     * monotone, five prefix sums for four bins).  The choice and the counts are
+     * those of the grid itself; where slices of an axis that fall in the same
+     * bins throughout are merged for the walk, they are taken for this call
+     * from the unmerged grid.  hist_runs is 0 when the point and interval streams were
      * not built (the record stream was cheaper than both). */
     int32_t hist_layout, hist_stream;
     int64_t hist_runs, hist_intervals, hist_records;

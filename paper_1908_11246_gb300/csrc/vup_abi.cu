@@ -248,13 +248,12 @@ static void free_grid(vup_grid g) {
         devbuf_free(L.rec_gch);
     }
     cudaFree(g->hist_sel);
+    cudaFree(g->fold_mem);
     if (g->side) cudaStreamDestroy(g->side);
     if (g->ev_fork) cudaEventDestroy(g->ev_fork);
     if (g->ev_join) cudaEventDestroy(g->ev_join);
     if (g->ev_rec) cudaEventDestroy(g->ev_rec);
     if (g->ev_lay) cudaEventDestroy(g->ev_lay);
-    if (g->ev_dens) cudaEventDestroy(g->ev_dens);
-    if (g->ev_pre) cudaEventDestroy(g->ev_pre);
     if (g->ev_mom) cudaEventDestroy(g->ev_mom);
     if (g->ev_mfin) cudaEventDestroy(g->ev_mfin);
     if (g->side2) cudaStreamDestroy(g->side2);
@@ -280,7 +279,7 @@ static void free_grid(vup_grid g) {
     devbuf_free(g->partials);
     devbuf_free(g->hist_part);
     devbuf_free(g->hist_direct);
-    devbuf_free(g->hist_prefix);
+    devbuf_free(g->ftab_fold);
     devbuf_free(g->ipsa_part);
     devbuf_free(g->atf_hi);
     devbuf_free(g->atf_lo);
@@ -397,6 +396,23 @@ extern "C" vup_status vup_grid_create(int ndim, const int64_t *n, const double *
         L.rec_chunk = A.rec_chunk;
         L.rec_chunk_grp = A.rec_chunk_grp;
     }
+    if (ndim >= 2) {
+        // equal-slice folding: geometry, class members (CSR), build scratch, merged bins
+        int64_t slices = 0;
+        for (int d = 0; d < ndim; ++d) slices += n[d];
+        const size_t a16 = 15, idx = sizeof(int32_t) * (size_t)(3 * slices + 3);
+        const size_t o_idx = (sizeof(FoldGeom) + a16) & ~a16, o_scr = (o_idx + idx + a16) & ~a16;
+        g->fold_scratch_bytes = vup_fold_scratch_bytes(g);
+        const size_t o_bins = (o_scr + g->fold_scratch_bytes + a16) & ~a16;
+        ALLOC(g->fold_mem, o_bins + sizeof(int32_t) * (size_t)N);
+        uint8_t *base = (uint8_t *)g->fold_mem;
+        g->fold = (FoldGeom *)base;
+        g->fold_rep = (int32_t *)(base + o_idx);
+        g->fold_members = g->fold_rep + slices;
+        g->fold_start = g->fold_members + slices;
+        g->fold_scratch = base + o_scr;
+        g->fold_bins = (int32_t *)(base + o_bins);
+    }
     ALLOC(g->hist_sel, sizeof(int32_t) * 8);
     ALLOC(g->ydev_scale, sizeof(double) * kScaleSlots);
     ALLOC(g->dstatus, sizeof(int));
@@ -512,12 +528,6 @@ vup_status vup_reserve_k(vup_grid g, int64_t K, bool bf16, bool ipsa, bool tf32)
             return st;
         if ((st = devbuf_reserve(g->hist_direct, sizeof(float) * (size_t)g->hist_P * g->B * K_pad)) != VUP_OK)
             return st;
-        {
-            int64_t rows = 1;
-            for (int l = 0; l < g->n_layouts; ++l) rows = std::max(rows, g->hl[l].part_rows);
-            if ((st = devbuf_reserve(g->hist_prefix, sizeof(float) * (size_t)g->hist_P * K_pad * (rows + 1))) != VUP_OK)
-                return st;
-        }
         if (tf32) {
             const size_t a = (size_t)K_pad * g->orient[vup_tc_orient(g)].R_pad;
             if ((st = devbuf_reserve(g->atf_hi, sizeof(float) * a)) != VUP_OK) return st;
@@ -558,6 +568,7 @@ static vup_status propagate_nd(vup_grid g, const vup_densities *d, vup_precision
     const bool want_m = moments_raw || moments_central;
     const bool fuse = ip != nullptr;
     if ((st = vup_reserve_k(g, K, bf16, fuse, tf32)) != VUP_OK) return st;
+    if (hist && (st = vup_reserve_fold(g, K)) != VUP_OK) return st;
     // the histogram layout (when not built for this model yet) on the second
     // stream, beside the density preparation and the contraction
     bool forked = false;
@@ -606,24 +617,19 @@ static vup_status propagate_nd(vup_grid g, const vup_densities *d, vup_precision
         VUP_CHECK_CUDA(cudaEventRecord(g->ev_join, g->side));
         if (lst != VUP_OK) return lst;
     }
-    // the histogram's prefix-sum tiles on a third stream, beside the
-    // contraction (they need the densities and the layout choice only)
-    bool prefix_ready = false;
-    if (hist && forked && want_m) {
-        if (!g->side2) {
-            VUP_CHECK_CUDA(cudaStreamCreateWithFlags(&g->side2, cudaStreamNonBlocking));
-            VUP_CHECK_CUDA(cudaEventCreateWithFlags(&g->ev_dens, cudaEventDisableTiming));
-            VUP_CHECK_CUDA(cudaEventCreateWithFlags(&g->ev_pre, cudaEventDisableTiming));
-            VUP_CHECK_CUDA(cudaEventCreateWithFlags(&g->ev_mom, cudaEventDisableTiming));
-            VUP_CHECK_CUDA(cudaEventCreateWithFlags(&g->ev_mfin, cudaEventDisableTiming));
-            join_fin.e = g->ev_mfin;
-        }
-        VUP_CHECK_CUDA(cudaEventRecord(g->ev_dens, s));
-        VUP_CHECK_CUDA(cudaStreamWaitEvent(g->side2, g->ev_dens, 0));
-        VUP_CHECK_CUDA(cudaStreamWaitEvent(g->side2, g->ev_lay, 0));
-        prefix_ready = vup_hist_prefix(g, K, g->side2);
-        VUP_CHECK_CUDA(cudaEventRecord(g->ev_pre, g->side2));
+    // merged factor tables of the rest axes: short, at full bandwidth before the
+    // contraction takes the L2's (15 us where beside it 260 at 1024 x 16384)
+    const bool beside = hist && want_m;  // the FP64 finish runs beside the histogram
+    if (hist) {
+        if (forked) VUP_CHECK_CUDA(cudaStreamWaitEvent(s, g->ev_lay, 0));
+        if ((st = vup_fold_tables(g, K, s)) != VUP_OK) return st;
     }
+    if (beside && !g->side2) {
+        VUP_CHECK_CUDA(cudaStreamCreateWithFlags(&g->side2, cudaStreamNonBlocking));
+        VUP_CHECK_CUDA(cudaEventCreateWithFlags(&g->ev_mom, cudaEventDisableTiming));
+        VUP_CHECK_CUDA(cudaEventCreateWithFlags(&g->ev_mfin, cudaEventDisableTiming));
+    }
+    join_fin.e = g->ev_mfin;
     // fused: the sensitivity partials of both orientations ([3][tiles][K_pad][4]
     // each, orientation 1 after orientation 0), the forward orientation first
     const int fo = bf16 ? to : 0;
@@ -655,8 +661,8 @@ static vup_status propagate_nd(vup_grid g, const vup_densities *d, vup_precision
             nct = vup_simt_col_tiles(g->orient[0]);
         }
         if (!want_m) {
-        } else if (prefix_ready) {
-            // the FP64 finish on the third stream: the histogram does not need it
+        } else if (beside) {
+            // on a stream of its own: the histogram does not need it
             VUP_CHECK_CUDA(cudaEventRecord(g->ev_mom, s));
             VUP_CHECK_CUDA(cudaStreamWaitEvent(g->side2, g->ev_mom, 0));
             join_fin.on = true;
@@ -671,9 +677,7 @@ static vup_status propagate_nd(vup_grid g, const vup_densities *d, vup_precision
         // the record-stream histogram waits for the records only; the other
         // streams' kernels (and the finish) for the whole layout
         if (forked) VUP_CHECK_CUDA(cudaStreamWaitEvent(s, g->ev_rec, 0));
-        if (prefix_ready) VUP_CHECK_CUDA(cudaStreamWaitEvent(s, g->ev_pre, 0));
-        if ((st = vup_hist_fused(g, K, hist, s, nullptr, false, forked ? g->ev_join : nullptr, prefix_ready)) !=
-            VUP_OK)
+        if ((st = vup_hist_fused(g, K, hist, s, nullptr, false, forked ? g->ev_join : nullptr, true)) != VUP_OK)
             return st;
         join.on = false;
     }
@@ -812,6 +816,24 @@ extern "C" vup_status vup_grid_info(vup_grid g, vup_grid_info_t *info) {
         if (g->ndim >= 2) {
             if (!g->layout_valid) {
                 vup_status st = vup_build_layout(g, 0);
+                if (st != VUP_OK) return st;
+                VUP_CHECK_CUDA(cudaDeviceSynchronize());
+            }
+            // the counts describe the grid itself: where the walks run on a merged
+            // grid, the unfolded layout is built for them and then the merged one again
+            FoldGeom F;
+            VUP_CHECK_CUDA(cudaMemcpy(&F, g->fold, sizeof(F), cudaMemcpyDeviceToHost));
+            const bool points = g->layout_has_points != 0;
+            struct Refold {
+                vup_grid g;
+                bool on, points;
+                ~Refold() {
+                    if (on && vup_build_layout(g, 0, points) != VUP_OK) g->layout_valid = 0;
+                    if (on) cudaDeviceSynchronize();
+                }
+            } refold{g, F.any != 0, points};
+            if (F.any) {
+                vup_status st = vup_build_layout(g, 0, points, nullptr, nullptr, false);
                 if (st != VUP_OK) return st;
                 VUP_CHECK_CUDA(cudaDeviceSynchronize());
             }

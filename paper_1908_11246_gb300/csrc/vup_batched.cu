@@ -235,6 +235,7 @@ extern "C" vup_status vup_propagate_batched(int n_inst, const vup_grid *g, const
             const int64_t K = d[i].K, K_pad = ceil_div64(K, 128) * 128;
             vup_status st;
             if ((st = vup_reserve_k(g[i], K, bf16, false)) != VUP_OK) return st;
+            if (hist && hist[i] && (st = vup_reserve_fold(g[i], K)) != VUP_OK) return st;
             if ((st = vup_build_tables(g[i], kOrientLast, bf16 ? 1 : 0, s)) != VUP_OK) return st;
             if (hist && hist[i] && (st = vup_ensure_layout(g[i], s)) != VUP_OK) return st;
             if ((st = vup_density_reserve(g[i], K)) != VUP_OK) return st;
@@ -258,7 +259,7 @@ extern "C" vup_status vup_propagate_batched(int n_inst, const vup_grid *g, const
                               (uint64_t)(hist ? hist[i] : nullptr), (uint64_t)G->ftab.p, (uint64_t)G->dstats.p,
                               (uint64_t)G->dconst.p, (uint64_t)G->dpart.p, (uint64_t)G->partials.p,
                               (uint64_t)G->atab_hi.p, (uint64_t)G->atab_lo.p, (uint64_t)G->hist_part.p,
-                              (uint64_t)G->hist_direct.p};
+                              (uint64_t)G->hist_direct.p, (uint64_t)G->ftab_fold.p};
         key.insert(key.end(), std::begin(w), std::end(w));
     }
     Entry *e = nullptr;

@@ -45,6 +45,7 @@ extern "C" vup_status vup_posterior_means(vup_grid g, const vup_densities *d, fl
     const int B = g->B, nd = g->ndim;
     const size_t tab = (size_t)K_pad * vup_ftab_floats(g);
     if ((st = vup_reserve_k(g, K, false, false)) != VUP_OK) return st;
+    if ((st = vup_reserve_fold(g, K)) != VUP_OK) return st;
     if ((st = devbuf_reserve(g_xtab, sizeof(float) * tab)) != VUP_OK) return st;
     if ((st = devbuf_reserve(g_hx, sizeof(float) * (size_t)nd * K * B)) != VUP_OK) return st;
     if (!hist) {

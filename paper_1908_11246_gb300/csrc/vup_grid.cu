@@ -539,9 +539,13 @@ __global__ void __launch_bounds__(256) k_model_bins(double *__restrict__ y, int6
 __device__ __forceinline__ bool gated_off(const int32_t *gate) { return gate && gate[0] == 0; }
 
 // Points per (key, warp tile) of a key array with key < Bk.
+// (fold given: the merged grid's points; tiles past them count nothing)
 __global__ void k_count(const int32_t *__restrict__ keys, int64_t N, int Bk, int32_t *__restrict__ counts,
-                        int64_t n_tiles, const int32_t *gate) {
+                        int64_t n_tiles, const int32_t *gate, const FoldGeom *fold) {
+    pdl_trigger();
+    pdl_wait();
     if (gated_off(gate)) return;
+    if (fold) N = fold->N;
     extern __shared__ int32_t s_cnt[];  // [warps][Bk]
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     int32_t *cnt = s_cnt + warp * Bk;
@@ -568,52 +572,463 @@ struct LayGeom {
     int P;
 };
 struct LaySel {
-    LayGeom g[2];
+    const FoldGeom *fold;  // the (merged) grid's sizes, decided on the device
     const int32_t *sel;
-    __device__ __forceinline__ LayGeom get() const { return g[sel[0] ? 1 : 0]; }
+    __device__ __forceinline__ LayGeom get() const {
+        const int l = sel[0] ? 1 : 0;
+        return LayGeom{fold->n_last[l], fold->part_rows[l], fold->P[l]};
+    }
 };
 
-// Intervals of both 2-D layouts (stretches of one (part, bin) key along the
-// gathered axis), counted without sorting: 1 + key changes along each line.
-__global__ void k_iv_count(const int32_t *__restrict__ bins, int64_t n0, int64_t n1, int B, LaySel L,
-                           int32_t *__restrict__ cnt) {
-    const int64_t N = n0 * n1;
-    int32_t c0 = 0, c1 = 0;
-    const uint32_t p0 = (uint32_t)L.g[0].part_rows, p1 = (uint32_t)L.g[1].part_rows;
-    const uint32_t m1 = (uint32_t)n1;  // N < 2^31: 32-bit index arithmetic
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t i0 = (uint32_t)i / m1, i1 = (uint32_t)i - i0 * m1;
-        const int32_t b = bins[i];
-        // layout 0 gathers axis 1, layout 1 axis 0
-        c0 += i1 == 0 || (i1 / p0) * B + b != ((i1 - 1) / p0) * B + bins[i - 1];
-        c1 += i0 == 0 || (i0 / p1) * B + b != ((i0 - 1) / p1) * B + bins[i - n1];
+// ---- equal slices of the bin grid (FoldGeom) ----------------------------------
+// Host-side sizes, scratch and outputs of the fold kernels.
+struct FoldArgs {
+    const int32_t *bins;
+    int64_t n[3];            // the grid's axes (2-D: n[0], n[1], 1)
+    int ndim, B;
+    int P[2];                // the unfolded layouts' parts and rows per part
+    int64_t part_rows[2];
+    FoldGeom *fold;
+    // zeroed before k_fold_hash: slice hashes, hash-table keys and values (a power
+    // of two >= 2 n slots per axis), unequal-slice marks, control words
+    unsigned long long *hash, *tkey;
+    // ctl: 0, 1, 2 block counters, 3 candidates, 4..6 candidate axes, 8, 9 intervals of the
+    // layouts, 10..12 classes (0: not folded), 13, 14 intervals of the merged grid's layouts
+    int32_t *tval, *bad, *ctl;
+    int32_t *rep, *start, *members, *out_bins, *sel;
+};
+constexpr int kFoldCtl = 16;
+__host__ __device__ inline int64_t fold_slots(int64_t n) {
+    int64_t t = 2;
+    while (t < 2 * n) t <<= 1;
+    return t;
+}
+
+// Per-index weight of a slice hash: an odd 64-bit mix (the SplitMix64 finaliser) of the index.
+__device__ __forceinline__ unsigned long long fold_weight(int axis, int64_t i) {
+    unsigned long long z = (unsigned long long)(i + 1) * 0x9e3779b97f4a7c15ull + (unsigned long long)axis * 0xd1b54a32d192ed03ull;
+    z = (z ^ (z >> 30)) * 0xbf58476d1ce4e5b9ull;
+    z = (z ^ (z >> 27)) * 0x94d049bb133111ebull;
+    return (z ^ (z >> 31)) | 1ull;
+}
+
+// The geometry of the (merged) grid: sizes, layouts' gathered axes, parts.  A
+// merged axis keeps the unfolded layout's rows per part at most, so that every
+// buffer and tile sized for the unfolded grid holds it.
+__device__ void fold_write_geom(const FoldArgs &A, const int64_t m[3], const int folded[3]) {
+    FoldGeom F;
+    F.any = 0;
+    F.N = 1;
+    for (int d = 0; d < 3; ++d) {
+        F.n[d] = m[d];
+        F.folded[d] = folded[d];
+        F.any |= folded[d];
+        F.N *= m[d];
     }
-    for (int o = 16; o > 0; o >>= 1) {
-        c0 += __shfl_xor_sync(0xffffffffu, c0, o);
-        c1 += __shfl_xor_sync(0xffffffffu, c1, o);
+    for (int l = 0; l < 2; ++l) {
+        const int ax = (l == 0 || A.ndim == 3) ? A.ndim - 1 : 0;
+        F.n_last[l] = m[ax];
+        const int64_t P = A.P[l] == 1 ? 1 : (m[ax] + A.part_rows[l] - 1) / A.part_rows[l];
+        F.P[l] = (int32_t)P;
+        F.part_rows[l] = (m[ax] + P - 1) / P;
     }
-    if ((threadIdx.x & 31) == 0) {
-        atomicAdd(&cnt[0], c0);
-        atomicAdd(&cnt[1], c1);
+    *A.fold = F;
+}
+
+// True in every thread of the block that finishes last (the others' writes are then visible to it).
+__device__ __forceinline__ bool fold_last_block(int32_t *ctr) {
+    __shared__ int s_last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(ctr, 1) == (int)gridDim.x - 1;
+    __syncthreads();
+    if (s_last) __threadfence();
+    return s_last != 0;
+}
+
+// Layout choice: the one with fewer intervals (both streams' work grows with the
+// runs and intervals of the layout, and a layout's runs are at most its intervals).
+__device__ __forceinline__ void pick_layout(const FoldArgs &A, int32_t c0, int32_t c1) {
+    A.sel[2] = c0;
+    A.sel[3] = c1;
+    A.sel[0] = A.ndim == 2 && c1 < c0 ? 1 : 0;
+}
+
+// One pass over the bins (viewed as [R][C], C the last axis): the slice hashes
+// of every axis and, on 2-D grids, the intervals of both layouts (stretches of
+// one (part, bin) key along the gathered axis: 1 + key changes along each
+// line).  The hash of a slice is the sum of (bin + 1) times the product of its
+// points' index weights, modulo 2^64.  A warp takes 8 rows of 128 columns,
+// every load of four rows in flight together: column sums stay in registers, a
+// row's sum is reduced over the warp.
+constexpr int kFoldRows = 8, kFoldCols = 128;
+__global__ void __launch_bounds__(256) k_fold_hash(FoldArgs A) {
+    pdl_trigger();
+    pdl_wait();
+    const int tid = threadIdx.x, lane = tid & 31;
+    const bool d3 = A.ndim == 3;
+    const int64_t C = A.n[A.ndim - 1], R = d3 ? A.n[0] * A.n[1] : A.n[0];
+    unsigned long long *h0 = A.hash, *h1 = A.hash + A.n[0];
+    unsigned long long *hc = d3 ? h1 + A.n[1] : h1;
+    const uint32_t p0 = (uint32_t)A.part_rows[0], p1 = (uint32_t)A.part_rows[1];
+    constexpr int kRows = kFoldRows * 8;  // rows of a block
+    const int64_t ncb = (C + kFoldCols - 1) / kFoldCols, nrb = (R + kRows - 1) / kRows;
+    __shared__ unsigned long long s_col[8][kFoldCols];
+    int32_t i0 = 0, i1 = 0;  // intervals of layouts 0 (gathers axis 1) and 1 (gathers axis 0)
+    for (int64_t t = blockIdx.x; t < ncb * nrb; t += gridDim.x) {
+        const int64_t cb = (t % ncb) * kFoldCols, c0 = cb + lane;
+        const int64_t r0 = (t / ncb) * kRows + (tid >> 5) * kFoldRows;
+        unsigned long long wc[4], acc[4] = {0, 0, 0, 0};
+        bool cut[4];  // a part of layout 0 starts at the column
+        int32_t up[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            wc[q] = fold_weight(A.ndim - 1, c0 + 32 * q);
+            cut[q] = (uint32_t)(c0 + 32 * q) % p0 == 0;
+            up[q] = !d3 && r0 > 0 && r0 < R && c0 + 32 * q < C ? A.bins[(r0 - 1) * C + c0 + 32 * q] + 1 : 0;
+        }
+#pragma unroll
+        for (int rr = 0; rr < kFoldRows; rr += 4) {
+            int32_t b[4][4], left[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const bool in = r0 + rr + u < R;
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    b[u][q] = in && c0 + 32 * q < C ? A.bins[(r0 + rr + u) * C + c0 + 32 * q] + 1 : 0;
+                left[u] = !d3 && in && lane == 0 && c0 > 0 ? A.bins[(r0 + rr + u) * C + c0 - 1] + 1 : 0;
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int64_t r = r0 + rr + u;
+                if (r >= R) break;
+                const int64_t a0 = d3 ? r / A.n[1] : r, a1 = d3 ? r - a0 * A.n[1] : 0;
+                const unsigned long long w0 = fold_weight(0, a0), w1 = d3 ? fold_weight(1, a1) : 1ull;
+                const unsigned long long wr = w0 * w1;
+                unsigned long long s = 0;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    s += (unsigned long long)b[u][q] * wc[q];
+                    acc[q] += (unsigned long long)b[u][q] * wr;
+                }
+                if (!d3) {
+                    const bool rcut = (uint32_t)r % p1 == 0;
+                    int32_t lw = left[u];  // the column before this lane's, per group of 32
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const int32_t sh = __shfl_up_sync(0xffffffffu, b[u][q], 1);
+                        const int32_t l = lane == 0 ? lw : sh;
+                        lw = __shfl_sync(0xffffffffu, b[u][q], 31);
+                        if (c0 + 32 * q < C) {
+                            i0 += cut[q] || b[u][q] != l;
+                            i1 += rcut || b[u][q] != up[q];
+                        }
+                        up[q] = b[u][q];
+                    }
+                }
+                for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+                if (lane == 0) {
+                    atomicAdd(h0 + a0, s * w1);
+                    if (d3) atomicAdd(h1 + a1, s * w0);
+                }
+            }
+        }
+        // the warps' column sums to one atomic per column
+#pragma unroll
+        for (int q = 0; q < 4; ++q) s_col[tid >> 5][lane + 32 * q] = acc[q];
+        __syncthreads();
+        if (tid < kFoldCols && cb + tid < C) {
+            unsigned long long v = 0;
+#pragma unroll
+            for (int w = 0; w < 8; ++w) v += s_col[w][tid];
+            atomicAdd(hc + cb + tid, v);
+        }
+        __syncthreads();
+    }
+    if (d3) return;
+    i0 = __reduce_add_sync(0xffffffffu, i0);
+    i1 = __reduce_add_sync(0xffffffffu, i1);
+    if (lane == 0) {
+        atomicAdd(&A.ctl[8], i0);
+        atomicAdd(&A.ctl[9], i1);
     }
 }
 
-// Layout choice: the one with fewer intervals (both streams' work grows with
-// the runs and intervals of the layout, and a layout's runs are at most its
-// intervals).
-__global__ void k_pick_layout(const int32_t *cnt, int32_t *sel) { sel[0] = cnt[1] < cnt[0] ? 1 : 0; }
+// Block d: the first index with each slice hash of axis d (an open-addressing
+// table in L2); an axis with more than 5/8 distinct hashes is no candidate.
+// Without a candidate (or with `enable` 0) the geometry is the grid's own and
+// the counted layout is picked; the kernels below then return at once.
+__global__ void __launch_bounds__(1024) k_fold_reps(FoldArgs A, int enable) {
+    pdl_trigger();
+    pdl_wait();
+    __shared__ int s_cnt;
+    const int d = blockIdx.x, tid = threadIdx.x;
+    const int64_t n = A.n[d], T = fold_slots(n);
+    int64_t off = 0, toff = 0;
+    for (int q = 0; q < d; ++q) {
+        off += A.n[q];
+        toff += fold_slots(A.n[q]);
+    }
+    int cand = 0;
+    if (enable) {
+        unsigned long long *tk = A.tkey + toff;
+        int32_t *tv = A.tval + toff;
+        if (tid == 0) s_cnt = 0;
+        for (int64_t a = tid; a < n; a += blockDim.x) {
+            unsigned long long h = A.hash[off + a];
+            h = h ? h : 1ull;  // 0 marks a free slot
+            int64_t sl = (int64_t)(h >> 20) & (T - 1);
+            for (int64_t probe = 0; probe < T; ++probe) {
+                const unsigned long long old = atomicCAS(tk + sl, 0ull, h);
+                if (old == 0ull || old == h) break;
+                sl = (sl + 1) & (T - 1);
+            }
+            atomicMax(tv + sl, 0x7fffffff - (int32_t)a);  // the first index has the largest value
+            A.rep[off + a] = (int32_t)sl;
+        }
+        __syncthreads();
+        int mine = 0;
+        for (int64_t a = tid; a < n; a += blockDim.x) {
+            const int32_t first = 0x7fffffff - __ldcg(tv + A.rep[off + a]);
+            A.rep[off + a] = first;
+            mine += first == (int32_t)a;
+        }
+        atomicAdd(&s_cnt, mine);
+        __syncthreads();
+        cand = (int64_t)s_cnt * 8 <= 5 * n;
+    }
+    if (tid == 0) {
+        A.ctl[4 + d] = cand;
+        if (cand) atomicAdd(&A.ctl[3], 1);
+    }
+    if (!fold_last_block(A.ctl)) return;
+    if (tid == 0 && atomicAdd(&A.ctl[3], 0) == 0) {
+        const int64_t m[3] = {A.n[0], A.n[1], A.n[2]};
+        const int none[3] = {0, 0, 0};
+        fold_write_geom(A, m, none);
+        pick_layout(A, A.ctl[8], A.ctl[9]);
+    }
+}
+
+// Every slice of a candidate axis compared with the first of its hash, point by
+// point; one that differs anywhere is marked and stays a class of its own.  A
+// warp takes rows of 128 columns (loads of four rows in flight).
+__global__ void __launch_bounds__(256) k_fold_verify(FoldArgs A) {
+    pdl_trigger();
+    pdl_wait();
+    if (A.ctl[3] == 0) return;  // uniform: nothing to merge
+    const int lane = threadIdx.x & 31;
+    const bool d3 = A.ndim == 3;
+    const int64_t C = A.n[A.ndim - 1], n1 = d3 ? A.n[1] : 1, R = A.n[0] * n1;
+    const int32_t *rep0 = A.rep, *rep1 = A.rep + A.n[0], *repc = d3 ? rep1 + A.n[1] : rep1;
+    int32_t *bad0 = A.bad, *bad1 = A.bad + A.n[0], *badc = d3 ? bad1 + A.n[1] : bad1;
+    const bool f0 = A.ctl[4], f1 = d3 && A.ctl[5], fc = A.ctl[4 + A.ndim - 1];
+    const int64_t ncb = (C + kFoldCols - 1) / kFoldCols, nrb = (R + kFoldRows - 1) / kFoldRows;
+    const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
+    for (int64_t t = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); t < ncb * nrb; t += nw) {
+        const int64_t c0 = (t % ncb) * kFoldCols + lane, r0 = (t / ncb) * kFoldRows;
+        int32_t rc[4];
+        bool bad[4] = {false, false, false, false};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int64_t c = c0 + 32 * q;
+            rc[q] = fc && c < C ? repc[c] : (int32_t)c;
+        }
+#pragma unroll 4
+        for (int u = 0; u < kFoldRows; ++u) {
+            const int64_t r = r0 + u;
+            if (r >= R) break;
+            const int64_t a0 = r / n1, a1 = r - a0 * n1;
+            const int64_t q0 = f0 ? rep0[a0] : a0, q1 = f1 ? rep1[a1] : a1;
+            bool b0 = false, b1 = false;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int64_t c = c0 + 32 * q;
+                if (c >= C) continue;
+                const int32_t b = A.bins[r * C + c];
+                if (q0 != a0) b0 |= A.bins[(q0 * n1 + a1) * C + c] != b;
+                if (q1 != a1) b1 |= A.bins[(a0 * n1 + q1) * C + c] != b;
+                if (rc[q] != (int32_t)c) bad[q] |= A.bins[r * C + rc[q]] != b;
+            }
+            if (b0) bad0[a0] = 1;
+            if (b1) bad1[a1] = 1;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (bad[q]) badc[c0 + 32 * q] = 1;
+    }
+}
+
+// Block d numbers the classes of axis d in index order and lists their members
+// (CSR, ascending, so that the merged factors are summed in a fixed order);
+// the last block writes the merged geometry.  Shared memory: class cursors
+// (fold_cap(n) ints), then the class of every index (16 bits: at most 20480).
+__global__ void __launch_bounds__(1024) k_fold_number(FoldArgs A) {
+    pdl_trigger();
+    pdl_wait();
+    if (A.ctl[3] == 0) return;  // uniform: nothing to merge
+    extern __shared__ int32_t s_cur[];
+    __shared__ int32_t s_w[32];
+    const int d = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    int64_t off = 0, soff = 0;
+    for (int q = 0; q < d; ++q) {
+        off += A.n[q];
+        soff += A.n[q] + 1;
+    }
+    const int64_t n = A.n[d], cap = fold_cap(n);
+    uint16_t *s_cls = reinterpret_cast<uint16_t *>(s_cur + cap);
+    const int32_t *rep = A.rep + off, *bad = A.bad + off;
+    int32_t *start = A.start + soff, *mem = A.members + off;
+    int32_t base = 0;
+    if (A.ctl[4 + d]) {  // uniform
+        for (int64_t a0 = 0; a0 < n; a0 += blockDim.x) {
+            const int64_t a = a0 + tid;
+            const bool head = a < n && (rep[a] == (int32_t)a || bad[a]);
+            const unsigned bal = __ballot_sync(0xffffffffu, head);
+            if (lane == 0) s_w[warp] = __popc(bal);
+            __syncthreads();
+            int32_t before = base, total = 0;
+            for (int w = 0; w < 32; ++w) {
+                if (w < warp) before += s_w[w];
+                total += s_w[w];
+            }
+            if (head) s_cls[a] = (uint16_t)(before + __popc(bal & ((1u << lane) - 1u)));
+            base += total;
+            __syncthreads();
+        }
+    }
+    const bool fold = base > 0 && base <= cap;  // (otherwise too many differ)
+    if (fold) {
+        for (int64_t c = tid; c < base; c += blockDim.x) s_cur[c] = 0;
+        __syncthreads();
+        for (int64_t a = tid; a < n; a += blockDim.x) {
+            // (a head's entry is only read, the others' only written here)
+            if (rep[a] != (int32_t)a && !bad[a]) s_cls[a] = s_cls[rep[a]];
+            atomicAdd(&s_cur[s_cls[a]], 1);
+        }
+        __syncthreads();
+        if (warp == 0) {
+            // offsets, then the members in index order (one warp: equal classes ranked by lane)
+            int32_t run = 0;
+            for (int64_t c0 = 0; c0 < base; c0 += 32) {
+                const int64_t c = c0 + lane;
+                const int32_t v = c < base ? s_cur[c] : 0;
+                int32_t x = v;
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int32_t t = __shfl_up_sync(0xffffffffu, x, o);
+                    if (lane >= o) x += t;
+                }
+                if (c < base) {
+                    s_cur[c] = run + x - v;
+                    start[c] = run + x - v;
+                }
+                run += __shfl_sync(0xffffffffu, x, 31);
+            }
+            if (lane == 0) start[base] = run;
+            __syncwarp();
+            for (int64_t a0 = 0; a0 < n; a0 += 32) {
+                const int64_t a = a0 + lane;
+                const int32_t cls = a < n ? (int32_t)s_cls[a] : -1 - lane;
+                const unsigned peers = __match_any_sync(0xffffffffu, cls);
+                const unsigned below = peers & ((1u << lane) - 1u);
+                int32_t pos = 0;
+                if (a < n) pos = s_cur[cls] + __popc(below);
+                __syncwarp();
+                if (a < n) {
+                    mem[pos] = (int32_t)a;
+                    if (below == 0) s_cur[cls] += __popc(peers);
+                }
+                __syncwarp();
+            }
+        }
+        __syncthreads();
+        for (int64_t c = tid; c < base; c += blockDim.x) mem[s_cur[c] - 1] |= kFoldLast;  // cursors end at the next class
+    }
+    if (tid == 0) A.ctl[10 + d] = fold ? base : 0;
+    if (!fold_last_block(A.ctl + 1)) return;
+    if (tid == 0) {
+        int64_t m[3] = {A.n[0], A.n[1], A.n[2]};
+        int folded[3] = {0, 0, 0};
+        int any = 0;
+        for (int q = 0; q < A.ndim; ++q) {
+            const int32_t v = __ldcg(A.ctl + 10 + q);
+            if (v) {
+                m[q] = v;
+                folded[q] = any = 1;
+            }
+        }
+        fold_write_geom(A, m, folded);
+        if (!any) pick_layout(A, A.ctl[8], A.ctl[9]);
+    }
+}
+
+// The merged bins, when an axis is folded, and on 2-D grids the intervals of
+// both layouts of the merged grid; the last block picks the layout.
+__global__ void __launch_bounds__(256) k_fold_bins(FoldArgs A) {
+    pdl_trigger();
+    pdl_wait();
+    const FoldGeom F = *A.fold;
+    if (!F.any) return;
+    const uint32_t m1 = (uint32_t)(A.ndim == 3 ? F.n[1] : 1), mc = (uint32_t)F.n[A.ndim - 1];
+    const uint32_t n1 = (uint32_t)(A.ndim == 3 ? A.n[1] : 1), nc = (uint32_t)A.n[A.ndim - 1];
+    const int dc = A.ndim - 1;
+    // first member of a class (the slice that stands for it)
+    const int32_t *mem0 = A.members, *st0 = A.start;
+    const int32_t *mem1 = A.members + A.n[0], *st1 = A.start + A.n[0] + 1;
+    const int32_t *memc = A.ndim == 3 ? mem1 + A.n[1] : mem1, *stc = A.ndim == 3 ? st1 + A.n[1] + 1 : st1;
+    auto at = [&](uint32_t a0, uint32_t a1, uint32_t c) -> int32_t {
+        const int64_t b0 = F.folded[0] ? mem0[st0[a0]] & (kFoldLast - 1) : (int32_t)a0;
+        const int64_t b1 = A.ndim == 3 && F.folded[1] ? mem1[st1[a1]] & (kFoldLast - 1) : (int32_t)a1;
+        const int64_t bc = F.folded[dc] ? memc[stc[c]] & (kFoldLast - 1) : (int32_t)c;
+        return A.bins[(b0 * n1 + b1) * nc + bc];
+    };
+    int32_t c0 = 0, c1 = 0;
+    const uint32_t p0 = (uint32_t)F.part_rows[0], p1 = (uint32_t)F.part_rows[1];
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < F.N; i += (int64_t)gridDim.x * blockDim.x) {
+        const uint32_t r = (uint32_t)i / mc, c = (uint32_t)i - r * mc;
+        const uint32_t a0 = r / m1, a1 = r - a0 * m1;
+        const int32_t b = at(a0, a1, c);
+        A.out_bins[i] = b;
+        if (A.ndim == 2) {
+            // layout 0 gathers axis 1, layout 1 axis 0
+            c0 += c % p0 == 0 || b != at(a0, 0, c - 1);
+            c1 += a0 % p1 == 0 || b != at(a0 - 1, 0, c);
+        }
+    }
+    if (A.ndim == 2) {
+        c0 = __reduce_add_sync(0xffffffffu, c0);
+        c1 = __reduce_add_sync(0xffffffffu, c1);
+        if ((threadIdx.x & 31) == 0) {
+            atomicAdd(&A.ctl[13], c0);
+            atomicAdd(&A.ctl[14], c1);
+        }
+    }
+    if (!fold_last_block(A.ctl + 2)) return;
+    if (threadIdx.x == 0) pick_layout(A, atomicAdd(&A.ctl[13], 0), atomicAdd(&A.ctl[14], 0));
+}
+
+// The bins the layout is built from: the merged ones where an axis is folded.
+struct LayBins {
+    const int32_t *full, *merged;
+    __device__ __forceinline__ const int32_t *get(const FoldGeom *f) const { return f->any ? merged : full; }
+};
 
 // Sort keys of the chosen layout: key = part of the gathered index * B + bin,
 // in the layout's flat order.  bins is viewed as an [R][C] matrix (C = the
 // last axis); layout 1 (2-D) walks its transpose.  32 x 32 tiles go through
 // shared memory so that reads and writes are coalesced either way.
-__global__ void k_layout_keys(const int32_t *__restrict__ bins, int64_t R, int64_t C, int B, LaySel L,
-                              int32_t *__restrict__ keys, const int32_t *gate) {
+__global__ void k_layout_keys(LayBins bin_src, int ndim, int B, LaySel L, int32_t *__restrict__ keys,
+                              const int32_t *gate) {
+    pdl_trigger();
+    pdl_wait();
     if (gated_off(gate)) return;
+    const int32_t *bins = bin_src.get(L.fold);
+    const int64_t C = L.fold->n[ndim - 1], R = L.fold->N / C;
     __shared__ int32_t t[32][33];
     const bool tr = L.sel[0] != 0;  // uniform over the grid
     const LayGeom G = L.get();
     const int64_t cb = (int64_t)blockIdx.x * 32;
+    if (cb >= C) return;
     for (int64_t rb = (int64_t)blockIdx.y * 32; rb < R; rb += (int64_t)gridDim.y * 32) {
         for (int yy = threadIdx.y; yy < 32; yy += blockDim.y) {
             const int64_t r = rb + yy, c = cb + threadIdx.x;
@@ -639,8 +1054,11 @@ __global__ void k_layout_keys(const int32_t *__restrict__ bins, int64_t R, int64
 // caller asked for one of them.  The record stream is then chosen at once
 // (sel[1] = 2, before the rest of the layout is built); otherwise the choice
 // waits for the run counts (sel[1] = -1 meanwhile) and is one of the others.
-__global__ void k_need_keys(const int32_t *n_rec, const int32_t *n_iv, int64_t N, int nf, int force,
+__global__ void k_need_keys(const int32_t *n_rec, const int32_t *n_iv, const FoldGeom *fold, int nf, int force,
                             int force_keys, int32_t *sel, int32_t *n_runs) {
+    pdl_trigger();
+    pdl_wait();
+    const int64_t N = fold->N;
     const int64_t c_iv = 19 * (int64_t)n_iv[0];
     const int64_t c_rec = (16 + 6 * nf) * (int64_t)n_rec[0] + 6 * ((int64_t)n_iv[0] + 2 * (int64_t)n_rec[0]);
     const int need = force_keys || force == 0 || force == 1 || (force < 0 && !(c_rec < 4 * N && c_rec <= c_iv));
@@ -659,8 +1077,12 @@ __global__ void k_need_keys(const int32_t *n_rec, const int32_t *n_iv, int64_t N
 // interval count).  After the key sort: the point or the
 // interval stream, whichever costs less (unless forced), when the record
 // stream was not chosen before it.
-__global__ void k_pick_stream(const int32_t *n_runs, const int32_t *n_iv, int64_t N, int force, int32_t *sel) {
+__global__ void k_pick_stream(const int32_t *n_runs, const int32_t *n_iv, const FoldGeom *fold, int force,
+                              int32_t *sel) {
+    pdl_trigger();
+    pdl_wait();
     if (sel[4] == 0) return;  // the record stream, chosen before the key sort
+    const int64_t N = fold->N;
     const int64_t c_pt = 4 * N + 20 * (int64_t)n_runs[0];
     const int64_t c_iv = 19 * (int64_t)n_iv[0];
     sel[1] = (force == 0 || force == 1) ? force : (c_iv < c_pt ? 1 : 0);
@@ -670,8 +1092,11 @@ __global__ void k_pick_stream(const int32_t *n_runs, const int32_t *n_iv, int64_
 // equal keys inside a step are ranked by lane with __match_any_sync.
 __global__ void k_sort_scatter(const int32_t *__restrict__ keys, int64_t N, int Bk, const int32_t *gate,
                                const int32_t *__restrict__ starts, int64_t n_tiles,
-                               int32_t *__restrict__ perm) {
+                               int32_t *__restrict__ perm, const FoldGeom *fold) {
+    pdl_trigger();
+    pdl_wait();
     if (gated_off(gate)) return;
+    if (fold) N = fold->N;
     extern __shared__ int32_t s_cnt[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     int32_t *cnt = s_cnt + warp * Bk;
@@ -733,6 +1158,8 @@ __device__ __forceinline__ T block_excl_scan(T v, T *s_warp, T &total) {
 template <typename T>
 __global__ void k_scan_blocks(const T *__restrict__ in, T *__restrict__ out, int64_t L, T *__restrict__ block_sums,
                               const int32_t *gate) {
+    pdl_trigger();
+    pdl_wait();
     if (gated_off(gate)) return;
     __shared__ T s_warp[32];
     const int64_t base = (int64_t)blockIdx.x * kScanBlock + (int64_t)threadIdx.x * kScanItems;
@@ -753,11 +1180,22 @@ __global__ void k_scan_blocks(const T *__restrict__ in, T *__restrict__ out, int
 
 template <typename T>
 __global__ void k_scan_add(T *__restrict__ out, int64_t L, const T *__restrict__ block_off, const int32_t *gate) {
+    pdl_trigger();
+    pdl_wait();
     if (gated_off(gate)) return;
     const int64_t base = (int64_t)blockIdx.x * kScanBlock;
     const T add = block_off[blockIdx.x];
-    for (int j = threadIdx.x; j < kScanBlock; j += blockDim.x)
-        if (base + j < L) out[base + j] += add;
+    T v[kScanItems];  // every load in flight together
+#pragma unroll
+    for (int j = 0; j < kScanItems; ++j) {
+        const int64_t e = base + j * kScanThreads + threadIdx.x;
+        v[j] = e < L ? out[e] : T(0);
+    }
+#pragma unroll
+    for (int j = 0; j < kScanItems; ++j) {
+        const int64_t e = base + j * kScanThreads + threadIdx.x;
+        if (e < L) out[e] = v[j] + add;
+    }
 }
 
 // ---- runs, intervals and chunks of the segmented histogram ------------------
@@ -767,9 +1205,12 @@ __global__ void k_scan_add(T *__restrict__ out, int64_t L, const T *__restrict__
 // along one line of the grid).  One flag word per sorted point holds both
 // start flags (run: bit 0, interval: bit 32), so a single 64-bit scan numbers
 // runs (low half) and intervals (high half).
-__global__ void k_layout_flags(const int32_t *__restrict__ perm, const int32_t *__restrict__ keys, int64_t N,
-                               LaySel L, unsigned long long *__restrict__ flags, const int32_t *gate) {
+__global__ void k_layout_flags(const int32_t *__restrict__ perm, const int32_t *__restrict__ keys, LaySel L,
+                               unsigned long long *__restrict__ flags, const int32_t *gate) {
+    pdl_trigger();
+    pdl_wait();
     if (gated_off(gate)) return;
+    const int64_t N = L.fold->N;
     const int64_t n_last = L.get().n_last;
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < N;
          t += (int64_t)gridDim.x * blockDim.x) {
@@ -791,14 +1232,17 @@ __global__ void k_layout_flags(const int32_t *__restrict__ perm, const int32_t *
 // order instead) | run-end / key-end flags (bits 30, 31); the interval words
 // (first row << shift; (last row + 1) << shift | the flags of its last point)
 // and each interval's rest index.
-__global__ void k_layout_build(const int32_t *__restrict__ perm, const int32_t *__restrict__ keys, int64_t N,
-                               LaySel L, int shift, const unsigned long long *__restrict__ flags,
+__global__ void k_layout_build(const int32_t *__restrict__ perm, const int32_t *__restrict__ keys, LaySel L,
+                               int shift, const unsigned long long *__restrict__ flags,
                                const unsigned long long *__restrict__ excl, int32_t *__restrict__ run_start,
                                int32_t *__restrict__ run_rest, int32_t *__restrict__ run_bin,
                                uint32_t *__restrict__ hpt, int32_t *__restrict__ n_runs, uint2 *__restrict__ ipt,
                                int32_t *__restrict__ iv_rest, int32_t *__restrict__ n_iv, const int32_t *gate) {
+    pdl_trigger();
+    pdl_wait();
     if (gated_off(gate)) return;
     const LayGeom G = L.get();
+    const int64_t N = L.fold->N;
     const uint32_t rmask = (1u << kRowBits) - 1u;
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < N;
          t += (int64_t)gridDim.x * blockDim.x) {
@@ -858,10 +1302,13 @@ __device__ __forceinline__ uint32_t rest_code(int32_t rest, int ndim, int64_t n1
 }
 __global__ void k_layout_encode(const int32_t *__restrict__ run_start, const int32_t *__restrict__ run_rest,
                                 const int32_t *__restrict__ n_runs_p, const int32_t *__restrict__ iv_rest,
-                                const int32_t *__restrict__ n_iv_p, int ndim, int64_t n1, int shift,
+                                const int32_t *__restrict__ n_iv_p, int ndim, const FoldGeom *fold, int shift,
                                 uint32_t *__restrict__ hpt, uint2 *__restrict__ ipt, int run_ahead,
                                 const int32_t *gate) {
+    pdl_trigger();
+    pdl_wait();
     if (gated_off(gate)) return;
+    const int64_t n1 = ndim == 3 ? fold->n[1] : 1;
     const int32_t n_runs = n_runs_p[0], n_iv = n_iv_p[0];
     const int32_t n = n_runs > n_iv ? n_runs : n_iv;
     for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < n; x += (int64_t)gridDim.x * blockDim.x) {
@@ -871,18 +1318,32 @@ __global__ void k_layout_encode(const int32_t *__restrict__ run_start, const int
     }
 }
 
+// Start of chunk cc of C over n elements: n cc / C, rounded down to whole
+// chunks of `least` elements where n / C is less (some chunks are then empty,
+// spread evenly): a chunk's cut keys or groups cost partial rows, which short
+// chunks would make the larger part of the work.
+constexpr int kChunkPoints = 256, kChunkRecords = 24;
+__device__ __forceinline__ int64_t chunk_at(int64_t n, int64_t cc, int64_t C, int64_t least) {
+    int64_t t = n * cc / C;
+    if (n < C * least && cc < C) t = t / least * least;
+    return t;
+}
+
 // Chunks, C per part: chunk c of part p starts at the first run whose first
 // point is >= lo_p + (hi_p - lo_p) c / C, [lo_p, hi_p) being the part's
 // points; chunk_iv[c] is its first interval (chunks start on runs, which
 // start intervals).  Entry P C is the end.
 __global__ void k_chunks(const int32_t *__restrict__ run_start, const int32_t *__restrict__ n_runs_p,
                          const int32_t *__restrict__ koff, int B, LaySel L, int C,
-                         const unsigned long long *__restrict__ excl, int64_t N, const int32_t *__restrict__ n_iv_p,
+                         const unsigned long long *__restrict__ excl, const int32_t *__restrict__ n_iv_p,
                          int32_t *__restrict__ chunk_pt, int32_t *__restrict__ chunk_run,
                          int32_t *__restrict__ chunk_iv, const int32_t *gate) {
+    pdl_trigger();
+    pdl_wait();
     if (gated_off(gate)) return;
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     const int P = L.get().P;
+    const int64_t N = L.fold->N;
     if (c > P * C) return;
     const int32_t n_runs = n_runs_p[0];
     int32_t r;
@@ -891,7 +1352,7 @@ __global__ void k_chunks(const int32_t *__restrict__ run_start, const int32_t *_
     } else {
         const int p = c / C, cc = c - p * C;
         const int64_t lo = koff[p * B], hi = koff[(p + 1) * B];
-        const int64_t target = lo + ((hi - lo) * (int64_t)cc) / C;
+        const int64_t target = lo + chunk_at(hi - lo, cc, C, kChunkPoints);
         int32_t a = 0, b = n_runs;  // first r in [0, n_runs] with run_start[r] >= target
         while (a < b) {
             int32_t mid = (a + b) >> 1;
@@ -907,8 +1368,11 @@ __global__ void k_chunks(const int32_t *__restrict__ run_start, const int32_t *_
 
 // Key offsets of a counting sort: koff[b] = starts[b * n_tiles], koff[Bk] = N.
 __global__ void k_koff(const int32_t *__restrict__ starts, int64_t n_tiles, int Bk, int64_t N,
-                       int32_t *__restrict__ koff, const int32_t *gate) {
+                       int32_t *__restrict__ koff, const int32_t *gate, const FoldGeom *fold) {
+    pdl_trigger();
+    pdl_wait();
     if (gated_off(gate)) return;
+    if (fold) N = fold->N;
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b < Bk) koff[b] = starts[(int64_t)b * n_tiles];
     else if (b == Bk) koff[b] = (int32_t)N;
@@ -916,6 +1380,8 @@ __global__ void k_koff(const int32_t *__restrict__ starts, int64_t n_tiles, int 
 
 __global__ void k_chunk_bins(const int32_t *__restrict__ chunk_run, const int32_t *__restrict__ run_bin, LaySel L,
                              int C, int32_t *__restrict__ chunk_bin, const int32_t *gate) {
+    pdl_trigger();
+    pdl_wait();
     if (gated_off(gate)) return;
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= L.get().P * C) return;
@@ -936,6 +1402,8 @@ __device__ __forceinline__ int chunk_holding(const int32_t *chunk_pt, int n, int
 }
 __global__ void k_key_chunks(const int32_t *__restrict__ koff, LaySel L, int B, const int32_t *__restrict__ chunk_pt,
                              int C, int2 *__restrict__ out, const int32_t *gate) {
+    pdl_trigger();
+    pdl_wait();
     if (gated_off(gate)) return;
     const int key = blockIdx.x * blockDim.x + threadIdx.x;
     const int P = L.get().P;
@@ -978,22 +1446,24 @@ constexpr uint32_t kRecEnd = 1u << 31;  // last record of its group
 // inside the part): bin 8q + j holds rows [B_j, B_j+1) when the bins rise
 // along the line, [B_j+1, B_j) when they fall.
 struct RecGeom {
-    int64_t R, C;
     int GB;       // groups of kRecBins bins per part
     int64_t NL;   // line stride of the count matrix (the most lines of either layout)
     int64_t cap;  // slots per segment (the most part rows)
-    int ndim;
-    int64_t n1;   // 3-D rest code: line = a0 n1 + a1 -> a0 | a1 << 15
+    int ndim;     // 3-D rest code: line = a0 n1 + a1 -> a0 | a1 << 15
 };
 
 constexpr int kWalkWarps = 8;  // segments (warps) per block of the record walk
-__global__ void __launch_bounds__(kWalkWarps * 32) k_rec_walk(const int32_t *__restrict__ bins, RecGeom Q, LaySel L,
+__global__ void __launch_bounds__(kWalkWarps * 32) k_rec_walk(LayBins bin_src, RecGeom Q, LaySel L,
                                                               int32_t *__restrict__ cnt, int32_t *__restrict__ n_iv,
                                                               uint4 *__restrict__ tmp, int32_t *__restrict__ seg_n) {
+    pdl_trigger();
+    pdl_wait();
     extern __shared__ int32_t s_rank[];  // [warps][GB]: records so far of each group of the part
     const bool tr = L.sel[0] != 0;
     const LayGeom G = L.get();
-    const int64_t n_lines = tr ? Q.C : Q.R;
+    const int32_t *bins = bin_src.get(L.fold);
+    const int64_t C = L.fold->n[Q.ndim - 1];
+    const int64_t n_lines = tr ? C : L.fold->N / C;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // one warp per segment; the warps of a block walk consecutive lines of one part
     const int64_t seg = (int64_t)blockIdx.x * kWalkWarps + warp;
@@ -1004,8 +1474,8 @@ __global__ void __launch_bounds__(kWalkWarps * 32) k_rec_walk(const int32_t *__r
     int32_t *rank = s_rank + warp * Q.GB;
     for (int q = lane; q < Q.GB; q += 32) rank[q] = 0;
     __syncwarp();
-    const int64_t stride = tr ? Q.C : 1;
-    const int32_t *src = bins + (tr ? line : line * Q.C);
+    const int64_t stride = tr ? C : 1;
+    const int32_t *src = bins + (tr ? line : line * C);
     uint4 *slot = tmp + 2 * seg * Q.cap;
 
     // record state, the same in every lane; lane j < 8 holds st_j, the first
@@ -1100,13 +1570,15 @@ __global__ void __launch_bounds__(kWalkWarps * 32) k_rec_walk(const int32_t *__r
 // the record kRunAhead places later, group, 0), and its rest index (the
 // line).  One warp per segment.
 __global__ void k_rec_scatter(const uint4 *__restrict__ tmp, const int32_t *__restrict__ seg_n, RecGeom Q,
-                              LaySel L, const int32_t *__restrict__ starts, const int32_t *__restrict__ goff,
-                              const int32_t *__restrict__ n_rec_p, uint4 *__restrict__ rec,
-                              int32_t *__restrict__ rec_rest) {
+                              LaySel L, const int32_t *__restrict__ starts, const int32_t *__restrict__ counts,
+                              int64_t Lr, int n_groups, uint4 *__restrict__ rec, int32_t *__restrict__ rec_rest) {
+    pdl_trigger();
+    pdl_wait();
     const bool tr = L.sel[0] != 0;
     const LayGeom G = L.get();
-    const int64_t n_seg = (int64_t)G.P * (tr ? Q.C : Q.R);
-    const int32_t n_rec = n_rec_p[0];
+    const int64_t C = L.fold->n[Q.ndim - 1], n1 = Q.ndim == 3 ? L.fold->n[1] : 1;
+    const int64_t n_seg = (int64_t)G.P * (tr ? C : L.fold->N / C);
+    const int32_t n_rec = starts[Lr - 1] + counts[Lr - 1];
     const int lane = threadIdx.x & 31;
     const int64_t w0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -1123,76 +1595,68 @@ __global__ void k_rec_scatter(const uint4 *__restrict__ tmp, const int32_t *__re
             const int64_t pos = (int64_t)starts[(int64_t)g * Q.NL + line] + v.w;
             rec[2 * pos] = u;
             uint32_t *w1 = reinterpret_cast<uint32_t *>(rec + 2 * pos + 1);
-            w1[0] = v.x | (pos + 1 == goff[g + 1] ? kRecEnd : 0u);
+            const int64_t g_end = (int)g + 1 < n_groups ? starts[(int64_t)(g + 1) * Q.NL] : n_rec;
+            w1[0] = v.x | (pos + 1 == g_end ? kRecEnd : 0u);
             if (pos + kRunAhead >= n_rec) w1[1] = 0u;
             w1[2] = g;
             w1[3] = 0u;
             const uint32_t code =
-                Q.ndim == 3 ? (uint32_t)(line / Q.n1) | ((uint32_t)(line % Q.n1) << 15) : (uint32_t)line;
+                Q.ndim == 3 ? (uint32_t)(line / n1) | ((uint32_t)(line % n1) << 15) : (uint32_t)line;
             if (pos >= kRunAhead) reinterpret_cast<uint32_t *>(rec + 2 * (pos - kRunAhead) + 1)[1] = code;
             rec_rest[pos] = (int32_t)line;
         }
     }
 }
 
-// First record of every group (n_groups + 2 entries: the last two = the
-// record count) from the scanned (group, line) counts.
-__global__ void k_rec_goff(const int32_t *__restrict__ starts, const int32_t *__restrict__ counts, int64_t Lr,
-                           int64_t NL, int n_groups, int32_t *__restrict__ goff, int32_t *__restrict__ n_rec) {
-    const int32_t total = starts[Lr - 1] + counts[Lr - 1];
-    for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < n_groups + 2; g += gridDim.x * blockDim.x)
-        goff[g] = g < n_groups ? starts[g * NL] : total;
-    if (blockIdx.x == 0 && threadIdx.x == 0) n_rec[0] = total;
-}
-
-// Record chunks, C per part (equal record counts; records cost alike):
-// chunk c of part p starts at record lo_p + (hi_p - lo_p) c / C; its first and
-// last groups (-1 when empty); entry P C is the end.  A group may be cut by
-// chunk bounds, like a key of the point stream.
-__global__ void k_rec_chunks(const int32_t *__restrict__ goff, const int32_t *__restrict__ n_rec_p, int GB,
-                             LaySel L, int C, const uint4 *__restrict__ rec, int32_t *__restrict__ chunk_rec,
-                             int32_t *__restrict__ chunk_grp) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
+// The record stream's tables from the scanned (group, line) counts, one launch:
+// the first record of every group (n_groups + 2 entries: the last two = the
+// record count); the record chunks, C per part (equal record counts; records
+// cost alike): chunk c of part p starts at record lo_p + chunk_at(.., c), with
+// its first and last groups (-1 when empty), entry P C is the end -- a group may
+// be cut by chunk bounds, like a key of the point stream; and the first and
+// last chunk holding records of each group (-1, -1 for an empty group).
+__global__ void k_rec_tables(const int32_t *__restrict__ starts, const int32_t *__restrict__ counts, int64_t Lr,
+                             int64_t NL, int n_groups, int GB, LaySel L, int C, const uint4 *__restrict__ rec,
+                             int32_t *__restrict__ goff, int32_t *__restrict__ n_rec, int32_t *__restrict__ chunk_rec,
+                             int32_t *__restrict__ chunk_grp, int2 *__restrict__ gch) {
+    pdl_trigger();
+    pdl_wait();
     const int P = L.get().P;
-    if (c > P * C) return;
-    int32_t r;
-    if (c == P * C) {
-        r = n_rec_p[0];
-    } else {
+    const int32_t total = starts[Lr - 1] + counts[Lr - 1];
+    auto first = [&](int g) -> int32_t { return g < n_groups ? starts[g * NL] : total; };
+    auto bound = [&](int c) -> int32_t {  // first record of chunk c
+        if (c >= P * C) return total;
         const int p = c / C, cc = c - p * C;
-        const int64_t lo = goff[p * GB], hi = goff[(p + 1) * GB];
-        r = (int32_t)(lo + ((hi - lo) * (int64_t)cc) / C);
-    }
-    chunk_rec[c] = r;
-    if (c < P * C) {
-        const int p = c / C, cc = c - p * C;
-        const int64_t lo = goff[p * GB], hi = goff[(p + 1) * GB];
-        const int32_t r1 = (int32_t)(lo + ((hi - lo) * (int64_t)(cc + 1)) / C);
+        const int64_t lo = first(p * GB), hi = first((p + 1) * GB);
+        return (int32_t)(lo + chunk_at(hi - lo, cc, C, kChunkRecords));
+    };
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
+    if (i == 0) n_rec[0] = total;
+    for (int g = i; g < n_groups + 2; g += step) goff[g] = first(g);
+    for (int c = i; c <= P * C; c += step) {
+        const int32_t r = bound(c);
+        chunk_rec[c] = r;
+        if (c == P * C) break;
+        const int32_t r1 = bound(c + 1);
         chunk_grp[2 * c] = r1 > r ? (int32_t)rec[2 * (int64_t)r + 1].z : -1;
         chunk_grp[2 * c + 1] = r1 > r ? (int32_t)rec[2 * (int64_t)(r1 - 1) + 1].z : -1;
     }
-}
-
-// First and last chunk holding records of each group (-1, -1 for an empty group).
-__global__ void k_rec_group_chunks(const int32_t *__restrict__ goff, int n_groups,
-                                   const int32_t *__restrict__ chunk_rec, LaySel L, int C, int2 *__restrict__ out) {
-    const int gr = blockIdx.x * blockDim.x + threadIdx.x;
-    if (gr >= n_groups) return;
-    const int n_chunks = L.get().P * C;  // the chosen layout's chunks
-    const int32_t o0 = goff[gr], o1 = goff[gr + 1];
-    if (o0 == o1) {
-        out[gr] = make_int2(-1, -1);
-        return;
-    }
-    auto holding = [&](int32_t t) {  // last c in [0, n_chunks) with chunk_rec[c] <= t
-        int lo = 0, hi = n_chunks;
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (chunk_rec[mid] <= t) lo = mid; else hi = mid;
+    for (int g = i; g < n_groups; g += step) {
+        const int32_t o0 = first(g), o1 = first(g + 1);
+        if (o0 == o1) {
+            gch[g] = make_int2(-1, -1);
+            continue;
         }
-        return lo;
-    };
-    out[gr] = make_int2(holding(o0), holding(o1 - 1));
+        auto holding = [&](int32_t t) {  // last chunk of the group's part that starts at or before t
+            int lo = g / GB * C, hi = lo + C;
+            while (hi - lo > 1) {
+                const int mid = (lo + hi) >> 1;
+                if (bound(mid) <= t) lo = mid; else hi = mid;
+            }
+            return lo;
+        };
+        gch[g] = make_int2(holding(o0), holding(o1 - 1));
+    }
 }
 
 // ---- power tables -----------------------------------------------------------
@@ -1363,17 +1827,17 @@ static vup_status scan_exclusive(const T *in, T *out, int64_t L, T *scratch, cud
                                  const int32_t *gate = nullptr) {
     const int64_t nb = ceil_div64(L, kScanBlock);
     if (nb <= 1) {
-        k_scan_blocks<T><<<1, kScanThreads, 0, s>>>(in, out, L, nullptr, gate);
+        VUP_CHECK_CUDA(launch_pdl(k_scan_blocks<T>, dim3(1), dim3(kScanThreads), 0, s, in, out, L, nullptr, gate));
         VUP_CHECK_LAUNCH();
         return VUP_OK;
     }
     T *sums = scratch;
     T *sums_scan = scratch + nb + 32;
-    k_scan_blocks<T><<<(unsigned)nb, kScanThreads, 0, s>>>(in, out, L, sums, gate);
+    VUP_CHECK_CUDA(launch_pdl(k_scan_blocks<T>, dim3((unsigned)nb), dim3(kScanThreads), 0, s, in, out, L, sums, gate));
     VUP_CHECK_LAUNCH();
     vup_status st = scan_exclusive<T>(sums, sums_scan, nb, scratch + 2 * nb + 64, s, gate);
     if (st != VUP_OK) return st;
-    k_scan_add<T><<<(unsigned)nb, 256, 0, s>>>(out, L, sums_scan, gate);
+    VUP_CHECK_CUDA(launch_pdl(k_scan_add<T>, dim3((unsigned)nb), dim3(kScanThreads), 0, s, out, L, sums_scan, gate));
     VUP_CHECK_LAUNCH();
     return VUP_OK;
 }
@@ -1477,7 +1941,7 @@ static int sort_warps(int Bk) { return std::max(1, std::min(kSortWarps, 32768 / 
 // (Bk + 1 entries) when koff is not null.  `counts` must hold 2 Bk n_tiles + 8.
 static vup_status counting_sort(vup_grid g, const int32_t *keys, int Bk, int32_t *perm, int32_t *koff,
                                 int32_t *counts, int32_t *scratch, bool counts_ready, cudaStream_t s,
-                                const int32_t *gate = nullptr) {
+                                const int32_t *gate = nullptr, const FoldGeom *fold = nullptr) {
     const int64_t N = g->N;
     const int64_t n_tiles = ceil_div64(N, kSortTile);
     const int64_t L = (int64_t)Bk * n_tiles;
@@ -1490,15 +1954,15 @@ static vup_status counting_sort(vup_grid g, const int32_t *keys, int Bk, int32_t
         VUP_CHECK_CUDA(cudaFuncSetAttribute(k_sort_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     }
     if (!counts_ready) {
-        k_count<<<blocks, 32 * nw, smem, s>>>(keys, N, Bk, counts, n_tiles, gate);
+        VUP_CHECK_CUDA(launch_pdl(k_count, dim3(blocks), dim3(32 * nw), smem, s, keys, N, Bk, counts, n_tiles, gate, fold));
         VUP_CHECK_LAUNCH();
     }
     vup_status st = scan_exclusive(counts, starts, L, scratch, s, gate);
     if (st != VUP_OK) return st;
-    k_sort_scatter<<<blocks, 32 * nw, smem, s>>>(keys, N, Bk, gate, starts, n_tiles, perm);
+    VUP_CHECK_CUDA(launch_pdl(k_sort_scatter, dim3(blocks), dim3(32 * nw), smem, s, keys, N, Bk, gate, starts, n_tiles, perm, fold));
     VUP_CHECK_LAUNCH();
     if (koff) {
-        k_koff<<<(Bk + 1 + 255) / 256, 256, 0, s>>>(starts, n_tiles, Bk, N, koff, gate);
+        VUP_CHECK_CUDA(launch_pdl(k_koff, dim3((Bk + 1 + 255) / 256), dim3(256), 0, s, starts, n_tiles, Bk, N, koff, gate, fold));
         VUP_CHECK_LAUNCH();
     }
     return VUP_OK;
@@ -1607,12 +2071,53 @@ vup_status vup_launch_grid_finish(vup_grid g, cudaStream_t s) {
     return VUP_OK;
 }
 
+// The scratch of a layout build's equal-slice search: hashes and table keys
+// (64-bit), table values, marks and control words (32-bit).
+size_t vup_fold_scratch_bytes(const vup_grid_s *g) {
+    int64_t n = 0, t = 0;
+    for (int d = 0; d < g->ndim; ++d) {
+        n += g->n[d];
+        t += fold_slots(g->n[d]);
+    }
+    return sizeof(unsigned long long) * (size_t)(n + t) + sizeof(int32_t) * (size_t)(t + n + kFoldCtl);
+}
+
+static FoldArgs fold_args(vup_grid g) {
+    FoldArgs A{};
+    int64_t n = 0, t = 0;
+    for (int d = 0; d < 3; ++d) A.n[d] = d < g->ndim ? g->n[d] : 1;
+    for (int d = 0; d < g->ndim; ++d) {
+        n += g->n[d];
+        t += fold_slots(g->n[d]);
+    }
+    A.bins = g->bins;
+    A.ndim = g->ndim;
+    A.B = g->B;
+    for (int l = 0; l < 2; ++l) {
+        const auto &h = g->hl[l < g->n_layouts ? l : 0];
+        A.P[l] = h.P;
+        A.part_rows[l] = h.part_rows;
+    }
+    A.fold = g->fold;
+    A.hash = reinterpret_cast<unsigned long long *>(g->fold_scratch);
+    A.tkey = A.hash + n;
+    A.tval = reinterpret_cast<int32_t *>(A.tkey + t);
+    A.bad = A.tval + t;
+    A.ctl = A.bad + n;
+    A.rep = g->fold_rep;
+    A.start = g->fold_start;
+    A.members = g->fold_members;
+    A.out_bins = g->fold_bins;
+    A.sel = g->hist_sel;
+    return A;
+}
+
 // The histogram layout of a 2-D / 3-D grid (sorted point and interval
 // streams, chunks, the natural bin offsets) for the current bins.  Built on
 // first use after a model evaluation (the histogram, the bin offsets), so a
 // caller may run it on a second stream beside the density preparation.
 vup_status vup_build_layout(vup_grid g, cudaStream_t s, bool points_needed, cudaEvent_t records_done,
-                            cudaEvent_t layout_picked) {
+                            cudaEvent_t layout_picked, bool fold) {
     const int64_t N = g->N;
     const int B = g->B;
     // two timed parts: up to the record-stream decision, and the key-sorted streams
@@ -1629,21 +2134,31 @@ vup_status vup_build_layout(vup_grid g, cudaStream_t s, bool points_needed, cuda
         const int C = g->n_chunks;
         auto &HL = g->hl[0];
         LaySel L;
-        for (int l = 0; l < 2; ++l) {
-            const auto &h = g->hl[l < g->n_layouts ? l : 0];
-            L.g[l] = LayGeom{h.n_last, h.part_rows, h.P};
-        }
+        L.fold = g->fold;
         L.sel = g->hist_sel;
-        int32_t *iv_cnt = g->hist_sel + 2;
-        if (g->n_layouts > 1) {
-            // the layout with fewer intervals (counted without sorting)
-            VUP_CHECK_CUDA(cudaMemsetAsync(iv_cnt, 0, 2 * sizeof(int32_t), s));
-            k_iv_count<<<blocks, 256, 0, s>>>(g->bins, g->n[0], g->n[1], B, L, iv_cnt);
-            VUP_CHECK_LAUNCH();
-            k_pick_layout<<<1, 1, 0, s>>>(iv_cnt, g->hist_sel);
-            VUP_CHECK_LAUNCH();
+        {
+            // equal slices merged, then the layout with fewer intervals (counted without sorting)
+            const FoldArgs A = fold_args(g);
+            VUP_CHECK_CUDA(cudaMemsetAsync(g->fold_scratch, 0, g->fold_scratch_bytes, s));
+            const int64_t tasks = ceil_div64(A.n[g->ndim - 1], kFoldCols) *
+                                  ceil_div64(N / A.n[g->ndim - 1], kFoldRows);
+            const int tb = (int)std::min<int64_t>(ceil_div64(tasks, 8), (int64_t)vup_num_sms() * 8);
+            VUP_CHECK_CUDA(launch_pdl(k_fold_hash, dim3(tb), dim3(256), 0, s, A));
+            VUP_CHECK_CUDA(launch_pdl(k_fold_reps, dim3(g->ndim), dim3(1024), 0, s, A, fold ? 1 : 0));
             launches += 2;
+            if (fold) {
+                size_t sm = 0;
+                for (int d = 0; d < g->ndim; ++d)
+                    sm = std::max(sm, sizeof(int32_t) * (size_t)fold_cap(g->n[d]) + sizeof(uint16_t) * (size_t)g->n[d]);
+                if (sm > 48 * 1024)
+                    VUP_CHECK_CUDA(cudaFuncSetAttribute(k_fold_number, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+                VUP_CHECK_CUDA(launch_pdl(k_fold_verify, dim3(tb), dim3(256), 0, s, A));
+                VUP_CHECK_CUDA(launch_pdl(k_fold_number, dim3(g->ndim), dim3(1024), sm, s, A));
+                VUP_CHECK_CUDA(launch_pdl(k_fold_bins, dim3(blocks), dim3(256), 0, s, A));
+                launches += 3;
+            }
         }
+        const LayBins lb{g->bins, g->fold_bins};
         if (layout_picked) VUP_CHECK_CUDA(cudaEventRecord(layout_picked, s));
         const int rb = (int)std::min<int64_t>(ceil_div64(N, 256), (int64_t)vup_num_sms() * 8);
         const int64_t Cn = HL.n_last, Rn = N / Cn;  // bins as [R][C], C = the last axis
@@ -1677,41 +2192,28 @@ vup_status vup_build_layout(vup_grid g, cudaStream_t s, bool points_needed, cuda
             int32_t *rcnt = (int32_t *)g->rec_tmp.p, *rstart = rcnt + Lr, *seg_n = rcnt + 2 * Lr;
             uint4 *rslot = reinterpret_cast<uint4 *>(rcnt + ints);
             RecGeom Q;
-            Q.R = Rn;
-            Q.C = Cn;
             Q.GB = GB;
             Q.NL = NL;
             Q.cap = cap;
             Q.ndim = g->ndim;
-            Q.n1 = g->ndim == 3 ? g->n[1] : 1;
             VUP_CHECK_CUDA(cudaMemsetAsync(rcnt, 0, sizeof(int32_t) * (size_t)Lr, s));
             VUP_CHECK_CUDA(cudaMemsetAsync(HL.n_iv, 0, sizeof(int32_t), s));
             const size_t wsm = sizeof(int32_t) * (size_t)kWalkWarps * GB;
             if (wsm > 48 * 1024)
                 VUP_CHECK_CUDA(cudaFuncSetAttribute(k_rec_walk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wsm));
-            k_rec_walk<<<(unsigned)ceil_div64(walkers, kWalkWarps), kWalkWarps * 32, wsm, s>>>(g->bins, Q, L, rcnt,
-                                                                                             HL.n_iv, rslot, seg_n);
+            VUP_CHECK_CUDA(launch_pdl(k_rec_walk, dim3((unsigned)ceil_div64(walkers, kWalkWarps)), dim3(kWalkWarps * 32), wsm, s, lb, Q, L, rcnt,
+                                                                                             HL.n_iv, rslot, seg_n));
             VUP_CHECK_LAUNCH();
             if ((st = scan_exclusive(rcnt, rstart, Lr, scratch, s)) != VUP_OK) return st;
-            k_rec_goff<<<(n_groups + 2 + 255) / 256, 256, 0, s>>>(rstart, rcnt, Lr, NL, n_groups,
-                                                                  (int32_t *)HL.rec_goff.p, HL.n_rec);
+            VUP_CHECK_CUDA(launch_pdl(k_rec_scatter, dim3((unsigned)std::min<int64_t>(ceil_div64(walkers, 8), (int64_t)vup_num_sms() * 16)), dim3(256), 0, s, rslot, seg_n, Q, L, rstart, rcnt, Lr, n_groups, (uint4 *)HL.rec.p,
+                                 (int32_t *)HL.rec_rest.p));
             VUP_CHECK_LAUNCH();
-            k_rec_scatter<<<(unsigned)std::min<int64_t>(ceil_div64(walkers, 8), (int64_t)vup_num_sms() * 16), 256, 0,
-                            s>>>(rslot, seg_n, Q, L, rstart, (const int32_t *)HL.rec_goff.p, HL.n_rec,
-                                 (uint4 *)HL.rec.p, (int32_t *)HL.rec_rest.p);
-            VUP_CHECK_LAUNCH();
-            // chunks of records (the same count per part as the other streams' chunks / 4)
             const int Cr = g->n_chunks_rec;
-            k_rec_chunks<<<(P_sel * Cr + 1 + 127) / 128, 128, 0, s>>>((const int32_t *)HL.rec_goff.p, HL.n_rec, GB, L,
-                                                                      Cr, (const uint4 *)HL.rec.p, HL.rec_chunk,
-                                                                      HL.rec_chunk_grp);
+            VUP_CHECK_CUDA(launch_pdl(k_rec_tables, dim3((std::max(n_groups + 2, P_sel * Cr + 1) + 127) / 128), dim3(128), 0, s, rstart, rcnt, Lr, NL, n_groups, GB, L, Cr, (const uint4 *)HL.rec.p, (int32_t *)HL.rec_goff.p, HL.n_rec,
+                HL.rec_chunk, HL.rec_chunk_grp, (int2 *)HL.rec_gch.p));
             VUP_CHECK_LAUNCH();
-            k_rec_group_chunks<<<(n_groups + 127) / 128, 128, 0, s>>>((const int32_t *)HL.rec_goff.p, n_groups,
-                                                                       HL.rec_chunk, L, Cr,
-                                                                       (int2 *)HL.rec_gch.p);
-            VUP_CHECK_LAUNCH();
-            // walk, scan, first records, scatter, chunks, group chunks, gate
-            launches += 2 + scan_launches(Lr) + 2 + 2 + 1;
+            // walk, scan, scatter, tables, gate
+            launches += 1 + scan_launches(Lr) + 2 + 1;
         }
         // the key-sorted point and interval streams, unless the record stream is
         // cheaper than both (every kernel below then returns at once); the
@@ -1719,8 +2221,8 @@ vup_status vup_build_layout(vup_grid g, cudaStream_t s, bool points_needed, cuda
         // means -- and where the shared-memory kernels cannot run
         const int32_t *gate = g->hist_sel + 4;
         const bool force_keys = points_needed || !vup_hist_tile_fits(g);
-        k_need_keys<<<1, 1, 0, s>>>(HL.n_rec, HL.n_iv, N, g->ndim - 1, g->hist_force, force_keys ? 1 : 0,
-                                    g->hist_sel, HL.n_runs);
+        VUP_CHECK_CUDA(launch_pdl(k_need_keys, dim3(1), dim3(1), 0, s, HL.n_rec, HL.n_iv, g->fold, g->ndim - 1, g->hist_force, force_keys ? 1 : 0,
+                                    g->hist_sel, HL.n_runs));
         VUP_CHECK_LAUNCH();
         // a caller may start the record-stream histogram from here on
         prof_rec->launches = launches;
@@ -1730,38 +2232,38 @@ vup_status vup_build_layout(vup_grid g, cudaStream_t s, bool points_needed, cuda
         ProfScope prof("layout_sort_runs", s, 0);
         // sort keys of the chosen layout in its order, stable counting sort
         dim3 tg((unsigned)ceil_div64(Cn, 32), (unsigned)std::min<int64_t>(ceil_div64(Rn, 32), 65535));
-        k_layout_keys<<<tg, dim3(32, 8), 0, s>>>(g->bins, Rn, Cn, B, L, HL.keys_own, gate);
+        VUP_CHECK_CUDA(launch_pdl(k_layout_keys, tg, dim3(32, 8), 0, s, lb, g->ndim, B, L, HL.keys_own, gate));
         VUP_CHECK_LAUNCH();
         HL.keys = HL.keys_own;
-        st = counting_sort(g, HL.keys, Bk_max, HL.perm, HL.koff, counts, scratch, false, s, gate);
+        st = counting_sort(g, HL.keys, Bk_max, HL.perm, HL.koff, counts, scratch, false, s, gate, g->fold);
         if (st != VUP_OK) return st;
         // runs and intervals: one flag word per point, one 64-bit scan
         st = devbuf_reserve(g->lay_tmp, sizeof(unsigned long long) * 2 * (size_t)N);
         if (st != VUP_OK) return st;
         auto *flags = (unsigned long long *)g->lay_tmp.p;
         auto *excl = flags + N;
-        k_layout_flags<<<rb, 256, 0, s>>>(HL.perm, HL.keys, N, L, flags, gate);
+        VUP_CHECK_CUDA(launch_pdl(k_layout_flags, dim3(rb), dim3(256), 0, s, HL.perm, HL.keys, L, flags, gate));
         VUP_CHECK_LAUNCH();
         st = scan_exclusive<unsigned long long>(flags, excl, N, (unsigned long long *)g->scan_tmp.p, s, gate);
         if (st != VUP_OK) return st;
-        k_layout_build<<<rb, 256, 0, s>>>(HL.perm, HL.keys, N, L, kRowShift, flags, excl, HL.run_start, HL.run_rest,
-                                          HL.run_bin, HL.hpt, HL.n_runs, HL.ipt, HL.iv_rest, HL.n_iv, gate);
+        VUP_CHECK_CUDA(launch_pdl(k_layout_build, dim3(rb), dim3(256), 0, s, HL.perm, HL.keys, L, kRowShift, flags, excl, HL.run_start, HL.run_rest,
+                                          HL.run_bin, HL.hpt, HL.n_runs, HL.ipt, HL.iv_rest, HL.n_iv, gate));
         VUP_CHECK_LAUNCH();
         // run-end words carry the rest code of the run kRunAhead places later
         // (their factors come from L2, loaded that far ahead), or of the next
         // run when the 3-D point stream stages the rest factors in shared memory
         const int run_ahead = vup_hist_rest_staged(g) ? 1 : kRunAhead;
-        k_layout_encode<<<rb, 256, 0, s>>>(HL.run_start, HL.run_rest, HL.n_runs, HL.iv_rest, HL.n_iv, g->ndim,
-                                           g->ndim == 3 ? g->n[1] : 1, kRowShift, HL.hpt, HL.ipt, run_ahead, gate);
+        VUP_CHECK_CUDA(launch_pdl(k_layout_encode, dim3(rb), dim3(256), 0, s, HL.run_start, HL.run_rest, HL.n_runs, HL.iv_rest, HL.n_iv, g->ndim,
+                                           g->fold, kRowShift, HL.hpt, HL.ipt, run_ahead, gate));
         VUP_CHECK_LAUNCH();
         // chunks of every part
         const int PC = g->hist_P * C;
-        k_chunks<<<(PC + 1 + 127) / 128, 128, 0, s>>>(HL.run_start, HL.n_runs, HL.koff, B, L, C, excl, N, HL.n_iv,
-                                                       HL.chunk_pt, HL.chunk_run, HL.chunk_iv, gate);
+        VUP_CHECK_CUDA(launch_pdl(k_chunks, dim3((PC + 1 + 127) / 128), dim3(128), 0, s, HL.run_start, HL.n_runs, HL.koff, B, L, C, excl, HL.n_iv,
+                                                       HL.chunk_pt, HL.chunk_run, HL.chunk_iv, gate));
         VUP_CHECK_LAUNCH();
-        k_chunk_bins<<<(PC + 127) / 128, 128, 0, s>>>(HL.chunk_run, HL.run_bin, L, C, HL.chunk_bin, gate);
+        VUP_CHECK_CUDA(launch_pdl(k_chunk_bins, dim3((PC + 127) / 128), dim3(128), 0, s, HL.chunk_run, HL.run_bin, L, C, HL.chunk_bin, gate));
         VUP_CHECK_LAUNCH();
-        k_key_chunks<<<(Bk_max + 127) / 128, 128, 0, s>>>(HL.koff, L, B, HL.chunk_pt, C, HL.key_chunks, gate);
+        VUP_CHECK_CUDA(launch_pdl(k_key_chunks, dim3((Bk_max + 127) / 128), dim3(128), 0, s, HL.koff, L, B, HL.chunk_pt, C, HL.key_chunks, gate));
         VUP_CHECK_LAUNCH();
         st = vup_pick_hist_layout(g, s);
         if (st != VUP_OK) return st;
@@ -1771,6 +2273,7 @@ vup_status vup_build_layout(vup_grid g, cudaStream_t s, bool points_needed, cuda
         prof.launches = launches;
     }
     g->layout_valid = 1;
+    g->layout_unfolded = fold ? 0 : 1;
     g->layout_has_points = points_needed || g->ndim == 1;
     return VUP_OK;
 }
@@ -1781,7 +2284,7 @@ vup_status vup_ensure_layout(vup_grid g, cudaStream_t s, bool points_needed) {
 }
 
 vup_status vup_pick_hist_layout(vup_grid g, cudaStream_t s) {
-    k_pick_stream<<<1, 1, 0, s>>>(g->hl[0].n_runs, g->hl[0].n_iv, g->N, g->hist_force, g->hist_sel);
+    VUP_CHECK_CUDA(launch_pdl(k_pick_stream, dim3(1), dim3(1), 0, s, g->hl[0].n_runs, g->hl[0].n_iv, g->fold, g->hist_force, g->hist_sel));
     VUP_CHECK_LAUNCH();
     return VUP_OK;
 }

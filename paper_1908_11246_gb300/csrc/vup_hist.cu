@@ -40,6 +40,7 @@ constexpr uint32_t kRunEnd = 1u << 30, kBinEnd = 1u << 31;
 constexpr uint32_t kFlags = kRunEnd | kBinEnd;
 constexpr uint32_t kSpin = 1u << 26;
 constexpr int kPF = 16;                      // runs prefetched per block (global fallback)
+constexpr int kHistCtr = 5;                  // hist_sel[5..7]: the item counters of the three streams' walks
 constexpr int kRecBinsH = 8;                 // bins per record group (the layout builder's kRecBins)
 
 struct LayoutArgs {
@@ -54,6 +55,7 @@ struct LayoutArgs {
     const uint4 *rec;      // record stream (two uint4 per record)
     const int32_t *rec_rest, *rec_goff;
     const int2 *rec_gch;   // first / last chunk holding each group
+    const int32_t *n_rec, *n_iv;
     const int32_t *rec_chunk, *rec_chunk_grp;
     const float *g_last;   // factor table of the gathered axis  [n_last][K_pad]
     const float *g0, *g1;  // rest-axis factor tables (g1 only for 3-D)
@@ -61,18 +63,27 @@ struct LayoutArgs {
     int64_t n1;            // size of the second rest axis (3-D)
     int64_t n0;            // rows of g0 (the first rest axis)
     int P;
+    int ax_last, ax0, ax1; // the axes behind g_last, g0 and g1
+    // members of the gathered axis' classes (CSR), null when it is not folded: its
+    // rows of g_last are then summed as a tile is filled
+    const int32_t *cls_start, *cls_members;
 };
 
+// (n_last, part_rows, n0, n1, P and the factor tables of L0 / L1 are the unfolded
+// grid's; pick() replaces them by the merged grid's, known on the device)
 struct HistArgs {
     LayoutArgs L0, L1;
+    const FoldGeom *fold;
+    const float *ftab, *ftab_fold;  // factor tables and merged factor tables, axis d at off / foff[d] rows
+    int64_t off[3], foff[3];
+    const int32_t *fold_start, *fold_members;  // class members per axis, as laid out by the layout build
     const int32_t *sel;   // device: chosen layout, stream (1 = intervals)
     const DensStats *ds;
     int ndim;
     int64_t K, K_pad;
     int B;
     int C;                // chunks per part
-    int group_chunks;     // chunks per work item (a multiple of kGroupChunks dividing C)
-    int rec_sets;         // record stream: work items per part (each a range of the part's record chunks)
+    int sets;             // batched form: work items per part and density tile (each a range of its chunks)
     int C_rec;            // record chunks per part
     int GB;               // record groups per part: ceil(B / kRecBins)
     int points_only;      // 1: point stream whatever the layout choice says
@@ -81,12 +92,31 @@ struct HistArgs {
     float *hist;          // [K][B]
     float *part;          // [P * C][2][K_pad]
     float *direct;        // [P][K][B] (P > 1)
-    const float *prefix;  // prefix-sum tiles [P][K_pad / 128][pre_rows][128] (null: each CTA sums its own)
-    int64_t pre_rows;     // rows of a prefix tile (the most part rows + 1)
     int *dstatus;
 };
 
-__device__ __forceinline__ LayoutArgs pick(const HistArgs &A) { return A.sel[0] ? A.L1 : A.L0; }
+// The chosen layout on the merged grid.
+__device__ __forceinline__ LayoutArgs pick(const HistArgs &A) {
+    const int l = A.sel[0] ? 1 : 0;
+    LayoutArgs H = l ? A.L1 : A.L0;
+    const FoldGeom *F = A.fold;
+    H.n_last = F->n_last[l];
+    H.part_rows = F->part_rows[l];
+    H.P = F->P[l];
+    if (F->any) {
+        if (F->folded[H.ax_last]) {
+            H.cls_start = A.fold_start + A.off[H.ax_last] + H.ax_last;
+            H.cls_members = A.fold_members + A.off[H.ax_last];
+        }
+        if (F->folded[H.ax0]) H.g0 = A.ftab_fold + A.foff[H.ax0] * A.K_pad;
+        H.n0 = F->n[H.ax0];
+        if (A.ndim == 3) {
+            if (F->folded[H.ax1]) H.g1 = A.ftab_fold + A.foff[H.ax1] * A.K_pad;
+            H.n1 = F->n[H.ax1];
+        }
+    }
+    return H;
+}
 
 using namespace vup_async;
 
@@ -115,12 +145,13 @@ __host__ __device__ inline size_t hist_warp_bytes() { return (size_t)2 * kWin * 
 // record stream with 16 warps of up to 128 registers (more of its five
 // gathers and four accumulators in flight per warp; measured faster when the
 // rest-factor table stays in L2, slower when its rows come from HBM and more
-// warps hide the latency), 4 point stream of a 3-D grid with both rest-axis
-// factor tables staged in shared memory.  The others run 20 warps of 96
-// registers.  Each fills the register file of the one CTA per SM that the
+// warps hide the latency), 4 and 5 point and record stream of a 3-D grid with
+// both rest-axis factor tables staged in shared memory.  The others run 20
+// warps of 96 registers.  Each fills the register file of the one CTA per SM that the
 // tile allows.
-__host__ __device__ constexpr int hist_warps(int mode) { return (mode == 2 || mode == 3) ? 16 : kHistWarps; }
-__host__ __device__ constexpr int hist_stream_of(int mode) { return mode == 3 ? 2 : (mode == 4 ? 0 : mode); }
+__host__ __device__ constexpr int hist_warps(int mode) { return (mode == 2 || mode == 3 || mode == 5) ? 16 : kHistWarps; }
+__host__ __device__ constexpr int hist_stream_of(int mode) { return (mode == 3 || mode == 5) ? 2 : (mode == 4 ? 0 : mode); }
+__host__ __device__ constexpr bool hist_staged(int mode) { return mode == 4 || mode == 5; }
 __host__ __device__ inline size_t hist_smem_bytes(int64_t rows, int warps = kHistWarps) {
     return hist_tile_bytes(rows) + warps * hist_warp_bytes() + warps * 2 * sizeof(uint64_t);
 }
@@ -201,6 +232,106 @@ __device__ __forceinline__ void fma4(float4 &a, float4 w, float4 b) {
     a = from_pairs(lo, hi);
 }
 
+// Sums of four densities per lane as FP32 TwoSum pairs.
+struct PairSum4 {
+    float4 h, l;
+    __device__ __forceinline__ void clear() { h = l = make_float4(0.f, 0.f, 0.f, 0.f); }
+    __device__ __forceinline__ void add(float4 x) {
+        two_sum_acc(h.x, l.x, x.x);
+        two_sum_acc(h.y, l.y, x.y);
+        two_sum_acc(h.z, l.z, x.z);
+        two_sum_acc(h.w, l.w, x.w);
+    }
+    // v z, the product unrounded
+    __device__ __forceinline__ void add_scaled(float4 v, float4 z) {
+        one(h.x, l.x, v.x, z.x);
+        one(h.y, l.y, v.y, z.y);
+        one(h.z, l.z, v.z, z.z);
+        one(h.w, l.w, v.w, z.w);
+    }
+    __device__ __forceinline__ float4 value() const {
+        return make_float4(h.x + l.x, h.y + l.y, h.z + l.z, h.w + l.w);
+    }
+    static __device__ __forceinline__ void one(float &h, float &l, float v, float z) {
+        const float s = fmaf(v, z, h);
+        const float b = s - h;
+        l += (h - (s - b)) + fmaf(v, z, -b);
+        h = s;
+    }
+};
+
+// Factor of one class of a folded axis (four densities): its members' factors
+// summed in index order as FP32 TwoSum pairs, rounded once.
+__device__ __forceinline__ float4 class_factor(const float *__restrict__ col, int64_t K_pad,
+                                               const int32_t *__restrict__ members, int32_t m0, int32_t m1) {
+    PairSum4 t;
+    t.clear();
+    for (int32_t m = m0; m < m1; m += 4) {
+        float4 v[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            v[q] = m + q < m1 ? ld4(col + (int64_t)(members[m + q] & (kFoldLast - 1)) * K_pad)
+                              : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) t.add(v[q]);
+    }
+    return t.value();
+}
+
+// One warp's rows of a tile: rows m0 .. m1 - 1 of the gathered axis' factor
+// table (src: this lane's four densities of row 0), or with `members` the
+// members m0 .. m1 - 1 of the rows' classes in class order (each class' last
+// one flagged), whose factors are summed per class.  Every row goes to dst
+// (SCALED: times the normalisers iz, else its scaled value into the sum that
+// tot receives, [h, l][lane]); eight rows' loads are in flight per warp (16, in
+// line or not, and packed pair arithmetic measured slower: 121 - 144 us against
+// 113 for the walk of 1024 x 1024 points x 16384 densities).
+template <bool SCALED, int AHEAD>
+__device__ __forceinline__ void tile_rows_in(const float *__restrict__ src, int64_t K_pad,
+                                              const int32_t *__restrict__ members, int32_t m0, int32_t m1, float4 iz,
+                                              float *dst, float4 *tot) {
+    const int lane = threadIdx.x & 31;
+    PairSum4 t;
+    t.clear();
+    PairSum4 c;
+    c.clear();
+    // lane u holds the u-th entry of a batch of 32
+    int32_t e = members && m0 + lane < m1 ? members[m0 + lane] : 0;
+    for (int32_t m = m0; m < m1; m += 32) {
+        const int32_t e_next = members && m + 32 + lane < m1 ? members[m + 32 + lane] : 0;
+        const int n = min(32, m1 - m);
+        for (int u0 = 0; u0 < n; u0 += AHEAD) {
+            float4 v[AHEAD];
+            int32_t r[AHEAD];
+#pragma unroll
+            for (int u = 0; u < AHEAD; ++u) {
+                r[u] = members ? __shfl_sync(0xffffffffu, e, u0 + u) : ((m + u0 + u) | kFoldLast);
+                v[u] = u0 + u < n ? ld4(src + (int64_t)(r[u] & (kFoldLast - 1)) * K_pad)
+                                  : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+#pragma unroll
+            for (int u = 0; u < AHEAD; ++u) {
+                if (u0 + u < n) {
+                    float4 x = v[u];
+                    if (members) {
+                        c.add(x);
+                        x = c.value();
+                    }
+                    if (r[u] & kFoldLast) {
+                        c.clear();
+                        if (!SCALED) t.add_scaled(x, iz);
+                        *reinterpret_cast<float4 *>(dst) = SCALED ? mul4(x, iz) : x;
+                        dst += kKT;
+                    }
+                }
+            }
+        }
+        e = e_next;
+    }
+    tot[lane] = t.h;
+    tot[32 + lane] = t.l;
+}
+
 // Per-item context, kept in shared memory: the chosen layout, the output
 // pointers and sizes.  Warps read it on demand, so none of it occupies
 // registers across the point loop.
@@ -209,12 +340,11 @@ struct ItemCtx {
     float *part;   // [P * C][2][K_pad] partial sums of keys cut by chunk bounds
     float *direct; // [P * B][K_pad] sums of keys held by one chunk
     int64_t K, K_pad;
-    int B, C, group_chunks, rec_sets, C_rec, GB;
+    int B, C, C_rec, GB;
     int mode;      // 0: point stream, tile holds factors; 1: interval stream, tile holds prefix sums
     int rest_smem;  // (3-D point stream) rest-axis factors [n0][kKT], [n1][kKT] after the staging buffers
     int64_t rest_n0;
-    const float *prefix;
-    int64_t pre_rows;
+    int64_t pre_rows;  // rows of a prefix tile (debug build's bound)
     int *dstatus;
 };
 
@@ -400,9 +530,10 @@ __device__ __noinline__ void flush_group(const ItemCtx *X, int c, int p, int64_t
     for (int j = 0; j < kRecBinsH; ++j)
         if (shared || b0 + j < X->B) *reinterpret_cast<float4 *>(row + j * K_pad) = a[j];
 }
-template <int NF>
+// RS: the rest-axis factor rows are read from shared memory (w0s, w1s).
+template <int NF, bool RS>
 __device__ __forceinline__ bool rec_chunk_walk(const ItemCtx &X, int c, int p, int64_t k, const float *ws,
-                                               uint32_t *win, uint64_t *mbar, uint32_t &wseq, volatile int *abort) {
+                                               const float *w0s, const float *w1s, uint32_t *win, uint64_t *mbar, uint32_t &wseq, volatile int *abort) {
     const LayoutArgs &H = X.H;
     const int lane = threadIdx.x & 31;
     const int32_t r0 = H.rec_chunk[c], r1 = H.rec_chunk[c + 1];
@@ -437,6 +568,7 @@ __device__ __forceinline__ bool rec_chunk_walk(const ItemCtx &X, int c, int p, i
     auto rest2 = [&](uint32_t a0, uint32_t a1) -> float4 {
         if (!VUP_DBG_IN(a0, H.n0, X.dstatus)) a0 = 0;
         if (!VUP_DBG_IN(a1, H.n1, X.dstatus)) a1 = 0;
+        if (RS) return mul4(ld4(w0s + a0 * kKT), ld4(w1s + a1 * kKT));
         return mul4(row4(g0b, a0), row4(g1b, a1));
     };
     auto rest1 = [&](uint32_t a0) -> float4 {
@@ -491,12 +623,13 @@ __device__ __forceinline__ bool rec_chunk_walk(const ItemCtx &X, int c, int p, i
             for (int j = 0; j <= kRecBinsH; ++j) rw[j] = 0;
 #endif
         const float4 fs = (v.x & kRecNegFlag) ? make_float4(-f.x, -f.y, -f.z, -f.w) : f;
-        // each half of the group is skipped when it holds no bin (its
+        // each half (3-D: quarter, a line there holds 2.5 bins of a group where a
+        // 2-D one holds 6) of the group is skipped when it holds no bin (its
         // boundaries then all equal its first)
+        constexpr int kH = RS ? 2 : kRecBinsH / 2;
         float4 prev = gather(wsl + (rw[0] << kRowShift));
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            constexpr int kH = kRecBinsH / 2;
+        for (int h = 0; h < kRecBinsH / kH; ++h) {
             if (rw[kH * h + kH] != rw[kH * h]) {
 #pragma unroll
                 for (int j = kH * h; j < kH * h + kH; ++j) {
@@ -556,14 +689,13 @@ __device__ __forceinline__ bool rec_chunk_walk(const ItemCtx &X, int c, int p, i
     return true;
 }
 
-// One work item: part p, chunk group cg (kGroupChunks chunks, drawn by the
-// warps one at a time) and
-// the 128 densities from k0 of the instance *Ap (kernel parameter or global
+// One work item: part p, range cg of G of the part's chunks (drawn by the
+// warps one at a time) and the 128 densities from k0 of the instance *Ap (kernel parameter or global
 // memory).  Called by every thread of the CTA; `wseq` counts the staging
 // windows this warp has consumed so far (it keeps the per-warp mbarrier
 // phases consistent across items).
 template <int NF, int MODE>
-__device__ __forceinline__ void hist_item(const HistArgs *Ap, int p, int cg, int64_t k0, uint8_t *sm,
+__device__ __forceinline__ void hist_item(const HistArgs *Ap, int p, int cg, int G, int64_t k0, uint8_t *sm,
                                           int64_t tile_rows, uint32_t &wseq, volatile int *abort, ItemCtx &X,
                                           float *s_invz, int *next_chunk) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -580,23 +712,20 @@ __device__ __forceinline__ void hist_item(const HistArgs *Ap, int p, int cg, int
     if (threadIdx.x == 0) {
         const HistArgs &A = *Ap;
         *next_chunk = 0;
-        X.H = A.sel[0] ? A.L1 : A.L0;
+        X.H = pick(A);
         X.part = A.part;
         X.direct = A.direct;
         X.K = A.K;
         X.K_pad = A.K_pad;
         X.B = A.B;
         X.C = A.C;
-        X.group_chunks = A.group_chunks;
-        X.rec_sets = A.rec_sets;
         X.C_rec = A.C_rec;
         X.GB = A.GB;
         X.mode = hist_stream_of(MODE);
-        X.prefix = A.prefix;
-        X.pre_rows = A.pre_rows;
+        X.pre_rows = X.H.part_rows + 1;
         X.dstatus = A.dstatus;
-        X.rest_smem = MODE == 4 ? 1 : 0;
-        X.rest_n0 = A.rest_n0;
+        X.rest_smem = hist_staged(MODE) ? 1 : 0;
+        X.rest_n0 = X.H.n0;
     }
     if (threadIdx.x < kKT) s_invz[threadIdx.x] = inv_z(*Ap, k0 + threadIdx.x);
     __syncthreads();
@@ -607,20 +736,26 @@ __device__ __forceinline__ void hist_item(const HistArgs *Ap, int p, int cg, int
     // normaliser 1 / prod_d Z_d
     const int64_t row0 = (int64_t)p * H.part_rows;
     const int64_t nrows = min(H.part_rows, H.n_last - row0);
-    constexpr bool kPrefixTile = hist_stream_of(MODE) != 0;  // interval / record streams: prefix sums
-    const bool pre = kPrefixTile && X.prefix != nullptr;     // the prefix sums come ready-made
-    if (pre) {
-        const float *src = X.prefix + ((int64_t)p * (X.K_pad / kKT) + k0 / kKT) * X.pre_rows * kKT;
-        for (int64_t e = threadIdx.x; e < (nrows + 1) * (kKT / 4); e += blockDim.x) cp_async16(ws + e * 4, src + e * 4);
-    } else {
-        const float *src = H.g_last + row0 * X.K_pad + k0;
-        const int64_t K_pad = X.K_pad;
-        for (int64_t e = threadIdx.x; e < nrows * (kKT / 4); e += blockDim.x) {
-            const int64_t a = e / (kKT / 4), cc = e % (kKT / 4);
-            cp_async16(ws + a * kKT + cc * 4, src + a * K_pad + cc * 4);
-        }
+    // every warp fills its share of the rows; the interval and record
+    // streams then turn the columns into exclusive prefix sums P[0..nrows]
+    // (each P the TwoSum pair of the rows before it, rounded once to FP32), so
+    // that rows a .. b - 1 sum to P[b] - P[a]: the warps' totals first (kept in
+    // the idle staging buffers), then each warp again from the totals before
+    // it.  (Prefix tiles from a kernel of their own cost 60 us at 1024 rows x
+    // 16384 densities, or five times that beside the contraction, whose
+    // operands take the L2 bandwidth; the scan here costs an item 3 us.)
+    const float4 iz4 = ld4(s_invz + 4 * lane);
+    const int32_t a0 = (int32_t)(nrows * warp / kWarps), a1 = (int32_t)(nrows * (warp + 1) / kWarps);
+    PairSum4 t;
+    t.clear();
+    {
+        const int32_t *members = H.cls_start ? H.cls_members : nullptr;
+        const int32_t m0 = members ? H.cls_start[row0 + a0] : (int32_t)row0 + a0;
+        const int32_t m1 = members ? H.cls_start[row0 + a1] : (int32_t)row0 + a1;
+        tile_rows_in<hist_stream_of(MODE) == 0, 8>(H.g_last + k, X.K_pad, members, m0, m1, iz4,
+                                                       ws + (int64_t)a0 * kKT + 4 * lane, reinterpret_cast<float4 *>(win));
     }
-    if (MODE == 4) {
+    if (hist_staged(MODE)) {
         // the k-tile's rows of both rest-axis factor tables (unnormalised)
         float *rs = reinterpret_cast<float *>(sm + hist_smem_bytes(tile_rows, kWarps));
         const int64_t n0 = X.rest_n0, n1 = H.n1, K_pad = X.K_pad;
@@ -629,56 +764,29 @@ __device__ __forceinline__ void hist_item(const HistArgs *Ap, int p, int cg, int
             const float *src = a < n0 ? H.g0 + a * K_pad : H.g1 + (a - n0) * K_pad;
             cp_async16(rs + a * kKT + cc * 4, src + k0 + cc * 4);
         }
+        cp_async_commit();
     }
-    cp_async_commit();
-    if (!pre && threadIdx.x < kKT) ws[nrows * kKT + threadIdx.x] = 0.f;
-    cp_async_wait_all();
-    __syncthreads();
-    if (pre) {
-        // the staging buffers are next written by bulk copies (async proxy)
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    } else if (kPrefixTile) {
-        // interval stream: every column becomes the exclusive prefix sums
-        // P[0..nrows] of its scaled factors (compensated sums, each P rounded
-        // once to FP32), so that rows a .. b - 1 sum to P[b] - P[a].  The
-        // rows are cut into kScanSegs segments, one thread per (segment,
-        // column): segment totals first (kept in the idle staging buffers),
-        // then each segment rescanned from the sum of the totals before it.
-        constexpr int kScanSegs = kWarps * 32 / kKT;
-        const int col = threadIdx.x % kKT, sg = threadIdx.x / kKT;
-        const int64_t rs = (nrows + kScanSegs - 1) / kScanSegs;
-        const int64_t a0 = min(nrows, sg * rs), a1 = min(nrows, a0 + rs);
-        const float iz = s_invz[col];
-        float *tcol = ws + col;
-        float2 *segsum = reinterpret_cast<float2 *>(sm + tb);  // [kScanSegs][kKT]
-        auto add = [](float &sh, float &sl, float v) {
-            const float t = sh + v, bb = t - sh;
-            sl += (sh - (t - bb)) + (v - bb);
-            sh = t;
-        };
-        {
-            float sh = 0.f, sl = 0.f;
-            for (int64_t a = a0; a < a1; ++a) add(sh, sl, tcol[a * kKT] * iz);
-            segsum[sg * kKT + col] = make_float2(sh, sl);
-        }
-        __syncthreads();
-        float oh = 0.f, ol = 0.f;
-        for (int q = 0; q < sg; ++q) {
-            const float2 v = segsum[q * kKT + col];
-            add(oh, ol, v.x);
-            ol += v.y;
-        }
-        for (int64_t a = a0; a < a1; ++a) {
-            const float v = tcol[a * kKT] * iz;
-            tcol[a * kKT] = oh + ol;
-            add(oh, ol, v);
-        }
-        if (a1 == nrows && (a0 < a1 || sg == 0)) tcol[nrows * kKT] = oh + ol;
-        // the staging buffers are next written by bulk copies (async proxy)
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    if (hist_stream_of(MODE) == 0) {
+        if (threadIdx.x < kKT) ws[nrows * kKT + threadIdx.x] = 0.f;
     } else {
-        for (int64_t e = threadIdx.x; e < nrows * kKT; e += blockDim.x) ws[e] *= s_invz[e % kKT];
+        __syncthreads();
+        t.clear();
+        for (int w = 0; w < warp; ++w) {
+            const float4 *o = reinterpret_cast<const float4 *>(sm + tb + (size_t)w * hist_warp_bytes());
+            t.add(o[lane]);
+            add4(t.l, o[32 + lane]);
+        }
+        float *q = ws + (int64_t)a0 * kKT + 4 * lane;
+        for (int32_t a = a0; a < a1; ++a, q += kKT) {
+            const float4 x = ld4(q);
+            *reinterpret_cast<float4 *>(q) = t.value();
+            t.add_scaled(x, iz4);
+        }
+        if (warp == kWarps - 1) *reinterpret_cast<float4 *>(q) = t.value();
+        // the staging buffers are next written by bulk copies (async proxy)
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
+    if (hist_staged(MODE)) cp_async_wait_all();
     __syncthreads();
 
     // the item's chunks are handed out one at a time (at least kChunksPerWarp per warp
@@ -866,21 +974,24 @@ __device__ __forceinline__ void hist_item(const HistArgs *Ap, int p, int cg, int
     };
     if constexpr (hist_stream_of(MODE) == 2) {
         // this item's range of the part's record chunks, handed out one at a time
-        const int c_lo = (int)((int64_t)cg * X.C_rec / X.rec_sets), c_hi = (int)((int64_t)(cg + 1) * X.C_rec / X.rec_sets);
+        const int c_lo = (int)((int64_t)cg * X.C_rec / G), c_hi = (int)((int64_t)(cg + 1) * X.C_rec / G);
         for (;;) {
             int ci = 0;
             if (lane == 0) ci = atomicAdd(next_chunk, 1);
             ci = __shfl_sync(0xffffffffu, ci, 0);
             if (c_lo + ci >= c_hi) break;
-            if (!rec_chunk_walk<NF>(X, p * X.C_rec + c_lo + ci, p, k, ws, win, mbar, wseq, abort)) return;
+            const float *w0s = reinterpret_cast<const float *>(sm + hist_smem_bytes(tile_rows, kWarps)) + 4 * lane;
+            if (!rec_chunk_walk<NF, hist_staged(MODE)>(X, p * X.C_rec + c_lo + ci, p, k, ws, w0s,
+                                                       w0s + X.rest_n0 * kKT, win, mbar, wseq, abort))
+                return;
         }
     } else {
         for (;;) {
             int ci = 0;
             if (lane == 0) ci = atomicAdd(next_chunk, 1);
             ci = __shfl_sync(0xffffffffu, ci, 0);
-            if (ci >= X.group_chunks) break;
-            const int wc = cg * X.group_chunks + ci;
+            const int wc = (int)((int64_t)cg * X.C / G) + ci;
+            if (wc >= (int)((int64_t)(cg + 1) * X.C / G)) break;
             bool ok;
             if constexpr (MODE == 1) ok = iv_chunk<NF>(X, p * X.C + wc, p, k, ws, win, mbar, wseq, abort);
             else ok = run_chunk(wc);
@@ -907,30 +1018,88 @@ __device__ __forceinline__ void hist_init_mbar(uint8_t *sm, int64_t tile_rows, i
 // unless the caller asked for points).
 __device__ __forceinline__ int hist_stream(const HistArgs &A) { return A.points_only ? 0 : A.sel[1]; }
 
-// One CTA per item, it = (k-tile * P + part) * G + chunk group, so that
-// CTAs running together share k-tiles (rest-factor rows stay in L2) and the
-// hardware hands items to SMs as they free up (item costs vary; a static
-// split of items over persistent CTAs measured 12 % slower on the 3-D
-// workload).  Each stream is its own kernel (their register allocations
-// stay apart); the host launches both and every CTA of the one the device
-// did not choose returns at once.
+// Work items per (part, density tile) of a walk over n elements (points,
+// intervals or records) per part in C chunks: the split G that ends first by
+//   ceil(items / CTAs) (tile + max(n thr / G, ceil(C / G / warps) n / C thr warps / 2))
+// SM cycles: the tile's copy (about 10 cycles per 512-byte row after a 3000-cycle
+// start), the walk at its measured rate thr per element and 128 densities, or,
+// where an item has fewer chunks than warps, at half a warp's share of it
+// (latency).  Few density tiles are cut into up to C items (a 200 x 328 grid
+// with 225 densities ran on 2 CTAs), many into as few as fill the last wave.
+// One warp evaluates 32 candidates at a time; every CTA finds the same G.
+__device__ __forceinline__ int hist_split(int64_t n, int C, int64_t tiles, int64_t rows, int warps, float thr,
+                                          int ctas) {
+    const int lane = threadIdx.x & 31;
+    float best = 3.0e38f;
+    int bg = 1;
+    for (int g = 1 + lane; g <= C; g += 32) {
+        const float waves = (float)((tiles * g + ctas - 1) / ctas);
+        const float ch = (float)(((C + g - 1) / g + warps - 1) / warps);
+        const float walk = (float)n * thr;
+        const float t = waves * (3000.f + 10.f * (float)rows +
+                                 fmaxf(walk / (float)g, ch * walk / (float)C * 0.5f * (float)warps));
+        if (t < best) {
+            best = t;
+            bg = g;
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const float ot = __shfl_xor_sync(0xffffffffu, best, o);
+        const int og = __shfl_xor_sync(0xffffffffu, bg, o);
+        if (ot < best || (ot == best && og < bg)) {
+            best = ot;
+            bg = og;
+        }
+    }
+    return bg;
+}
+// Measured SM cycles per element and 128 densities of each stream's walk.
+__host__ __device__ constexpr float hist_rate(int mode) {
+    return hist_stream_of(mode) == 2 ? 55.f : (mode == 1 ? 19.f : 6.f);
+}
+
+// Persistent CTAs, one per SM (the tile fills its shared memory), drawing the
+// items it = (k-tile * P + part) * G + range in order from a counter, so that
+// CTAs running together share k-tiles (rest-factor rows stay in L2) and an SM
+// takes the next item as it frees up (item costs vary; a static split of
+// items over the CTAs measured 12 % slower on the 3-D workload).  The counters
+// are zeroed by the merged-table kernel, which runs before the walks of every
+// call.  Each stream is its own kernel (their register allocations stay
+// apart); the host launches every stream's and the CTAs of those the device
+// did not choose return at once (a CTA per item instead cost 32 us for each of
+// them at 65536 densities of a 2048 x 2048 grid).
 template <int NF, int MODE>
 __global__ void __launch_bounds__(hist_warps(MODE) * 32, 1)
-    k_hist_smem(const __grid_constant__ HistArgs A, int64_t tile_rows, int P, int G, int n_items) {
+    k_hist_smem(const __grid_constant__ HistArgs A, int64_t tile_rows, int nkt, int *__restrict__ next_item) {
     pdl_trigger();
     pdl_wait();
     if (hist_stream(A) != hist_stream_of(MODE)) return;  // uniform
     extern __shared__ __align__(128) uint8_t sm[];
     __shared__ ItemCtx X;
     __shared__ float s_invz[kKT];
-    __shared__ int abort, next_chunk;
+    __shared__ int abort, next_chunk, s_item, s_G;
     if (threadIdx.x == 0) abort = 0;
     hist_init_mbar(sm, tile_rows, hist_warps(MODE));
+    const int P = A.fold->P[A.sel[0] ? 1 : 0];
+    if (threadIdx.x < 32) {
+        const LayoutArgs &L = A.sel[0] ? A.L1 : A.L0;
+        const int64_t n = hist_stream_of(MODE) == 2 ? L.n_rec[0] : (MODE == 1 ? L.n_iv[0] : A.fold->N);
+        const int C = hist_stream_of(MODE) == 2 ? A.C_rec : A.C;
+        const int G = hist_split(n / P, C, (int64_t)nkt * P, A.fold->part_rows[A.sel[0] ? 1 : 0], hist_warps(MODE),
+                                 hist_rate(MODE), gridDim.x);
+        if (threadIdx.x == 0) s_G = G;
+    }
     uint32_t wseq = 0;
-    for (int it = blockIdx.x; it < n_items; it += gridDim.x) {
+    for (;;) {
+        __syncthreads();  // the previous item's readers of s_item are done
+        if (threadIdx.x == 0) s_item = atomicAdd(next_item, 1);
+        __syncthreads();
+        const int G = s_G, it = s_item;
+        if (it >= (int64_t)nkt * P * G || abort) return;
         const int cg = it % G, pk = it / G;
         const int p = pk % P, kt = pk / P;
-        hist_item<NF, MODE>(&A, p, cg, (int64_t)kt * kKT, sm, tile_rows, wseq, &abort, X, s_invz, &next_chunk);
+        hist_item<NF, MODE>(&A, p, cg, G, (int64_t)kt * kKT, sm, tile_rows, wseq, &abort, X, s_invz, &next_chunk);
     }
 }
 
@@ -1014,8 +1183,8 @@ __global__ void __launch_bounds__(hist_warps(MODE) * 32, 1) k_hist_batched(const
         const int it = s_it;
         if (it >= n_items) break;
         const HistItem w = items[list[it]];
-        hist_item<NF, MODE>(insts + w.inst, w.p, w.cg, (int64_t)w.kt * kKT, sm, tile_rows, wseq, &abort, X, s_invz,
-                            &next_chunk);
+        hist_item<NF, MODE>(insts + w.inst, w.p, w.cg, insts[w.inst].sets, (int64_t)w.kt * kKT, sm, tile_rows, wseq,
+                            &abort, X, s_invz, &next_chunk);
     }
 }
 
@@ -1028,9 +1197,9 @@ __global__ void __launch_bounds__(kHistWarps * 32, 1) k_hist_global(HistArgs A, 
     if (p >= H.P) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t k = (int64_t)blockIdx.y * kKT + 4 * lane;
-    // chunks cg * group_chunks + j * kHistWarps + warp
-    for (int j = 0; j < A.group_chunks / kHistWarps; ++j) {
-        const int c = p * A.C + cg * A.group_chunks + j * kHistWarps + warp;
+    const int group = A.C / G;  // chunks of a block: cg * group + j * kHistWarps + warp
+    for (int j = 0; j < group / kHistWarps; ++j) {
+        const int c = p * A.C + cg * group + j * kHistWarps + warp;
         const int32_t p0 = H.chunk_pt[c], p1 = H.chunk_pt[c + 1];
         if (p0 >= p1) continue;
         const int32_t r0 = H.chunk_run[c], r1 = H.chunk_run[c + 1];
@@ -1058,8 +1227,11 @@ __global__ void __launch_bounds__(kHistWarps * 32, 1) k_hist_global(HistArgs A, 
                 const int32_t r = rb + u;
                 if (r >= r1) break;
                 float4 acc = zero4;
-                for (int32_t q = H.run_start[r]; q < H.run_start[r + 1]; ++q)
-                    add4(acc, ld4(wl + (int64_t)(H.perm[q] % H.n_last) * A.K_pad));
+                for (int32_t q = H.run_start[r]; q < H.run_start[r + 1]; ++q) {
+                    const int64_t a = H.perm[q] % H.n_last;
+                    add4(acc, H.cls_start ? class_factor(wl, A.K_pad, H.cls_members, H.cls_start[a], H.cls_start[a + 1])
+                                          : ld4(wl + a * A.K_pad));
+                }
                 fma4(bacc, w[u], acc);
                 const int32_t nk = r + 1 < r1 ? H.run_bin[r + 1] : -1;
                 if (nk != cur_key) {
@@ -1070,52 +1242,6 @@ __global__ void __launch_bounds__(kHistWarps * 32, 1) k_hist_global(HistArgs A, 
             }
         }
     }
-}
-
-// Prefix-sum tiles of the interval and record streams, once per (part,
-// density): thread (p, k) walks the part's rows of the gathered-axis factor
-// table, each factor scaled by the density's normaliser 1 / prod_d Z_d, and
-// writes the exclusive prefix sums P[0..nrows] (compensated, each P rounded
-// once to FP32) so that rows a .. b - 1 sum to P[b] - P[a].  Tile (p, k-tile)
-// is one contiguous block of pre_rows x 128 floats, copied as is into the
-// histogram kernel's shared memory.  Returns at once when the device chose
-// the point stream, whose tile holds the scaled factors themselves.  Loads
-// and stores are marked evict-first: the kernel runs beside the contraction,
-// whose operands should keep L2.
-__device__ __forceinline__ void prefix_tile(const HistArgs &A, const LayoutArgs &H, float *__restrict__ out, int p,
-                                            int64_t k) {
-    const int64_t row0 = (int64_t)p * H.part_rows;
-    const int64_t nrows = min(H.part_rows, H.n_last - row0);
-    const float iz = inv_z(A, k);
-    const float *src = H.g_last + row0 * A.K_pad + k;
-    float *dst = out + ((int64_t)p * (A.K_pad / kKT) + k / kKT) * A.pre_rows * kKT + (k % kKT);
-    float sh = 0.f, sl = 0.f;
-    constexpr int kAhead = 32;  // rows loaded ahead (the walk is bound by loads in flight)
-    for (int64_t a = 0; a < nrows; a += kAhead) {
-        float v[kAhead];
-#pragma unroll
-        for (int u = 0; u < kAhead; ++u) v[u] = a + u < nrows ? __ldcs(src + (a + u) * A.K_pad) : 0.f;
-#pragma unroll
-        for (int u = 0; u < kAhead; ++u) {
-            if (a + u >= nrows) break;
-            __stcs(dst + (a + u) * kKT, sh + sl);
-            const float x = v[u] * iz;
-            const float t = sh + x, bb = t - sh;
-            sl += (sh - (t - bb)) + (x - bb);
-            sh = t;
-        }
-    }
-    __stcs(dst + nrows * kKT, sh + sl);
-}
-
-__global__ void __launch_bounds__(128) k_prefix_tiles(const __grid_constant__ HistArgs A, float *__restrict__ out,
-                                                      int gate_stream) {
-    if (A.points_only || (gate_stream && A.sel[1] == 0)) return;
-    const LayoutArgs &H = A.sel[0] ? A.L1 : A.L0;
-    // tiles (p, k-tile) strided over the grid
-    const int64_t nkt = A.K_pad / kKT;
-    for (int64_t u = blockIdx.x; u < (int64_t)H.P * nkt; u += gridDim.x)
-        prefix_tile(A, H, out, (int)(u / nkt), (u % nkt) * kKT + threadIdx.x);
 }
 
 // Finish H[k, b]: for every part, the key (part, b) is either empty, summed
@@ -1135,7 +1261,7 @@ __device__ __forceinline__ void hist_finish_tiles(const HistArgs &A, int64_t kt0
     __shared__ int2 s_cc[kFinMaxP][kFinB];
     const LayoutArgs &H = A.sel[0] ? A.L1 : A.L0;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int P = H.P;
+    const int P = A.fold->P[A.sel[0] ? 1 : 0];
     const bool recs = !A.points_only && A.sel[1] == 2;  // record stream: every non-empty group wrote its rows
     // the chunk range of every (part, bin) key of the bin tile; on the record
     // stream that of the part's group of the bin
@@ -1296,7 +1422,7 @@ static HistArgs hist_args_for(vup_grid g, int64_t K, float *hist, int64_t &rows,
         return ft + off;
     };
     HistArgs A{};
-    A.group_chunks = kGroupChunks;
+    A.sets = 1;
     rows = 0;
     P_max = 1;
     for (int l = 0; l < 2; ++l) {
@@ -1315,6 +1441,8 @@ static HistArgs hist_args_for(vup_grid g, int64_t K, float *hist, int64_t &rows,
         La.ipt = HL.ipt;
         La.iv_rest = HL.iv_rest;
         La.chunk_iv = HL.chunk_iv;
+        La.n_rec = HL.n_rec;
+        La.n_iv = HL.n_iv;
         La.rec = (const uint4 *)g->hl[0].rec.p;  // the built layout's arrays
         La.rec_rest = (const int32_t *)g->hl[0].rec_rest.p;
         La.rec_goff = (const int32_t *)g->hl[0].rec_goff.p;
@@ -1336,12 +1464,23 @@ static HistArgs hist_args_for(vup_grid g, int64_t K, float *hist, int64_t &rows,
         La.n_last = HL.n_last;
         La.part_rows = HL.part_rows;
         La.P = HL.P;
+        La.ax_last = HL.last_axis;
+        La.ax0 = nd == 3 ? 0 : 1 - HL.last_axis;
+        La.ax1 = nd == 3 ? 1 : La.ax0;
         rows = std::max(rows, HL.part_rows);
         P_max = std::max(P_max, HL.P);
     }
+    A.fold = g->fold;
+    A.ftab = ft;
+    A.ftab_fold = (const float *)g->ftab_fold.p;
+    A.fold_start = g->fold_start;
+    A.fold_members = g->fold_members;
+    for (int d = 0; d < nd; ++d) {
+        A.off[d] = d ? A.off[d - 1] + g->n[d - 1] : 0;
+        A.foff[d] = d ? A.foff[d - 1] + fold_cap(g->n[d - 1]) : 0;
+    }
     A.sel = g->hist_sel;
     A.GB = (int)ceil_div64(g->B, kRecBinsH);
-    A.rec_sets = 1;
     A.C_rec = g->n_chunks_rec;
     A.ds = (const DensStats *)g->dstats.p;
     A.ndim = nd;
@@ -1356,15 +1495,83 @@ static HistArgs hist_args_for(vup_grid g, int64_t K, float *hist, int64_t &rows,
     return A;
 }
 
-bool vup_hist_prefix(vup_grid g, int64_t K, cudaStream_t s) {
-    if (!vup_hist_tile_fits(g)) return false;
-    int64_t rows;
-    int P_max;
-    HistArgs A = hist_args_for(g, K, nullptr, rows, P_max);
-    A.pre_rows = rows + 1;
-    VUP_PROF("hist_prefix", s, 1);
-    k_prefix_tiles<<<(unsigned)(P_max * (A.K_pad / 128)), 128, 0, s>>>(A, (float *)g->hist_prefix.p, 0);
-    return cudaGetLastError() == cudaSuccess;
+// Merged factor tables (FoldGeom) of the folded rest axes of the chosen layout
+// (the gathered axis' classes are summed where its tiles are made).  HBM
+// bound: it reads a folded axis' factors once and writes 5/8 of that at most;
+// a grid-stride walk over (axis, class, 512 densities), so that a grid without
+// folded axes costs an empty launch.
+struct FoldTabArgs {
+    const FoldGeom *fold;
+    const int32_t *sel;
+    const int32_t *start, *members;
+    const float *ftab;
+    float *out;
+    int64_t n[3], K_pad;
+    int ndim;
+    int *ctr;  // the walks' item counters, zeroed here (or null)
+};
+__device__ __forceinline__ void fold_table_rows(const FoldTabArgs &T, int64_t first, int64_t step) {
+    const int64_t kb = (T.K_pad + 511) / 512;
+    const int gathered = T.ndim == 2 && T.sel[0] ? 0 : T.ndim - 1;
+    int64_t off = 0, foff = 0;
+    for (int d = 0; d < T.ndim; ++d) {
+        if (T.fold->folded[d] && d != gathered) {
+            const int64_t rows = T.fold->n[d];
+            for (int64_t u = first; u < rows * kb; u += step) {
+                const int64_t c = u / kb, k = (u - c * kb) * 512 + 4 * threadIdx.x;
+                if (k >= T.K_pad) continue;
+                const int32_t *st = T.start + off + d + c;
+                *reinterpret_cast<float4 *>(T.out + (foff + c) * T.K_pad + k) =
+                    class_factor(T.ftab + off * T.K_pad + k, T.K_pad, T.members + off, st[0], st[1]);
+            }
+        }
+        off += T.n[d];
+        foff += fold_cap(T.n[d]);
+    }
+}
+__global__ void __launch_bounds__(128) k_fold_tables(const __grid_constant__ FoldTabArgs T) {
+    if (blockIdx.x == 0 && threadIdx.x < 3) T.ctr[threadIdx.x] = 0;
+    if (!T.fold->any) return;
+    fold_table_rows(T, blockIdx.x, gridDim.x);
+}
+// Batched form: block y serves instance y.
+__global__ void __launch_bounds__(128) k_fold_tables_batched(const FoldTabArgs *__restrict__ jobs) {
+    const FoldTabArgs &T = jobs[blockIdx.y];
+    if (!T.fold->any) return;
+    fold_table_rows(T, blockIdx.x, gridDim.x);
+}
+
+static FoldTabArgs fold_tab_args(vup_grid g, int64_t K) {
+    FoldTabArgs T{};
+    T.fold = g->fold;
+    T.sel = g->hist_sel;
+    T.start = g->fold_start;
+    T.members = g->fold_members;
+    T.ftab = (const float *)g->ftab.p;
+    T.out = (float *)g->ftab_fold.p;
+    T.K_pad = ceil_div64(K, 128) * 128;
+    T.ndim = g->ndim;
+    for (int d = 0; d < 3; ++d) T.n[d] = d < g->ndim ? g->n[d] : 0;
+    return T;
+}
+
+vup_status vup_reserve_fold(vup_grid g, int64_t K) {
+    int64_t rows = 0;
+    for (int d = 0; d < g->ndim; ++d) rows += fold_cap(g->n[d]);
+    return devbuf_reserve(g->ftab_fold, sizeof(float) * (size_t)rows * (size_t)(ceil_div64(K, 128) * 128));
+}
+
+vup_status vup_fold_tables(vup_grid g, int64_t K, cudaStream_t s, const float *ftab) {
+    FoldTabArgs T = fold_tab_args(g, K);
+    if (ftab) T.ftab = ftab;
+    T.ctr = g->hist_sel + kHistCtr;
+    int64_t rows = 0;
+    for (int d = 0; d < g->ndim; ++d) rows += fold_cap(g->n[d]);
+    const int64_t blocks = std::min<int64_t>(rows * ceil_div64(T.K_pad, 512), (int64_t)vup_num_sms() * 16);
+    VUP_PROF("hist_fold_tables", s, 1);
+    k_fold_tables<<<(unsigned)blocks, 128, 0, s>>>(T);
+    VUP_CHECK_LAUNCH();
+    return VUP_OK;
 }
 
 bool vup_hist_rest_staged(const vup_grid_s *g) {
@@ -1374,7 +1581,7 @@ bool vup_hist_rest_staged(const vup_grid_s *g) {
 }
 
 vup_status vup_hist_fused(vup_grid g, int64_t K, float *hist, cudaStream_t s, const float *ftab,
-                          bool points_only, cudaEvent_t keys_ready, bool prefix_ready) {
+                          bool points_only, cudaEvent_t keys_ready, bool tables_ready) {
     const int nd = g->ndim;
     int64_t rows;
     int P_max;
@@ -1390,57 +1597,23 @@ vup_status vup_hist_fused(vup_grid g, int64_t K, float *hist, cudaStream_t s, co
     // the global-memory fallback walks points whatever the device chose
     points_only = points_only || !in_smem;
     A.points_only = points_only ? 1 : 0;
-    // items: G groups of C / G chunks per part, G dividing C / kGroupChunks,
-    // chosen for the fewest idle SM slots in the last wave (one CTA per SM)
-    const int S = A.C / kGroupChunks, nkt = (int)ceil_div64(K, kKT), sms = vup_num_sms();
-    int G = S;
-    double best = -1.0;
-    for (int gg = S; gg >= 1; --gg) {
-        if (S % gg) continue;
-        const int64_t items = (int64_t)P_max * gg * nkt;
-        const double eff = (double)items / (double)(ceil_div64(items, sms) * sms);
-        if (eff > best + 0.02) {
-            best = eff;
-            G = gg;
-        }
-    }
-    A.group_chunks = A.C / G;
-    const int n_items = P_max * G * nkt;
-    // record stream: S items per part, each a range of its record chunks, S for
-    // the fullest last wave
-    int Sr = 1;
-    {
-        double best_r = -1.0;
-        for (int ss = 1; ss <= std::max(1, A.C_rec / hist_warps(3)); ++ss) {  // at least a chunk per warp
-            const int64_t items = (int64_t)P_max * ss * nkt;
-            const double eff = (double)items / (double)(ceil_div64(items, sms) * sms);
-            if (eff > best_r + 0.02) {
-                best_r = eff;
-                Sr = ss;
-            }
-        }
-    }
-    A.rec_sets = Sr;
-    const int n_items_rec = P_max * Sr * nkt;
-    if (in_smem && !points_only && !ftab) {
-        // prefix-sum tiles for the interval and record streams (the kernel
-        // returns at once when the device chose the point stream)
-        A.prefix = (const float *)g->hist_prefix.p;
-        A.pre_rows = rows + 1;
-        if (!prefix_ready) {
-            VUP_PROF("hist_prefix", s, 1);
-            k_prefix_tiles<<<(unsigned)(P_max * (A.K_pad / 128)), 128, 0, s>>>(A, (float *)g->hist_prefix.p, 1);
-            VUP_CHECK_LAUNCH();
-        }
+    const int nkt = (int)ceil_div64(K, kKT), sms = vup_num_sms();
+    if (!tables_ready) {
+        vup_status st = vup_fold_tables(g, K, s, ftab);
+        if (st != VUP_OK) return st;
     }
     {
         VUP_PROF("hist_segmented", s, in_smem && !points_only ? 3 : 1);
         if (in_smem) {
-            auto launch = [&](auto kern, int gg, int items, int mode) -> vup_status {
-                const size_t sm_bytes = hist_smem_bytes(rows, hist_warps(mode)) + (mode == 4 ? rest_bytes : 0);
+            // (at most one item per part, density tile and chunk)
+            const int64_t most = (int64_t)P_max * nkt * std::max(A.C, A.C_rec);
+            const unsigned ctas = (unsigned)std::min<int64_t>(sms, most);
+            auto launch = [&](auto kern, int mode) -> vup_status {
+                const size_t sm_bytes =
+                    hist_smem_bytes(rows, hist_warps(mode)) + (hist_staged(mode) ? rest_bytes : 0);
                 VUP_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_bytes));
-                VUP_CHECK_CUDA(launch_pdl(kern, dim3(items), dim3(hist_warps(mode) * 32), sm_bytes, s, A, rows,
-                                          P_max, gg, items));
+                VUP_CHECK_CUDA(launch_pdl(kern, dim3(ctas), dim3(hist_warps(mode) * 32), sm_bytes, s, A, rows, nkt,
+                                          (int *)g->hist_sel + kHistCtr + hist_stream_of(mode)));
                 return VUP_OK;
             };
             vup_status st;
@@ -1450,24 +1623,34 @@ vup_status vup_hist_fused(vup_grid g, int64_t K, float *hist, cudaStream_t s, co
                 for (int l = 0; l < g->n_layouts; ++l) rest_rows = std::max(rest_rows, g->N / g->hl[l].n_last);
                 if (nd == 3) rest_rows = g->n[0] + g->n[1];
                 const bool l2_rest = (double)rest_rows * A.K_pad * 4.0 <= 96.0 * 1024 * 1024;
-                if (l2_rest)
-                    st = nd == 3 ? launch(k_hist_smem<2, 3>, Sr, n_items_rec, 3)
-                                 : launch(k_hist_smem<1, 3>, Sr, n_items_rec, 3);
-                else
-                    st = nd == 3 ? launch(k_hist_smem<2, 2>, Sr, n_items_rec, 2)
-                                 : launch(k_hist_smem<1, 2>, Sr, n_items_rec, 2);
+                if (A.rest_smem) st = launch(k_hist_smem<2, 5>, 5);
+                else if (l2_rest) st = nd == 3 ? launch(k_hist_smem<2, 3>, 3) : launch(k_hist_smem<1, 3>, 3);
+                else st = nd == 3 ? launch(k_hist_smem<2, 2>, 2) : launch(k_hist_smem<1, 2>, 2);
                 if (st != VUP_OK) return st;
             }
             if (keys_ready) VUP_CHECK_CUDA(cudaStreamWaitEvent(s, keys_ready, 0));
-            st = nd == 3 ? (A.rest_smem ? launch(k_hist_smem<2, 4>, G, n_items, 4)
-                                        : launch(k_hist_smem<2, 0>, G, n_items, 0))
-                         : launch(k_hist_smem<1, 0>, G, n_items, 0);
+            st = nd == 3 ? (A.rest_smem ? launch(k_hist_smem<2, 4>, 4) : launch(k_hist_smem<2, 0>, 0))
+                         : launch(k_hist_smem<1, 0>, 0);
             if (st != VUP_OK) return st;
             if (!points_only) {
-                st = nd == 3 ? launch(k_hist_smem<2, 1>, G, n_items, 1) : launch(k_hist_smem<1, 1>, G, n_items, 1);
+                st = nd == 3 ? launch(k_hist_smem<2, 1>, 1) : launch(k_hist_smem<1, 1>, 1);
                 if (st != VUP_OK) return st;
             }
         } else {
+            // G groups of C / G chunks per part, G dividing C / kGroupChunks, for the
+            // fewest idle SM slots in the last wave
+            const int S = A.C / kGroupChunks;
+            int G = S;
+            double best = -1.0;
+            for (int gg = S; gg >= 1; --gg) {
+                if (S % gg) continue;
+                const int64_t items = (int64_t)P_max * gg * nkt;
+                const double eff = (double)items / (double)(ceil_div64(items, sms) * sms);
+                if (eff > best + 0.02) {
+                    best = eff;
+                    G = gg;
+                }
+            }
             if (keys_ready) VUP_CHECK_CUDA(cudaStreamWaitEvent(s, keys_ready, 0));
             dim3 grd((unsigned)(P_max * G), (unsigned)nkt);
             k_hist_global<<<grd, kHistWarps * 32, 0, s>>>(A, G);
@@ -1499,6 +1682,7 @@ bool vup_hist_batchable(vup_grid g) {
 // instance's (part, chunk group, density tile) items, longest first, and one
 // finishing launch.
 struct HistPlan {
+    DevBuf fold;                      // FoldTabArgs of every instance
     DevBuf args, items, fitems, ctr;  // ctr: next item of each stream's launch, then each stream's item count
     DevBuf lists;                     // [3][n_items] each stream's items (k_hist_split_items)
     int n_inst = 0, n_items = 0, n_fitems = 0;
@@ -1516,9 +1700,8 @@ vup_status vup_hist_plan(int n, const vup_grid *gs, const int64_t *Ks, float *co
         args[i] = hist_args_for(gs[i], Ks[i], hists[i], rows, P_max);
         if (!hists[i]) continue;
         rows_max = std::max(rows_max, rows);
-        args[i].group_chunks = kGroupChunks;
         const int G = args[i].C / kGroupChunks;
-        args[i].rec_sets = G;  // record stream: item cg takes the cg-th of G ranges of the part's record chunks
+        args[i].sets = G;
         const int64_t nkt = ceil_div64(Ks[i], kKT);
         // cost of one item: points per chunk x densities per tile
         const int64_t cost = gs[i]->N / std::max<int64_t>(1, (int64_t)P_max * args[i].C);
@@ -1537,12 +1720,16 @@ vup_status vup_hist_plan(int n, const vup_grid *gs, const int64_t *Ks, float *co
     P->n_fitems = (int)fin.size();
     P->rows = rows_max;
     vup_status st;
+    std::vector<FoldTabArgs> folds(n);
+    for (int i = 0; i < n; ++i) folds[i] = fold_tab_args(gs[i], Ks[i]);
     if ((st = devbuf_reserve(P->args, sizeof(HistArgs) * n)) != VUP_OK ||
+        (st = devbuf_reserve(P->fold, sizeof(FoldTabArgs) * n)) != VUP_OK ||
         (st = devbuf_reserve(P->items, sizeof(HistItem) * std::max<size_t>(1, items.size()))) != VUP_OK ||
         (st = devbuf_reserve(P->fitems, sizeof(int4) * std::max<size_t>(1, fin.size()))) != VUP_OK ||
         (st = devbuf_reserve(P->ctr, sizeof(int) * 6)) != VUP_OK ||
         (st = devbuf_reserve(P->lists, sizeof(int32_t) * 3 * std::max<size_t>(1, items.size()))) != VUP_OK) {
         devbuf_free(P->args);
+        devbuf_free(P->fold);
         devbuf_free(P->items);
         devbuf_free(P->fitems);
         devbuf_free(P->ctr);
@@ -1551,6 +1738,7 @@ vup_status vup_hist_plan(int n, const vup_grid *gs, const int64_t *Ks, float *co
         return st;
     }
     VUP_CHECK_CUDA(cudaMemcpy(P->args.p, args.data(), sizeof(HistArgs) * n, cudaMemcpyHostToDevice));
+    VUP_CHECK_CUDA(cudaMemcpy(P->fold.p, folds.data(), sizeof(FoldTabArgs) * n, cudaMemcpyHostToDevice));
     VUP_CHECK_CUDA(cudaMemcpy(P->items.p, items.data(), sizeof(HistItem) * items.size(), cudaMemcpyHostToDevice));
     VUP_CHECK_CUDA(cudaMemcpy(P->fitems.p, fin.data(), sizeof(int4) * fin.size(), cudaMemcpyHostToDevice));
     // the largest tile any plan may use, so that graphs of earlier plans stay launchable
@@ -1568,6 +1756,7 @@ void vup_hist_plan_free(void *plan) {
     HistPlan *P = (HistPlan *)plan;
     if (!P) return;
     devbuf_free(P->args);
+    devbuf_free(P->fold);
     devbuf_free(P->items);
     devbuf_free(P->fitems);
     devbuf_free(P->ctr);
@@ -1581,7 +1770,12 @@ vup_status vup_hist_batched(void *plan, cudaStream_t s) {
     const size_t smem = hist_smem_bytes(P->rows);
     if (smem > 220 * 1024) return VUP_ERR_UNSUPPORTED;
     {
-        VUP_PROF("hist_segmented_batched", s, 4);
+        VUP_PROF("hist_segmented_batched", s, 5);
+        for (int i0 = 0; i0 < P->n_inst; i0 += 65535) {  // (the grid's y limit)
+            const unsigned ny = (unsigned)std::min(65535, P->n_inst - i0);
+            k_fold_tables_batched<<<dim3(32, ny), 128, 0, s>>>((const FoldTabArgs *)P->fold.p + i0);
+            VUP_CHECK_LAUNCH();
+        }
         const int grid = std::max(1, std::min(P->n_items, vup_num_sms()));
         int *ctr = (int *)P->ctr.p, *counts = ctr + 3;
         const int32_t *lists = (const int32_t *)P->lists.p;

@@ -197,6 +197,30 @@ struct Orient {
 // derivatives of axis 1).
 enum { kOrientLast = 0, kOrientFirst = 1, kNumOrient = 2 };
 
+// Histogram grid with equal slices folded (device memory, rewritten with every
+// layout build).  Two indices of one axis whose slices of the bin grid are
+// equal (every point of one falls in the bin of its counterpart: mirror
+// images of an even or periodic model, an axis the model ignores) contribute
+// to the same bins, and a product density's weights factor over axes, so
+//   sum_i W[k,i] 1[bin_i = b]
+// keeps its value when the slices are merged into one whose factor is the sum
+// of theirs.  The histogram runs on the merged grid: its layout, its walks
+// and its factor tables (class c of a folded axis: the sum of its members'
+// factors).  Nothing is assumed of the model; slices are compared point by
+// point.  An axis is folded when its classes number at most 5/8 of its
+// indices (a mirror symmetry halves it), since a merged table costs one read
+// of the axis' factors.
+struct FoldGeom {
+    int64_t n[3];                   // merged sizes (the grid's own where an axis is not folded)
+    int64_t N;                      // their product
+    int64_t n_last[2], part_rows[2];  // layouts' gathered axis and its parts
+    int32_t P[2];
+    int32_t folded[3];              // 1: the axis' merged factor table is used
+    int32_t any;
+};
+constexpr int32_t kFoldLast = 1 << 30;  // flags the last member of a class in its list
+__host__ __device__ inline int64_t fold_cap(int64_t n) { return (5 * n + 7) / 8; }  // most classes of a folded axis
+
 struct vup_grid_s {
     int device = 0;
     int ndim = 0;
@@ -228,8 +252,8 @@ struct vup_grid_s {
     // (forked from and joined back into the caller's stream)
     cudaStream_t side = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_rec = nullptr;
-    cudaStream_t side2 = nullptr;                       // the prefix-sum tiles beside the contraction
-    cudaEvent_t ev_lay = nullptr, ev_dens = nullptr, ev_pre = nullptr, ev_mom = nullptr, ev_mfin = nullptr;
+    cudaStream_t side2 = nullptr;                       // the FP64 moments finish beside the histogram
+    cudaEvent_t ev_lay = nullptr, ev_mom = nullptr, ev_mfin = nullptr;
 
     // counting-sort scratch
     DevBuf sort_counts, scan_tmp, lay_tmp, rec_tmp;
@@ -276,9 +300,20 @@ struct vup_grid_s {
         int32_t *rec_chunk_grp = nullptr;  // [P * n_chunks_rec * 2] first / last group of each chunk
         int32_t *n_rec = nullptr;      // [1] device
     } hl[2];
+    // equal-slice folding of the bin grid (2-D / 3-D): one allocation holding
+    // the device geometry, the class members per axis (CSR: start, members),
+    // the build's scratch (zeroed first) and the merged bins
+    void *fold_mem = nullptr;
+    FoldGeom *fold = nullptr;
+    int32_t *fold_rep = nullptr, *fold_start = nullptr, *fold_members = nullptr, *fold_bins = nullptr;
+    uint8_t *fold_scratch = nullptr;
+    size_t fold_scratch_bytes = 0;
+    int layout_unfolded = 0;       // the current layout was built without folding (vup_grid_info's counts)
     int hist_P = 1;                // max parts over layouts (scratch sizing)
     int n_layouts = 1;
-    int32_t *hist_sel = nullptr;   // [4] device: chosen layout, 1 = interval stream, intervals of layouts 0 / 1
+    // [8] device: chosen layout, stream, intervals of layouts 0 / 1, key streams built,
+    // item counters of the three streams' walks
+    int32_t *hist_sel = nullptr;
     int hist_force = -1;           // -1 auto, 0 points only, 1 intervals only
     int32_t n_chunks = 0;
     int32_t n_chunks_rec = 0;      // record chunks per part (records are several times fewer than points)
@@ -296,7 +331,7 @@ struct vup_grid_s {
     // per-K scratch (density constants, factor tables, partials)
     int64_t K_cap = 0;
     DevBuf dconst, dstats, dpart, ftab, atab_hi, atab_lo, partials, hist_part, hist_direct, ipsa_part;
-    DevBuf hist_prefix;  // prefix-sum tiles of the gathered axis [P][K_pad / 128][rows + 1][128]
+    DevBuf ftab_fold;    // merged factor tables of the folded axes, axis d at fold_off(d) rows of K_pad
     DevBuf atf_hi, atf_lo;         // TF32 split of the A operand [K_pad][R_pad]
 
     // supplied-weights path: the grid points in blocks of 256, each block's
@@ -322,8 +357,10 @@ vup_status vup_pick_hist_layout(vup_grid g, cudaStream_t s);
 // records_done (optional) is recorded on s once the record stream is complete
 // (the key-sorted streams follow); layout_picked (optional) once the layout
 // (hist_sel[0]) is chosen.
+// fold: merge equal slices of the bin grid first (FoldGeom).
 vup_status vup_build_layout(vup_grid g, cudaStream_t s, bool points_needed = false,
-                            cudaEvent_t records_done = nullptr, cudaEvent_t layout_picked = nullptr);
+                            cudaEvent_t records_done = nullptr, cudaEvent_t layout_picked = nullptr,
+                            bool fold = true);
 vup_status vup_ensure_layout(vup_grid g, cudaStream_t s, bool points_needed = false);
 // every layout's part tile fits the shared-memory histogram kernels
 bool vup_hist_tile_fits(vup_grid g);
@@ -354,15 +391,15 @@ vup_status vup_moments_finish(vup_grid g, int64_t K, int n_col_tiles, double *ra
 // the numerators and denominators of ratios do).
 // keys_ready (optional): an event the point and interval kernels (and the
 // finish) wait for; the record-stream kernel is launched before that wait.
-// prefix_ready: vup_hist_prefix already wrote the prefix-sum tiles for
-// these densities (on a stream s has waited for).
+// tables_ready: vup_fold_tables already ran for these densities.
 vup_status vup_hist_fused(vup_grid g, int64_t K, float *hist, cudaStream_t s, const float *ftab = nullptr,
-                          bool points_only = false, cudaEvent_t keys_ready = nullptr, bool prefix_ready = false);
-// The interval and record streams' prefix-sum tiles of the chosen layout for K
-// densities (after their preparation and the layout choice), whichever
-// stream the device picks later; false when the grid's histogram does not
-// run the shared-memory kernels (nothing launched).
-bool vup_hist_prefix(vup_grid g, int64_t K, cudaStream_t s);
+                          bool points_only = false, cudaEvent_t keys_ready = nullptr, bool tables_ready = false);
+// Merged factor tables of the folded rest axes (nothing to do where none is
+// folded), read by the walks, whose item counters the call also zeroes;
+// scratch for them.
+vup_status vup_fold_tables(vup_grid g, int64_t K, cudaStream_t s, const float *ftab = nullptr);
+vup_status vup_reserve_fold(vup_grid g, int64_t K);
+size_t vup_fold_scratch_bytes(const vup_grid_s *g);
 vup_status vup_propagate_1d(vup_grid g, const vup_densities *d, double *raw, double *central,
                             float *hist, cudaStream_t s);
 vup_status vup_ipsa_1d(vup_grid g, const vup_densities *d, const double *grad, float *dmu,
