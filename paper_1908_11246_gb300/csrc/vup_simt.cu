@@ -67,73 +67,91 @@ __device__ __forceinline__ float epi_weight(const EpiArgs &ep, int64_t K_pad, in
     return e;
 }
 
-// One 128 (densities) x 128 (columns (q, j)) tile.  Each thread owns 8 rows
-// x 8 columns (2 rest points x 4 powers): the GEMM part accumulates kChain
-// reduction terms per plain FP32 chain, then folds the chain into
-// out[row][j] += w(row, q) * chain with Kahan compensation; the 16 column
-// threads of a row are reduced in FP64 and the tile writes one FP32 partial
-// per (row, power) for the FP64 finish.
+// One tile of TM densities x 128 columns (q, j).  Each thread owns 4 densities x
+// 8 columns (2 rest points x 4 powers): the GEMM part accumulates kChain
+// reduction terms per plain FP32 chain, then folds the chain into out[density][j]
+// += w(density, q) * chain with Kahan compensation; the 16 column threads of a
+// row are reduced in FP64 and the tile writes one FP32 partial per (row, power)
+// for the FP64 finish.
+//
+// The FP32 pipes bound it: a chain costs 8 multiply-adds and 4 operations of
+// fold, so at most 2/3 of the multiply-add rate.  4 x 8 values per thread leave
+// room for 16 warps per SM (8 x 8 values, 8 warps: 888 us at 900 x 1100 points, K
+// = 3000; packed FP32 pairs: 1169; this form: 814).  NPL = 3 forms the IPSA sums
+// (weights e, e u, e u^2) from one set of chains, 8 + 12 operations per chain
+// instead of 3 (8 + 4), on tiles of 64 densities (the three planes' sums take
+// the registers; 500 x 400 points, K = 2000, both orientations: 1009 -> 590 us).
+template <int NPL>
+struct SimtShape {
+    static constexpr int kTM = NPL == 3 ? 64 : 128;  // densities of a tile
+    static constexpr int kThreads = 4 * kTM;
+};
+template <int NPL>
 __device__ __forceinline__ void simt_tile(const float *__restrict__ A, const float *__restrict__ Zt, int64_t R,
                                           int64_t K_pad, int64_t ldz, const EpiArgs &ep, int64_t n_ct,
-                                          float *__restrict__ part, int64_t ct, int64_t row_tile, int wmode) {
-    __shared__ __align__(16) float As[2][BK][BM];
+                                          float *__restrict__ part, int64_t ct, int64_t row_tile) {
+    constexpr int TM = SimtShape<NPL>::kTM, kT = SimtShape<NPL>::kThreads;
+    constexpr int NB = BN * BK / 4 / kT;  // 16-byte pieces of the column tile per thread (one of the density tile)
+    __shared__ __align__(16) float As[2][BK][TM];
     __shared__ __align__(16) float Bs[2][BK][BN];
     const int tid = threadIdx.x;
     const int tx = tid & 15, ty = tid >> 4;
-    const int64_t k0 = row_tile * BM;
+    const int64_t k0 = row_tile * TM;
     const int64_t c0 = ct * BN;
-    auto row_of = [&](int i) { return k0 + (i < 4 ? ty * 4 + i : 64 + ty * 4 + (i - 4)); };
 
     // epilogue weights of the thread's rows and rest points, fixed for the tile
-    float w[8][2];
+    float w[NPL][4][2];
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
+    for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int gq = 0; gq < 2; ++gq) w[i][gq] = epi_weight(ep, K_pad, row_of(i), c0 / 4 + gq * 16 + tx, wmode);
+        for (int gq = 0; gq < 2; ++gq)
+#pragma unroll
+            for (int pl = 0; pl < NPL; ++pl) w[pl][i][gq] = epi_weight(ep, K_pad, k0 + ty * 4 + i, c0 / 4 + gq * 16 + tx, pl);
 
-    float acc[8][8];
-    float out[8][4], cmp[8][4];
+    float acc[4][8];
+    float out[NPL][4][4], cmp[NPL][4][4];
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
+    for (int pl = 0; pl < NPL; ++pl)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) out[i][j] = cmp[i][j] = 0.f;
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) out[pl][i][j] = cmp[pl][i][j] = 0.f;
     auto fold = [&]() {
 #pragma unroll
-        for (int i = 0; i < 8; ++i)
+        for (int pl = 0; pl < NPL; ++pl)
 #pragma unroll
-            for (int j = 0; j < 4; ++j)
+            for (int gq = 0; gq < 2; ++gq)
 #pragma unroll
-                for (int gq = 0; gq < 2; ++gq) {
-                    const float yv = fmaf(w[i][gq], acc[i][gq * 4 + j], -cmp[i][j]);
-                    const float t = out[i][j] + yv;
-                    cmp[i][j] = (t - out[i][j]) - yv;
-                    out[i][j] = t;
-                }
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const float yv = fmaf(w[pl][i][gq], acc[i][gq * 4 + j], -cmp[pl][i][j]);
+                        const float t = out[pl][i][j] + yv;
+                        cmp[pl][i][j] = (t - out[pl][i][j]) - yv;
+                        out[pl][i][j] = t;
+                    }
     };
 
-    float4 ra[2], rb[2];
+    float4 ra, rb[NB];
     auto load_regs = [&](int64_t r0) {
+        const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+        {
+            const int64_t r = r0 + tid / (TM / 4);
+            ra = r < R ? *reinterpret_cast<const float4 *>(A + r * K_pad + k0 + (tid % (TM / 4)) * 4) : zero;
+        }
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int e = tid + h * 256;
-            const int row = e >> 5, c4 = e & 31;
-            const int64_t r = r0 + row;
-            if (r < R) {
-                ra[h] = *reinterpret_cast<const float4 *>(A + r * K_pad + k0 + c4 * 4);
-                rb[h] = *reinterpret_cast<const float4 *>(Zt + r * ldz + c0 + c4 * 4);
-            } else {
-                ra[h] = make_float4(0.f, 0.f, 0.f, 0.f);
-                rb[h] = ra[h];
-            }
+        for (int h = 0; h < NB; ++h) {
+            const int e = tid + h * kT;
+            const int64_t r = r0 + (e >> 5);
+            rb[h] = r < R ? *reinterpret_cast<const float4 *>(Zt + r * ldz + c0 + (e & 31) * 4) : zero;
         }
     };
     auto store_smem = [&](int buf) {
+        *reinterpret_cast<float4 *>(&As[buf][tid / (TM / 4)][(tid % (TM / 4)) * 4]) = ra;
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int e = tid + h * 256;
-            const int row = e >> 5, c4 = e & 31;
-            *reinterpret_cast<float4 *>(&As[buf][row][c4 * 4]) = ra[h];
-            *reinterpret_cast<float4 *>(&Bs[buf][row][c4 * 4]) = rb[h];
+        for (int h = 0; h < NB; ++h) {
+            const int e = tid + h * kT;
+            *reinterpret_cast<float4 *>(&Bs[buf][e >> 5][(e & 31) * 4]) = rb[h];
         }
     };
 
@@ -146,19 +164,18 @@ __device__ __forceinline__ void simt_tile(const float *__restrict__ A, const flo
         if (rt + 1 < n_rt) load_regs((rt + 1) * BK);
 #pragma unroll
         for (int kk = 0; kk < BK; ++kk) {
-            float a[8], b[8];
+            float a[4], b[8];
             *reinterpret_cast<float4 *>(&a[0]) = *reinterpret_cast<const float4 *>(&As[buf][kk][ty * 4]);
-            *reinterpret_cast<float4 *>(&a[4]) = *reinterpret_cast<const float4 *>(&As[buf][kk][64 + ty * 4]);
             *reinterpret_cast<float4 *>(&b[0]) = *reinterpret_cast<const float4 *>(&Bs[buf][kk][tx * 4]);
             *reinterpret_cast<float4 *>(&b[4]) = *reinterpret_cast<const float4 *>(&Bs[buf][kk][64 + tx * 4]);
             if (kk % kChain == 0) {
 #pragma unroll
-                for (int i = 0; i < 8; ++i)
+                for (int i = 0; i < 4; ++i)
 #pragma unroll
                     for (int j = 0; j < 8; ++j) acc[i][j] = a[i] * b[j];
             } else {
 #pragma unroll
-                for (int i = 0; i < 8; ++i)
+                for (int i = 0; i < 4; ++i)
 #pragma unroll
                     for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
             }
@@ -172,38 +189,42 @@ __device__ __forceinline__ void simt_tile(const float *__restrict__ A, const flo
 
     // reduce over the 16 column threads of a half-warp (FP64)
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        double v[4];
+    for (int pl = 0; pl < NPL; ++pl)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            v[j] = (double)out[i][j] - (double)cmp[i][j];
-            v[j] += __shfl_xor_sync(0xffffffffu, v[j], 8);
-            v[j] += __shfl_xor_sync(0xffffffffu, v[j], 4);
-            v[j] += __shfl_xor_sync(0xffffffffu, v[j], 2);
-            v[j] += __shfl_xor_sync(0xffffffffu, v[j], 1);
+        for (int i = 0; i < 4; ++i) {
+            double v[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                v[j] = (double)out[pl][i][j] - (double)cmp[pl][i][j];
+                v[j] += __shfl_xor_sync(0xffffffffu, v[j], 8);
+                v[j] += __shfl_xor_sync(0xffffffffu, v[j], 4);
+                v[j] += __shfl_xor_sync(0xffffffffu, v[j], 2);
+                v[j] += __shfl_xor_sync(0xffffffffu, v[j], 1);
+            }
+            if (tx == 0)
+                *reinterpret_cast<float4 *>(part + (((int64_t)pl * n_ct + ct) * K_pad + k0 + ty * 4 + i) * 4) =
+                    make_float4((float)v[0], (float)v[1], (float)v[2], (float)v[3]);
         }
-        if (tx == 0)
-            *reinterpret_cast<float4 *>(part + (((int64_t)wmode * n_ct + ct) * K_pad + row_of(i)) * 4) =
-                make_float4((float)v[0], (float)v[1], (float)v[2], (float)v[3]);
-    }
 }
 
-// wmode 0: moments; 1, 2: the IPSA sums with weights e u and e u^2 (one
-// launch each, into partial slice wmode).
-__global__ void __launch_bounds__(256, 1)
+template <int NPL>
+__global__ void __launch_bounds__(SimtShape<NPL>::kThreads, 1)
 k_moments_simt(const float *__restrict__ A, const float *__restrict__ Zt, int64_t R, int64_t K_pad,
-               int64_t ldz, EpiArgs ep, int64_t n_ct, float *__restrict__ part, int wmode) {
-    simt_tile(A, Zt, R, K_pad, ldz, ep, n_ct, part, blockIdx.x, blockIdx.y, wmode);
+               int64_t ldz, EpiArgs ep, int64_t n_ct, float *__restrict__ part) {
+    // three planes (2-D grids: at most 1024 column tiles, but up to 65536 tiles of 64
+    // densities) put the densities on x, whose limit is larger
+    if (NPL == 3) simt_tile<NPL>(A, Zt, R, K_pad, ldz, ep, n_ct, part, blockIdx.y, blockIdx.x);
+    else simt_tile<NPL>(A, Zt, R, K_pad, ldz, ep, n_ct, part, blockIdx.x, blockIdx.y);
 }
 
 // Batched form: one persistent launch over the tiles of many instances,
 // longest reductions first (items[t] = (instance, column tile, row tile)).
-__global__ void __launch_bounds__(256, 1)
+__global__ void __launch_bounds__(SimtShape<1>::kThreads, 1)
 k_moments_simt_batched(const SimtJob *__restrict__ jobs, const int4 *__restrict__ items, int n_items) {
     for (int t = blockIdx.x; t < n_items; t += gridDim.x) {
         const int4 it = items[t];
         const SimtJob J = jobs[it.x];
-        simt_tile(J.A, J.Zt, J.R, J.K_pad, J.ldz, J.ep, J.n_ct, J.part, it.y, it.z, 0);
+        simt_tile<1>(J.A, J.Zt, J.R, J.K_pad, J.ldz, J.ep, J.n_ct, J.part, it.y, it.z);
         __syncthreads();
     }
 }
@@ -401,12 +422,14 @@ vup_status vup_moments_simt(vup_grid g, int64_t K, int orient, int n_out, float 
     const int64_t n_ct = vup_simt_col_tiles(o);
     const int64_t ldz = ceil_div64(o.NC, 128) * 128;
     EpiArgs ep = epi_for(g, orient, K_pad);
-    dim3 grd((unsigned)n_ct, (unsigned)(K_pad / BM));
-    VUP_PROF(n_out == 1 ? "moments_fp32_simt" : "ipsa_fp32_simt", s, n_out);
-    for (int wm = 0; wm < n_out; ++wm) {
-        k_moments_simt<<<grd, 256, 0, s>>>(A, g->zs[orient], o.R, K_pad, ldz, ep, n_ct, part, wm);
-        VUP_CHECK_LAUNCH();
-    }
+    VUP_PROF(n_out == 1 ? "moments_fp32_simt" : "ipsa_fp32_simt", s, 1);
+    if (n_out == 1)
+        k_moments_simt<1><<<dim3((unsigned)n_ct, (unsigned)(K_pad / SimtShape<1>::kTM)), SimtShape<1>::kThreads, 0, s>>>(
+            A, g->zs[orient], o.R, K_pad, ldz, ep, n_ct, part);
+    else
+        k_moments_simt<3><<<dim3((unsigned)(K_pad / SimtShape<3>::kTM), (unsigned)n_ct), SimtShape<3>::kThreads, 0, s>>>(
+            A, g->zs[orient], o.R, K_pad, ldz, ep, n_ct, part);
+    VUP_CHECK_LAUNCH();
     return VUP_OK;
 }
 
@@ -492,9 +515,9 @@ void vup_simt_plan_free(void *plan) {
 vup_status vup_simt_batched(void *plan, cudaStream_t s) {
     const SimtPlan *P = (const SimtPlan *)plan;
     if (P->n_items == 0) return VUP_OK;
-    const int grid = std::min(P->n_items, 2 * vup_num_sms());
+    const int grid = std::min(P->n_items, vup_num_sms());
     VUP_PROF("moments_fp32_simt_batched", s, 1);
-    k_moments_simt_batched<<<grid, 256, 0, s>>>((const SimtJob *)P->jobs.p, (const int4 *)P->items.p, P->n_items);
+    k_moments_simt_batched<<<grid, SimtShape<1>::kThreads, 0, s>>>((const SimtJob *)P->jobs.p, (const int4 *)P->items.p, P->n_items);
     VUP_CHECK_LAUNCH();
     return VUP_OK;
 }
