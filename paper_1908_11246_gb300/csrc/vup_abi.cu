@@ -280,6 +280,8 @@ static void free_grid(vup_grid g) {
     devbuf_free(g->hist_part);
     devbuf_free(g->hist_direct);
     devbuf_free(g->ftab_fold);
+    devbuf_free(g->post_tmp);
+    devbuf_free(g->post_x);
     devbuf_free(g->ipsa_part);
     devbuf_free(g->atf_hi);
     devbuf_free(g->atf_lo);

@@ -4,8 +4,9 @@
 // coordinates: the posterior mean of every input axis per output bin,
 //   post[k][b][d] = sum_{i in b} W[k,i] x_{d,i} / H[k,b].
 // The numerators are histograms of the densities with one axis' factor
-// table multiplied by that axis' coordinates, so each axis is one more pass
-// of the segmented histogram kernel; W is never formed.
+// table multiplied by that axis' coordinates; one walk of the point stream
+// forms them with H (vup_post_fused), or one pass each where the grid's tiles
+// do not fit shared memory.  W is never formed.
 #include "vup_internal.cuh"
 
 namespace {
@@ -44,16 +45,22 @@ extern "C" vup_status vup_posterior_means(vup_grid g, const vup_densities *d, fl
     const int64_t K = d->K, K_pad = ceil_div64(K, 128) * 128;
     const int B = g->B, nd = g->ndim;
     const size_t tab = (size_t)K_pad * vup_ftab_floats(g);
+    const bool one_pass = vup_hist_tile_fits(g);
     if ((st = vup_reserve_k(g, K, false, false)) != VUP_OK) return st;
     if ((st = vup_reserve_fold(g, K)) != VUP_OK) return st;
-    if ((st = devbuf_reserve(g_xtab, sizeof(float) * tab)) != VUP_OK) return st;
-    if ((st = devbuf_reserve(g_hx, sizeof(float) * (size_t)nd * K * B)) != VUP_OK) return st;
-    if (!hist) {
+    // a grid whose tiles do not fit shared memory: one histogram pass per axis
+    if (!one_pass && (st = devbuf_reserve(g_xtab, sizeof(float) * tab)) != VUP_OK) return st;
+    if (!one_pass && (st = devbuf_reserve(g_hx, sizeof(float) * (size_t)nd * K * B)) != VUP_OK) return st;
+    if (!one_pass && !hist) {
         if ((st = devbuf_reserve(g_hist, sizeof(float) * (size_t)K * B)) != VUP_OK) return st;
         hist = (float *)g_hist.p;
     }
     if ((st = vup_ensure_layout(g, s, true)) != VUP_OK) return st;  // the ratios walk the point stream
     if ((st = vup_density_prep(g, d, 0, s)) != VUP_OK) return st;
+    if (one_pass) {
+        bool done = false;
+        return vup_post_fused(g, K, hist, post, s, done);
+    }
     // point stream: the ratios need the relative accuracy of low-mass bins,
     // which differences of prefix sums (interval stream) do not keep
     if ((st = vup_hist_fused(g, K, hist, s, nullptr, true)) != VUP_OK) return st;

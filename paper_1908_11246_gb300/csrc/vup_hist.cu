@@ -1383,6 +1383,372 @@ __global__ void __launch_bounds__(256, 3) k_hist_finish_batched(const HistArgs *
     hist_finish_tiles(insts[it.x], (int64_t)it.y * kFinNK, it.z);
 }
 
+// ---- posterior sums ------------------------------------------------------------
+// One point-stream pass for everything the posterior means need: per bin the
+// sums of W and of W x_d for every axis d.  A CTA takes 64 densities: a tile
+// row holds, per lane, the factors of its two densities and the same times the
+// gathered axis' coordinate (a merged row: summed over its members), so one
+// 16-byte gather per point gives both; a run's two sums S0 = sum w and S1 =
+// sum w x are multiplied at its end by the rest axes' factors (H += f S0, the
+// gathered axis' sum += f S1, a rest axis' sum += f_x S0 with f_x its factor
+// times its coordinate).  Separate passes per axis gathered every point once for each
+// (three times on 2-D grids) and re-read the weighted tables: 1024 x 1024
+// points, K = 8192: 4.88 ms, 1.14 with equal slices merged, 0.59 in one pass.
+struct PostArgs {
+    HistArgs h;              // the histogram's arguments (tables, layout, scratch sizes)
+    const float *xs;         // coordinates of every axis, axis d from off[d]
+    const float *fx;         // rest factors times coordinate (merged), axis d at off[d] rows
+    float *part, *direct;    // [cut row or key][1 + ndim][K_pad]
+    float *hist, *post;      // [K][B] (or null), [K][B][ndim]
+};
+constexpr int kPostKT = 64;
+__device__ __forceinline__ float2 ld2(const float *q) { return *reinterpret_cast<const float2 *>(q); }
+
+// Rest factors f_x (and, of folded axes, the merged f into ftab_fold).
+__global__ void __launch_bounds__(128) k_post_tables(const __grid_constant__ PostArgs A, float *__restrict__ fx,
+                                                     float *__restrict__ f_merged, int *__restrict__ ctr) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) *ctr = 0;
+    const HistArgs &h = A.h;
+    const int64_t K_pad = h.K_pad, kb = (K_pad + 511) / 512;
+    const int gathered = h.ndim == 2 && h.sel[0] ? 0 : h.ndim - 1;
+    for (int d = 0; d < h.ndim; ++d) {
+        if (d == gathered) continue;
+        const bool folded = h.fold->folded[d] != 0;
+        const int64_t rows = h.fold->n[d], off = h.off[d];
+        for (int64_t u = blockIdx.x; u < rows * kb; u += gridDim.x) {
+            const int64_t c = u / kb, k = (u - c * kb) * 512 + 4 * threadIdx.x;
+            if (k >= K_pad) continue;
+            const int32_t *st = h.fold_start + off + d + c, *mem = h.fold_members + off;
+            const int32_t m0 = folded ? st[0] : 0, m1 = folded ? st[1] : 1;
+            PairSum4 f, x;
+            f.clear();
+            x.clear();
+            for (int32_t m = m0; m < m1; ++m) {
+                const int64_t a = folded ? mem[m] & (kFoldLast - 1) : c;
+                const float4 v = ld4(h.ftab + (off + a) * K_pad + k);
+                const float xa = A.xs[off + a];
+                f.add(v);
+                x.add(make_float4(v.x * xa, v.y * xa, v.z * xa, v.w * xa));
+            }
+            *reinterpret_cast<float4 *>(fx + (off + c) * K_pad + k) = x.value();
+            if (folded) *reinterpret_cast<float4 *>(f_merged + (h.foff[d] + c) * K_pad + k) = f.value();
+        }
+    }
+}
+
+// Midpoint coordinates of every axis, rounded once to FP32.
+struct AxisGeom {
+    int ndim;
+    int64_t n[3];
+    double lo[3], h[3];
+};
+__global__ void k_axis_coords(AxisGeom G, float *__restrict__ xs) {
+    int64_t off = 0;
+    for (int d = 0; d < G.ndim; ++d) {
+        for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < G.n[d]; a += (int64_t)gridDim.x * blockDim.x)
+            xs[off + a] = (float)__dadd_rn(G.lo[d], __dmul_rn((double)a + 0.5, G.h[d]));
+        off += G.n[d];
+    }
+}
+
+// Rest factors of one run for a lane's two densities: f, and f with one rest
+// axis' factor weighted by its coordinate.
+template <int NF>
+struct RunFactors {
+    float2 f, fx[NF];
+};
+
+// AHEAD: how many runs ahead a run-end word's rest code points (the layout's).
+template <int NF, int AHEAD>
+__global__ void __launch_bounds__(kHistWarps * 32, 1)
+    k_post_walk(const __grid_constant__ PostArgs A, int64_t tile_rows, int nkt, int *__restrict__ next_item) {
+    constexpr int NO = 2 + NF;  // sums per key: W, W x of the gathered axis, of the rest axes
+    extern __shared__ __align__(128) uint8_t sm[];
+    __shared__ LayoutArgs H;
+    __shared__ float s_iz[kPostKT];
+    __shared__ int abort, next_chunk, s_item, s_G;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t K_pad = A.h.K_pad;
+    const int C = A.h.C;
+    int *dstatus = A.h.dstatus;
+    if (threadIdx.x == 0) {
+        abort = 0;
+        H = pick(A.h);
+    }
+    hist_init_mbar(sm, tile_rows, kHistWarps);
+    uint64_t *mbar = hist_mbar(sm, tile_rows, kHistWarps);
+    float *ws = reinterpret_cast<float *>(sm);
+    uint32_t *win = reinterpret_cast<uint32_t *>(sm + hist_tile_bytes(tile_rows) + (size_t)warp * hist_warp_bytes());
+    __syncthreads();
+    const int P = H.P;
+    if (warp == 0) {
+        const int G = hist_split(A.h.fold->N / P, C, (int64_t)nkt * P, H.part_rows, kHistWarps, hist_rate(0), gridDim.x);
+        if (lane == 0) s_G = G;
+    }
+    uint32_t wseq = 0;
+    for (;;) {
+        __syncthreads();  // the previous item's readers of the tile and of s_item are done
+        if (threadIdx.x == 0) {
+            s_item = atomicAdd(next_item, 1);
+            next_chunk = 0;
+        }
+        __syncthreads();
+        const int G = s_G, it = s_item;
+        if (it >= (int64_t)nkt * P * G || abort) return;  // uniform
+        const int cg = it % G, pk = it / G, p = pk % P;
+        const int64_t k0 = (int64_t)(pk / P) * kPostKT, k = k0 + 2 * lane;
+        if (threadIdx.x < kPostKT) s_iz[threadIdx.x] = inv_z(A.h, k0 + threadIdx.x);
+        __syncthreads();
+        const int64_t row0 = (int64_t)p * H.part_rows;
+        const int32_t nrows = (int32_t)min(H.part_rows, H.n_last - row0);
+        {
+            // this warp's rows: (w, w', w x, w' x) of the lane's two densities, class members summed
+            const float2 iz = make_float2(s_iz[2 * lane], s_iz[2 * lane + 1]);
+            const float *xs = A.xs + A.h.off[H.ax_last], *src = H.g_last + k;
+            const int32_t a0 = nrows * warp / kHistWarps, a1 = nrows * (warp + 1) / kHistWarps;
+            const int32_t *members = H.cls_start ? H.cls_members : nullptr;
+            const int32_t m0 = members ? H.cls_start[row0 + a0] : (int32_t)row0 + a0;
+            const int32_t m1 = members ? H.cls_start[row0 + a1] : (int32_t)row0 + a1;
+            float *dst = ws + (int64_t)a0 * kKT + 4 * lane;
+            PairSum4 c;
+            c.clear();
+            for (int32_t m = m0; m < m1; m += 8) {
+                float2 v[8];
+                float x[8];
+                int32_t r[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    r[u] = m + u < m1 ? (members ? members[m + u] : (m + u) | kFoldLast) : 0;
+                    const int64_t a = r[u] & (kFoldLast - 1);
+                    v[u] = m + u < m1 ? ld2(src + a * K_pad) : make_float2(0.f, 0.f);
+                    x[u] = m + u < m1 ? xs[a] : 0.f;
+                }
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    c.add(make_float4(v[u].x, v[u].y, v[u].x * x[u], v[u].y * x[u]));
+                    if (r[u] & kFoldLast) {
+                        const float4 t = c.value();
+                        *reinterpret_cast<float4 *>(dst) = make_float4(t.x * iz.x, t.y * iz.y, t.z * iz.x, t.w * iz.y);
+                        dst += kKT;
+                        c.clear();
+                    }
+                }
+            }
+            if (threadIdx.x < kKT) ws[(int64_t)nrows * kKT + threadIdx.x] = 0.f;
+        }
+        __syncthreads();
+
+        const float *g0k = H.g0 + k, *x0k = A.fx + A.h.off[H.ax0] * K_pad + k;
+        const float *g1k = NF == 2 ? H.g1 + k : nullptr, *x1k = NF == 2 ? A.fx + A.h.off[H.ax1] * K_pad + k : nullptr;
+        auto factors = [&](uint32_t a0, uint32_t a1) -> RunFactors<NF> {
+            // (debug build: rows outside the factor tables are recorded and read as row 0)
+            if (!VUP_DBG_IN(a0, H.n0, dstatus)) a0 = 0;
+            if (NF == 2 && !VUP_DBG_IN(a1, H.n1, dstatus)) a1 = 0;
+            RunFactors<NF> R;
+            R.f = ld2(g0k + (int64_t)a0 * K_pad);
+            R.fx[0] = ld2(x0k + (int64_t)a0 * K_pad);
+            if constexpr (NF == 2) {
+                const float2 q = ld2(g1k + (int64_t)a1 * K_pad), qx = ld2(x1k + (int64_t)a1 * K_pad);
+                R.fx[1] = make_float2(R.f.x * qx.x, R.f.y * qx.y);
+                R.fx[0] = make_float2(R.fx[0].x * q.x, R.fx[0].y * q.y);
+                R.f = make_float2(R.f.x * q.x, R.f.y * q.y);
+            }
+            return R;
+        };
+        auto coded = [&](uint32_t u) -> RunFactors<NF> {
+            const uint32_t lo = u & 0x1ffu, hi = (u >> 18) & 0xfffu;
+            return NF == 2 ? factors(lo, hi) : factors(lo | (hi << 9), 0u);
+        };
+        const uint32_t wsl = smem_u32(ws) + lane * 16;
+        const uint32_t null_word = (uint32_t)nrows << kRowShift;  // zero row, no flags
+        auto gather = [&](uint32_t word) -> float4 {
+            uint32_t o = word & kOffMask;
+            if (!VUP_DBG_IN(o >> kRowShift, nrows + 1, dstatus)) o = null_word;
+            float4 v;
+            asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                         : "r"(wsl + o));
+            return v;
+        };
+        const int c_end = (int)((int64_t)(cg + 1) * C / G);
+        for (;;) {
+            int ci = 0;
+            if (lane == 0) ci = atomicAdd(&next_chunk, 1);
+            ci = __shfl_sync(0xffffffffu, ci, 0) + (int)((int64_t)cg * C / G);
+            if (ci >= c_end) break;
+            const int c = p * C + ci;
+            const int32_t p0 = H.chunk_pt[c], p1 = H.chunk_pt[c + 1];
+            if (p0 >= p1) continue;
+            const int32_t r0 = H.chunk_run[c], r1 = H.chunk_run[c + 1];
+            // keys cut by the chunk bounds can only be its first and last key
+            const int32_t first_key = H.chunk_bin[2 * c], last_key = H.chunk_bin[2 * c + 1];
+            const bool sh_first = H.koff[first_key] < p0 || H.koff[first_key + 1] > p1;
+            const bool sh_last = H.koff[last_key] < p0 || H.koff[last_key + 1] > p1;
+            const int32_t wb0 = p0 & ~(kWin - 1);
+            if (lane == 0) {
+                const int b0 = wseq & 1;
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // earlier reads of both buffers
+                bulk_copy(win + b0 * kWin, H.hpt + wb0, kWin * 4, &mbar[b0]);
+                if (wb0 + kWin < p1) bulk_copy(win + (b0 ^ 1) * kWin, H.hpt + wb0 + kWin, kWin * 4, &mbar[b0 ^ 1]);
+            }
+            __syncwarp();
+            RunFactors<NF> pf[AHEAD];  // of the current run and the next ones
+#pragma unroll
+            for (int q = 0; q < AHEAD; ++q) {
+                const int32_t rest = r0 + q < r1 ? H.run_rest[r0 + q] : 0;
+                const int32_t a0 = NF == 2 ? rest / (int32_t)H.n1 : rest;
+                pf[q] = factors((uint32_t)a0, NF == 2 ? (uint32_t)(rest - a0 * (int32_t)H.n1) : 0u);
+            }
+            int32_t r = r0, cur_key = first_key;
+            float4 s = make_float4(0.f, 0.f, 0.f, 0.f);  // S0, S1 of the current run
+            float2 acc[NO];
+#pragma unroll
+            for (int o = 0; o < NO; ++o) acc[o] = make_float2(0.f, 0.f);
+            auto flush = [&]() {
+                const bool first = cur_key == first_key;
+                const bool shared = first ? sh_first : (cur_key == last_key && sh_last);
+                float *dst = (shared ? A.part + ((int64_t)c * 2 + (first ? 0 : 1)) * NO * K_pad
+                                     : A.direct + (int64_t)cur_key * NO * K_pad) + k;
+                if (VUP_DBG_IN(cur_key, (int64_t)P * A.h.B, dstatus))
+#pragma unroll
+                    for (int o = 0; o < NO; ++o) *reinterpret_cast<float2 *>(dst + o * K_pad) = acc[o];
+#pragma unroll
+                for (int o = 0; o < NO; ++o) acc[o] = make_float2(0.f, 0.f);
+            };
+            auto fold_run = [&]() {
+                acc[0].x = fmaf(pf[0].f.x, s.x, acc[0].x);
+                acc[0].y = fmaf(pf[0].f.y, s.y, acc[0].y);
+                acc[1].x = fmaf(pf[0].f.x, s.z, acc[1].x);
+                acc[1].y = fmaf(pf[0].f.y, s.w, acc[1].y);
+#pragma unroll
+                for (int o = 0; o < NF; ++o) {
+                    acc[2 + o].x = fmaf(pf[0].fx[o].x, s.x, acc[2 + o].x);
+                    acc[2 + o].y = fmaf(pf[0].fx[o].y, s.y, acc[2 + o].y);
+                }
+                s = make_float4(0.f, 0.f, 0.f, 0.f);
+            };
+            auto run_end = [&](uint32_t u) {
+                fold_run();
+                if (u & kBinEnd) {
+                    flush();
+                    cur_key = r + 1 < r1 ? H.run_bin[r + 1] : -1;
+                }
+#pragma unroll
+                for (int q = 0; q + 1 < AHEAD; ++q) pf[q] = pf[q + 1];
+                pf[AHEAD - 1] = coded(u);
+                ++r;
+            };
+            auto group = [&](const uint4 v) {
+                const float4 a0 = gather(v.x), a1 = gather(v.y), a2 = gather(v.z), a3 = gather(v.w);
+                if (((v.x | v.y | v.z | v.w) & kFlags) == 0) {
+                    add4(s, a0);
+                    add4(s, a1);
+                    add4(s, a2);
+                    add4(s, a3);
+                } else {
+                    add4(s, a0);
+                    if (v.x & kFlags) run_end(v.x);
+                    add4(s, a1);
+                    if (v.y & kFlags) run_end(v.y);
+                    add4(s, a2);
+                    if (v.z & kFlags) run_end(v.z);
+                    add4(s, a3);
+                    if (v.w & kFlags) run_end(v.w);
+                }
+            };
+            for (int32_t wbase = wb0; wbase < p1; wbase += kWin, ++wseq) {
+                const int b = wseq & 1;
+                for (uint32_t i = 0; !mbar_try_wait(&mbar[b], (wseq >> 1) & 1); ++i) {
+                    if (i > kSpin || *(volatile int *)&abort) {  // a staged copy never landed: record and stop
+                        *(volatile int *)&abort = 1;
+                        atomicCAS(dstatus, 0, VUP_DSTAT_TIMEOUT);
+                        break;
+                    }
+                }
+                if (*(volatile int *)&abort) break;
+                const uint32_t *wv = win + b * kWin;
+                const int lo = (p0 > wbase ? p0 : wbase) - wbase;
+                const int hi = (p1 < wbase + kWin ? p1 : wbase + kWin) - wbase;
+                for (int pa = lo & ~3; pa < hi; pa += 4) {
+                    uint4 v = *reinterpret_cast<const uint4 *>(wv + pa);
+                    if (pa < lo || pa + 4 > hi) {  // cut by the chunk bounds: foreign points read the zero row
+                        if (pa + 0 < lo || pa + 0 >= hi) v.x = null_word;
+                        if (pa + 1 < lo || pa + 1 >= hi) v.y = null_word;
+                        if (pa + 2 < lo || pa + 2 >= hi) v.z = null_word;
+                        if (pa + 3 < lo || pa + 3 >= hi) v.w = null_word;
+                    }
+                    group(v);
+                }
+                __syncwarp();
+                if (lane == 0 && wbase + 2 * kWin < p1) {
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    bulk_copy(win + b * kWin, H.hpt + wbase + 2 * kWin, kWin * 4, &mbar[b]);
+                }
+            }
+            if (*(volatile int *)&abort) break;
+            if (cur_key >= 0) flush();  // (its last run ended with the chunk)
+        }
+    }
+}
+
+// H and the posterior means from the walk's sums (parts in order, cut keys from
+// their chunks' partials in chunk order, as the histogram's finish): 128
+// densities x 8 bins per CTA, a warp per bin.
+__global__ void __launch_bounds__(256) k_post_finish(const __grid_constant__ PostArgs A) {
+    __shared__ float tile[4][8][128 + 1];
+    const HistArgs &h = A.h;
+    const LayoutArgs &H = h.sel[0] ? h.L1 : h.L0;
+    const int P = h.fold->P[h.sel[0] ? 1 : 0], nd = h.ndim, no = 1 + nd;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int b = blockIdx.y * 8 + warp;
+    const int64_t k0 = (int64_t)blockIdx.x * 128, k = k0 + 4 * lane;
+    float4 t[4];
+#pragma unroll
+    for (int o = 0; o < 4; ++o) t[o] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (b < h.B)
+        for (int p = 0; p < P; ++p) {
+            const int32_t key = p * h.B + b;
+            const int2 cc = H.key_chunks[key];
+            if (cc.x < 0) continue;
+            if (cc.x == cc.y) {
+                const float *row = A.direct + (int64_t)key * no * h.K_pad + k;
+#pragma unroll
+                for (int o = 0; o < 4; ++o)
+                    if (o < no) add4(t[o], ld4(row + o * h.K_pad));
+                continue;
+            }
+            for (int c = cc.x; c <= cc.y; ++c) {
+                if (H.chunk_pt[c] >= H.chunk_pt[c + 1]) continue;
+                const int side = H.chunk_bin[2 * c] == key ? 0 : 1;
+                const float *row = A.part + ((int64_t)c * 2 + side) * no * h.K_pad + k;
+#pragma unroll
+                for (int o = 0; o < 4; ++o)
+                    if (o < no) add4(t[o], ld4(row + o * h.K_pad));
+            }
+        }
+#pragma unroll
+    for (int o = 0; o < 4; ++o) {
+        float *q = tile[o][warp] + 4 * lane;
+        q[0] = t[o].x;
+        q[1] = t[o].y;
+        q[2] = t[o].z;
+        q[3] = t[o].w;
+    }
+    __syncthreads();
+    // sum o > 0 belongs to an axis: 1 the gathered one, then the rest axes
+    const int bb = threadIdx.x & 7;
+    const int64_t bo = (int64_t)blockIdx.y * 8 + bb;
+    for (int kk = threadIdx.x >> 3; kk < 128; kk += 32) {
+        if (k0 + kk >= h.K || bo >= h.B) continue;
+        const int64_t e = (k0 + kk) * h.B + bo;
+        const float m = tile[0][bb][kk];
+        if (A.hist) A.hist[e] = m;
+        for (int d = 0; d < nd; ++d) {
+            const int o = d == H.ax_last ? 1 : (d == H.ax0 ? 2 : 3);
+            A.post[e * nd + d] = m > 0.f ? tile[o][bb][kk] / m : 0.f;
+        }
+    }
+}
+
 }  // namespace
 
 // Chunks per part: groups of kGroupChunks chunks, as many groups (1..16) as
@@ -1668,6 +2034,74 @@ bool vup_hist_tile_fits(vup_grid g) {
     for (int l = 0; l < g->n_layouts; ++l)
         if (hist_smem_bytes(g->hl[l].part_rows) > 220 * 1024) return false;
     return coded;
+}
+
+// H (or null) and posterior means of a 2-D / 3-D grid whose tiles fit shared
+// memory, from the densities' factor tables and the point stream; false when
+// they do not fit (nothing done).
+vup_status vup_post_fused(vup_grid g, int64_t K, float *hist, float *post, cudaStream_t s, bool &done) {
+    done = false;
+    if (!vup_hist_tile_fits(g)) return VUP_OK;
+    int64_t rows;
+    int P_max;
+    PostArgs A{};
+    A.h = hist_args_for(g, K, nullptr, rows, P_max);
+    A.h.points_only = 1;
+    const int nd = g->ndim, no = 1 + nd;
+    const int64_t K_pad = A.h.K_pad;
+    int64_t axis_rows = 0;
+    for (int d = 0; d < nd; ++d) axis_rows += g->n[d];
+    // scratch: f_x tables, then the cut rows and the keys' rows; the coordinates
+    const size_t f_fx = (size_t)axis_rows * K_pad, f_part = (size_t)P_max * A.h.C * 2 * no * K_pad;
+    const size_t f_dir = (size_t)P_max * A.h.B * no * K_pad;
+    vup_status st;
+    if ((st = devbuf_reserve(g->post_tmp, sizeof(float) * (f_fx + f_part + f_dir))) != VUP_OK) return st;
+    if ((st = devbuf_reserve(g->post_x, sizeof(float) * (size_t)axis_rows)) != VUP_OK) return st;
+    float *fx = (float *)g->post_tmp.p, *xs = (float *)g->post_x.p;
+    A.xs = xs;
+    A.fx = fx;
+    A.part = fx + f_fx;
+    A.direct = A.part + f_part;
+    A.hist = hist;
+    A.post = post;
+    AxisGeom G{};
+    G.ndim = nd;
+    int64_t n_max = 1;
+    for (int d = 0; d < nd; ++d) {
+        G.n[d] = g->n[d];
+        G.lo[d] = g->lo[d];
+        G.h[d] = (g->hi[d] - g->lo[d]) / (double)g->n[d];
+        n_max = std::max(n_max, g->n[d]);
+    }
+    int *ctr = g->hist_sel + kHistCtr;
+    {
+        VUP_PROF("posterior_axis_weights", s, 2);
+        k_axis_coords<<<(unsigned)ceil_div64(n_max, 128), 128, 0, s>>>(G, xs);
+        VUP_CHECK_LAUNCH();
+        const int64_t blocks = std::min<int64_t>(axis_rows * ceil_div64(K_pad, 512), (int64_t)vup_num_sms() * 16);
+        k_post_tables<<<(unsigned)blocks, 128, 0, s>>>(A, fx, (float *)g->ftab_fold.p, ctr);
+        VUP_CHECK_LAUNCH();
+    }
+    {
+        VUP_PROF("hist_segmented", s, 1);
+        const int nkt = (int)ceil_div64(K, kPostKT);
+        const size_t smem = hist_smem_bytes(rows);
+        const unsigned ctas = (unsigned)std::min<int64_t>(vup_num_sms(), (int64_t)P_max * nkt * A.h.C);
+        auto launch = [&](auto kern) -> vup_status {
+            VUP_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            kern<<<ctas, kHistWarps * 32, smem, s>>>(A, rows, nkt, ctr);
+            VUP_CHECK_LAUNCH();
+            return VUP_OK;
+        };
+        st = nd == 2 ? launch(k_post_walk<1, 4>)
+                     : (vup_hist_rest_staged(g) ? launch(k_post_walk<2, 1>) : launch(k_post_walk<2, 4>));
+        if (st != VUP_OK) return st;
+    }
+    VUP_PROF("posterior_finish", s, 1);
+    k_post_finish<<<dim3((unsigned)ceil_div64(K, 128), (unsigned)ceil_div64(g->B, 8)), 256, 0, s>>>(A);
+    VUP_CHECK_LAUNCH();
+    done = true;
+    return VUP_OK;
 }
 
 // A 2-D grid whose every part fits the shared-memory tile.

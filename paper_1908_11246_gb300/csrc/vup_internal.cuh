@@ -331,6 +331,7 @@ struct vup_grid_s {
     // per-K scratch (density constants, factor tables, partials)
     int64_t K_cap = 0;
     DevBuf dconst, dstats, dpart, ftab, atab_hi, atab_lo, partials, hist_part, hist_direct, ipsa_part;
+    DevBuf post_tmp, post_x;  // posterior means: weighted tables, sums per key; axis coordinates
     DevBuf ftab_fold;    // merged factor tables of the folded axes, axis d at fold_off(d) rows of K_pad
     DevBuf atf_hi, atf_lo;         // TF32 split of the A operand [K_pad][R_pad]
 
@@ -400,6 +401,7 @@ vup_status vup_hist_fused(vup_grid g, int64_t K, float *hist, cudaStream_t s, co
 vup_status vup_fold_tables(vup_grid g, int64_t K, cudaStream_t s, const float *ftab = nullptr);
 vup_status vup_reserve_fold(vup_grid g, int64_t K);
 size_t vup_fold_scratch_bytes(const vup_grid_s *g);
+vup_status vup_post_fused(vup_grid g, int64_t K, float *hist, float *post, cudaStream_t s, bool &done);
 vup_status vup_propagate_1d(vup_grid g, const vup_densities *d, double *raw, double *central,
                             float *hist, cudaStream_t s);
 vup_status vup_ipsa_1d(vup_grid g, const vup_densities *d, const double *grad, float *dmu,
