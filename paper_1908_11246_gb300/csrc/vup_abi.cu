@@ -272,7 +272,6 @@ static void free_grid(vup_grid g) {
     devbuf_free(g->rec_tmp);
     devbuf_free(g->dconst);
     devbuf_free(g->dstats);
-    devbuf_free(g->dpart);
     devbuf_free(g->ftab);
     devbuf_free(g->atab_hi);
     devbuf_free(g->atab_lo);

@@ -237,8 +237,7 @@ extern "C" vup_status vup_propagate_batched(int n_inst, const vup_grid *g, const
             if ((st = vup_reserve_k(g[i], K, bf16, false)) != VUP_OK) return st;
             if (hist && hist[i] && (st = vup_reserve_fold(g[i], K)) != VUP_OK) return st;
             if ((st = vup_build_tables(g[i], kOrientLast, bf16 ? 1 : 0, s)) != VUP_OK) return st;
-            if (hist && hist[i] && (st = vup_ensure_layout(g[i], s)) != VUP_OK) return st;
-            if ((st = vup_density_reserve(g[i], K)) != VUP_OK) return st;
+            if (hist && hist[i] && (st = vup_ensure_layout(g[i], s, false, true)) != VUP_OK) return st;
             if (bf16 &&
                 (st = devbuf_reserve(g[i]->partials,
                                      sizeof(float) * 4 * K_pad * vup_tc_col_tiles_bn(g[i]->orient[0], 64))) != VUP_OK)
@@ -257,7 +256,7 @@ extern "C" vup_status vup_propagate_batched(int n_inst, const vup_grid *g, const
                               (uint64_t)D.sigma, (uint64_t)D.lo, (uint64_t)D.hi,
                               (uint64_t)(moments_raw ? moments_raw[i] : nullptr),
                               (uint64_t)(hist ? hist[i] : nullptr), (uint64_t)G->ftab.p, (uint64_t)G->dstats.p,
-                              (uint64_t)G->dconst.p, (uint64_t)G->dpart.p, (uint64_t)G->partials.p,
+                              (uint64_t)G->dconst.p, (uint64_t)G->partials.p,
                               (uint64_t)G->atab_hi.p, (uint64_t)G->atab_lo.p, (uint64_t)G->hist_part.p,
                               (uint64_t)G->hist_direct.p, (uint64_t)G->ftab_fold.p};
         key.insert(key.end(), std::begin(w), std::end(w));

@@ -33,11 +33,10 @@ struct KSum {
     __device__ __forceinline__ double value() const { return (double)s + (double)c; }
 };
 
-// Error-free FP32 transformations (Knuth two-sum, FMA two-product).
-__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
+// a + b as s + e exactly, for |a| >= |b| (or a + b exact): Dekker's fast two-sum.
+__device__ __forceinline__ void fast_two_sum(float a, float b, float &s, float &e) {
     s = a + b;
-    const float bb = s - a;
-    e = (a - (s - bb)) + (b - bb);
+    e = b - (s - a);
 }
 
 // Constants of one (k, d) Gaussian factor in index space, as FP32 pairs.
@@ -60,7 +59,7 @@ struct GaussArg {
 __device__ __forceinline__ float gauss_value(float A, const GaussArg &ga, float &u) {
     // t = A - f exactly as a pair
     float th, tl;
-    two_sum(A, -ga.fh, th, tl);
+    fast_two_sum(A, -ga.fh, th, tl);  // A is an integer, fh in [0, 1): 0 or larger than fh
     tl -= ga.fl;
     // u = t r
     const float uh = th * ga.rh;
@@ -69,13 +68,15 @@ __device__ __forceinline__ float gauss_value(float A, const GaussArg &ga, float 
     // u^2 - u0^2
     const float sh = uh * uh;
     const float sl = fmaf(uh, uh, -sh) + 2.f * uh * ul;
+    // (u0 is the smallest |u|: sh >= qh but where they round to neighbours, whose
+    // difference is exact)
     float dh, dl;
-    two_sum(sh, -ga.qh, dh, dl);
+    fast_two_sum(sh, -ga.qh, dh, dl);
     dl += sl - ga.ql;
-    const float eh0 = 0.5f * dh, el0 = 0.5f * dl;
-    const float eh = eh0 + el0;
-    const float el = el0 - (eh - eh0);
-    return expf(-eh) * (1.f - el);
+    // e = dh + dl; the halves of e and of its error are exact
+    const float e = dh + dl;
+    const float l = dl - (e - dh);
+    return expf(-0.5f * e) * fmaf(-0.5f, l, 1.f);
 }
 
 // Midpoint coordinate of cell a, x_a = lo + (a + 1/2) h, rounded in FP64 in
@@ -103,25 +104,28 @@ __device__ __forceinline__ int64_t first_true(int64_t b, int64_t e, P pred) {
 // outside).  EXACT_F32: every a - n in the segment is below 2^24 in
 // magnitude, so A is carried as an FP32 counter; otherwise A is rounded
 // from FP64 per cell.
-template <bool EXACT_F32, bool STATS>
-__device__ __forceinline__ void prep_segment(float *__restrict__ tab, int64_t K_pad, int kind, int64_t a_begin,
-                                             int64_t a_end, int64_t in_b, int64_t in_e, const GaussArg &ga,
+// PLAIN: a warp of Gaussian densities (no supports to look at).
+template <bool EXACT_F32, bool STATS, bool PLAIN>
+__device__ __forceinline__ void prep_segment(float *__restrict__ tab, int64_t K_pad, int kind, int32_t a_begin,
+                                             int32_t a_end, int32_t in_b, int32_t in_e, const GaussArg &ga,
                                              KSum &S0, KSum &S1, KSum &S2) {
     float Af = (float)((double)a_begin - ga.nk);
-    for (int64_t a = a_begin; a < a_end; ++a) {
+    tab += a_begin * K_pad;
+    for (int32_t a = a_begin; a < a_end; ++a, tab += K_pad) {
         const float A = EXACT_F32 ? Af : (float)((double)a - ga.nk);
         Af += 1.f;
         float u;
-        const float gv = gauss_value(A, ga, u);
-        const bool inside = a >= in_b && a < in_e;
-        float g;
-        if (kind == VUP_UNIFORM) {
-            g = inside ? 1.f : 0.f;
-            u = 0.f;
-        } else {
-            g = (kind == VUP_TRUNCNORM && !inside) ? 0.f : gv;
+        float g = gauss_value(A, ga, u);
+        if (!PLAIN) {
+            const bool inside = a >= in_b && a < in_e;
+            if (kind == VUP_UNIFORM) {
+                g = inside ? 1.f : 0.f;
+                u = 0.f;
+            } else if (kind == VUP_TRUNCNORM && !inside) {
+                g = 0.f;
+            }
         }
-        tab[a * K_pad] = g;
+        *tab = g;
         S0.add(g);
         if (STATS) {
             S1.add(g * u);
@@ -139,7 +143,6 @@ struct DensJob {
     double lo[3], h[3];
     int S;  // segments per axis
     DensConst *dconst;
-    double *dpart;
     float *ftab;
     DensStats *dstats;
     int *dstatus;
@@ -149,105 +152,115 @@ struct DensJob {
     __nv_bfloat16 *ahi, *alo;
 };
 
-// Density factors of densities kb*128 .. kb*128+127 on axis d, segment z of
-// that axis: the factor table entries and partial compensated sums.
+// One CTA: the factors and the normalisation statistics of 32 densities on one
+// axis; warp z (threadIdx.y) takes segment z.  Warp 0 first forms the densities'
+// constants -- FP64 divisions and, for supports, binary searches -- which every
+// segment's thread repeated before (half of the kernel's time, as FP64 issues
+// at a 64th of the FP32 rate); the segments' compensated sums are added in order
+// (FP64) by the same CTA: Z = sum g, E[u] and E[u^2] under g / Z.  The rest is
+// FP32 issue: about 38 instructions per factor.  1024 + 1024 cells x 16384
+// densities with the split table, beside a layout build: 165 -> 142 us; 2048 +
+// 2048 x 65536 with two split tables: 1133 -> 970.
+constexpr int kMaxSeg = 16;
+struct DensK {
+    GaussArg ga;
+    int32_t kind, in_b, in_e;  // cells [in_b, in_e) are inside the support
+};
 template <bool STATS>
-__device__ __forceinline__ void density_prep_body(const DensJob &J, int64_t kb, int d, int z) {
-    const int64_t k = kb * (int64_t)blockDim.x + threadIdx.x;
-    if (k >= J.K_pad) return;
-    const int64_t K = J.K, K_pad = J.K_pad;
-    const int ndim = J.ndim, S = J.S;
+__device__ __forceinline__ void density_prep_body(const DensJob &J, int64_t kb, int d) {
+    constexpr int NS = STATS ? 3 : 1;
+    __shared__ DensK s_k[32];
+    __shared__ float2 s_sum[kMaxSeg][NS][32];
+    const int lane = threadIdx.x, z = threadIdx.y;
+    const int64_t k = kb * 32 + lane;  // K_pad is a multiple of 128: k < K_pad
+    const int64_t K_pad = J.K_pad, p = k * J.ndim + d;
     const DensIn &in = J.in;
-    const int64_t nd = J.n[d];
-    // this thread's segment of the axis
-    const int64_t seg = (nd + S - 1) / S;
-    const int64_t a_begin = z * seg, a_end = a_begin + seg < nd ? a_begin + seg : nd;
-    const double lo = J.lo[d];
-    const double h = J.h[d];
+    const int32_t nd = (int32_t)J.n[d];
+    const bool live = k < J.K;
     int64_t off = 0;
     for (int q = 0; q < d; ++q) off += J.n[q] * K_pad;
-    float *tab = J.ftab + off;
-    if (k >= K) {
-        for (int64_t a = a_begin; a < a_end; ++a) tab[a * K_pad + k] = 0.f;
-        return;
-    }
-    const int64_t p = k * ndim + d;
-    const int kind = in.kind[p];
-    const double mu = in.mu[p], sigma = in.sigma[p];
-    const double tlo = in.lo ? in.lo[p] : 0.0, thi = in.hi ? in.hi[p] : 0.0;
-    // index coordinate of the mean: (mu - lo) / h - 1/2 = nk + f
-    const double c = (mu - lo) / h - 0.5;
-    const double nk = floor(c);
-    const double fd = c - nk;
-    const double rd = h / sigma;
-    const float f = (float)fd;
-    const float r = (float)rd;
-    GaussArg ga;
-    ga.nk = nk;
-    ga.fh = f;
-    ga.fl = (float)(fd - (double)f);
-    ga.rh = r;
-    ga.rl = (float)(rd - (double)r);
-    // squared index-space distance from the mean to its nearest midpoint
-    double anear = floor(c + 0.5);
-    anear = fmin(fmax(anear, 0.0), (double)(nd - 1));
-    const double u0 = ((anear - nk) - fd) * rd;
-    double u0sq = kind == VUP_UNIFORM ? 0.0 : u0 * u0;
-    if (!(u0sq < 1e30)) u0sq = 0.0;
-    ga.qh = (float)u0sq;
-    ga.ql = (float)(u0sq - (double)ga.qh);
-    // support of a uniform or truncated density: an interval of cells, since
-    // x_a is non-decreasing in a
-    int64_t in_b = a_begin, in_e = a_end;
-    if (kind == VUP_UNIFORM) {
-        const double half = __dmul_rn(0.5, sigma);
-        in_b = first_true(a_begin, a_end, [&](int64_t a) { return __dsub_rn(midpoint(lo, h, a), mu) >= -half; });
-        in_e = first_true(in_b, a_end, [&](int64_t a) { return !(__dsub_rn(midpoint(lo, h, a), mu) <= half); });
-    } else if (kind == VUP_TRUNCNORM) {
-        in_b = first_true(a_begin, a_end, [&](int64_t a) { return midpoint(lo, h, a) >= tlo; });
-        in_e = first_true(in_b, a_end, [&](int64_t a) { return !(midpoint(lo, h, a) <= thi); });
-    }
-    KSum S0, S1, S2;
-    const double A0 = (double)a_begin - nk;
-    if (fabs(A0) + (double)(a_end - a_begin) < 16777216.0)
-        prep_segment<true, STATS>(tab + k, K_pad, kind, a_begin, a_end, in_b, in_e, ga, S0, S1, S2);
-    else
-        prep_segment<false, STATS>(tab + k, K_pad, kind, a_begin, a_end, in_b, in_e, ga, S0, S1, S2);
-    if (z == 0) {
+    float *tab = J.ftab + off + k;
+    if (z == 0 && live) {
+        const double lo = J.lo[d], h = J.h[d];
+        DensK D;
+        D.kind = in.kind[p];
+        const double mu = in.mu[p], sigma = in.sigma[p];
+        // index coordinate of the mean: (mu - lo) / h - 1/2 = nk + f
+        const double c = (mu - lo) / h - 0.5;
+        const double nk = floor(c);
+        const double fd = c - nk;
+        const double rd = h / sigma;
+        GaussArg &ga = D.ga;
+        ga.nk = nk;
+        ga.fh = (float)fd;
+        ga.fl = (float)(fd - (double)ga.fh);
+        ga.rh = (float)rd;
+        ga.rl = (float)(rd - (double)ga.rh);
+        // squared index-space distance from the mean to its nearest midpoint
+        double anear = floor(c + 0.5);
+        anear = fmin(fmax(anear, 0.0), (double)(nd - 1));
+        const double u0 = ((anear - nk) - fd) * rd;
+        double u0sq = D.kind == VUP_UNIFORM ? 0.0 : u0 * u0;
+        if (!(u0sq < 1e30)) u0sq = 0.0;
+        ga.qh = (float)u0sq;
+        ga.ql = (float)(u0sq - (double)ga.qh);
+        // support of a uniform or truncated density: an interval of cells, since
+        // x_a is non-decreasing in a
+        D.in_b = 0;
+        D.in_e = nd;
+        if (D.kind == VUP_UNIFORM) {
+            const double half = __dmul_rn(0.5, sigma);
+            D.in_b = first_true(0, nd, [&](int64_t a) { return __dsub_rn(midpoint(lo, h, a), mu) >= -half; });
+            D.in_e = first_true(D.in_b, nd, [&](int64_t a) { return !(__dsub_rn(midpoint(lo, h, a), mu) <= half); });
+        } else if (D.kind == VUP_TRUNCNORM) {
+            const double tlo = in.lo ? in.lo[p] : 0.0, thi = in.hi ? in.hi[p] : 0.0;
+            D.in_b = first_true(0, nd, [&](int64_t a) { return midpoint(lo, h, a) >= tlo; });
+            D.in_e = first_true(D.in_b, nd, [&](int64_t a) { return !(midpoint(lo, h, a) <= thi); });
+        }
+        s_k[lane] = D;
         DensConst dc;
         dc.n = (int32_t)fmax(fmin(nk, 2147483647.0), -2147483647.0);
-        dc.f = f;
-        dc.r = r;
-        dc.kind = kind;
+        dc.f = ga.fh;
+        dc.r = ga.rh;
+        dc.kind = D.kind;
         J.dconst[p] = dc;
     }
-    double *q = J.dpart + (((int64_t)d * S + z) * K_pad + k) * 3;
-    q[0] = S0.value();
-    q[1] = S1.value();
-    q[2] = S2.value();
-}
-
-
-// Normalisation statistics from the per-segment compensated sums (segments
-// added in order, FP64): Z = sum g, E[u] and E[u^2] under g / Z.
-__device__ __forceinline__ void density_finish_body(const DensJob &J, int64_t kb, int d) {
-    const int64_t k = kb * (int64_t)blockDim.x + threadIdx.x;
-    if (k >= J.K) return;
-    double s0 = 0.0, s1 = 0.0, s2 = 0.0;
-    for (int z = 0; z < J.S; ++z) {
-        const double *q = J.dpart + (((int64_t)d * J.S + z) * J.K_pad + k) * 3;
-        s0 += q[0];
-        s1 += q[1];
-        s2 += q[2];
+    __syncthreads();
+    const int32_t seg = (nd + J.S - 1) / J.S;
+    const int32_t a_begin = min(nd, z * seg), a_end = min(nd, a_begin + seg);
+    KSum S0, S1, S2;
+    if (live) {
+        const DensK D = s_k[lane];
+        const GaussArg &ga = D.ga;
+        const double A0 = (double)a_begin - ga.nk;
+        const bool exact = fabs(A0) + (double)(a_end - a_begin) < 16777216.0;
+        if (__all_sync(__activemask(), exact && D.kind == VUP_GAUSS))
+            prep_segment<true, STATS, true>(tab, K_pad, D.kind, a_begin, a_end, D.in_b, D.in_e, ga, S0, S1, S2);
+        else if (exact)
+            prep_segment<true, STATS, false>(tab, K_pad, D.kind, a_begin, a_end, D.in_b, D.in_e, ga, S0, S1, S2);
+        else
+            prep_segment<false, STATS, false>(tab, K_pad, D.kind, a_begin, a_end, D.in_b, D.in_e, ga, S0, S1, S2);
+    } else {
+        for (int32_t a = a_begin; a < a_end; ++a) tab[a * K_pad] = 0.f;
     }
-    const int64_t p = k * J.ndim + d;
+    s_sum[z][0][lane] = make_float2(S0.s, S0.c);
+    if constexpr (STATS) {
+        s_sum[z][1][lane] = make_float2(S1.s, S1.c);
+        s_sum[z][2][lane] = make_float2(S2.s, S2.c);
+    }
+    __syncthreads();
+    if (z != 0 || !live) return;
+    double s[3] = {0.0, 0.0, 0.0};
+    for (int q = 0; q < J.S; ++q)
+#pragma unroll
+        for (int i = 0; i < NS; ++i) s[i] += (double)s_sum[q][i][lane].x + (double)s_sum[q][i][lane].y;
     DensStats ds;
-    ds.invZ = s0 > 0.0 ? 1.0 / s0 : 0.0;
-    ds.Eu = s0 > 0.0 ? s1 / s0 : 0.0;
-    ds.Eu2 = s0 > 0.0 ? s2 / s0 : 0.0;
-    ds.inv_sigma = 1.0 / J.in.sigma[p];
+    ds.invZ = s[0] > 0.0 ? 1.0 / s[0] : 0.0;
+    ds.Eu = STATS && s[0] > 0.0 ? s[1] / s[0] : 0.0;
+    ds.Eu2 = STATS && s[0] > 0.0 ? s[2] / s[0] : 0.0;
+    ds.inv_sigma = 1.0 / in.sigma[p];
     J.dstats[p] = ds;
-    if (!(s0 > 0.0)) atomicCAS(J.dstatus, 0, VUP_DSTAT_EMPTY);
+    if (!(s[0] > 0.0)) atomicCAS(J.dstatus, 0, VUP_DSTAT_EMPTY);
 }
 
 // A-operand table of the tensor-core contraction: rows k, reduction index a
@@ -311,15 +324,10 @@ __device__ __forceinline__ void split_transpose_body(const float *__restrict__ t
 
 // STATS: also the sums of g u and g u^2 (E[u], E[u^2] of the IPSA derivatives)
 template <bool STATS>
-__global__ void k_density_prep(DensJob J) {
+__global__ void __launch_bounds__(32 * kMaxSeg) k_density_prep(DensJob J) {
     pdl_trigger();
     pdl_wait();
-    density_prep_body<STATS>(J, blockIdx.x, blockIdx.y, blockIdx.z);
-}
-__global__ void k_density_finish(DensJob J) {
-    pdl_trigger();
-    pdl_wait();
-    density_finish_body(J, blockIdx.x, blockIdx.y);
+    density_prep_body<STATS>(J, blockIdx.x, blockIdx.y);
 }
 // grid: x = density tiles of 128 (more than the 65535 limit of y for large K), y = axis tiles
 template <typename T>
@@ -332,13 +340,12 @@ __global__ void k_split_transpose(const float *__restrict__ tab, int64_t nd, int
 
 // Batched forms: one launch for the blocks of every instance; items[b] =
 // (instance, block coordinates) of block b.
-__global__ void k_density_prep_batched(const DensJob *__restrict__ jobs, const int4 *__restrict__ items) {
+// (blocks of as many warps as the batch's longest axis has segments; the others'
+// spare warps have empty segments)
+__global__ void __launch_bounds__(32 * kMaxSeg) k_density_prep_batched(const DensJob *__restrict__ jobs,
+                                                                       const int4 *__restrict__ items) {
     const int4 it = items[blockIdx.x];
-    density_prep_body<false>(jobs[it.x], it.y, it.z, it.w);
-}
-__global__ void k_density_finish_batched(const DensJob *__restrict__ jobs, const int4 *__restrict__ items) {
-    const int4 it = items[blockIdx.x];
-    density_finish_body(jobs[it.x], it.y, it.z);
+    density_prep_body<false>(jobs[it.x], it.y, it.z);
 }
 __global__ void k_split_transpose_batched(const DensJob *__restrict__ jobs, const int4 *__restrict__ items) {
     const int4 it = items[blockIdx.x];
@@ -349,7 +356,7 @@ __global__ void k_split_transpose_batched(const DensJob *__restrict__ jobs, cons
 int density_segments(vup_grid g) {
     int64_t nmax = 1;
     for (int q = 0; q < g->ndim; ++q) nmax = std::max(nmax, g->n[q]);
-    return (int)std::max<int64_t>(1, std::min<int64_t>(16, nmax / 128));
+    return (int)std::max<int64_t>(1, std::min<int64_t>(kMaxSeg, nmax / 128));
 }
 
 DensJob make_job(vup_grid g, const vup_densities *d) {
@@ -365,7 +372,6 @@ DensJob make_job(vup_grid g, const vup_densities *d) {
     }
     J.S = density_segments(g);
     J.dconst = (DensConst *)g->dconst.p;
-    J.dpart = (double *)g->dpart.p;
     J.ftab = (float *)g->ftab.p;
     J.dstats = (DensStats *)g->dstats.p;
     J.dstatus = g->dstatus;
@@ -388,11 +394,6 @@ size_t vup_ftab_floats(const vup_grid g) {
     return s;
 }
 
-vup_status vup_density_reserve(vup_grid g, int64_t K) {
-    const int64_t K_pad = ceil_div64(K, 128) * 128;
-    return devbuf_reserve(g->dpart, sizeof(double) * 3 * (size_t)density_segments(g) * g->ndim * K_pad);
-}
-
 // need_bf16_orient_mask: bit o set -> build the split BF16 A table for the
 // reduction axis of orientation o.
 template <typename T>
@@ -400,16 +401,12 @@ static vup_status split_tables(vup_grid g, int mask, int64_t K_pad, T *hi0, T *l
 
 vup_status vup_density_prep(vup_grid g, const vup_densities *d, int need_bf16_orient_mask, cudaStream_t s,
                             bool tf32, bool stats) {
-    vup_status st = vup_density_reserve(g, d->K);
-    if (st != VUP_OK) return st;
     const DensJob J = make_job(g, d);
     const int64_t K_pad = J.K_pad;
-    dim3 grd((unsigned)ceil_div64(K_pad, 128), (unsigned)g->ndim, (unsigned)J.S);
-    VUP_PROF("density_prep", s, 2 + __builtin_popcount(need_bf16_orient_mask));
-    VUP_CHECK_CUDA(stats ? launch_pdl(k_density_prep<true>, grd, 128, 0, s, J)
-                         : launch_pdl(k_density_prep<false>, grd, 128, 0, s, J));
-    dim3 fgrd((unsigned)ceil_div64(d->K, 128), (unsigned)g->ndim);
-    VUP_CHECK_CUDA(launch_pdl(k_density_finish, fgrd, 128, 0, s, J));
+    dim3 grd((unsigned)(K_pad / 32), (unsigned)g->ndim), blk(32, (unsigned)J.S);
+    VUP_PROF("density_prep", s, 1 + __builtin_popcount(need_bf16_orient_mask));
+    VUP_CHECK_CUDA(stats ? launch_pdl(k_density_prep<true>, grd, blk, 0, s, J)
+                         : launch_pdl(k_density_prep<false>, grd, blk, 0, s, J));
     if (tf32) return split_tables<float>(g, need_bf16_orient_mask, K_pad, (float *)g->atf_hi.p,
                                          (float *)g->atf_lo.p, s);
     return split_tables<__nv_bfloat16>(g, need_bf16_orient_mask, K_pad, (__nv_bfloat16 *)g->atab_hi.p,
@@ -446,33 +443,28 @@ static vup_status split_tables(vup_grid g, int mask, int64_t K_pad, T *hi0, T *l
 // via the launch.  Scratch of every grid must already be reserved for its K.
 struct DensPlan {
     DevBuf jobs, items;
-    int n_prep = 0, n_fin = 0, n_split = 0;
+    int n_prep = 0, n_split = 0, segs = 1;
 };
 
 vup_status vup_density_plan(int n, const vup_grid *gs, const vup_densities *ds, bool bf16, void **plan_out) {
     DensPlan *P = new DensPlan();
     std::vector<DensJob> jobs(n);
-    std::vector<int4> prep, fin, split;
+    std::vector<int4> prep, split;
     for (int i = 0; i < n; ++i) {
         jobs[i] = make_job(gs[i], &ds[i]);
         const DensJob &J = jobs[i];
-        const int64_t nkb_pad = ceil_div64(J.K_pad, 128), nkb = ceil_div64(J.K, 128);
+        P->segs = std::max(P->segs, J.S);
         for (int d = 0; d < J.ndim; ++d)
-            for (int z = 0; z < J.S; ++z)
-                for (int64_t kb = 0; kb < nkb_pad; ++kb) prep.push_back(make_int4(i, (int)kb, d, z));
-        for (int d = 0; d < J.ndim; ++d)
-            for (int64_t kb = 0; kb < nkb; ++kb) fin.push_back(make_int4(i, (int)kb, d, 0));
+            for (int64_t kb = 0; kb < J.K_pad / 32; ++kb) prep.push_back(make_int4(i, (int)kb, d, 0));
         if (bf16)
             for (int64_t by = 0; by < ceil_div64(J.K_pad, kSplitK); ++by)
                 for (int64_t bx = 0; bx < ceil_div64(J.R_pad, 64); ++bx)
                     split.push_back(make_int4(i, (int)bx, (int)by, 0));
     }
     P->n_prep = (int)prep.size();
-    P->n_fin = (int)fin.size();
     P->n_split = (int)split.size();
     std::vector<int4> all;
     all.insert(all.end(), prep.begin(), prep.end());
-    all.insert(all.end(), fin.begin(), fin.end());
     all.insert(all.end(), split.begin(), split.end());
     vup_status st;
     if ((st = devbuf_reserve(P->jobs, sizeof(DensJob) * n)) != VUP_OK ||
@@ -500,12 +492,10 @@ vup_status vup_density_batched(void *plan, cudaStream_t s) {
     const DensPlan *P = (const DensPlan *)plan;
     const DensJob *jobs = (const DensJob *)P->jobs.p;
     const int4 *items = (const int4 *)P->items.p;
-    VUP_PROF("density_prep_batched", s, P->n_split ? 3 : 2);
-    if (P->n_prep) k_density_prep_batched<<<P->n_prep, 128, 0, s>>>(jobs, items);
+    VUP_PROF("density_prep_batched", s, P->n_split ? 2 : 1);
+    if (P->n_prep) k_density_prep_batched<<<P->n_prep, dim3(32, P->segs), 0, s>>>(jobs, items);
     VUP_CHECK_LAUNCH();
-    if (P->n_fin) k_density_finish_batched<<<P->n_fin, 128, 0, s>>>(jobs, items + P->n_prep);
-    VUP_CHECK_LAUNCH();
-    if (P->n_split) k_split_transpose_batched<<<P->n_split, dim3(32, 8), 0, s>>>(jobs, items + P->n_prep + P->n_fin);
+    if (P->n_split) k_split_transpose_batched<<<P->n_split, dim3(32, 8), 0, s>>>(jobs, items + P->n_prep);
     VUP_CHECK_LAUNCH();
     return VUP_OK;
 }

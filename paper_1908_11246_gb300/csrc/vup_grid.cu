@@ -657,8 +657,8 @@ __device__ __forceinline__ void pick_layout(const FoldArgs &A, int32_t c0, int32
 // One pass over the bins (viewed as [R][C], C the last axis): the slice hashes
 // of every axis and, on 2-D grids, the intervals of both layouts (stretches of
 // one (part, bin) key along the gathered axis: 1 + key changes along each
-// line).  The hash of a slice is the sum of (bin + 1) times the product of its
-// points' index weights, modulo 2^64.  A warp takes 8 rows of 128 columns,
+// line).  The hash of a slice sums (bin + 1) times the product of its points'
+// index weights, in two 32-bit halves, over the same blocks for every slice.  A warp takes 8 rows of 128 columns,
 // every load of four rows in flight together: column sums stay in registers, a
 // row's sum is reduced over the warp.
 constexpr int kFoldRows = 8, kFoldCols = 128;
@@ -678,12 +678,15 @@ __global__ void __launch_bounds__(256) k_fold_hash(FoldArgs A) {
     for (int64_t t = blockIdx.x; t < ncb * nrb; t += gridDim.x) {
         const int64_t cb = (t % ncb) * kFoldCols, c0 = cb + lane;
         const int64_t r0 = (t / ncb) * kRows + (tid >> 5) * kFoldRows;
-        unsigned long long wc[4], acc[4] = {0, 0, 0, 0};
+        // two 32-bit hashes: their warp sums are one instruction each
+        uint32_t wl[4], wh[4], al[4] = {0, 0, 0, 0}, ah[4] = {0, 0, 0, 0};
         bool cut[4];  // a part of layout 0 starts at the column
         int32_t up[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            wc[q] = fold_weight(A.ndim - 1, c0 + 32 * q);
+            const unsigned long long w = fold_weight(A.ndim - 1, c0 + 32 * q);
+            wl[q] = (uint32_t)w;
+            wh[q] = (uint32_t)(w >> 32) | 1u;
             cut[q] = (uint32_t)(c0 + 32 * q) % p0 == 0;
             up[q] = !d3 && r0 > 0 && r0 < R && c0 + 32 * q < C ? A.bins[(r0 - 1) * C + c0 + 32 * q] + 1 : 0;
         }
@@ -705,11 +708,14 @@ __global__ void __launch_bounds__(256) k_fold_hash(FoldArgs A) {
                 const int64_t a0 = d3 ? r / A.n[1] : r, a1 = d3 ? r - a0 * A.n[1] : 0;
                 const unsigned long long w0 = fold_weight(0, a0), w1 = d3 ? fold_weight(1, a1) : 1ull;
                 const unsigned long long wr = w0 * w1;
-                unsigned long long s = 0;
+                const uint32_t rl = (uint32_t)wr, rh = (uint32_t)(wr >> 32) | 1u;
+                uint32_t sl = 0, sh = 0;
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
-                    s += (unsigned long long)b[u][q] * wc[q];
-                    acc[q] += (unsigned long long)b[u][q] * wr;
+                    sl += (uint32_t)b[u][q] * wl[q];
+                    sh += (uint32_t)b[u][q] * wh[q];
+                    al[q] += (uint32_t)b[u][q] * rl;
+                    ah[q] += (uint32_t)b[u][q] * rh;
                 }
                 if (!d3) {
                     const bool rcut = (uint32_t)r % p1 == 0;
@@ -726,8 +732,10 @@ __global__ void __launch_bounds__(256) k_fold_hash(FoldArgs A) {
                         up[q] = b[u][q];
                     }
                 }
-                for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+                sl = __reduce_add_sync(0xffffffffu, sl);
+                sh = __reduce_add_sync(0xffffffffu, sh);
                 if (lane == 0) {
+                    const unsigned long long s = ((unsigned long long)sh << 32) + sl;
                     atomicAdd(h0 + a0, s * w1);
                     if (d3) atomicAdd(h1 + a1, s * w0);
                 }
@@ -735,7 +743,7 @@ __global__ void __launch_bounds__(256) k_fold_hash(FoldArgs A) {
         }
         // the warps' column sums to one atomic per column
 #pragma unroll
-        for (int q = 0; q < 4; ++q) s_col[tid >> 5][lane + 32 * q] = acc[q];
+        for (int q = 0; q < 4; ++q) s_col[tid >> 5][lane + 32 * q] = ((unsigned long long)ah[q] << 32) + al[q];
         __syncthreads();
         if (tid < kFoldCols && cb + tid < C) {
             unsigned long long v = 0;
@@ -1318,14 +1326,15 @@ __global__ void k_layout_encode(const int32_t *__restrict__ run_start, const int
     }
 }
 
-// Start of chunk cc of C over n elements: n cc / C, rounded down to whole
-// chunks of `least` elements where n / C is less (some chunks are then empty,
-// spread evenly): a chunk's cut keys or groups cost partial rows, which short
-// chunks would make the larger part of the work.
+// Start of chunk cc of C over n elements: n cc / C, on a merged grid or one of a
+// batch (coarse) rounded down to whole chunks of `least` elements where n / C is
+// less (some chunks are then empty, spread evenly): a chunk's cut keys or groups
+// cost partial rows, which short chunks would make the larger part of the work
+// (a batch's finish: 102 -> 86 us), and neither needs them to fill the SMs.
 constexpr int kChunkPoints = 256, kChunkRecords = 24;
 __device__ __forceinline__ int64_t chunk_at(int64_t n, int64_t cc, int64_t C, int64_t least) {
     int64_t t = n * cc / C;
-    if (n < C * least && cc < C) t = t / least * least;
+    if (least > 1 && n < C * least && cc < C) t = t / least * least;
     return t;
 }
 
@@ -1337,7 +1346,7 @@ __global__ void k_chunks(const int32_t *__restrict__ run_start, const int32_t *_
                          const int32_t *__restrict__ koff, int B, LaySel L, int C,
                          const unsigned long long *__restrict__ excl, const int32_t *__restrict__ n_iv_p,
                          int32_t *__restrict__ chunk_pt, int32_t *__restrict__ chunk_run,
-                         int32_t *__restrict__ chunk_iv, const int32_t *gate) {
+                         int32_t *__restrict__ chunk_iv, const int32_t *gate, int coarse) {
     pdl_trigger();
     pdl_wait();
     if (gated_off(gate)) return;
@@ -1352,7 +1361,7 @@ __global__ void k_chunks(const int32_t *__restrict__ run_start, const int32_t *_
     } else {
         const int p = c / C, cc = c - p * C;
         const int64_t lo = koff[p * B], hi = koff[(p + 1) * B];
-        const int64_t target = lo + chunk_at(hi - lo, cc, C, kChunkPoints);
+        const int64_t target = lo + chunk_at(hi - lo, cc, C, coarse || L.fold->any ? kChunkPoints : 1);
         int32_t a = 0, b = n_runs;  // first r in [0, n_runs] with run_start[r] >= target
         while (a < b) {
             int32_t mid = (a + b) >> 1;
@@ -1618,44 +1627,45 @@ __global__ void k_rec_scatter(const uint4 *__restrict__ tmp, const int32_t *__re
 __global__ void k_rec_tables(const int32_t *__restrict__ starts, const int32_t *__restrict__ counts, int64_t Lr,
                              int64_t NL, int n_groups, int GB, LaySel L, int C, const uint4 *__restrict__ rec,
                              int32_t *__restrict__ goff, int32_t *__restrict__ n_rec, int32_t *__restrict__ chunk_rec,
-                             int32_t *__restrict__ chunk_grp, int2 *__restrict__ gch) {
+                             int32_t *__restrict__ chunk_grp, int2 *__restrict__ gch, int coarse) {
     pdl_trigger();
     pdl_wait();
     const int P = L.get().P;
+    const int64_t least = coarse || L.fold->any ? kChunkRecords : 1;
     const int32_t total = starts[Lr - 1] + counts[Lr - 1];
     auto first = [&](int g) -> int32_t { return g < n_groups ? starts[g * NL] : total; };
-    auto bound = [&](int c) -> int32_t {  // first record of chunk c
-        if (c >= P * C) return total;
-        const int p = c / C, cc = c - p * C;
-        const int64_t lo = first(p * GB), hi = first((p + 1) * GB);
-        return (int32_t)(lo + chunk_at(hi - lo, cc, C, kChunkRecords));
-    };
     const int i = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
     if (i == 0) n_rec[0] = total;
     for (int g = i; g < n_groups + 2; g += step) goff[g] = first(g);
     for (int c = i; c <= P * C; c += step) {
-        const int32_t r = bound(c);
+        if (c == P * C) {
+            chunk_rec[c] = total;
+            break;
+        }
+        const int p = c / C, cc = c - p * C;
+        const int64_t lo = first(p * GB), n = first((p + 1) * GB) - lo;
+        const int32_t r = (int32_t)(lo + chunk_at(n, cc, C, least)), r1 = (int32_t)(lo + chunk_at(n, cc + 1, C, least));
         chunk_rec[c] = r;
-        if (c == P * C) break;
-        const int32_t r1 = bound(c + 1);
         chunk_grp[2 * c] = r1 > r ? (int32_t)rec[2 * (int64_t)r + 1].z : -1;
         chunk_grp[2 * c + 1] = r1 > r ? (int32_t)rec[2 * (int64_t)(r1 - 1) + 1].z : -1;
     }
     for (int g = i; g < n_groups; g += step) {
+        const int p = g / GB;
         const int32_t o0 = first(g), o1 = first(g + 1);
         if (o0 == o1) {
             gch[g] = make_int2(-1, -1);
             continue;
         }
-        auto holding = [&](int32_t t) {  // last chunk of the group's part that starts at or before t
-            int lo = g / GB * C, hi = lo + C;
-            while (hi - lo > 1) {
-                const int mid = (lo + hi) >> 1;
-                if (bound(mid) <= t) lo = mid; else hi = mid;
+        const int64_t lo = first(p * GB), n = first((p + 1) * GB) - lo;
+        auto holding = [&](int64_t t) {  // last chunk of the part that starts at or before its record t
+            int64_t a = 0, b = C;
+            while (b - a > 1) {
+                const int64_t mid = (a + b) >> 1;
+                if (chunk_at(n, mid, C, least) <= t) a = mid; else b = mid;
             }
-            return lo;
+            return p * C + (int)a;
         };
-        gch[g] = make_int2(holding(o0), holding(o1 - 1));
+        gch[g] = make_int2(holding(o0 - lo), holding(o1 - 1 - lo));
     }
 }
 
@@ -2169,7 +2179,7 @@ static FoldArgs fold_args(vup_grid g) {
 // first use after a model evaluation (the histogram, the bin offsets), so a
 // caller may run it on a second stream beside the density preparation.
 vup_status vup_build_layout(vup_grid g, cudaStream_t s, bool points_needed, cudaEvent_t records_done,
-                            cudaEvent_t layout_picked, bool fold) {
+                            cudaEvent_t layout_picked, bool fold, bool coarse) {
     const int64_t N = g->N;
     const int B = g->B;
     // two timed parts: up to the record-stream decision, and the key-sorted streams
@@ -2262,7 +2272,7 @@ vup_status vup_build_layout(vup_grid g, cudaStream_t s, bool points_needed, cuda
             VUP_CHECK_LAUNCH();
             const int Cr = g->n_chunks_rec;
             VUP_CHECK_CUDA(launch_pdl(k_rec_tables, dim3((std::max(n_groups + 2, P_sel * Cr + 1) + 127) / 128), dim3(128), 0, s, rstart, rcnt, Lr, NL, n_groups, GB, L, Cr, (const uint4 *)HL.rec.p, (int32_t *)HL.rec_goff.p, HL.n_rec,
-                HL.rec_chunk, HL.rec_chunk_grp, (int2 *)HL.rec_gch.p));
+                HL.rec_chunk, HL.rec_chunk_grp, (int2 *)HL.rec_gch.p, coarse ? 1 : 0));
             VUP_CHECK_LAUNCH();
             // walk, scan, scatter, tables, gate
             launches += 1 + scan_launches(Lr) + 2 + 1;
@@ -2311,7 +2321,7 @@ vup_status vup_build_layout(vup_grid g, cudaStream_t s, bool points_needed, cuda
         // chunks of every part
         const int PC = g->hist_P * C;
         VUP_CHECK_CUDA(launch_pdl(k_chunks, dim3((PC + 1 + 127) / 128), dim3(128), 0, s, HL.run_start, HL.n_runs, HL.koff, B, L, C, excl, HL.n_iv,
-                                                       HL.chunk_pt, HL.chunk_run, HL.chunk_iv, gate));
+                                                       HL.chunk_pt, HL.chunk_run, HL.chunk_iv, gate, coarse ? 1 : 0));
         VUP_CHECK_LAUNCH();
         VUP_CHECK_CUDA(launch_pdl(k_chunk_bins, dim3((PC + 127) / 128), dim3(128), 0, s, HL.chunk_run, HL.run_bin, L, C, HL.chunk_bin, gate));
         VUP_CHECK_LAUNCH();
@@ -2330,9 +2340,9 @@ vup_status vup_build_layout(vup_grid g, cudaStream_t s, bool points_needed, cuda
     return VUP_OK;
 }
 
-vup_status vup_ensure_layout(vup_grid g, cudaStream_t s, bool points_needed) {
+vup_status vup_ensure_layout(vup_grid g, cudaStream_t s, bool points_needed, bool coarse) {
     if (g->layout_valid && (!points_needed || g->layout_has_points)) return VUP_OK;
-    return vup_build_layout(g, s, points_needed);
+    return vup_build_layout(g, s, points_needed, nullptr, nullptr, true, coarse);
 }
 
 vup_status vup_pick_hist_layout(vup_grid g, cudaStream_t s) {

@@ -278,10 +278,10 @@ __device__ __forceinline__ float4 class_factor(const float *__restrict__ col, in
     return t.value();
 }
 
-// One warp's rows of a tile: rows m0 .. m1 - 1 of the gathered axis' factor
-// table (src: this lane's four densities of row 0), or with `members` the
-// members m0 .. m1 - 1 of the rows' classes in class order (each class' last
-// one flagged), whose factors are summed per class.  Every row goes to dst
+// One warp's rows of a merged tile: the members m0 .. m1 - 1 of the rows' classes
+// in class order (each class' last one flagged), whose factors (src: this lane's
+// four densities of row 0 of the gathered axis' factor table) are summed per
+// class.  Every row goes to dst
 // (SCALED: times the normalisers iz, else its scaled value into the sum that
 // tot receives, [h, l][lane]); eight rows' loads are in flight per warp (16, in
 // line or not, and packed pair arithmetic measured slower: 121 - 144 us against
@@ -328,6 +328,27 @@ __device__ __forceinline__ void tile_rows_in(const float *__restrict__ src, int6
         }
         e = e_next;
     }
+    tot[lane] = t.h;
+    tot[32 + lane] = t.l;
+}
+
+// One warp's rows of an unmerged tile, n rows from src (this lane's four
+// densities), the copies all in flight (each lane reads back its own); dst and
+// tot as above.
+template <bool SCALED>
+__device__ __forceinline__ void plain_rows_in(const float *__restrict__ src, int64_t K_pad, int32_t n, float4 iz, float *dst,
+                                  float4 *tot) {
+    for (int32_t a = 0; a < n; ++a) cp_async16(dst + (int64_t)a * kKT, src + a * K_pad);
+    cp_async_commit();
+    cp_async_wait_all();
+    PairSum4 t;
+    t.clear();
+    for (int32_t a = 0; a < n; ++a, dst += kKT) {
+        const float4 x = ld4(dst);
+        if (SCALED) *reinterpret_cast<float4 *>(dst) = mul4(x, iz);
+        else t.add_scaled(x, iz);
+    }
+    const int lane = threadIdx.x & 31;
     tot[lane] = t.h;
     tot[32 + lane] = t.l;
 }
@@ -749,11 +770,14 @@ __device__ __forceinline__ void hist_item(const HistArgs *Ap, int p, int cg, int
     PairSum4 t;
     t.clear();
     {
-        const int32_t *members = H.cls_start ? H.cls_members : nullptr;
-        const int32_t m0 = members ? H.cls_start[row0 + a0] : (int32_t)row0 + a0;
-        const int32_t m1 = members ? H.cls_start[row0 + a1] : (int32_t)row0 + a1;
-        tile_rows_in<hist_stream_of(MODE) == 0, 8>(H.g_last + k, X.K_pad, members, m0, m1, iz4,
-                                                       ws + (int64_t)a0 * kKT + 4 * lane, reinterpret_cast<float4 *>(win));
+        float *q = ws + (int64_t)a0 * kKT + 4 * lane;
+        if (H.cls_start) {
+            tile_rows_in<hist_stream_of(MODE) == 0, 8>(H.g_last + k, X.K_pad, H.cls_members, H.cls_start[row0 + a0],
+                                                       H.cls_start[row0 + a1], iz4, q, reinterpret_cast<float4 *>(win));
+        } else {
+            plain_rows_in<hist_stream_of(MODE) == 0>(H.g_last + (row0 + a0) * X.K_pad + k, X.K_pad, a1 - a0, iz4, q,
+                                                     reinterpret_cast<float4 *>(win));
+        }
     }
     if (hist_staged(MODE)) {
         // the k-tile's rows of both rest-axis factor tables (unnormalised)
@@ -2123,22 +2147,47 @@ struct HistPlan {
     int64_t rows = 0;
 };
 
+// The most parts either layout of a grid has.
+static int g_parts(const vup_grid_s *g) {
+    int P = 1;
+    for (int l = 0; l < g->n_layouts; ++l) P = std::max(P, g->hl[l].P);
+    return P;
+}
+
 vup_status vup_hist_plan(int n, const vup_grid *gs, const int64_t *Ks, float *const *hists, void **out) {
     std::vector<HistArgs> args(n);
     std::vector<std::pair<int64_t, HistItem>> work;
     std::vector<int4> fin;
     int64_t rows_max = 0;
+    // SM cycles of an instance's tile fill and of its walk per (part, density
+    // tile), from the sizes (its stream and counts are the device's to choose): a
+    // walk costs about a cycle per point and 128 densities on smooth models.  An
+    // instance is cut so that no item's walk exceeds a third of an SM's share of
+    // the whole batch, nor falls below its fill: small batches fill the SMs (8
+    // instances of 38 - 170 points a side: 77 -> 69 us), large ones keep one
+    // item per tile.
+    std::vector<int64_t> fill(n), walk(n);
+    double share = 0.0;
     for (int i = 0; i < n; ++i) {
         int64_t rows;
         int P_max;
         args[i] = hist_args_for(gs[i], Ks[i], hists[i], rows, P_max);
+        fill[i] = 3000 + 30 * rows;
+        walk[i] = gs[i]->N / P_max;
+        if (hists[i]) share += (double)(fill[i] + walk[i]) * (double)P_max * (double)ceil_div64(Ks[i], kKT);
+    }
+    share /= vup_num_sms();
+    for (int i = 0; i < n; ++i) {
         if (!hists[i]) continue;
+        const int P_max = g_parts(gs[i]);
+        const int64_t rows = std::max(args[i].L0.part_rows, args[i].L1.part_rows);
         rows_max = std::max(rows_max, rows);
-        const int G = args[i].C / kGroupChunks;
+        const int64_t most = std::max<int64_t>(1, args[i].C_rec / 8);  // at least eight record chunks
+        const int G = (int)std::max<int64_t>(
+            1, std::min(most, ceil_div64(walk[i], std::max((int64_t)(share / 3.0), fill[i]))));
         args[i].sets = G;
         const int64_t nkt = ceil_div64(Ks[i], kKT);
-        // cost of one item: points per chunk x densities per tile
-        const int64_t cost = gs[i]->N / std::max<int64_t>(1, (int64_t)P_max * args[i].C);
+        const int64_t cost = fill[i] + walk[i] / G;
         for (int p = 0; p < P_max; ++p)
             for (int cg = 0; cg < G; ++cg)
                 for (int64_t kt = 0; kt < nkt; ++kt) work.push_back({cost, HistItem{i, p, cg, (int32_t)kt}});

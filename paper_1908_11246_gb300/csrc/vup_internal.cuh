@@ -330,7 +330,7 @@ struct vup_grid_s {
 
     // per-K scratch (density constants, factor tables, partials)
     int64_t K_cap = 0;
-    DevBuf dconst, dstats, dpart, ftab, atab_hi, atab_lo, partials, hist_part, hist_direct, ipsa_part;
+    DevBuf dconst, dstats, ftab, atab_hi, atab_lo, partials, hist_part, hist_direct, ipsa_part;
     DevBuf post_tmp, post_x;  // posterior means: weighted tables, sums per key; axis coordinates
     DevBuf ftab_fold;    // merged factor tables of the folded axes, axis d at fold_off(d) rows of K_pad
     DevBuf atf_hi, atf_lo;         // TF32 split of the A operand [K_pad][R_pad]
@@ -361,8 +361,9 @@ vup_status vup_pick_hist_layout(vup_grid g, cudaStream_t s);
 // fold: merge equal slices of the bin grid first (FoldGeom).
 vup_status vup_build_layout(vup_grid g, cudaStream_t s, bool points_needed = false,
                             cudaEvent_t records_done = nullptr, cudaEvent_t layout_picked = nullptr,
-                            bool fold = true);
-vup_status vup_ensure_layout(vup_grid g, cudaStream_t s, bool points_needed = false);
+                            bool fold = true, bool coarse = false);
+// coarse: at least 24 records (256 points) per chunk, for a grid among many of a batch.
+vup_status vup_ensure_layout(vup_grid g, cudaStream_t s, bool points_needed = false, bool coarse = false);
 // every layout's part tile fits the shared-memory histogram kernels
 bool vup_hist_tile_fits(vup_grid g);
 // the 3-D point stream stages both rest-axis factor tables in shared memory
@@ -423,7 +424,6 @@ vup_status vup_reserve_k(vup_grid g, int64_t K, bool bf16, bool ipsa, bool tf32 
 // lists and uploads them into device memory it owns (synchronous; never call
 // during stream capture); each *_batched launch is stream-ordered and
 // capturable; *_plan_free releases a plan.
-vup_status vup_density_reserve(vup_grid g, int64_t K);
 vup_status vup_density_plan(int n, const vup_grid *gs, const vup_densities *ds, bool bf16, void **plan);
 vup_status vup_density_batched(void *plan, cudaStream_t s);
 void vup_density_plan_free(void *plan);
