@@ -187,24 +187,28 @@ __device__ __forceinline__ void simt_tile(const float *__restrict__ A, const flo
         __syncthreads();
     }
 
-    // reduce over the 16 column threads of a half-warp (FP64)
+    // reduce over the 16 column threads of a half-warp (FP64): at each step a lane
+    // keeps half of its values and adds its partner's, so lane tx ends with value tx
+    // = 4 row + power (15 FP64 additions for 16 values, in the same tree as 64 of a
+    // butterfly per value, which took a tenth to a third of a tile's time)
 #pragma unroll
-    for (int pl = 0; pl < NPL; ++pl)
+    for (int pl = 0; pl < NPL; ++pl) {
+        double v[16];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            double v[4];
+        for (int i = 0; i < 4; ++i)
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                v[j] = (double)out[pl][i][j] - (double)cmp[pl][i][j];
-                v[j] += __shfl_xor_sync(0xffffffffu, v[j], 8);
-                v[j] += __shfl_xor_sync(0xffffffffu, v[j], 4);
-                v[j] += __shfl_xor_sync(0xffffffffu, v[j], 2);
-                v[j] += __shfl_xor_sync(0xffffffffu, v[j], 1);
+            for (int j = 0; j < 4; ++j) v[4 * i + j] = (double)out[pl][i][j] - (double)cmp[pl][i][j];
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) {
+            const bool up = (tx & o) != 0;
+#pragma unroll
+            for (int i = 0; i < o; ++i) {
+                const double keep = up ? v[i + o] : v[i], send = up ? v[i] : v[i + o];
+                v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
             }
-            if (tx == 0)
-                *reinterpret_cast<float4 *>(part + (((int64_t)pl * n_ct + ct) * K_pad + k0 + ty * 4 + i) * 4) =
-                    make_float4((float)v[0], (float)v[1], (float)v[2], (float)v[3]);
         }
+        part[(((int64_t)pl * n_ct + ct) * K_pad + k0 + ty * 4 + (tx >> 2)) * 4 + (tx & 3)] = (float)v[0];
+    }
 }
 
 template <int NPL>
