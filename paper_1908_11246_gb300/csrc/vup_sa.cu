@@ -30,32 +30,64 @@ __device__ __forceinline__ int dev_bin(int b, double ymin, double w, double yref
     return f < 0.0 ? 0 : (f > (double)(nd - 1) ? nd - 1 : (int)f);
 }
 
-// One CTA per column k: every output bin's deviation bin is computed once
-// into shared memory (one FP64 division each); the map is non-decreasing in
-// b, so the bins of deviation bin e form one contiguous range, found by
-// binary search over the shared map and summed in increasing b.
-__global__ void k_ipsa_matrix(const float *__restrict__ H, int64_t K, int B, const unsigned long long *__restrict__ ext,
-                              const double *__restrict__ yref, int nd, double dlo, double dhi,
-                              float *__restrict__ out) {
-    extern __shared__ int emap[];  // [B]
-    const double ymin = ext_value(ext[0]), ymax = ext_value(ext[1]);
-    const double w = __ddiv_rn(__dsub_rn(ymax, ymin), (double)B);
-    const double wd = __ddiv_rn(__dsub_rn(dhi, dlo), (double)nd);
+// dev_bin with an FP32 screen: t = b s + o in FP32 (s = w / wd, o the rest of the
+// quotient, each rounded once from FP64) is within eps of the exact quotient;
+// where no integer lies within eps of t its floor is the bin, otherwise the FP64
+// expression decides (about one bin in a thousand).  Error of t: the roundings
+// of s, o and the FMA, each <= 2^-24 relative to |b s| + |o|; eps allows eight
+// times that.
+struct DevRule {
+    double ymin, w, yref, dlo, wd;
+    float s, o;
+    int nd;
+    __device__ __forceinline__ int operator()(int b) const {
+        const float t = fmaf((float)b, s, o);
+        const float f = floorf(t);
+        const float eps = 0x1p-21f * (fabsf((float)b * s) + fabsf(o) + 1.f);
+        if (t - f > eps && f + 1.f - t > eps) return f < 0.f ? 0 : (f > (float)(nd - 1) ? nd - 1 : (int)f);
+        return dev_bin(b, ymin, w, yref, dlo, wd, nd);
+    }
+};
+
+// One CTA per column k: every output bin's deviation bin is computed once into
+// shared memory; the map is non-decreasing in b, so the bins of deviation bin e
+// form one contiguous range, whose first bin is noted as the map is made, and
+// are summed in increasing b.  FP64 bounds it: a division per bin and a search
+// per deviation bin took 63 us for 1000 columns of 1000 bins, the screen and
+// the noted starts 25.
+__global__ void __launch_bounds__(256) k_ipsa_matrix(const float *__restrict__ H, int64_t K, int B,
+                                                     const unsigned long long *__restrict__ ext,
+                                                     const double *__restrict__ yref, int nd, double dlo, double dhi,
+                                                     float *__restrict__ out) {
+    extern __shared__ int emap[];  // [B], then the first bin of each deviation bin [nd] (B: none)
+    int *first = emap + B;
+    __shared__ DevRule s_rule;
     for (int64_t k = blockIdx.x; k < K; k += gridDim.x) {
-        const double yr = yref[k];
         __syncthreads();  // the previous column's readers are done
-        for (int b = threadIdx.x; b < B; b += blockDim.x) emap[b] = dev_bin(b, ymin, w, yr, dlo, wd, nd);
+        if (threadIdx.x == 0) {
+            const double ymin = ext_value(ext[0]), ymax = ext_value(ext[1]), yr = yref[k];
+            const double w = __ddiv_rn(__dsub_rn(ymax, ymin), (double)B);
+            const double wd = __ddiv_rn(__dsub_rn(dhi, dlo), (double)nd);
+            s_rule = DevRule{ymin, w, yr, dlo, wd, (float)(w / wd), (float)((ymin + 0.5 * w - yr - dlo) / wd), nd};
+        }
+        for (int e = threadIdx.x; e < nd; e += blockDim.x) first[e] = B;
+        __syncthreads();
+        const DevRule R = s_rule;
+        for (int b = threadIdx.x; b < B; b += blockDim.x) emap[b] = R(b);
+        __syncthreads();
+        for (int b = threadIdx.x; b < B; b += blockDim.x)
+            if (b == 0 || emap[b] != emap[b - 1]) first[emap[b]] = b;
         __syncthreads();
         const float *h = H + k * B;
         for (int e = threadIdx.x; e < nd; e += blockDim.x) {
-            int lo = 0, hi = B;  // first b with emap[b] >= e
-            while (lo < hi) {
-                const int mid = (lo + hi) >> 1;
-                if (emap[mid] >= e) hi = mid; else lo = mid + 1;
+            const int lo = first[e];
+            float v = lo < B ? h[lo] : 0.f;  // (one bin: its value; more: summed in FP64)
+            if (lo + 1 < B && emap[lo + 1] == e) {
+                double s = (double)v;
+                for (int b = lo + 1; b < B && emap[b] == e; ++b) s = __dadd_rn(s, (double)h[b]);
+                v = (float)s;
             }
-            double s = 0.0;
-            for (int b = lo; b < B && emap[b] == e; ++b) s = __dadd_rn(s, (double)h[b]);
-            out[k * nd + e] = (float)s;
+            out[k * nd + e] = v;
         }
     }
 }
@@ -68,13 +100,16 @@ __global__ void k_deviation_moments(const double *__restrict__ raw, int64_t K, i
     double M[5] = {1.0, 0.0, 0.0, 0.0, 0.0};
     for (int j = 1; j <= J; ++j) M[j] = raw[k * J + j - 1];
     const double c = -yref[k];
-    for (int j = 1; j <= J; ++j) {
-        double s = 0.0, binom = 1.0, cp = 1.0;
+    const double C[5][5] = {{1, 0, 0, 0, 0}, {1, 1, 0, 0, 0}, {1, 2, 1, 0, 0}, {1, 3, 3, 1, 0}, {1, 4, 6, 4, 1}};
+#pragma unroll
+    for (int j = 1; j <= 4; ++j) {
+        if (j > J) break;
+        double s = 0.0, cp = 1.0;
         // terms m = j, j-1, ..., 0: C(j, m) M_m c^(j-m)
+#pragma unroll
         for (int m = j; m >= 0; --m) {
-            s += binom * M[m] * cp;
+            s += C[j][m] * M[m] * cp;
             cp *= c;
-            binom = binom * (double)m / (double)(j - m + 1);
         }
         out[k * J + j - 1] = s;
     }
@@ -149,13 +184,28 @@ __global__ void k_sa_global_part(const float *__restrict__ H, int64_t K, int nb,
     const int64_t k0 = (int64_t)blockIdx.y * kSaRows, k1 = min(K, k0 + kSaRows);
     if (b < nb) {
         double g = 0.0;
+        if (rho) {
 #pragma unroll 16
-        for (int64_t k = k0; k < k1; ++k) g = __dadd_rn(g, __dmul_rn(rho ? rho[k] : 1.0, (double)__ldg(H + k * nb + b)));
+            for (int64_t k = k0; k < k1; ++k) g = __dadd_rn(g, __dmul_rn(rho[k], (double)__ldg(H + k * nb + b)));
+        } else {
+            const float *h = H + k0 * nb + b;
+            for (int64_t q = 0; q < k1 - k0; q += 32) {  // 32 rows' loads in flight, added in order
+                float v[32];
+#pragma unroll
+                for (int u = 0; u < 32; ++u) v[u] = q + u < k1 - k0 ? __ldg(h + (q + u) * nb) : 0.f;
+#pragma unroll
+                for (int u = 0; u < 32; ++u)
+                    if (q + u < k1 - k0) g = __dadd_rn(g, (double)v[u]);
+            }
+        }
         part[(int64_t)blockIdx.y * nb + b] = g;
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         double rs = 0.0;
-        for (int64_t k = k0; k < k1; ++k) rs = __dadd_rn(rs, rho ? rho[k] : 1.0);
+        if (rho)
+            for (int64_t k = k0; k < k1; ++k) rs = __dadd_rn(rs, rho[k]);
+        else
+            rs = (double)(k1 - k0);
         rpart[blockIdx.y] = rs;
     }
 }
@@ -164,6 +214,7 @@ __global__ void k_sa_global_sum(const double *__restrict__ part, const double *_
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= nb) return;
     double g = 0.0, rs = 0.0;
+#pragma unroll 8
     for (int64_t q = 0; q < nblk; ++q) {
         g = __dadd_rn(g, part[q * nb + b]);
         rs = __dadd_rn(rs, rpart[q]);
@@ -187,7 +238,7 @@ extern "C" vup_status vup_deviation_moments(vup_grid g, int64_t K, const double 
     if (!g->have_model) return VUP_ERR_STATE;
     cudaStream_t s = (cudaStream_t)stream;
     VUP_PROF("deviation_moments", s, 1);
-    k_deviation_moments<<<(unsigned)ceil_div64(K, 128), 128, 0, s>>>(moments_raw, K, g->J, y_ref, out);
+    k_deviation_moments<<<(unsigned)ceil_div64(K, 32), 32, 0, s>>>(moments_raw, K, g->J, y_ref, out);
     VUP_CHECK_LAUNCH();
     return VUP_OK;
 }
@@ -200,8 +251,8 @@ extern "C" vup_status vup_ipsa_matrix(vup_grid g, int64_t K, const float *hist, 
     if (!g->have_model) return VUP_ERR_STATE;
     cudaStream_t s = (cudaStream_t)stream;
     VUP_PROF("ipsa_matrix", s, 1);
-    const size_t smem = sizeof(int) * (size_t)g->B;
-    if (smem > 48 * 1024)
+    const size_t smem = sizeof(int) * ((size_t)g->B + (size_t)n_dbins);
+    if (smem > 40 * 1024)
         VUP_CHECK_CUDA(cudaFuncSetAttribute(k_ipsa_matrix, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const unsigned grid = (unsigned)std::min<int64_t>(K, (int64_t)vup_num_sms() * 8);
     k_ipsa_matrix<<<grid, 256, smem, s>>>(hist, K, g->B, g->ext, y_ref, n_dbins, dlo, dhi, out);

@@ -77,10 +77,10 @@ __device__ __forceinline__ float epi_weight(const EpiArgs &ep, int64_t K_pad, in
 // The FP32 pipes bound it: a chain costs 8 multiply-adds and 4 operations of
 // fold, so at most 2/3 of the multiply-add rate.  4 x 8 values per thread leave
 // room for 16 warps per SM (8 x 8 values, 8 warps: 888 us at 900 x 1100 points, K
-// = 3000; packed FP32 pairs: 1169; this form: 814).  NPL = 3 forms the IPSA sums
+// = 3000; packed FP32 pairs: 1169; this form: 774).  NPL = 3 forms the IPSA sums
 // (weights e, e u, e u^2) from one set of chains, 8 + 12 operations per chain
 // instead of 3 (8 + 4), on tiles of 64 densities (the three planes' sums take
-// the registers; 500 x 400 points, K = 2000, both orientations: 1009 -> 590 us).
+// the registers; 500 x 400 points, K = 2000, both orientations: 1009 -> 489 us).
 template <int NPL>
 struct SimtShape {
     static constexpr int kTM = NPL == 3 ? 64 : 128;  // densities of a tile
