@@ -1331,7 +1331,19 @@ __global__ void k_layout_encode(const int32_t *__restrict__ run_start, const int
 // less (some chunks are then empty, spread evenly): a chunk's cut keys or groups
 // cost partial rows, which short chunks would make the larger part of the work
 // (a batch's finish: 102 -> 86 us), and neither needs them to fill the SMs.
-constexpr int kChunkPoints = 256, kChunkRecords = 24;
+// Records: as many whole rounds of one chunk for each of the walk's 16 warps as
+// keep the chunks at or under kChunkRecMost, so that no round leaves most warps
+// idle.  Walk + finish against chunks of 24 whatever their number: 1024 x 1024
+// points, K = 16384 (1165 records per part) 159 -> 147 us; 2048 x 2048, K = 65536
+// (1550) 950 -> 893; 1021 x 613, K = 9001 (1100) 119 -> 113; 32 uneven instances
+// 384 -> 360.  At most 48: 147 / 893 / 113 / 374; at most 100 (one round): 139 / 842 /
+// 125 / 366, where a part split between two CTAs leaves half their warps idle.
+constexpr int kChunkPoints = 256, kChunkRecLeast = 24, kChunkRecMost = 64, kRecWalkWarps = 16;
+__device__ __forceinline__ int64_t record_chunk(int64_t n) {
+    const int64_t round = (n + kRecWalkWarps - 1) / kRecWalkWarps;
+    const int64_t rounds = max((round + kChunkRecMost - 1) / kChunkRecMost, (int64_t)1);
+    return max((round + rounds - 1) / rounds, (int64_t)kChunkRecLeast);
+}
 __device__ __forceinline__ int64_t chunk_at(int64_t n, int64_t cc, int64_t C, int64_t least) {
     int64_t t = n * cc / C;
     if (least > 1 && n < C * least && cc < C) t = t / least * least;
@@ -1631,7 +1643,8 @@ __global__ void k_rec_tables(const int32_t *__restrict__ starts, const int32_t *
     pdl_trigger();
     pdl_wait();
     const int P = L.get().P;
-    const int64_t least = coarse || L.fold->any ? kChunkRecords : 1;
+    const bool whole = coarse || L.fold->any;
+    auto least_of = [&](int64_t n) -> int64_t { return whole ? record_chunk(n) : 1; };
     const int32_t total = starts[Lr - 1] + counts[Lr - 1];
     auto first = [&](int g) -> int32_t { return g < n_groups ? starts[g * NL] : total; };
     const int i = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
@@ -1644,6 +1657,7 @@ __global__ void k_rec_tables(const int32_t *__restrict__ starts, const int32_t *
         }
         const int p = c / C, cc = c - p * C;
         const int64_t lo = first(p * GB), n = first((p + 1) * GB) - lo;
+        const int64_t least = least_of(n);
         const int32_t r = (int32_t)(lo + chunk_at(n, cc, C, least)), r1 = (int32_t)(lo + chunk_at(n, cc + 1, C, least));
         chunk_rec[c] = r;
         chunk_grp[2 * c] = r1 > r ? (int32_t)rec[2 * (int64_t)r + 1].z : -1;
@@ -1656,7 +1670,7 @@ __global__ void k_rec_tables(const int32_t *__restrict__ starts, const int32_t *
             gch[g] = make_int2(-1, -1);
             continue;
         }
-        const int64_t lo = first(p * GB), n = first((p + 1) * GB) - lo;
+        const int64_t lo = first(p * GB), n = first((p + 1) * GB) - lo, least = least_of(n);
         auto holding = [&](int64_t t) {  // last chunk of the part that starts at or before its record t
             int64_t a = 0, b = C;
             while (b - a > 1) {

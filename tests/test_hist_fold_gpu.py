@@ -98,3 +98,22 @@ def test_merged_slices_batched():
         g.sync()
         ref = O.solve(p, rows=np.arange(p.K))["hist"]
         assert np.abs(hs.cpu().numpy() - ref).max() <= HIST_TOL
+
+
+# records per part from fewer than one chunk per warp to several rounds of chunks for every warp
+@pytest.mark.parametrize("n0,n1,B", [(24, 40, 8), (200, 300, 30), (401, 500, 60), (640, 900, 64), (1800, 1100, 500)])
+def test_record_chunks_match_oracle(n0, n1, B):
+    from paper_1908_11246_gb300 import vup
+    lo, hi = (-1.0, -1.0), (2.0, 2.0)
+    y = np.add.outer(np.linspace(-1, 1, n0) ** 2, 3 * np.abs(np.linspace(-1, 1, n1)))
+    K = 130
+    dens = I.random_densities(np.random.default_rng(90), K, lo, hi, kinds=(I.GAUSS,), sig=(0.2, 1.0), margin=0.1)
+    b, _, _ = O.bins(y.ravel(), B)
+    ref = O.propagate((n0, n1), lo, hi, y.ravel(), b, B, 4, dens, rows=np.arange(K))["hist"]
+    g = vup.Grid((n0, n1), lo, hi)
+    g.set_outputs(torch.as_tensor(y, device="cuda"), B)
+    g.set_hist_stream(2)
+    _, _, hs = g.propagate(vup.densities_to_device(dens), "fp32")
+    g.sync()
+    assert np.abs(hs.cpu().numpy() - ref).max() <= HIST_TOL
+    g.close()
