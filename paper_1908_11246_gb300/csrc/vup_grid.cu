@@ -1331,6 +1331,10 @@ __global__ void k_layout_encode(const int32_t *__restrict__ run_start, const int
 // less (some chunks are then empty, spread evenly): a chunk's cut keys or groups
 // cost partial rows, which short chunks would make the larger part of the work
 // (a batch's finish: 102 -> 86 us), and neither needs them to fill the SMs.
+// Points (and intervals, cut where points are): n / 512, at least 64, where the 80
+// or more slots then give a small grid's few density tiles a chunk for most warps
+// (8200 merged points, K = 225: walk 35 us at 256 points, 27 at 64 or 32), at most
+// 256 (131072 points, K = 16384: 765; 775 at 128 and 512).
 // Records: as many whole rounds of one chunk for each of the walk's 16 warps as
 // keep the chunks at or under kChunkRecMost, so that no round leaves most warps
 // idle.  Walk + finish against chunks of 24 whatever their number: 1024 x 1024
@@ -1338,7 +1342,10 @@ __global__ void k_layout_encode(const int32_t *__restrict__ run_start, const int
 // (1550) 950 -> 893; 1021 x 613, K = 9001 (1100) 119 -> 113; 32 uneven instances
 // 384 -> 360.  At most 48: 147 / 893 / 113 / 374; at most 100 (one round): 139 / 842 /
 // 125 / 366, where a part split between two CTAs leaves half their warps idle.
-constexpr int kChunkPoints = 256, kChunkRecLeast = 24, kChunkRecMost = 64, kRecWalkWarps = 16;
+constexpr int kChunkPtsLeast = 64, kChunkPtsMost = 256, kChunkRecLeast = 24, kChunkRecMost = 64, kRecWalkWarps = 16;
+__device__ __forceinline__ int64_t point_chunk(int64_t n) {
+    return min(max(n / 512, (int64_t)kChunkPtsLeast), (int64_t)kChunkPtsMost);
+}
 __device__ __forceinline__ int64_t record_chunk(int64_t n) {
     const int64_t round = (n + kRecWalkWarps - 1) / kRecWalkWarps;
     const int64_t rounds = max((round + kChunkRecMost - 1) / kChunkRecMost, (int64_t)1);
@@ -1373,7 +1380,7 @@ __global__ void k_chunks(const int32_t *__restrict__ run_start, const int32_t *_
     } else {
         const int p = c / C, cc = c - p * C;
         const int64_t lo = koff[p * B], hi = koff[(p + 1) * B];
-        const int64_t target = lo + chunk_at(hi - lo, cc, C, coarse || L.fold->any ? kChunkPoints : 1);
+        const int64_t target = lo + chunk_at(hi - lo, cc, C, coarse || L.fold->any ? point_chunk(hi - lo) : 1);
         int32_t a = 0, b = n_runs;  // first r in [0, n_runs] with run_start[r] >= target
         while (a < b) {
             int32_t mid = (a + b) >> 1;
