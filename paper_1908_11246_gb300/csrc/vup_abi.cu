@@ -215,40 +215,17 @@ extern "C" const char *vup_version(void) { return "vup-gb300 0.1 (sm_103a)"; }
 extern "C" const char *vup_last_error_detail(void) { return g_last_err; }
 
 static void free_grid(vup_grid g) {
-    cudaFree(g->y);
-    cudaFree(g->axis_terms);
-    cudaFree(g->ext);
-    cudaFree(g->bins);
-    cudaFree(g->perm);
+    cudaFree(g->arena);
     cudaFree(g->offsets);
-    {  // the built layout's arrays (hl[1] aliases them)
+    {  // the built layout's arrays outside the arena (hl[1] aliases them)
         auto &L = g->hl[0];
-        if (L.perm != g->perm) cudaFree(L.perm);
-        cudaFree(L.keys_own);
         cudaFree(L.koff);
         cudaFree(L.key_chunks);
-        cudaFree(L.hpt);
-        cudaFree(L.run_start);
-        cudaFree(L.run_rest);
-        cudaFree(L.run_bin);
-        cudaFree(L.n_runs);
-        cudaFree(L.chunk_pt);
-        cudaFree(L.chunk_run);
-        cudaFree(L.chunk_bin);
-        cudaFree(L.ipt);
-        cudaFree(L.iv_rest);
-        cudaFree(L.n_iv);
-        cudaFree(L.chunk_iv);
-        cudaFree(L.n_rec);
-        cudaFree(L.rec_chunk);
-        cudaFree(L.rec_chunk_grp);
         devbuf_free(L.rec);
         devbuf_free(L.rec_rest);
         devbuf_free(L.rec_goff);
         devbuf_free(L.rec_gch);
     }
-    cudaFree(g->hist_sel);
-    cudaFree(g->fold_mem);
     if (g->side) cudaStreamDestroy(g->side);
     if (g->ev_fork) cudaEventDestroy(g->ev_fork);
     if (g->ev_join) cudaEventDestroy(g->ev_join);
@@ -257,8 +234,6 @@ static void free_grid(vup_grid g) {
     if (g->ev_mom) cudaEventDestroy(g->ev_mom);
     if (g->ev_mfin) cudaEventDestroy(g->ev_mfin);
     if (g->side2) cudaStreamDestroy(g->side2);
-    cudaFree(g->ydev_scale);
-    cudaFree(g->dstatus);
     for (int o = 0; o < kNumOrient; ++o) {
         cudaFree(g->ztf_hi[o]);
         cudaFree(g->ztf_lo[o]);
@@ -333,14 +308,23 @@ extern "C" vup_status vup_grid_create(int ndim, const int64_t *n, const double *
     g->n_chunks = vup_hist_chunks_for(N, p_all);
     g->n_chunks_rec = vup_hist_rec_chunks_for(g->n_chunks);
     const int C = g->n_chunks;
-    cudaError_t e = cudaSuccess;
-#define ALLOC(ptr, bytes) \
-    if (e == cudaSuccess) e = vup_dev_malloc((void **)&(ptr), (bytes))
-    ALLOC(g->y, sizeof(double) * N);
-    ALLOC(g->axis_terms, sizeof(double2) * (size_t)(g->n[0] + (ndim > 1 ? g->n[1] : 0) + (ndim > 2 ? g->n[2] : 0)));
-    ALLOC(g->ext, sizeof(unsigned long long) * 3);  // range keys (min, max) and a grid-barrier counter
-    ALLOC(g->bins, sizeof(int32_t) * N);
-    ALLOC(g->perm, sizeof(int32_t) * N);
+    // every array whose size the grid fixes, in one device allocation (256-byte
+    // aligned pieces): one call to the driver instead of thirty
+    struct Piece {
+        void **p;
+        size_t at;
+    };
+    std::vector<Piece> pieces;
+    size_t total = 0;
+    auto place = [&](auto &ptr, size_t bytes) {
+        pieces.push_back({(void **)&ptr, total});
+        total += (bytes + 255) & ~(size_t)255;
+    };
+    place(g->y, sizeof(double) * N);
+    place(g->axis_terms, sizeof(double2) * (size_t)(g->n[0] + (ndim > 1 ? g->n[1] : 0) + (ndim > 2 ? g->n[2] : 0)));
+    place(g->ext, sizeof(unsigned long long) * 3);  // range keys (min, max) and a grid-barrier counter
+    place(g->bins, sizeof(int32_t) * N);
+    place(g->perm, sizeof(int32_t) * N);
     g->n_layouts = ndim == 2 ? 2 : 1;
     int p_max = 1;
     for (int l = 0; l < g->n_layouts; ++l) {
@@ -351,29 +335,50 @@ extern "C" vup_status vup_grid_create(int ndim, const int64_t *n, const double *
     }
     {
         auto &L = g->hl[0];  // arrays of the one layout built per model
-        ALLOC(L.hpt, sizeof(uint32_t) * (N + 512));  // tail slack for whole staged windows
-        ALLOC(L.run_start, sizeof(int32_t) * (N + 1));
-        ALLOC(L.run_rest, sizeof(int32_t) * N);
-        ALLOC(L.run_bin, sizeof(int32_t) * N);
-        ALLOC(L.n_runs, sizeof(int32_t));
-        ALLOC(L.chunk_pt, sizeof(int32_t) * (p_max * C + 1));
-        ALLOC(L.chunk_run, sizeof(int32_t) * (p_max * C + 1));
-        ALLOC(L.chunk_bin, sizeof(int32_t) * 2 * p_max * C);
+        place(L.hpt, sizeof(uint32_t) * (N + 512));  // tail slack for whole staged windows
+        place(L.run_start, sizeof(int32_t) * (N + 1));
+        place(L.run_rest, sizeof(int32_t) * N);
+        place(L.run_bin, sizeof(int32_t) * N);
+        place(L.n_runs, sizeof(int32_t));
+        place(L.chunk_pt, sizeof(int32_t) * (p_max * C + 1));
+        place(L.chunk_run, sizeof(int32_t) * (p_max * C + 1));
+        place(L.chunk_bin, sizeof(int32_t) * 2 * p_max * C);
         if (ndim >= 2) {
-            ALLOC(L.perm, sizeof(int32_t) * N);
-            ALLOC(L.keys_own, sizeof(int32_t) * N);
-            ALLOC(L.ipt, sizeof(uint2) * (N + 128));  // tail slack for whole staged windows
-            ALLOC(L.iv_rest, sizeof(int32_t) * N);
-            ALLOC(L.n_iv, sizeof(int32_t));
-            ALLOC(L.chunk_iv, sizeof(int32_t) * (p_max * C + 1));
-            ALLOC(L.n_rec, sizeof(int32_t));
-            ALLOC(L.rec_chunk, sizeof(int32_t) * (p_max * g->n_chunks_rec + 1));
-            ALLOC(L.rec_chunk_grp, sizeof(int32_t) * 2 * p_max * g->n_chunks_rec);
+            place(L.perm, sizeof(int32_t) * N);
+            place(L.keys_own, sizeof(int32_t) * N);
+            place(L.ipt, sizeof(uint2) * (N + 128));  // tail slack for whole staged windows
+            place(L.iv_rest, sizeof(int32_t) * N);
+            place(L.n_iv, sizeof(int32_t));
+            place(L.chunk_iv, sizeof(int32_t) * (p_max * C + 1));
+            place(L.n_rec, sizeof(int32_t));
+            place(L.rec_chunk, sizeof(int32_t) * (p_max * g->n_chunks_rec + 1));
+            place(L.rec_chunk_grp, sizeof(int32_t) * 2 * p_max * g->n_chunks_rec);
+        }
+    }
+    // equal-slice folding: geometry, class members (CSR), build scratch, merged bins
+    int64_t slices = 0;
+    for (int d = 0; d < ndim; ++d) slices += n[d];
+    if (ndim >= 2) {
+        g->fold_scratch_bytes = vup_fold_scratch_bytes(g);
+        place(g->fold, sizeof(FoldGeom));
+        place(g->fold_rep, sizeof(int32_t) * (size_t)(3 * slices + 3));
+        place(g->fold_scratch, g->fold_scratch_bytes);
+        place(g->fold_bins, sizeof(int32_t) * (size_t)N);
+    }
+    place(g->hist_sel, sizeof(int32_t) * 8);
+    place(g->ydev_scale, sizeof(double) * kScaleSlots);
+    place(g->dstatus, sizeof(int));
+    cudaError_t e = vup_dev_malloc(&g->arena, total);
+    if (e == cudaSuccess) {
+        for (const Piece &q : pieces) *q.p = (uint8_t *)g->arena + q.at;
+        if (ndim >= 2) {
+            g->fold_members = g->fold_rep + slices;
+            g->fold_start = g->fold_members + slices;
             // words past the stream's end are read by whole-window staging and
             // masked; zero keeps their rest codes valid indices
-            if (e == cudaSuccess) e = cudaMemset(L.ipt, 0, sizeof(uint2) * (N + 128));
+            e = cudaMemset(g->hl[0].ipt, 0, sizeof(uint2) * (N + 128));
         } else {
-            L.perm = g->perm;
+            g->hl[0].perm = g->perm;
         }
     }
     if (g->n_layouts > 1) {
@@ -397,27 +402,6 @@ extern "C" vup_status vup_grid_create(int ndim, const int64_t *n, const double *
         L.rec_chunk = A.rec_chunk;
         L.rec_chunk_grp = A.rec_chunk_grp;
     }
-    if (ndim >= 2) {
-        // equal-slice folding: geometry, class members (CSR), build scratch, merged bins
-        int64_t slices = 0;
-        for (int d = 0; d < ndim; ++d) slices += n[d];
-        const size_t a16 = 15, idx = sizeof(int32_t) * (size_t)(3 * slices + 3);
-        const size_t o_idx = (sizeof(FoldGeom) + a16) & ~a16, o_scr = (o_idx + idx + a16) & ~a16;
-        g->fold_scratch_bytes = vup_fold_scratch_bytes(g);
-        const size_t o_bins = (o_scr + g->fold_scratch_bytes + a16) & ~a16;
-        ALLOC(g->fold_mem, o_bins + sizeof(int32_t) * (size_t)N);
-        uint8_t *base = (uint8_t *)g->fold_mem;
-        g->fold = (FoldGeom *)base;
-        g->fold_rep = (int32_t *)(base + o_idx);
-        g->fold_members = g->fold_rep + slices;
-        g->fold_start = g->fold_members + slices;
-        g->fold_scratch = base + o_scr;
-        g->fold_bins = (int32_t *)(base + o_bins);
-    }
-    ALLOC(g->hist_sel, sizeof(int32_t) * 8);
-    ALLOC(g->ydev_scale, sizeof(double) * kScaleSlots);
-    ALLOC(g->dstatus, sizeof(int));
-#undef ALLOC
     if (e == cudaSuccess) e = cudaMemset(g->dstatus, 0, sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(g->hist_sel, 0, sizeof(int32_t) * 8);
     if (e != cudaSuccess) {

@@ -303,7 +303,6 @@ struct vup_grid_s {
     // equal-slice folding of the bin grid (2-D / 3-D): one allocation holding
     // the device geometry, the class members per axis (CSR: start, members),
     // the build's scratch (zeroed first) and the merged bins
-    void *fold_mem = nullptr;
     FoldGeom *fold = nullptr;
     int32_t *fold_rep = nullptr, *fold_start = nullptr, *fold_members = nullptr, *fold_bins = nullptr;
     uint8_t *fold_scratch = nullptr;
@@ -314,6 +313,7 @@ struct vup_grid_s {
     // [8] device: chosen layout, stream, intervals of layouts 0 / 1, key streams built,
     // item counters of the three streams' walks
     int32_t *hist_sel = nullptr;
+    void *arena = nullptr;  // the device memory behind every array whose size the grid fixes
     int hist_force = -1;           // -1 auto, 0 points only, 1 intervals only
     int32_t n_chunks = 0;
     int32_t n_chunks_rec = 0;      // record chunks per part (records are several times fewer than points)
