@@ -215,12 +215,8 @@ def roofline_for(name, ms, n_work, units, pk, workload, hist_units=None):
     it that do the work (the histogram's launch for the stream the device did
     not choose returns at once and is not counted); units: dist-points one
     working launch covers (every contraction launch, moments or one IPSA
-    orientation, covers all K x N); hist_units: bytes one histogram pass moves
-    through the SM's L1 data pipe by its algorithm (per density: 4 per point +
-    4 per rest-factor row per run on the point stream; 8 of prefix sums + 4 per
-    rest-factor row per interval on the interval stream; on the record stream
-    4 per prefix sum a record needs -- one per bin it holds and one more, the
-    intervals plus the records in all -- + 4 per rest-factor row per record)."""
+    orientation, covers all K x N); hist_units: bytes one histogram pass needs
+    through the SM's L1 data pipe (walk_bytes)."""
     per = ms / max(n_work, 1) * 1e-3
     tr = traffic_for(name, workload)
     if name.startswith(("moments_bf16", "ipsa_bf16", "moments_tf32")):
@@ -246,15 +242,58 @@ def roofline_for(name, ms, n_work, units, pk, workload, hist_units=None):
         peak = pk["gather_gbs"]
         a = (hist_units or 4.0 * units) / per / 1e9
         return {"bound": "alu", "achieved": a, "peak": peak, "unit": "GB/s", "frac": a / peak, "traffic": tr,
-                "note": "bytes through the L1 data pipe that the walk needs per pass (per density: point stream "
-                        "4 per point + 4 per rest-factor row per run; interval stream 8 of prefix sums + 4 per "
-                        "rest-factor row per interval; record stream 4 per prefix sum it needs (one per bin a "
-                        "record holds + one per record) + 4 per rest-factor row "
-                        "per record); peak = shared-memory 512-byte row gathers measured by "
+                "note": "bytes through the L1 data pipe of the cheapest walk of the bin grid, equal slices "
+                        "merged (per density: points 4 each + 4 per rest-factor row per run; intervals 8 of "
+                        "prefix sums + 4 per rest-factor row; records 4 per prefix sum needed (one per bin a "
+                        "record holds + one) + 4 per rest-factor row; posterior sums: 8 per point + 8 per "
+                        "rest-factor row per run); peak = shared-memory 512-byte row gathers measured by "
                         "vup_measure_peak(1) in this run"}
     a = 4.0 * units / per / 1e9
     return {"bound": "hbm", "achieved": a, "peak": pk["hbm"], "unit": "GB/s", "frac": a / pk["hbm"],
             "traffic": tr, "note": f"4 B/dist-point; peak = measured copy bandwidth, of {pk['source']}"}
+
+
+def merged_bins(b):
+    """The bin grid with the equal slices of each axis merged into one, where an axis keeps
+    at most 5/8 of its slices by that (the library's rule for its histogram)."""
+    src = b
+    for d in range(b.ndim):
+        rows = np.ascontiguousarray(np.moveaxis(src, d, 0)).reshape(src.shape[d], -1)
+        keep = np.sort(np.unique([hash(r.tobytes()) for r in rows], return_index=True)[1])
+        if len(keep) <= (5 * src.shape[d] + 7) // 8:
+            b = np.take(b, keep, axis=d)
+    return b
+
+
+def stretch_counts(lines):
+    """(intervals, runs, records) of a bin array [line][row]: stretches of one bin along a line,
+    distinct (line, bin) pairs, and maximal monotone sequences of stretches of one line inside one
+    group of eight bins."""
+    first = np.ones(lines.shape, bool)
+    first[:, 1:] = lines[:, 1:] != lines[:, :-1]
+    v = lines[first].astype(np.int64)
+    line = np.nonzero(first)[0]
+    q = v // 8
+    same1 = np.zeros(v.size, bool)
+    same1[1:] = (line[1:] == line[:-1]) & (q[1:] == q[:-1])
+    turn = np.zeros(v.size, bool)
+    turn[2:] = same1[2:] & same1[1:-1] & ((v[2:] > v[1:-1]) != (v[1:-1] > v[:-2]))
+    s = np.sort(lines, axis=1)
+    return int(v.size), lines.shape[0] + int((s[:, 1:] != s[:, :-1]).sum()), int((~same1 | turn).sum())
+
+
+def walk_bytes(bins, points_only=False):
+    """Bytes per density that the cheapest histogram walk of a 2-D / 3-D bin grid needs through
+    the L1 data pipe: the grid's equal slices merged; on 2-D grids the gathered axis with fewer
+    intervals, on 3-D grids the last.  points_only: the posterior sums' walk (two sums per point
+    and two factors per rest axis and run)."""
+    b = merged_bins(bins)
+    nf = b.ndim - 1
+    axes = (1, 0) if b.ndim == 2 else (2,)
+    n_iv, n_runs, n_rec = min(stretch_counts(np.moveaxis(b, a, -1).reshape(-1, b.shape[a])) for a in axes)
+    if points_only:
+        return 8 * b.size + 8 * nf * n_runs
+    return min(4 * b.size + 4 * nf * n_runs, n_iv * (8 + 4 * nf), 4 * (n_iv + n_rec) + 4 * nf * n_rec)
 
 
 ROOF_GROUPS = ("moments_bf16", "moments_fp32", "moments_tf32", "ipsa_bf16", "ipsa_fp32", "hist_seg", "weights")
@@ -306,7 +345,6 @@ class SingleGrid:
         self.ipsa = name == "c4"
         self.sa = name == "ipsa"
         self.bayes = name == "bayes"
-        self.hist_passes = 1 + prob.ndim if self.bayes else 1  # posterior means: H, then one pass per axis
         self.prec = prec
         self.g = vup.Grid(prob.n, prob.lo, prob.hi)
         K, J, B, nd_ = prob.K, prob.n_moments, prob.n_bins, prob.ndim
@@ -685,7 +723,7 @@ def main():
     # overlap others and are not candidates)
     cands = {k: v for k, v in prof.items() if k.startswith(ROOF_GROUPS)}
     dominant = max(cands.items(), key=lambda kv: kv[1][1])[0] if cands else None
-    # gathers of one histogram launch on the stream each grid's layout chose
+    # bytes one histogram pass needs (the streams named are those of the unmerged grids' layouts)
     hist_units, streams = 0, set()
     points_only = getattr(work, "bayes", False)  # posterior means walk the point stream
     for g, K in work.hist_grids():
@@ -693,17 +731,12 @@ def main():
         if info.ndim >= 2:
             mode = 0 if points_only else info.hist_stream
             streams.add(("points", "intervals", "records")[mode])
-            nf = info.ndim - 1  # rest-factor rows per run, interval or record
-            if mode == 2:
-                hist_units += K * (4 * (info.hist_intervals + info.hist_records) + 4 * nf * info.hist_records)
-            elif mode == 1:
-                hist_units += K * info.hist_intervals * (8 + 4 * nf)
-            else:
-                hist_units += K * (4 * info.N + 4 * nf * info.hist_runs)
+            hist_units += K * walk_bytes(g.array("bins").cpu().numpy().reshape(g.n), points_only)
+
     def n_work(k, launches):
-        # histogram: one working launch per pass (the other stream's launch exits at once)
+        # histogram: one working launch per step (the other streams' launches exit at once)
         if k.startswith("hist_seg"):
-            return args.steps * getattr(work, "hist_passes", 1)
+            return args.steps
         # the supplied-weights group is one pass per step over several launches
         # (power table, the W stream, the finish): its bytes are per pass
         if k.startswith("weights"):
@@ -749,8 +782,8 @@ def main():
         "kernels": {"per_step": per_step, "stage_ms_per_step": stage, "roofline": kern_roof,
                     "timing": ("CUDA events per kernel group inside the timed region, on each group's own "
                                "stream: the layout build runs on a second stream beside the density "
-                               "preparation and the contraction, the prefix tiles and the FP64 moments finish "
-                               "on a third (the finish waits there for SM room beside the histogram), so "
+                               "preparation and the contraction, the FP64 moments finish on a third "
+                               "beside the histogram, so "
                                "group spans overlap and can add up to more than ms_per_step") if profile_live
                     else "per-stage CUDA events from a second pass of the same steps (stage by stage)"},
         "fp32_arm": fp32_arm,
