@@ -362,7 +362,7 @@ vup_status vup_pick_hist_layout(vup_grid g, cudaStream_t s);
 vup_status vup_build_layout(vup_grid g, cudaStream_t s, bool points_needed = false,
                             cudaEvent_t records_done = nullptr, cudaEvent_t layout_picked = nullptr,
                             bool fold = true, bool coarse = false);
-// coarse: at least 24 records (256 points) per chunk, for a grid among many of a batch.
+// coarse: longer record and point chunks, as on merged grids, for a grid among many of a batch.
 vup_status vup_ensure_layout(vup_grid g, cudaStream_t s, bool points_needed = false, bool coarse = false);
 // every layout's part tile fits the shared-memory histogram kernels
 bool vup_hist_tile_fits(vup_grid g);
