@@ -9,10 +9,10 @@
 // FP64 arithmetic bounds this path: the GPU issues about two FP64 operations
 // per clock and SM, so its time is the number of them.  The density is evaluated once per
 // point (it was evaluated for each of the three sums: 338 us for 256 densities
-// on 4096 points, now 71), in 4 operations up to the exponent and 11 for a
-// table-driven exponential; points whose Gaussian cannot reach half the
-// smallest FP32 number are skipped (six of seven points at sigma = 1/200 of the
-// domain, none at 1/20); and sums add across warps and few lanes, as
+// on 4096 points, now 88), in 4 operations up to the exponent and 11 for a
+// table-driven exponential; points whose Gaussian is 0 in FP64, beyond 38.6
+// sigma, are skipped (three of five points at sigma = 1/200 of the domain, none
+// at 1/40); and sums add across warps and few lanes, as
 // a step of a shuffle tree costs an FP64 operation on all 32 lanes (full-warp
 // trees, with every warp forming the density's constants, took 116 us).
 #include "vup_internal.cuh"
@@ -37,7 +37,6 @@ struct P1 {
 struct Geo1 {
     int64_t n;
     double lo, h;
-    double cut;  // 104 + ln n
 };
 
 // 2^(j / 64), j = 0 .. 63, each rounded to FP64
@@ -95,7 +94,13 @@ struct Dens1 {
     int32_t b, e;  // the points evaluated; the others' density is 0
 };
 
-__device__ __forceinline__ Dens1 dens_of(const P1 &p, const Geo1 &G, int64_t k) {
+__device__ __forceinline__ bool finite_key(unsigned long long k) {  // an end of the outputs' range (ordered key)
+    const unsigned long long u = (k >> 63) ? (k & 0x7fffffffffffffffull) : ~k;
+    return isfinite(__longlong_as_double((long long)u));
+}
+
+__device__ __forceinline__ Dens1 dens_of(const P1 &p, const Geo1 &G, const unsigned long long *__restrict__ ext,
+                                         int64_t k) {
     Dens1 D;
     D.kind = p.kind[k];
     D.mu = p.mu[k];
@@ -111,9 +116,15 @@ __device__ __forceinline__ Dens1 dens_of(const P1 &p, const Geo1 &G, int64_t k) 
     D.q = v0 * v0;
     D.b = 0;
     D.e = (int32_t)G.n;
-    if (D.kind == VUP_GAUSS) {
-        // exp(q - v^2) / Z with Z >= 1: below 2^-150 / n for q - v^2 < -(104 + ln n)
-        const double hw = sqrt(D.q + G.cut) / D.r + 1.0;
+    if (D.kind == VUP_GAUSS && finite_key(ext[0]) && finite_key(ext[1])) {
+        // exp(q - v^2) is 0 in FP64 below q - v^2 = -745.2: such points add nothing to
+        // any sum, however large their output (a bound of FP32's range, right for the
+        // histogram, lost 84 % of E[y^4] of y = exp(80 x) at sigma = 0.05).  0.8 and
+        // 2^-46 q allow for the rounding of q - v^2, a cell and 2^-50 for that of the
+        // window.  (With an output that is not finite every point is evaluated: 0 times
+        // it is not a number.)
+        const double h0 = sqrt(D.q + (746.0 + 0x1p-46 * D.q)) / D.r;
+        const double hw = h0 + 1.0 + 0x1p-50 * (h0 + fabs(c));
         const double b = floor(c - hw), e = ceil(c + hw) + 1.0;
         if (b > 0.0) D.b = (int32_t)fmin(b, (double)G.n);
         if (e < (double)G.n) D.e = (int32_t)fmax(e, 0.0);
@@ -167,7 +178,8 @@ __device__ __forceinline__ void cluster_sums(cg::cluster_group &cl, const double
 }
 
 template <bool kIpsa>
-__global__ void __launch_bounds__(kThreads) k_1d(P1 p, Geo1 G, const double *__restrict__ y,
+__global__ void __launch_bounds__(kThreads) k_1d(P1 p, Geo1 G, const unsigned long long *__restrict__ ext,
+                                                 const double *__restrict__ y,
                                                  const int32_t *__restrict__ perm,
                                                  const int32_t *__restrict__ offsets, int B, int J,
                                                  double *__restrict__ raw, double *__restrict__ central,
@@ -182,7 +194,7 @@ __global__ void __launch_bounds__(kThreads) k_1d(P1 p, Geo1 G, const double *__r
     const int n_cta = (int)cl.num_blocks(), rank = (int)cl.block_rank();
     const int64_t k = blockIdx.x / n_cta;
     if (threadIdx.x < 64) s_tab[threadIdx.x] = kExpTab[threadIdx.x];
-    if (threadIdx.x == 64) s_dens = dens_of(p, G, k);  // one warp's FP64 work, not every warp's
+    if (threadIdx.x == 64) s_dens = dens_of(p, G, ext, k);  // one warp's FP64 work, not every warp's
     __syncthreads();
     const Dens1 D = s_dens;
     const int32_t len = D.e - D.b, per = (len + n_cta - 1) / n_cta;
@@ -326,9 +338,9 @@ vup_status launch_1d(vup_grid g, int64_t K, cudaStream_t s, Args... args) {
 vup_status vup_propagate_1d(vup_grid g, const vup_densities *d, double *raw, double *central, float *hist,
                             cudaStream_t s) {
     const P1 p{d->kind, d->mu, d->sigma, d->lo, d->hi};
-    const Geo1 G{g->n[0], g->lo[0], (g->hi[0] - g->lo[0]) / (double)g->n[0], 104.0 + log((double)g->n[0])};
+    const Geo1 G{g->n[0], g->lo[0], (g->hi[0] - g->lo[0]) / (double)g->n[0]};
     VUP_PROF("vup_1d_fp64", s, 1);
-    return launch_1d<false>(g, d->K, s, p, G, (const double *)g->y, (const int32_t *)g->perm,
+    return launch_1d<false>(g, d->K, s, p, G, (const unsigned long long *)g->ext, (const double *)g->y, (const int32_t *)g->perm,
                             (const int32_t *)g->offsets, g->B, g->J, raw, central, hist, (const double *)nullptr,
                             (float *)nullptr, (float *)nullptr, g->dstatus);
 }
@@ -336,9 +348,9 @@ vup_status vup_propagate_1d(vup_grid g, const vup_densities *d, double *raw, dou
 vup_status vup_ipsa_1d(vup_grid g, const vup_densities *d, const double *grad, float *dmu, float *dsg,
                        cudaStream_t s) {
     const P1 p{d->kind, d->mu, d->sigma, d->lo, d->hi};
-    const Geo1 G{g->n[0], g->lo[0], (g->hi[0] - g->lo[0]) / (double)g->n[0], 104.0 + log((double)g->n[0])};
+    const Geo1 G{g->n[0], g->lo[0], (g->hi[0] - g->lo[0]) / (double)g->n[0]};
     VUP_PROF("ipsa_1d_fp64", s, 1);
-    return launch_1d<true>(g, d->K, s, p, G, (const double *)g->y, (const int32_t *)g->perm,
+    return launch_1d<true>(g, d->K, s, p, G, (const unsigned long long *)g->ext, (const double *)g->y, (const int32_t *)g->perm,
                            (const int32_t *)g->offsets, g->B, g->J, (double *)nullptr, (double *)nullptr,
                            (float *)nullptr, grad, dmu, dsg, g->dstatus);
 }
