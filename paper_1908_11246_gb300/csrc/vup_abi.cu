@@ -377,6 +377,7 @@ extern "C" vup_status vup_grid_create(int ndim, const int64_t *n, const double *
             // words past the stream's end are read by whole-window staging and
             // masked; zero keeps their rest codes valid indices
             e = cudaMemset(g->hl[0].ipt, 0, sizeof(uint2) * (N + 128));
+            if (e == cudaSuccess) e = cudaMemset(g->fold, 0, sizeof(FoldGeom));  // nothing merged before a layout is built
         } else {
             g->hl[0].perm = g->perm;
         }

@@ -1924,7 +1924,7 @@ __global__ void __launch_bounds__(128) k_fold_tables(const __grid_constant__ Fol
     if (!T.fold->any) return;
     fold_table_rows(T, blockIdx.x, gridDim.x);
 }
-// Batched form: block y serves instance y.
+// Batched form: block y serves the y-th instance with a histogram.
 __global__ void __launch_bounds__(128) k_fold_tables_batched(const FoldTabArgs *__restrict__ jobs) {
     const FoldTabArgs &T = jobs[blockIdx.y];
     if (!T.fold->any) return;
@@ -2140,10 +2140,10 @@ bool vup_hist_batchable(vup_grid g) {
 // instance's (part, chunk group, density tile) items, longest first, and one
 // finishing launch.
 struct HistPlan {
-    DevBuf fold;                      // FoldTabArgs of every instance
+    DevBuf fold;                      // FoldTabArgs of every instance that wants a histogram
     DevBuf args, items, fitems, ctr;  // ctr: next item of each stream's launch, then each stream's item count
     DevBuf lists;                     // [3][n_items] each stream's items (k_hist_split_items)
-    int n_inst = 0, n_items = 0, n_fitems = 0;
+    int n_inst = 0, n_fold = 0, n_items = 0, n_fitems = 0;
     int64_t rows = 0;
 };
 
@@ -2203,10 +2203,14 @@ vup_status vup_hist_plan(int n, const vup_grid *gs, const int64_t *Ks, float *co
     P->n_fitems = (int)fin.size();
     P->rows = rows_max;
     vup_status st;
-    std::vector<FoldTabArgs> folds(n);
-    for (int i = 0; i < n; ++i) folds[i] = fold_tab_args(gs[i], Ks[i]);
+    // merged tables only where a histogram is asked for: the other instances' layouts
+    // need not exist, nor their tables hold this K
+    std::vector<FoldTabArgs> folds;
+    for (int i = 0; i < n; ++i)
+        if (hists[i]) folds.push_back(fold_tab_args(gs[i], Ks[i]));
+    P->n_fold = (int)folds.size();
     if ((st = devbuf_reserve(P->args, sizeof(HistArgs) * n)) != VUP_OK ||
-        (st = devbuf_reserve(P->fold, sizeof(FoldTabArgs) * n)) != VUP_OK ||
+        (st = devbuf_reserve(P->fold, sizeof(FoldTabArgs) * std::max<size_t>(1, folds.size()))) != VUP_OK ||
         (st = devbuf_reserve(P->items, sizeof(HistItem) * std::max<size_t>(1, items.size()))) != VUP_OK ||
         (st = devbuf_reserve(P->fitems, sizeof(int4) * std::max<size_t>(1, fin.size()))) != VUP_OK ||
         (st = devbuf_reserve(P->ctr, sizeof(int) * 6)) != VUP_OK ||
@@ -2221,7 +2225,7 @@ vup_status vup_hist_plan(int n, const vup_grid *gs, const int64_t *Ks, float *co
         return st;
     }
     VUP_CHECK_CUDA(cudaMemcpy(P->args.p, args.data(), sizeof(HistArgs) * n, cudaMemcpyHostToDevice));
-    VUP_CHECK_CUDA(cudaMemcpy(P->fold.p, folds.data(), sizeof(FoldTabArgs) * n, cudaMemcpyHostToDevice));
+    VUP_CHECK_CUDA(cudaMemcpy(P->fold.p, folds.data(), sizeof(FoldTabArgs) * folds.size(), cudaMemcpyHostToDevice));
     VUP_CHECK_CUDA(cudaMemcpy(P->items.p, items.data(), sizeof(HistItem) * items.size(), cudaMemcpyHostToDevice));
     VUP_CHECK_CUDA(cudaMemcpy(P->fitems.p, fin.data(), sizeof(int4) * fin.size(), cudaMemcpyHostToDevice));
     // the largest tile any plan may use, so that graphs of earlier plans stay launchable
@@ -2254,8 +2258,8 @@ vup_status vup_hist_batched(void *plan, cudaStream_t s) {
     if (smem > 220 * 1024) return VUP_ERR_UNSUPPORTED;
     {
         VUP_PROF("hist_segmented_batched", s, 5);
-        for (int i0 = 0; i0 < P->n_inst; i0 += 65535) {  // (the grid's y limit)
-            const unsigned ny = (unsigned)std::min(65535, P->n_inst - i0);
+        for (int i0 = 0; i0 < P->n_fold; i0 += 65535) {  // (the grid's y limit)
+            const unsigned ny = (unsigned)std::min(65535, P->n_fold - i0);
             k_fold_tables_batched<<<dim3(32, ny), 128, 0, s>>>((const FoldTabArgs *)P->fold.p + i0);
             VUP_CHECK_LAUNCH();
         }

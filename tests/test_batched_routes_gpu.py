@@ -1,0 +1,76 @@
+"""Batches whose instances want different outputs, against the FP64 oracle: an
+instance without a histogram may have no layout yet, or merged tables from an
+earlier call with fewer densities."""
+import numpy as np
+import pytest
+
+from oracle import oracle as O
+from paper_1908_11246_gb300 import inputs as I
+from tests import helpers as Hp
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _build():
+    from paper_1908_11246_gb300 import build
+    build.build()
+
+
+def _poly(i, n, K, even):
+    lo, hi = (-1.0, -2.0), (1.0, 2.0)
+    theta = (0.0, 0.0, 1.0, 0.0, 2.0) if even else (0.0, 1.0, 0.5, 0.3, 0.2)
+    dens = I.random_densities(np.random.default_rng(600 + i), K, lo, hi, sig=(0.1, 0.8))
+    return I.Problem(f"poly{i}", n, lo, hi, I.MODEL_POLY, theta, dens, 60)
+
+
+def _check(p, raw, hist, precision):
+    rows = np.arange(p.K)
+    res = O.solve(p, rows=rows, threads=Hp.oracle_threads())
+    if raw is not None:
+        scale = Hp.abs_moment_scale(p, res["y"], rows)
+        Hp.check_moments(raw.cpu().numpy(), res["raw"], scale, Hp.TOL[precision], what=p.name)
+    if hist is not None:
+        amb = Hp.ambiguous_points(res["y"], res["bins"], p.n_bins)
+        Hp.check_hist(hist.cpu().numpy(), res["hist"], Hp.ambiguous_mass(p, amb, rows))
+
+
+@pytest.mark.parametrize("precision", ["fp32", "bf16x3"])
+def test_instances_without_histogram(precision):
+    """0: merged tables from a call with fewer densities; 1: no layout, on memory
+    of closed grids; 2, 3: histograms with and without merged slices; 4: nothing wanted."""
+    from paper_1908_11246_gb300 import vup
+    for n in ((64, 90), (130, 91)):  # closed grids leave their merged sizes behind in freed memory
+        p = _poly(9, n, 200, True)
+        g = vup.Grid(p.n, p.lo, p.hi)
+        g.eval_model(p.model_id, p.theta, p.n_bins)
+        g.propagate(vup.densities_to_device(p.dens), precision)
+        g.sync()
+        g.close()
+    probs = [_poly(0, (130, 91), 3000, True), _poly(1, (64, 90), 700, True), _poly(2, (120, 80), 500, True),
+             _poly(3, (77, 130), 300, False), _poly(4, (40, 50), 260, True)]
+    grids, dds = [], []
+    for p in probs:
+        g = vup.Grid(p.n, p.lo, p.hi)
+        g.eval_model(p.model_id, p.theta, p.n_bins)
+        grids.append(g)
+        dds.append(vup.densities_to_device(p.dens))
+    few = _poly(7, (130, 91), 100, True)
+    _check(few, *grids[0].propagate(vup.densities_to_device(few.dens), precision, central=False)[::2], precision)
+    raws, hists = vup.batched_outputs(grids, dds)
+    hists[0] = hists[1] = hists[4] = raws[4] = raws[3] = None
+    for _ in range(2):  # the second call replays the graph
+        for t in raws + hists:
+            if t is not None:
+                t.fill_(-1)
+        vup.propagate_batched(grids, dds, precision, out=(raws, hists))
+        for g in grids:
+            g.sync()
+        for p, r, h in zip(probs, raws, hists):
+            _check(p, r, h, precision)
+    # and the instances without a histogram in a call of their own
+    for p, g, dd in zip(probs, grids, dds):
+        r, _, h = g.propagate(dd, precision, central=False)
+        g.sync()
+        _check(p, r, h, precision)
+        g.close()
