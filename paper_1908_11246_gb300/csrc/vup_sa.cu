@@ -75,8 +75,10 @@ __global__ void __launch_bounds__(256) k_ipsa_matrix(const float *__restrict__ H
         const DevRule R = s_rule;
         for (int b = threadIdx.x; b < B; b += blockDim.x) emap[b] = R(b);
         __syncthreads();
-        for (int b = threadIdx.x; b < B; b += blockDim.x)
-            if (b == 0 || emap[b] != emap[b - 1]) first[emap[b]] = b;
+        for (int b = threadIdx.x; b < B; b += blockDim.x) {
+            const int e = emap[b];  // (negative where the deviation is not a number: in no bin)
+            if (e >= 0 && (b == 0 || e != emap[b - 1])) first[e] = b;
+        }
         __syncthreads();
         const float *h = H + k * B;
         for (int e = threadIdx.x; e < nd; e += blockDim.x) {
