@@ -35,15 +35,18 @@ __device__ __forceinline__ int dev_bin(int b, double ymin, double w, double yref
 // where no integer lies within eps of t its floor is the bin, otherwise the FP64
 // expression decides (about one bin in a thousand).  Error of t: the roundings
 // of s, o and the FMA, each <= 2^-24 relative to |b s| + |o|; eps allows eight
-// times that.
+// times that.  Beside it the FP64 expression's own roundings, and those of o, which
+// grow with the values that cancel in them: at most 8 units of 2^-53 (|ymin| +
+// |ymax| + |yref| + |dlo|) / wd in all, of which eps (e64) allows twice; outputs
+// of 1e12 with a range of 3 move bins without it.
 struct DevRule {
     double ymin, w, yref, dlo, wd;
-    float s, o;
+    float s, o, e64;
     int nd;
     __device__ __forceinline__ int operator()(int b) const {
         const float t = fmaf((float)b, s, o);
         const float f = floorf(t);
-        const float eps = 0x1p-21f * (fabsf((float)b * s) + fabsf(o) + 1.f);
+        const float eps = fmaf(0x1p-21f, fabsf((float)b * s) + fabsf(o) + 1.f, e64);
         if (t - f > eps && f + 1.f - t > eps) return f < 0.f ? 0 : (f > (float)(nd - 1) ? nd - 1 : (int)f);
         return dev_bin(b, ymin, w, yref, dlo, wd, nd);
     }
@@ -68,7 +71,9 @@ __global__ void __launch_bounds__(256) k_ipsa_matrix(const float *__restrict__ H
             const double ymin = ext_value(ext[0]), ymax = ext_value(ext[1]), yr = yref[k];
             const double w = __ddiv_rn(__dsub_rn(ymax, ymin), (double)B);
             const double wd = __ddiv_rn(__dsub_rn(dhi, dlo), (double)nd);
-            s_rule = DevRule{ymin, w, yr, dlo, wd, (float)(w / wd), (float)((ymin + 0.5 * w - yr - dlo) / wd), nd};
+            const double mag = fabs(ymin) + fabs(ymax) + fabs(yr) + fabs(dlo);
+            s_rule = DevRule{ymin, w, yr, dlo, wd, (float)(w / wd), (float)((ymin + 0.5 * w - yr - dlo) / wd),
+                             (float)(0x1p-49 * mag / wd), nd};
         }
         for (int e = threadIdx.x; e < nd; e += blockDim.x) first[e] = B;
         __syncthreads();

@@ -1,6 +1,7 @@
 """IPSA matrix columns whose estimated value is not finite: NaN puts a column's
 mass in no deviation bin, an infinity in the first or last; the other columns
-are the oracle's bit for bit."""
+are the oracle's bit for bit.  And outputs whose size dwarfs their range, where
+the FP64 expression of a deviation bin is itself rounded by part of a bin."""
 import numpy as np
 import pytest
 import torch
@@ -56,4 +57,24 @@ def test_outputs_that_are_not_finite():
                         20, -1.0, 1.0, out)
     g.sync()
     assert (out == 0).all()
+    g.close()
+
+
+@pytest.mark.parametrize("offset", [0.0, 1e6, -1e9, 3e9, 1e12, -1e15])
+@pytest.mark.parametrize("B, nd", [(1000, 1000), (333, 2048), (4096, 700)])
+def test_offset_outputs_match_oracle(offset, B, nd):
+    from paper_1908_11246_gb300 import vup
+    rng = np.random.default_rng(B + nd)
+    y = np.linspace(-1.0, 2.0, 3000).reshape(60, 50) + offset
+    g = _grid(y, B)
+    info = g.info()
+    hist = rng.random((60, B)).astype(np.float32)
+    yref = offset + rng.uniform(-1.0, 2.0, 60)
+    for dlo, dhi in ((-3.0, 3.0), (-0.7, 4.1)):
+        out = torch.empty((60, nd), dtype=torch.float32, device="cuda")
+        vup.vup_ipsa_matrix(g.h, torch.as_tensor(hist, device="cuda"), torch.as_tensor(yref, device="cuda"), nd, dlo,
+                            dhi, out)
+        g.sync()
+        want = O.ipsa_matrix(hist.astype(np.float64), info.ymin, info.ymax, yref, nd, dlo, dhi)
+        np.testing.assert_array_equal(out.cpu().numpy(), want.astype(np.float32))
     g.close()
