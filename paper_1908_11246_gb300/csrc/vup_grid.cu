@@ -1326,11 +1326,14 @@ __global__ void k_layout_encode(const int32_t *__restrict__ run_start, const int
     }
 }
 
-// Start of chunk cc of C over n elements: n cc / C, on a merged grid or one of a
-// batch (coarse) rounded down to whole chunks of `least` elements where n / C is
-// less (some chunks are then empty, spread evenly): a chunk's cut keys or groups
-// cost partial rows, which short chunks would make the larger part of the work
-// (a batch's finish: 102 -> 86 us), and neither needs them to fill the SMs.
+// Start of chunk cc of C over n elements: n cc / C, on a merged grid rounded down
+// to whole chunks of `least` elements where n / C is less (some chunks are then
+// empty, spread evenly): a chunk's cut keys or groups cost partial rows, which
+// short chunks would make the larger part of the work, and a merged grid does not
+// need them to fill the SMs.  The rule looks at the grid alone, so that a
+// histogram's sums do not depend on which call built the layout (whole chunks on
+// every grid of a batch took 32 uneven unmerged instances from 714 to 663 us, but
+// left the one-instance call that followed with other bits).
 // Points (and intervals, cut where points are): n / 512, at least 64, where the 80
 // or more slots then give a small grid's few density tiles a chunk for most warps
 // (8200 merged points, K = 225: walk 35 us at 256 points, 27 at 64 or 32), at most
@@ -1339,11 +1342,9 @@ __global__ void k_layout_encode(const int32_t *__restrict__ run_start, const int
 // keep the chunks at or under kChunkRecMost, so that no round leaves most warps
 // idle.  Walk + finish against chunks of 24 whatever their number: 1024 x 1024
 // points, K = 16384 (1165 records per part) 159 -> 147 us; 2048 x 2048, K = 65536
-// (1550) 950 -> 893; 1021 x 613, K = 9001 (1100) 119 -> 113; 32 uneven instances
-// 384 -> 360.  At most 48: 147 / 893 / 113 / 374; at most 100 (one round): 139 / 842 /
-// 125 / 366, where a part split between two CTAs leaves half their warps idle.
-// At least 8: a batch of ten instances of at most 169 x 169 points 117.5 -> 113.4 us a
-// pass against at least 24, larger batches unchanged or 1 % faster.
+// (1550) 950 -> 893; 1021 x 613, K = 9001 (1100) 119 -> 113.  At most 48: 147 / 893 /
+// 113; at most 100 (one round): 139 / 842 / 125, where a part split between two CTAs
+// leaves half their warps idle.  At least 8.
 constexpr int kChunkPtsLeast = 64, kChunkPtsMost = 256, kChunkRecLeast = 8, kChunkRecMost = 64, kRecWalkWarps = 16;
 __device__ __forceinline__ int64_t point_chunk(int64_t n) {
     return min(max(n / 512, (int64_t)kChunkPtsLeast), (int64_t)kChunkPtsMost);
@@ -1367,7 +1368,7 @@ __global__ void k_chunks(const int32_t *__restrict__ run_start, const int32_t *_
                          const int32_t *__restrict__ koff, int B, LaySel L, int C,
                          const unsigned long long *__restrict__ excl, const int32_t *__restrict__ n_iv_p,
                          int32_t *__restrict__ chunk_pt, int32_t *__restrict__ chunk_run,
-                         int32_t *__restrict__ chunk_iv, const int32_t *gate, int coarse) {
+                         int32_t *__restrict__ chunk_iv, const int32_t *gate) {
     pdl_trigger();
     pdl_wait();
     if (gated_off(gate)) return;
@@ -1382,7 +1383,7 @@ __global__ void k_chunks(const int32_t *__restrict__ run_start, const int32_t *_
     } else {
         const int p = c / C, cc = c - p * C;
         const int64_t lo = koff[p * B], hi = koff[(p + 1) * B];
-        const int64_t target = lo + chunk_at(hi - lo, cc, C, coarse || L.fold->any ? point_chunk(hi - lo) : 1);
+        const int64_t target = lo + chunk_at(hi - lo, cc, C, L.fold->any ? point_chunk(hi - lo) : 1);
         int32_t a = 0, b = n_runs;  // first r in [0, n_runs] with run_start[r] >= target
         while (a < b) {
             int32_t mid = (a + b) >> 1;
@@ -1648,12 +1649,12 @@ __global__ void k_rec_scatter(const uint4 *__restrict__ tmp, const int32_t *__re
 __global__ void k_rec_tables(const int32_t *__restrict__ starts, const int32_t *__restrict__ counts, int64_t Lr,
                              int64_t NL, int n_groups, int GB, LaySel L, int C, const uint4 *__restrict__ rec,
                              int32_t *__restrict__ goff, int32_t *__restrict__ n_rec, int32_t *__restrict__ chunk_rec,
-                             int32_t *__restrict__ chunk_grp, int2 *__restrict__ gch, int coarse) {
+                             int32_t *__restrict__ chunk_grp, int2 *__restrict__ gch) {
     pdl_trigger();
     pdl_wait();
     const int P = L.get().P;
-    const bool whole = coarse || L.fold->any;
-    auto least_of = [&](int64_t n) -> int64_t { return whole ? record_chunk(n) : 1; };
+    const bool merged = L.fold->any != 0;
+    auto least_of = [&](int64_t n) -> int64_t { return merged ? record_chunk(n) : 1; };
     const int32_t total = starts[Lr - 1] + counts[Lr - 1];
     auto first = [&](int g) -> int32_t { return g < n_groups ? starts[g * NL] : total; };
     const int i = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
@@ -2202,7 +2203,7 @@ static FoldArgs fold_args(vup_grid g) {
 // first use after a model evaluation (the histogram, the bin offsets), so a
 // caller may run it on a second stream beside the density preparation.
 vup_status vup_build_layout(vup_grid g, cudaStream_t s, bool points_needed, cudaEvent_t records_done,
-                            cudaEvent_t layout_picked, bool fold, bool coarse) {
+                            cudaEvent_t layout_picked, bool fold) {
     const int64_t N = g->N;
     const int B = g->B;
     // two timed parts: up to the record-stream decision, and the key-sorted streams
@@ -2295,7 +2296,7 @@ vup_status vup_build_layout(vup_grid g, cudaStream_t s, bool points_needed, cuda
             VUP_CHECK_LAUNCH();
             const int Cr = g->n_chunks_rec;
             VUP_CHECK_CUDA(launch_pdl(k_rec_tables, dim3((std::max(n_groups + 2, P_sel * Cr + 1) + 127) / 128), dim3(128), 0, s, rstart, rcnt, Lr, NL, n_groups, GB, L, Cr, (const uint4 *)HL.rec.p, (int32_t *)HL.rec_goff.p, HL.n_rec,
-                HL.rec_chunk, HL.rec_chunk_grp, (int2 *)HL.rec_gch.p, coarse ? 1 : 0));
+                HL.rec_chunk, HL.rec_chunk_grp, (int2 *)HL.rec_gch.p));
             VUP_CHECK_LAUNCH();
             // walk, scan, scatter, tables, gate
             launches += 1 + scan_launches(Lr) + 2 + 1;
@@ -2344,7 +2345,7 @@ vup_status vup_build_layout(vup_grid g, cudaStream_t s, bool points_needed, cuda
         // chunks of every part
         const int PC = g->hist_P * C;
         VUP_CHECK_CUDA(launch_pdl(k_chunks, dim3((PC + 1 + 127) / 128), dim3(128), 0, s, HL.run_start, HL.n_runs, HL.koff, B, L, C, excl, HL.n_iv,
-                                                       HL.chunk_pt, HL.chunk_run, HL.chunk_iv, gate, coarse ? 1 : 0));
+                                                       HL.chunk_pt, HL.chunk_run, HL.chunk_iv, gate));
         VUP_CHECK_LAUNCH();
         VUP_CHECK_CUDA(launch_pdl(k_chunk_bins, dim3((PC + 127) / 128), dim3(128), 0, s, HL.chunk_run, HL.run_bin, L, C, HL.chunk_bin, gate));
         VUP_CHECK_LAUNCH();
@@ -2358,14 +2359,13 @@ vup_status vup_build_layout(vup_grid g, cudaStream_t s, bool points_needed, cuda
         prof.launches = launches;
     }
     g->layout_valid = 1;
-    g->layout_unfolded = fold ? 0 : 1;
     g->layout_has_points = points_needed || g->ndim == 1;
     return VUP_OK;
 }
 
-vup_status vup_ensure_layout(vup_grid g, cudaStream_t s, bool points_needed, bool coarse) {
+vup_status vup_ensure_layout(vup_grid g, cudaStream_t s, bool points_needed) {
     if (g->layout_valid && (!points_needed || g->layout_has_points)) return VUP_OK;
-    return vup_build_layout(g, s, points_needed, nullptr, nullptr, true, coarse);
+    return vup_build_layout(g, s, points_needed);
 }
 
 vup_status vup_pick_hist_layout(vup_grid g, cudaStream_t s) {

@@ -307,7 +307,6 @@ struct vup_grid_s {
     int32_t *fold_rep = nullptr, *fold_start = nullptr, *fold_members = nullptr, *fold_bins = nullptr;
     uint8_t *fold_scratch = nullptr;
     size_t fold_scratch_bytes = 0;
-    int layout_unfolded = 0;       // the current layout was built without folding (vup_grid_info's counts)
     int hist_P = 1;                // max parts over layouts (scratch sizing)
     int n_layouts = 1;
     // [8] device: chosen layout, stream, intervals of layouts 0 / 1, key streams built,
@@ -361,9 +360,8 @@ vup_status vup_pick_hist_layout(vup_grid g, cudaStream_t s);
 // fold: merge equal slices of the bin grid first (FoldGeom).
 vup_status vup_build_layout(vup_grid g, cudaStream_t s, bool points_needed = false,
                             cudaEvent_t records_done = nullptr, cudaEvent_t layout_picked = nullptr,
-                            bool fold = true, bool coarse = false);
-// coarse: longer record and point chunks, as on merged grids, for a grid among many of a batch.
-vup_status vup_ensure_layout(vup_grid g, cudaStream_t s, bool points_needed = false, bool coarse = false);
+                            bool fold = true);
+vup_status vup_ensure_layout(vup_grid g, cudaStream_t s, bool points_needed = false);
 // every layout's part tile fits the shared-memory histogram kernels
 bool vup_hist_tile_fits(vup_grid g);
 // the 3-D point stream stages both rest-axis factor tables in shared memory

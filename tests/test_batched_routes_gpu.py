@@ -74,3 +74,48 @@ def test_instances_without_histogram(precision):
         g.sync()
         _check(p, r, h, precision)
         g.close()
+
+
+def _oscillators():
+    return I.oscillator_batch(23, n_inst=8, side=(24, 400), kk=(40, 900), n_bins=128) + [_poly(5, (90, 61), 300, True)]
+
+
+def _grids(probs):
+    from paper_1908_11246_gb300 import vup
+    out = []
+    for p in probs:
+        g = vup.Grid(p.n, p.lo, p.hi)
+        g.eval_model(p.model_id, p.theta, p.n_bins, p.n_moments)
+        out.append(g)
+    return out
+
+
+def test_histograms_do_not_depend_on_which_call_came_first():
+    """One instance alone, in a batch, in a batch first and then alone, and alone
+    after vup_grid_info has looked at the counts: the same bits, on grids of each
+    order's own (the documented identity of the batched and the one-instance path)."""
+    from paper_1908_11246_gb300 import vup
+    probs = _oscillators()
+    dds = [vup.densities_to_device(p.dens) for p in probs]
+
+    def alone(grids):
+        return [g.propagate(dd, "fp32", moments=False, central=False)[2] for g, dd in zip(grids, dds)]
+
+    def batch(grids):
+        return vup.propagate_batched(grids, dds, "fp32", moments=False)[1]
+
+    def looked_at(grids):
+        for g in grids:
+            g.info()
+        return alone(grids)
+
+    first, second, third, fourth = (_grids(probs) for _ in range(4))
+    results = dict(alone=alone(first), batch_after_alone=batch(first), batch=batch(second), alone_after_batch=alone(second),
+                   looked_at=looked_at(third), batch_after_look=batch(third))
+    batch(fourth)
+    results["batch_then_look_then_alone"] = looked_at(fourth)
+    import torch
+    torch.cuda.synchronize()
+    for name, hs in results.items():
+        for p, a, b in zip(probs, results["alone"], hs):
+            np.testing.assert_array_equal(b.cpu().numpy(), a.cpu().numpy(), err_msg=f"{name} {p.name}")
