@@ -328,7 +328,7 @@ vup_status launch_1d(vup_grid g, int64_t K, cudaStream_t s, Args... args) {
     cfg.attrs = at;
     cfg.numAttrs = 1;
     if (smem > 40 * 1024)
-        VUP_CHECK_CUDA(cudaFuncSetAttribute(k_1d<kIpsa>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        VUP_CHECK_CUDA(smem_allow(k_1d<kIpsa>));
     VUP_CHECK_CUDA(cudaLaunchKernelEx(&cfg, k_1d<kIpsa>, args...));
     return VUP_OK;
 }

@@ -2036,8 +2036,8 @@ static vup_status counting_sort(vup_grid g, const int32_t *keys, int Bk, int32_t
     const size_t smem = sizeof(int32_t) * (size_t)Bk * nw;
     const unsigned blocks = (unsigned)ceil_div64(n_tiles, nw);
     if (smem > 48 * 1024) {
-        VUP_CHECK_CUDA(cudaFuncSetAttribute(k_count, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        VUP_CHECK_CUDA(cudaFuncSetAttribute(k_sort_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        VUP_CHECK_CUDA(smem_allow(k_count));
+        VUP_CHECK_CUDA(smem_allow(k_sort_scatter));
     }
     if (!counts_ready) {
         VUP_CHECK_CUDA(launch_pdl(k_count, dim3(blocks), dim3(32 * nw), smem, s, keys, N, Bk, counts, n_tiles, gate, fold));
@@ -2131,8 +2131,7 @@ vup_status vup_launch_grid_finish(vup_grid g, cudaStream_t s) {
             const int nw = sort_warps(B);
             const size_t smem = sizeof(int32_t) * (size_t)B * nw;
             if (smem > 48 * 1024)
-                VUP_CHECK_CUDA(
-                    cudaFuncSetAttribute(k_bins_count, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+                VUP_CHECK_CUDA(smem_allow(k_bins_count));
             k_bins_count<<<(unsigned)ceil_div64(n_tiles, nw), 32 * nw, smem, s>>>(g->y, N, B, g->ext, g->bins,
                                                                                 counts, n_tiles);
         } else if (!bins_done) {
@@ -2237,7 +2236,7 @@ vup_status vup_build_layout(vup_grid g, cudaStream_t s, bool points_needed, cuda
                 for (int d = 0; d < g->ndim; ++d)
                     sm = std::max(sm, sizeof(int32_t) * (size_t)fold_cap(g->n[d]) + sizeof(uint16_t) * (size_t)g->n[d]);
                 if (sm > 48 * 1024)
-                    VUP_CHECK_CUDA(cudaFuncSetAttribute(k_fold_number, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+                    VUP_CHECK_CUDA(smem_allow(k_fold_number));
                 VUP_CHECK_CUDA(launch_pdl(k_fold_verify, dim3(tb), dim3(256), 0, s, A));
                 VUP_CHECK_CUDA(launch_pdl(k_fold_number, dim3(g->ndim), dim3(1024), sm, s, A));
                 VUP_CHECK_CUDA(launch_pdl(k_fold_bins, dim3(blocks), dim3(256), 0, s, A));
@@ -2286,7 +2285,7 @@ vup_status vup_build_layout(vup_grid g, cudaStream_t s, bool points_needed, cuda
             VUP_CHECK_CUDA(cudaMemsetAsync(HL.n_iv, 0, sizeof(int32_t), s));
             const size_t wsm = sizeof(int32_t) * (size_t)kWalkWarps * GB;
             if (wsm > 48 * 1024)
-                VUP_CHECK_CUDA(cudaFuncSetAttribute(k_rec_walk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wsm));
+                VUP_CHECK_CUDA(smem_allow(k_rec_walk));
             VUP_CHECK_CUDA(launch_pdl(k_rec_walk, dim3((unsigned)ceil_div64(walkers, kWalkWarps)), dim3(kWalkWarps * 32), wsm, s, lb, Q, L, rcnt,
                                                                                              HL.n_iv, rslot, seg_n));
             VUP_CHECK_LAUNCH();

@@ -1967,7 +1967,7 @@ vup_status vup_fold_tables(vup_grid g, int64_t K, cudaStream_t s, const float *f
 bool vup_hist_rest_staged(const vup_grid_s *g) {
     if (g->ndim != 3 || g->hl[0].last_axis != 2 || g->n[0] > 512 || g->n[1] > 4096) return false;
     const size_t rest_bytes = (size_t)(g->n[0] + g->n[1]) * kKT * sizeof(float);
-    return hist_smem_bytes(g->hl[0].part_rows, hist_warps(4)) + rest_bytes <= 220 * 1024;
+    return hist_smem_bytes(g->hl[0].part_rows, hist_warps(4)) + rest_bytes <= kSmemMost;
 }
 
 vup_status vup_hist_fused(vup_grid g, int64_t K, float *hist, cudaStream_t s, const float *ftab,
@@ -1979,7 +1979,7 @@ vup_status vup_hist_fused(vup_grid g, int64_t K, float *hist, cudaStream_t s, co
     const size_t smem = hist_smem_bytes(rows);
     // run-end words encode the rest index in 21 bits (3-D: a0 < 512, a1 < 4096)
     const bool coded = nd == 2 || (g->n[0] <= 512 && g->n[1] <= 4096);
-    const bool in_smem = smem <= 220 * 1024 && coded;
+    const bool in_smem = smem <= kSmemMost && coded;
     // 3-D point stream: both rest-axis factor tiles in shared memory when they fit beside the tile
     const size_t rest_bytes = nd == 3 ? (size_t)(g->n[0] + g->n[1]) * kKT * sizeof(float) : 0;
     A.rest_n0 = nd == 3 ? g->n[0] : 0;
@@ -2001,7 +2001,7 @@ vup_status vup_hist_fused(vup_grid g, int64_t K, float *hist, cudaStream_t s, co
             auto launch = [&](auto kern, int mode) -> vup_status {
                 const size_t sm_bytes =
                     hist_smem_bytes(rows, hist_warps(mode)) + (hist_staged(mode) ? rest_bytes : 0);
-                VUP_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_bytes));
+                VUP_CHECK_CUDA(smem_allow(kern));
                 VUP_CHECK_CUDA(launch_pdl(kern, dim3(ctas), dim3(hist_warps(mode) * 32), sm_bytes, s, A, rows, nkt,
                                           (int *)g->hist_sel + kHistCtr + hist_stream_of(mode)));
                 return VUP_OK;
@@ -2056,7 +2056,7 @@ vup_status vup_hist_fused(vup_grid g, int64_t K, float *hist, cudaStream_t s, co
 bool vup_hist_tile_fits(vup_grid g) {
     const bool coded = g->ndim == 2 || (g->n[0] <= 512 && g->n[1] <= 4096);
     for (int l = 0; l < g->n_layouts; ++l)
-        if (hist_smem_bytes(g->hl[l].part_rows) > 220 * 1024) return false;
+        if (hist_smem_bytes(g->hl[l].part_rows) > kSmemMost) return false;
     return coded;
 }
 
@@ -2112,7 +2112,7 @@ vup_status vup_post_fused(vup_grid g, int64_t K, float *hist, float *post, cudaS
         const size_t smem = hist_smem_bytes(rows);
         const unsigned ctas = (unsigned)std::min<int64_t>(vup_num_sms(), (int64_t)P_max * nkt * A.h.C);
         auto launch = [&](auto kern) -> vup_status {
-            VUP_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            VUP_CHECK_CUDA(smem_allow(kern));
             kern<<<ctas, kHistWarps * 32, smem, s>>>(A, rows, nkt, ctr);
             VUP_CHECK_LAUNCH();
             return VUP_OK;
@@ -2132,7 +2132,7 @@ vup_status vup_post_fused(vup_grid g, int64_t K, float *hist, float *post, cudaS
 bool vup_hist_batchable(vup_grid g) {
     if (g->ndim != 2) return false;
     for (int l = 0; l < g->n_layouts; ++l)
-        if (hist_smem_bytes(g->hl[l].part_rows) > 220 * 1024) return false;
+        if (hist_smem_bytes(g->hl[l].part_rows) > kSmemMost) return false;
     return true;
 }
 
@@ -2229,12 +2229,9 @@ vup_status vup_hist_plan(int n, const vup_grid *gs, const int64_t *Ks, float *co
     VUP_CHECK_CUDA(cudaMemcpy(P->items.p, items.data(), sizeof(HistItem) * items.size(), cudaMemcpyHostToDevice));
     VUP_CHECK_CUDA(cudaMemcpy(P->fitems.p, fin.data(), sizeof(int4) * fin.size(), cudaMemcpyHostToDevice));
     // the largest tile any plan may use, so that graphs of earlier plans stay launchable
-    VUP_CHECK_CUDA(
-        cudaFuncSetAttribute(k_hist_batched<1, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
-    VUP_CHECK_CUDA(
-        cudaFuncSetAttribute(k_hist_batched<1, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
-    VUP_CHECK_CUDA(
-        cudaFuncSetAttribute(k_hist_batched<1, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
+    VUP_CHECK_CUDA(smem_allow(k_hist_batched<1, 0>));
+    VUP_CHECK_CUDA(smem_allow(k_hist_batched<1, 1>));
+    VUP_CHECK_CUDA(smem_allow(k_hist_batched<1, 2>));
     *out = P;
     return VUP_OK;
 }
@@ -2255,7 +2252,7 @@ vup_status vup_hist_batched(void *plan, cudaStream_t s) {
     const HistPlan *P = (const HistPlan *)plan;
     if (P->n_items == 0) return VUP_OK;
     const size_t smem = hist_smem_bytes(P->rows);
-    if (smem > 220 * 1024) return VUP_ERR_UNSUPPORTED;
+    if (smem > kSmemMost) return VUP_ERR_UNSUPPORTED;
     {
         VUP_PROF("hist_segmented_batched", s, 5);
         for (int i0 = 0; i0 < P->n_fold; i0 += 65535) {  // (the grid's y limit)

@@ -44,6 +44,16 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<Args &&>(args)...);
 }
 
+// Dynamic shared memory past a kernel's default limit has to be allowed, and
+// what is allowed belongs to the kernel, not to the launch: each call allows
+// the same most (no kernel here asks for more), as a call that set its own
+// size could lower it between another thread's setting and launch.
+constexpr int kSmemMost = 220 * 1024;
+template <typename... KArgs>
+inline cudaError_t smem_allow(void (*kernel)(KArgs...)) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMost);
+}
+
 void vup_set_last_cuda_error(cudaError_t e, const char *expr, const char *file, int line);
 
 // Every device allocation of the library goes through vup_dev_malloc, which

@@ -260,7 +260,7 @@ extern "C" vup_status vup_ipsa_matrix(vup_grid g, int64_t K, const float *hist, 
     VUP_PROF("ipsa_matrix", s, 1);
     const size_t smem = sizeof(int) * ((size_t)g->B + (size_t)n_dbins);
     if (smem > 40 * 1024)
-        VUP_CHECK_CUDA(cudaFuncSetAttribute(k_ipsa_matrix, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        VUP_CHECK_CUDA(smem_allow(k_ipsa_matrix));
     const unsigned grid = (unsigned)std::min<int64_t>(K, (int64_t)vup_num_sms() * 8);
     k_ipsa_matrix<<<grid, 256, smem, s>>>(hist, K, g->B, g->ext, y_ref, n_dbins, dlo, dhi, out);
     VUP_CHECK_LAUNCH();
