@@ -374,10 +374,6 @@ extern "C" vup_status vup_grid_create(int ndim, const int64_t *n, const double *
         if (ndim >= 2) {
             g->fold_members = g->fold_rep + slices;
             g->fold_start = g->fold_members + slices;
-            // words past the stream's end are read by whole-window staging and
-            // masked; zero keeps their rest codes valid indices
-            e = cudaMemset(g->hl[0].ipt, 0, sizeof(uint2) * (N + 128));
-            if (e == cudaSuccess) e = cudaMemset(g->fold, 0, sizeof(FoldGeom));  // nothing merged before a layout is built
         } else {
             g->hl[0].perm = g->perm;
         }
@@ -403,8 +399,26 @@ extern "C" vup_status vup_grid_create(int ndim, const int64_t *n, const double *
         L.rec_chunk = A.rec_chunk;
         L.rec_chunk_grp = A.rec_chunk_grp;
     }
-    if (e == cudaSuccess) e = cudaMemset(g->dstatus, 0, sizeof(int));
-    if (e == cudaSuccess) e = cudaMemset(g->hist_sel, 0, sizeof(int32_t) * 8);
+    // cleared before the handle is returned, on a stream of their own: queued on the
+    // default stream they could wait behind a caller's work there and land in the
+    // middle of this grid's calls on another stream
+    if (e == cudaSuccess) {
+        cudaStream_t cs = nullptr;
+        e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
+        auto clear = [&](void *q, size_t bytes) {
+            if (e == cudaSuccess) e = cudaMemsetAsync(q, 0, bytes, cs);
+        };
+        clear(g->dstatus, sizeof(int));
+        clear(g->hist_sel, sizeof(int32_t) * 8);
+        if (ndim >= 2) {
+            // words past the stream's end are read by whole-window staging and
+            // masked; zero keeps their rest codes valid indices
+            clear(g->hl[0].ipt, sizeof(uint2) * (N + 128));
+            clear(g->fold, sizeof(FoldGeom));  // nothing merged before a layout is built
+        }
+        if (e == cudaSuccess) e = cudaStreamSynchronize(cs);
+        if (cs) cudaStreamDestroy(cs);
+    }
     if (e != cudaSuccess) {
         vup_set_last_cuda_error(e, "vup_grid_create", __FILE__, __LINE__);
         cudaGetLastError();
