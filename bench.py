@@ -723,13 +723,13 @@ def main():
     # overlap others and are not candidates)
     cands = {k: v for k, v in prof.items() if k.startswith(ROOF_GROUPS)}
     dominant = max(cands.items(), key=lambda kv: kv[1][1])[0] if cands else None
-    # bytes one histogram pass needs (the streams named are those of the unmerged grids' layouts)
+    # bytes one histogram pass needs, and the streams walked
     hist_units, streams = 0, set()
     points_only = getattr(work, "bayes", False)  # posterior means walk the point stream
     for g, K in work.hist_grids():
         info = g.info()
         if info.ndim >= 2:
-            mode = 0 if points_only else info.hist_stream
+            mode = 0 if points_only else g.hist_walk().stream
             streams.add(("points", "intervals", "records")[mode])
             hist_units += K * walk_bytes(g.array("bins").cpu().numpy().reshape(g.n), points_only)
 

@@ -400,11 +400,12 @@ typedef struct {
      * layout 0 gathers the last axis, layout 1 axis 0 (2-D only); stream 0
      * walks sorted points, stream 1 sorted intervals (stretches of one bin
      * along the gathered axis, summed as differences of prefix sums), stream
-     * 2 records (stretches of one line over a group of 4 consecutive bins,
-     * monotone, five prefix sums for four bins).  The choice and the counts are
+     * 2 records (stretches of one line over a group of 8 consecutive bins,
+     * monotone, nine prefix sums for eight bins).  The choice and the counts are
      * those of the grid itself; where slices of an axis that fall in the same
-     * bins throughout are merged for the walk, they are taken for this call
-     * from the unmerged grid.  hist_runs is 0 when the point and interval streams were
+     * bins throughout are merged for the walk (vup_hist_walk tells what then
+     * runs), the first call per model builds the unmerged layout for them.
+     * hist_runs is 0 when the point and interval streams were
      * not built (the record stream was cheaper than both). */
     int32_t hist_layout, hist_stream;
     int64_t hist_runs, hist_intervals, hist_records;
@@ -413,6 +414,21 @@ typedef struct {
     double yshift;
 } vup_grid_info_t;
 vup_status vup_grid_info(vup_grid g, vup_grid_info_t *info);
+
+/*
+ * The walk that the histograms of a 2-D / 3-D grid run for the current model:
+ * the sizes of the grid it runs on (slices of an axis that fall in the same bins
+ * throughout are merged where that leaves at most 5/8 of them; N their
+ * product), and layout, stream and counts as in vup_grid_info_t, of that
+ * grid.  Builds the layout if no call has; synchronises the device.
+ * VUP_ERR_INVALID_ARG for a 1-D grid, VUP_ERR_STATE without a model.
+ */
+typedef struct {
+    int64_t n[3], N;
+    int32_t layout, stream;
+    int64_t runs, intervals, records;
+} vup_hist_walk_t;
+vup_status vup_hist_walk(vup_grid g, vup_hist_walk_t *walk);
 
 /*
  * Histogram stream choice of a 2-D / 3-D grid: -1 (default) picks, per model,

@@ -788,6 +788,31 @@ extern "C" vup_status vup_sync(vup_grid g, vup_stream_t stream) {
     }
 }
 
+// The merged sizes of the grid's current layout, built when it is not.
+static vup_status current_layout(vup_grid g, FoldGeom &F) {
+    if (!g->layout_valid) {
+        vup_status st = vup_build_layout(g, 0);
+        if (st != VUP_OK) return st;
+    }
+    VUP_CHECK_CUDA(cudaDeviceSynchronize());
+    VUP_CHECK_CUDA(cudaMemcpy(&F, g->fold, sizeof(F), cudaMemcpyDeviceToHost));
+    return VUP_OK;
+}
+
+// Choice and counts of the layout built last.
+static vup_status layout_counts(vup_grid g, LayoutCounts &c) {
+    int32_t sel[2] = {0, 0};
+    VUP_CHECK_CUDA(cudaDeviceSynchronize());
+    VUP_CHECK_CUDA(cudaMemcpy(sel, g->hist_sel, sizeof(sel), cudaMemcpyDeviceToHost));
+    const auto &HL = g->hl[0];  // the built layout's arrays
+    VUP_CHECK_CUDA(cudaMemcpy(&c.runs, HL.n_runs, sizeof(int32_t), cudaMemcpyDeviceToHost));
+    VUP_CHECK_CUDA(cudaMemcpy(&c.intervals, HL.n_iv, sizeof(int32_t), cudaMemcpyDeviceToHost));
+    VUP_CHECK_CUDA(cudaMemcpy(&c.records, HL.n_rec, sizeof(int32_t), cudaMemcpyDeviceToHost));
+    c.layout = sel[0];
+    c.stream = sel[1];
+    return VUP_OK;
+}
+
 extern "C" vup_status vup_grid_info(vup_grid g, vup_grid_info_t *info) {
     if (!g || !info) return VUP_ERR_INVALID_ARG;
     memset(info, 0, sizeof(*info));
@@ -814,42 +839,51 @@ extern "C" vup_status vup_grid_info(vup_grid g, vup_grid_info_t *info) {
         info->yscale = sc[kScaleS];
         info->yshift = sc[kScaleC];
         if (g->ndim >= 2) {
-            if (!g->layout_valid) {
-                vup_status st = vup_build_layout(g, 0);
-                if (st != VUP_OK) return st;
-                VUP_CHECK_CUDA(cudaDeviceSynchronize());
-            }
-            // the counts describe the grid itself: where the walks run on a merged
-            // grid, the unfolded layout is built for them and then the merged one again
+            // the counts describe the grid itself: where the walks run on a merged grid,
+            // the unmerged layout is built for them, once per model, and then the merged
+            // one again
             FoldGeom F;
-            VUP_CHECK_CUDA(cudaMemcpy(&F, g->fold, sizeof(F), cudaMemcpyDeviceToHost));
-            const bool points = g->layout_has_points != 0;
-            struct Refold {
-                vup_grid g;
-                bool on, points;
-                ~Refold() {
-                    if (on && vup_build_layout(g, 0, points) != VUP_OK) g->layout_valid = 0;
-                    if (on) cudaDeviceSynchronize();
-                }
-            } refold{g, F.any != 0, points};
-            if (F.any) {
-                vup_status st = vup_build_layout(g, 0, points, nullptr, nullptr, false);
-                if (st != VUP_OK) return st;
+            vup_status st = current_layout(g, F);
+            if (st != VUP_OK) return st;
+            const int points = g->layout_has_points != 0;
+            if (!F.any) {
+                if ((st = layout_counts(g, g->info_counts)) != VUP_OK) return st;
+            } else if (g->info_points != points) {
+                st = vup_build_layout(g, 0, points, nullptr, nullptr, false);
+                if (st == VUP_OK) st = layout_counts(g, g->info_counts);
+                const vup_status back = vup_build_layout(g, 0, points);
+                if (back != VUP_OK) g->layout_valid = 0;
                 VUP_CHECK_CUDA(cudaDeviceSynchronize());
+                if (st != VUP_OK) return st;
+                if (back != VUP_OK) return back;
+                g->info_points = points;
             }
-            int32_t sel[2] = {0, 0}, nr = 0, ni = 0, nrec = 0;
-            VUP_CHECK_CUDA(cudaMemcpy(sel, g->hist_sel, sizeof(sel), cudaMemcpyDeviceToHost));
-            const auto &HL = g->hl[0];  // the built layout's arrays
-            VUP_CHECK_CUDA(cudaMemcpy(&nr, HL.n_runs, sizeof(int32_t), cudaMemcpyDeviceToHost));
-            VUP_CHECK_CUDA(cudaMemcpy(&ni, HL.n_iv, sizeof(int32_t), cudaMemcpyDeviceToHost));
-            VUP_CHECK_CUDA(cudaMemcpy(&nrec, HL.n_rec, sizeof(int32_t), cudaMemcpyDeviceToHost));
-            info->hist_layout = sel[0];
-            info->hist_stream = sel[1];
-            info->hist_runs = nr;
-            info->hist_intervals = ni;
-            info->hist_records = nrec;
+            const LayoutCounts &c = g->info_counts;
+            info->hist_layout = c.layout;
+            info->hist_stream = c.stream;
+            info->hist_runs = c.runs;
+            info->hist_intervals = c.intervals;
+            info->hist_records = c.records;
         }
     }
+    return VUP_OK;
+}
+
+extern "C" vup_status vup_hist_walk(vup_grid g, vup_hist_walk_t *walk) {
+    if (!g || !walk || g->ndim < 2) return VUP_ERR_INVALID_ARG;
+    if (!g->have_model) return VUP_ERR_STATE;
+    VUP_CHECK_CUDA(cudaDeviceSynchronize());
+    FoldGeom F;
+    LayoutCounts c;
+    vup_status st = current_layout(g, F);
+    if (st != VUP_OK || (st = layout_counts(g, c)) != VUP_OK) return st;
+    for (int d = 0; d < 3; ++d) walk->n[d] = F.n[d];
+    walk->N = F.N;
+    walk->layout = c.layout;
+    walk->stream = vup_hist_tile_fits(g) ? c.stream : 0;  // (the kernel without shared-memory tiles walks points)
+    walk->runs = c.runs;
+    walk->intervals = c.intervals;
+    walk->records = c.records;
     return VUP_OK;
 }
 
@@ -857,7 +891,10 @@ extern "C" vup_status vup_set_hist_stream(vup_grid g, int32_t stream_kind, vup_s
     if (!g || g->ndim < 2 || stream_kind < -1 || stream_kind > 2) return VUP_ERR_INVALID_ARG;
     // the layout is rebuilt on next use with the choice (a forced point or
     // interval stream needs the key-sorted streams a record choice skips)
-    if (stream_kind != g->hist_force) g->layout_valid = g->ndim == 1;
+    if (stream_kind != g->hist_force) {
+        g->layout_valid = g->ndim == 1;
+        g->info_points = -1;
+    }
     g->hist_force = stream_kind;
     return VUP_OK;
 }

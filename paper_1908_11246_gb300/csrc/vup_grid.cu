@@ -2150,6 +2150,7 @@ vup_status vup_launch_grid_finish(vup_grid g, cudaStream_t s) {
         launches += 2 + scan_launches((int64_t)B * n_tiles);
     }
     g->layout_valid = g->ndim == 1;
+    g->info_points = -1;
     prof.launches = launches;
     for (int o = 0; o < kNumOrient; ++o) g->have_tab[o][0] = g->have_tab[o][1] = g->have_tab[o][2] = 0;
     if (bins_done) g->have_tab[vup_tc_orient(g)][1] = 1;  // written with the bins

@@ -231,6 +231,11 @@ struct FoldGeom {
 constexpr int32_t kFoldLast = 1 << 30;  // flags the last member of a class in its list
 __host__ __device__ inline int64_t fold_cap(int64_t n) { return (5 * n + 7) / 8; }  // most classes of a folded axis
 
+// Choice and counts of a histogram layout (host copies).
+struct LayoutCounts {
+    int32_t layout = 0, stream = 0, runs = 0, intervals = 0, records = 0;
+};
+
 struct vup_grid_s {
     int device = 0;
     int ndim = 0;
@@ -256,6 +261,10 @@ struct vup_grid_s {
     int natural_valid = 0;         // perm holds the stable sort by bin
     int layout_valid = 0;          // the histogram layout matches the current bins
     int layout_has_points = 0;     // ... and its key-sorted streams were built on request
+    // vup_grid_info's counts of a merged grid's unmerged layout, kept until the next
+    // model or stream choice: layout_has_points of their build (-1: none)
+    int info_points = -1;
+    LayoutCounts info_counts;
     int range_ready = 0;           // ext holds the range of y (reduced by the model kernels)
     int bins_ready = 0;            // the model kernel also wrote the bins and the power-table scale
     // second stream for the layout build beside the density preparation

@@ -29,7 +29,7 @@ ABI_SYMBOLS = [
     "vup_grid_create", "vup_grid_destroy", "vup_eval_model", "vup_set_outputs", "vup_propagate",
     "vup_propagate_weights", "vup_propagate_weights_noalloc", "vup_ipsa_sensitivity", "vup_propagate_ipsa", "vup_propagate_batched", "vup_batched_report", "vup_sync", "vup_selftest_wait", "vup_model_at",
     "vup_deviation_moments", "vup_ipsa_matrix", "vup_sa_fields", "vup_posterior_means",
-    "vup_grid_info", "vup_set_hist_stream", "vup_set_weights_form", "vup_grid_copy", "vup_status_string", "vup_version", "vup_profile",
+    "vup_grid_info", "vup_hist_walk", "vup_set_hist_stream", "vup_set_weights_form", "vup_grid_copy", "vup_status_string", "vup_version", "vup_profile",
     "vup_profile_read", "vup_profile_timeline", "vup_last_error_detail", "vup_debug_fail_alloc",
     "vup_measure_peak",
 ]
@@ -46,6 +46,11 @@ class vup_grid_info_t(C.Structure):
                 ("yscale", C.c_double), ("have_model", C.c_int32), ("hist_layout", C.c_int32),
                 ("hist_stream", C.c_int32), ("hist_runs", C.c_int64), ("hist_intervals", C.c_int64),
                 ("hist_records", C.c_int64), ("yshift", C.c_double)]
+
+
+class vup_hist_walk_t(C.Structure):
+    _fields_ = [("n", C.c_int64 * 3), ("N", C.c_int64), ("layout", C.c_int32), ("stream", C.c_int32),
+                ("runs", C.c_int64), ("intervals", C.c_int64), ("records", C.c_int64)]
 
 
 class VUPError(RuntimeError):
@@ -85,6 +90,7 @@ def lib():
         l.vup_sa_fields.argtypes = [i64, C.c_int, vp, C.c_double, vp, vp, vp, vp, vp]
         l.vup_posterior_means.argtypes = [vp, C.POINTER(vup_densities), vp, vp, vp]
         l.vup_grid_info.argtypes = [vp, C.POINTER(vup_grid_info_t)]
+        l.vup_hist_walk.argtypes = [vp, C.POINTER(vup_hist_walk_t)]
         l.vup_set_hist_stream.argtypes = [vp, C.c_int32, vp]
         l.vup_set_weights_form.argtypes = [vp, C.c_int32]
         l.vup_grid_copy.argtypes = [vp, C.c_int, vp, C.c_size_t, vp]
@@ -304,6 +310,12 @@ def vup_grid_info(h):
     return info
 
 
+def vup_hist_walk(h):
+    walk = vup_hist_walk_t()
+    _check(lib().vup_hist_walk(h, C.byref(walk)), "vup_hist_walk")
+    return walk
+
+
 def vup_set_hist_stream(h, kind: int, stream=None):
     """Histogram stream choice: -1 auto, 0 sorted points, 1 sorted intervals, 2 records."""
     _check(lib().vup_set_hist_stream(h, int(kind), _stream(stream)), "vup_set_hist_stream")
@@ -409,6 +421,10 @@ class Grid:
 
     def info(self):
         return vup_grid_info(self.h)
+
+    def hist_walk(self):
+        """What the grid's histograms walk: merged sizes, layout, stream and counts."""
+        return vup_hist_walk(self.h)
 
     def set_hist_stream(self, kind: int, stream=None):
         """-1: automatic choice; 0: sorted points; 1: sorted intervals; 2: records."""
