@@ -1867,7 +1867,7 @@ static HistArgs hist_args_for(vup_grid g, int64_t K, float *hist, int64_t &rows,
     A.fold_members = g->fold_members;
     for (int d = 0; d < nd; ++d) {
         A.off[d] = d ? A.off[d - 1] + g->n[d - 1] : 0;
-        A.foff[d] = d ? A.foff[d - 1] + fold_cap(g->n[d - 1]) : 0;
+        A.foff[d] = fold_row(nd, g->n, d);
     }
     A.sel = g->hist_sel;
     A.GB = (int)ceil_div64(g->B, kRecBinsH);
@@ -1903,10 +1903,10 @@ struct FoldTabArgs {
 __device__ __forceinline__ void fold_table_rows(const FoldTabArgs &T, int64_t first, int64_t step) {
     const int64_t kb = (T.K_pad + 511) / 512;
     const int gathered = T.ndim == 2 && T.sel[0] ? 0 : T.ndim - 1;
-    int64_t off = 0, foff = 0;
+    int64_t off = 0;
     for (int d = 0; d < T.ndim; ++d) {
         if (T.fold->folded[d] && d != gathered) {
-            const int64_t rows = T.fold->n[d];
+            const int64_t rows = T.fold->n[d], foff = fold_row(T.ndim, T.n, d);
             for (int64_t u = first; u < rows * kb; u += step) {
                 const int64_t c = u / kb, k = (u - c * kb) * 512 + 4 * threadIdx.x;
                 if (k >= T.K_pad) continue;
@@ -1916,7 +1916,6 @@ __device__ __forceinline__ void fold_table_rows(const FoldTabArgs &T, int64_t fi
             }
         }
         off += T.n[d];
-        foff += fold_cap(T.n[d]);
     }
 }
 __global__ void __launch_bounds__(128) k_fold_tables(const __grid_constant__ FoldTabArgs T) {
@@ -1946,8 +1945,7 @@ static FoldTabArgs fold_tab_args(vup_grid g, int64_t K) {
 }
 
 vup_status vup_reserve_fold(vup_grid g, int64_t K) {
-    int64_t rows = 0;
-    for (int d = 0; d < g->ndim; ++d) rows += fold_cap(g->n[d]);
+    const int64_t rows = fold_row(g->ndim, g->n, g->ndim);
     return devbuf_reserve(g->ftab_fold, sizeof(float) * (size_t)rows * (size_t)(ceil_div64(K, 128) * 128));
 }
 
@@ -1955,8 +1953,7 @@ vup_status vup_fold_tables(vup_grid g, int64_t K, cudaStream_t s, const float *f
     FoldTabArgs T = fold_tab_args(g, K);
     if (ftab) T.ftab = ftab;
     T.ctr = g->hist_sel + kHistCtr;
-    int64_t rows = 0;
-    for (int d = 0; d < g->ndim; ++d) rows += fold_cap(g->n[d]);
+    const int64_t rows = fold_row(g->ndim, g->n, g->ndim);
     const int64_t blocks = std::min<int64_t>(rows * ceil_div64(T.K_pad, 512), (int64_t)vup_num_sms() * 16);
     VUP_PROF("hist_fold_tables", s, 1);
     k_fold_tables<<<(unsigned)blocks, 128, 0, s>>>(T);

@@ -230,6 +230,15 @@ struct FoldGeom {
 };
 constexpr int32_t kFoldLast = 1 << 30;  // flags the last member of a class in its list
 __host__ __device__ inline int64_t fold_cap(int64_t n) { return (5 * n + 7) / 8; }  // most classes of a folded axis
+// First row of axis d's merged factor table, and the rows of all (d = ndim).  Only
+// the rest axes have one: of a 2-D grid's two axes one is gathered, so both start at
+// row 0; of three the last is gathered.
+__host__ __device__ inline int64_t fold_row(int ndim, const int64_t *n, int d) {
+    if (ndim == 2) return d < 2 ? 0 : (fold_cap(n[0]) > fold_cap(n[1]) ? fold_cap(n[0]) : fold_cap(n[1]));
+    int64_t r = 0;
+    for (int q = 0; q < d && q < ndim - 1; ++q) r += fold_cap(n[q]);
+    return r;
+}
 
 // Choice and counts of a histogram layout (host copies).
 struct LayoutCounts {
@@ -350,7 +359,7 @@ struct vup_grid_s {
     int64_t K_cap = 0;
     DevBuf dconst, dstats, ftab, atab_hi, atab_lo, partials, hist_part, hist_direct, ipsa_part;
     DevBuf post_tmp, post_x;  // posterior means: weighted tables, sums per key; axis coordinates
-    DevBuf ftab_fold;    // merged factor tables of the folded axes, axis d at fold_off(d) rows of K_pad
+    DevBuf ftab_fold;    // merged factor tables of the folded rest axes, axis d at fold_row(d) rows of K_pad
     DevBuf atf_hi, atf_lo;         // TF32 split of the A operand [K_pad][R_pad]
 
     // supplied-weights path: the grid points in blocks of 256, each block's
