@@ -351,12 +351,14 @@ vup_status vup_sa_fields(int64_t K, int n_bins, const float *hist, double level,
  * each with posterior probability W[k,i] / H[k,b] by Bayes' theorem): the
  * posterior mean of every input axis per output bin,
  *   post[k][b][d] = sum_{i in bin b} W[k,i] x_{d,i} / H[k,b]  (0 where H = 0),
- * from FP32 segmented sums: one histogram pass for H and one per axis with
- * that axis' factors weighted by its coordinates (W is never formed).
+ * from FP32 segmented sums (W is never formed): one walk over the points sums
+ * the weights and the weights times each axis' coordinate per bin; a grid whose
+ * tiles do not fit shared memory takes one histogram pass for H and one per axis.
  *   hist [K][B] float (device, or NULL): receives H as well;
  *   post [K][B][ndim] float (device).
  * ndim >= 2 (VUP_ERR_UNSUPPORTED for 1-D grids).  The first call with a
- * larger K than before allocates library scratch.
+ * larger K than before allocates library scratch: the axes' weighted factors,
+ * and the walk's sums for as many densities as 512 MB hold.
  */
 vup_status vup_posterior_means(vup_grid g, const vup_densities *d, float *hist, float *post, vup_stream_t stream);
 

@@ -57,10 +57,7 @@ extern "C" vup_status vup_posterior_means(vup_grid g, const vup_densities *d, fl
     }
     if ((st = vup_ensure_layout(g, s, true)) != VUP_OK) return st;  // the ratios walk the point stream
     if ((st = vup_density_prep(g, d, 0, s)) != VUP_OK) return st;
-    if (one_pass) {
-        bool done = false;
-        return vup_post_fused(g, K, hist, post, s, done);
-    }
+    if (one_pass) return vup_post_fused(g, K, hist, post, s);
     // point stream: the ratios need the relative accuracy of low-mass bins,
     // which differences of prefix sums (interval stream) do not keep
     if ((st = vup_hist_fused(g, K, hist, s, nullptr, true)) != VUP_OK) return st;

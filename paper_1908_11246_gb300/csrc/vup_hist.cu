@@ -1422,10 +1422,16 @@ struct PostArgs {
     HistArgs h;              // the histogram's arguments (tables, layout, scratch sizes)
     const float *xs;         // coordinates of every axis, axis d from off[d]
     const float *fx;         // rest factors times coordinate (merged), axis d at off[d] rows
-    float *part, *direct;    // [cut row or key][1 + ndim][K_pad]
+    float *part, *direct;    // [cut row or key][1 + ndim][kb] of the densities k0 .. k0 + kb - 1
+    int64_t k0, kb;
     float *hist, *post;      // [K][B] (or null), [K][B][ndim]
 };
 constexpr int kPostKT = 64;
+// The sums of a walk, (1 + ndim) floats per cut row or key and density, are kept for
+// as many densities as this many bytes hold (at least 128); the walk and its finish
+// run once per such block (1024 x 1024 points, 256 bins: 25 KB per density, one
+// block up to 21000 densities; 6 parts of 5000 bins: 0.37 MB, blocks of 1408).
+constexpr size_t kPostSums = (size_t)512 << 20;
 __device__ __forceinline__ float2 ld2(const float *q) { return *reinterpret_cast<const float2 *>(q); }
 
 // Rest factors f_x (and, of folded axes, the merged f into ftab_fold).
@@ -1520,7 +1526,7 @@ __global__ void __launch_bounds__(kHistWarps * 32, 1)
         const int G = s_G, it = s_item;
         if (it >= (int64_t)nkt * P * G || abort) return;  // uniform
         const int cg = it % G, pk = it / G, p = pk % P;
-        const int64_t k0 = (int64_t)(pk / P) * kPostKT, k = k0 + 2 * lane;
+        const int64_t k0 = A.k0 + (int64_t)(pk / P) * kPostKT, k = k0 + 2 * lane;
         if (threadIdx.x < kPostKT) s_iz[threadIdx.x] = inv_z(A.h, k0 + threadIdx.x);
         __syncthreads();
         const int64_t row0 = (int64_t)p * H.part_rows;
@@ -1630,11 +1636,11 @@ __global__ void __launch_bounds__(kHistWarps * 32, 1)
             auto flush = [&]() {
                 const bool first = cur_key == first_key;
                 const bool shared = first ? sh_first : (cur_key == last_key && sh_last);
-                float *dst = (shared ? A.part + ((int64_t)c * 2 + (first ? 0 : 1)) * NO * K_pad
-                                     : A.direct + (int64_t)cur_key * NO * K_pad) + k;
+                float *dst = (shared ? A.part + ((int64_t)c * 2 + (first ? 0 : 1)) * NO * A.kb
+                                     : A.direct + (int64_t)cur_key * NO * A.kb) + (k - A.k0);
                 if (VUP_DBG_IN(cur_key, (int64_t)P * A.h.B, dstatus))
 #pragma unroll
-                    for (int o = 0; o < NO; ++o) *reinterpret_cast<float2 *>(dst + o * K_pad) = acc[o];
+                    for (int o = 0; o < NO; ++o) *reinterpret_cast<float2 *>(dst + o * A.kb) = acc[o];
 #pragma unroll
                 for (int o = 0; o < NO; ++o) acc[o] = make_float2(0.f, 0.f);
             };
@@ -1724,7 +1730,7 @@ __global__ void __launch_bounds__(256) k_post_finish(const __grid_constant__ Pos
     const int P = h.fold->P[h.sel[0] ? 1 : 0], nd = h.ndim, no = 1 + nd;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int b = blockIdx.y * 8 + warp;
-    const int64_t k0 = (int64_t)blockIdx.x * 128, k = k0 + 4 * lane;
+    const int64_t k0 = A.k0 + (int64_t)blockIdx.x * 128, k = k0 + 4 * lane;
     float4 t[4];
 #pragma unroll
     for (int o = 0; o < 4; ++o) t[o] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -1734,19 +1740,19 @@ __global__ void __launch_bounds__(256) k_post_finish(const __grid_constant__ Pos
             const int2 cc = H.key_chunks[key];
             if (cc.x < 0) continue;
             if (cc.x == cc.y) {
-                const float *row = A.direct + (int64_t)key * no * h.K_pad + k;
+                const float *row = A.direct + (int64_t)key * no * A.kb + (k - A.k0);
 #pragma unroll
                 for (int o = 0; o < 4; ++o)
-                    if (o < no) add4(t[o], ld4(row + o * h.K_pad));
+                    if (o < no) add4(t[o], ld4(row + o * A.kb));
                 continue;
             }
             for (int c = cc.x; c <= cc.y; ++c) {
                 if (H.chunk_pt[c] >= H.chunk_pt[c + 1]) continue;
                 const int side = H.chunk_bin[2 * c] == key ? 0 : 1;
-                const float *row = A.part + ((int64_t)c * 2 + side) * no * h.K_pad + k;
+                const float *row = A.part + ((int64_t)c * 2 + side) * no * A.kb + (k - A.k0);
 #pragma unroll
                 for (int o = 0; o < 4; ++o)
-                    if (o < no) add4(t[o], ld4(row + o * h.K_pad));
+                    if (o < no) add4(t[o], ld4(row + o * A.kb));
             }
         }
 #pragma unroll
@@ -2058,11 +2064,8 @@ bool vup_hist_tile_fits(vup_grid g) {
 }
 
 // H (or null) and posterior means of a 2-D / 3-D grid whose tiles fit shared
-// memory, from the densities' factor tables and the point stream; false when
-// they do not fit (nothing done).
-vup_status vup_post_fused(vup_grid g, int64_t K, float *hist, float *post, cudaStream_t s, bool &done) {
-    done = false;
-    if (!vup_hist_tile_fits(g)) return VUP_OK;
+// memory, from the densities' factor tables and the point stream.
+vup_status vup_post_fused(vup_grid g, int64_t K, float *hist, float *post, cudaStream_t s) {
     int64_t rows;
     int P_max;
     PostArgs A{};
@@ -2073,16 +2076,17 @@ vup_status vup_post_fused(vup_grid g, int64_t K, float *hist, float *post, cudaS
     int64_t axis_rows = 0;
     for (int d = 0; d < nd; ++d) axis_rows += g->n[d];
     // scratch: f_x tables, then the cut rows and the keys' rows; the coordinates
-    const size_t f_fx = (size_t)axis_rows * K_pad, f_part = (size_t)P_max * A.h.C * 2 * no * K_pad;
-    const size_t f_dir = (size_t)P_max * A.h.B * no * K_pad;
+    const size_t f_fx = (size_t)axis_rows * K_pad, f_part = (size_t)P_max * A.h.C * 2 * no;
+    const size_t f_dir = (size_t)P_max * A.h.B * no;  // (both per density)
+    A.kb = std::min<int64_t>(K_pad, std::max<int64_t>(1, (int64_t)(kPostSums / (sizeof(float) * 128 * (f_part + f_dir)))) * 128);
     vup_status st;
-    if ((st = devbuf_reserve(g->post_tmp, sizeof(float) * (f_fx + f_part + f_dir))) != VUP_OK) return st;
+    if ((st = devbuf_reserve(g->post_tmp, sizeof(float) * (f_fx + (f_part + f_dir) * A.kb))) != VUP_OK) return st;
     if ((st = devbuf_reserve(g->post_x, sizeof(float) * (size_t)axis_rows)) != VUP_OK) return st;
     float *fx = (float *)g->post_tmp.p, *xs = (float *)g->post_x.p;
     A.xs = xs;
     A.fx = fx;
     A.part = fx + f_fx;
-    A.direct = A.part + f_part;
+    A.direct = A.part + f_part * A.kb;
     A.hist = hist;
     A.post = post;
     AxisGeom G{};
@@ -2103,25 +2107,28 @@ vup_status vup_post_fused(vup_grid g, int64_t K, float *hist, float *post, cudaS
         k_post_tables<<<(unsigned)blocks, 128, 0, s>>>(A, fx, (float *)g->ftab_fold.p, ctr);
         VUP_CHECK_LAUNCH();
     }
-    {
-        VUP_PROF("hist_segmented", s, 1);
-        const int nkt = (int)ceil_div64(K, kPostKT);
-        const size_t smem = hist_smem_bytes(rows);
-        const unsigned ctas = (unsigned)std::min<int64_t>(vup_num_sms(), (int64_t)P_max * nkt * A.h.C);
-        auto launch = [&](auto kern) -> vup_status {
-            VUP_CHECK_CUDA(smem_allow(kern));
-            kern<<<ctas, kHistWarps * 32, smem, s>>>(A, rows, nkt, ctr);
-            VUP_CHECK_LAUNCH();
-            return VUP_OK;
-        };
-        st = nd == 2 ? launch(k_post_walk<1, 4>)
-                     : (vup_hist_rest_staged(g) ? launch(k_post_walk<2, 1>) : launch(k_post_walk<2, 4>));
-        if (st != VUP_OK) return st;
+    for (A.k0 = 0; A.k0 < K; A.k0 += A.kb) {
+        const int64_t nk = std::min(A.kb, K - A.k0);
+        if (A.k0) VUP_CHECK_CUDA(cudaMemsetAsync(ctr, 0, sizeof(int), s));  // (the tables' kernel zeroed it for the first)
+        {
+            VUP_PROF("hist_segmented", s, 1);
+            const int nkt = (int)ceil_div64(nk, kPostKT);
+            const size_t smem = hist_smem_bytes(rows);
+            const unsigned ctas = (unsigned)std::min<int64_t>(vup_num_sms(), (int64_t)P_max * nkt * A.h.C);
+            auto launch = [&](auto kern) -> vup_status {
+                VUP_CHECK_CUDA(smem_allow(kern));
+                kern<<<ctas, kHistWarps * 32, smem, s>>>(A, rows, nkt, ctr);
+                VUP_CHECK_LAUNCH();
+                return VUP_OK;
+            };
+            st = nd == 2 ? launch(k_post_walk<1, 4>)
+                         : (vup_hist_rest_staged(g) ? launch(k_post_walk<2, 1>) : launch(k_post_walk<2, 4>));
+            if (st != VUP_OK) return st;
+        }
+        VUP_PROF("posterior_finish", s, 1);
+        k_post_finish<<<dim3((unsigned)ceil_div64(nk, 128), (unsigned)ceil_div64(g->B, 8)), 256, 0, s>>>(A);
+        VUP_CHECK_LAUNCH();
     }
-    VUP_PROF("posterior_finish", s, 1);
-    k_post_finish<<<dim3((unsigned)ceil_div64(K, 128), (unsigned)ceil_div64(g->B, 8)), 256, 0, s>>>(A);
-    VUP_CHECK_LAUNCH();
-    done = true;
     return VUP_OK;
 }
 

@@ -428,7 +428,7 @@ vup_status vup_hist_fused(vup_grid g, int64_t K, float *hist, cudaStream_t s, co
 vup_status vup_fold_tables(vup_grid g, int64_t K, cudaStream_t s, const float *ftab = nullptr);
 vup_status vup_reserve_fold(vup_grid g, int64_t K);
 size_t vup_fold_scratch_bytes(const vup_grid_s *g);
-vup_status vup_post_fused(vup_grid g, int64_t K, float *hist, float *post, cudaStream_t s, bool &done);
+vup_status vup_post_fused(vup_grid g, int64_t K, float *hist, float *post, cudaStream_t s);
 vup_status vup_propagate_1d(vup_grid g, const vup_densities *d, double *raw, double *central,
                             float *hist, cudaStream_t s);
 vup_status vup_ipsa_1d(vup_grid g, const vup_densities *d, const double *grad, float *dmu,

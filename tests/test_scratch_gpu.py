@@ -60,3 +60,29 @@ def test_merged_tables_are_those_of_the_rest_axes(n, K):
     assert _used() == before
     g.sync()
     g.close()
+
+
+@pytest.mark.parametrize("n, K, B", [((300, 2000), 3000, 5000), ((20, 24, 900), 2500, 8192)])
+def test_posterior_sums_are_held_for_blocks_of_densities(n, K, B):
+    """Many keys (6 and 3 parts x B bins): the walk's sums stay within 512 MB beside the
+    weighted factors, and the blocks' seams give what calls of a few densities give."""
+    from paper_1908_11246_gb300 import vup
+    nd = len(n)
+    g, dd, B = _setup(n, K, B)
+    K_pad = -(-K // 128) * 128
+    hist = torch.empty((K, B), dtype=torch.float32, device="cuda")
+    post = torch.empty((K, B, nd), dtype=torch.float32, device="cuda")
+    g.propagate(dd, "fp32", moments=False, central=False)  # the scratch of a propagation
+    torch.cuda.empty_cache()
+    before = _used()
+    vup.vup_posterior_means(g.h, vup.make_densities(dd), hist, post)
+    assert _used() - before <= 4 * sum(n) * K_pad + 512 * MB + 6 * MB
+    for k0 in [*range(0, K - 200, 97), K - 200]:
+        part = {q: v[k0:k0 + 200].contiguous() for q, v in dd.items()}
+        h, p = torch.empty_like(hist[:200]), torch.empty_like(post[:200])
+        vup.vup_posterior_means(g.h, vup.make_densities(part), h, p)
+        torch.cuda.synchronize()
+        # the same sums in the same order, whatever the block
+        assert torch.equal(h, hist[k0:k0 + 200]) and torch.equal(p, post[k0:k0 + 200])
+    g.sync()
+    g.close()
