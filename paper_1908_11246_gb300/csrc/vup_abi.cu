@@ -265,6 +265,29 @@ static void free_grid(vup_grid g) {
     delete g;
 }
 
+// Zeroes device memory and waits for it, on a non-blocking stream that new grids
+// share (one per device, made by the first: making and destroying one per grid took
+// 20 us of a grid's 85; made anew where a device reset took it away).
+static cudaError_t clear_now(const std::vector<std::pair<void *, size_t>> &pieces) {
+    static std::mutex mu;
+    static std::map<int, cudaStream_t> streams;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    std::lock_guard<std::mutex> lk(mu);
+    for (int tries = 0; tries < 2; ++tries) {
+        cudaStream_t &s = streams[dev];
+        if (e == cudaSuccess && !s) e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
+        for (const auto &q : pieces)
+            if (e == cudaSuccess) e = cudaMemsetAsync(q.first, 0, q.second, s);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        if (e != cudaErrorInvalidResourceHandle && e != cudaErrorContextIsDestroyed) break;
+        cudaGetLastError();
+        s = nullptr;
+        e = cudaSuccess;
+    }
+    return e;
+}
+
 extern "C" vup_status vup_grid_create(int ndim, const int64_t *n, const double *lo, const double *hi,
                                       vup_grid *out) {
     if (!out || !n || !lo || !hi || ndim < 1 || ndim > 3) return VUP_ERR_INVALID_ARG;
@@ -399,25 +422,18 @@ extern "C" vup_status vup_grid_create(int ndim, const int64_t *n, const double *
         L.rec_chunk = A.rec_chunk;
         L.rec_chunk_grp = A.rec_chunk_grp;
     }
-    // cleared before the handle is returned, on a stream of their own: queued on the
-    // default stream they could wait behind a caller's work there and land in the
-    // middle of this grid's calls on another stream
+    // cleared before the handle is returned, not on the default stream: there they
+    // could wait behind a caller's work and land in the middle of this grid's calls on
+    // another stream
     if (e == cudaSuccess) {
-        cudaStream_t cs = nullptr;
-        e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
-        auto clear = [&](void *q, size_t bytes) {
-            if (e == cudaSuccess) e = cudaMemsetAsync(q, 0, bytes, cs);
-        };
-        clear(g->dstatus, sizeof(int));
-        clear(g->hist_sel, sizeof(int32_t) * 8);
+        std::vector<std::pair<void *, size_t>> zero = {{g->dstatus, sizeof(int)}, {g->hist_sel, sizeof(int32_t) * 8}};
         if (ndim >= 2) {
             // words past the stream's end are read by whole-window staging and
             // masked; zero keeps their rest codes valid indices
-            clear(g->hl[0].ipt, sizeof(uint2) * (N + 128));
-            clear(g->fold, sizeof(FoldGeom));  // nothing merged before a layout is built
+            zero.push_back({g->hl[0].ipt, sizeof(uint2) * (N + 128)});
+            zero.push_back({g->fold, sizeof(FoldGeom)});  // nothing merged before a layout is built
         }
-        if (e == cudaSuccess) e = cudaStreamSynchronize(cs);
-        if (cs) cudaStreamDestroy(cs);
+        e = clear_now(zero);
     }
     if (e != cudaSuccess) {
         vup_set_last_cuda_error(e, "vup_grid_create", __FILE__, __LINE__);
