@@ -9,7 +9,7 @@
 // FP64 arithmetic bounds this path: the GPU issues about two FP64 operations
 // per clock and SM, so its time is the number of them.  The density is evaluated once per
 // point (it was evaluated for each of the three sums: 338 us for 256 densities
-// on 4096 points, now 88), in 4 operations up to the exponent and 11 for a
+// on 4096 points, now 88), in 4 operations up to the exponent and 12 for a
 // table-driven exponential; points whose Gaussian is 0 in FP64, beyond 38.6
 // sigma, are skipped (three of five points at sigma = 1/200 of the domain, none
 // at 1/40); and sums add across warps and few lanes, as
@@ -62,9 +62,11 @@ __constant__ double kExpTab[64] = {
 // exp(x) for x <= 0, table-driven (P. T. P. Tang, "Table-driven implementation
 // of the exponential function in IEEE floating-point arithmetic", ACM TOMS 15,
 // 1989): x = (64 m + j) ln2 / 64 + r, |r| <= ln2 / 128, exp(x) = 2^m 2^(j/64)
-// (1 + r + r^2/2 + .. + r^5/120); the truncation is below 4e-17, the whole
-// within 1.2 ulp (host check against 40 digits).  tab: the table in shared memory.  Results below the normal
-// range take the library function.
+// (1 + r + r^2/2 + .. + r^6/720).  Within 1.02 ulp: half an ulp each of the table
+// and of the last rounding, 0.01 of r and of the polynomial, 1e-4 of its truncation
+// (without r^6/720 the truncation is 0.3 ulp and results were up to 1.27 ulp off;
+// tests/test_fp64_forms.py compares with 40 digits).  tab: the table in shared
+// memory.  Results below the normal range take the library function.
 __device__ __forceinline__ double exp_neg(double x, const double *tab) {
     if (!(x > -700.0)) return exp(x);
     constexpr double kMagic = 6755399441055744.0;  // 1.5 2^52: the sum's low bits are round(x 64 / ln2)
@@ -73,7 +75,8 @@ __device__ __forceinline__ double exp_neg(double x, const double *tab) {
     const double kd = t - kMagic;
     double r = fma(kd, -0x1.62e42fee00000p-7, x);
     r = fma(kd, -0x1.a39ef35793c76p-39, r);
-    double q = fma(r, 1.0 / 120.0, 1.0 / 24.0);
+    double q = fma(r, 1.0 / 720.0, 1.0 / 120.0);
+    q = fma(q, r, 1.0 / 24.0);
     q = fma(q, r, 1.0 / 6.0);
     q = fma(q, r, 0.5);
     q = fma(q, r * r, r);

@@ -1731,8 +1731,9 @@ struct Store<Tf32Pair> {
 // a / s with inv = 1 / s rounded: the quotient estimate corrected once by its
 // exact remainder (P. Markstein, "Computation of elementary functions on the
 // IBM RISC System/6000 processor", IBM J. Res. Dev. 34, 1990); equal to the
-// correctly rounded quotient on 60000 random pairs (host check).  Operands whose exponents
-// could make the remainder inexact take the division.
+// correctly rounded quotient (tests/test_fp64_forms.py: random pairs and quotients
+// beside the midpoint of two doubles).  Operands whose exponents could make the
+// remainder inexact take the division.
 __device__ __forceinline__ bool mid_exponent(double v) {
     return (uint32_t)((__double2hiint(v) >> 20) & 0x7ff) - 200u < 1640u;
 }
