@@ -718,7 +718,7 @@ __device__ __forceinline__ bool rec_chunk_walk(const ItemCtx &X, int c, int p, i
 template <int NF, int MODE>
 __device__ __forceinline__ void hist_item(const HistArgs *Ap, int p, int cg, int G, int64_t k0, uint8_t *sm,
                                           int64_t tile_rows, uint32_t &wseq, volatile int *abort, ItemCtx &X,
-                                          float *s_invz, int *next_chunk) {
+                                          float4 *s_invz, int *next_chunk) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t k = k0 + 4 * lane;
     float *ws = reinterpret_cast<float *>(sm);
@@ -748,7 +748,7 @@ __device__ __forceinline__ void hist_item(const HistArgs *Ap, int p, int cg, int
         X.rest_smem = hist_staged(MODE) ? 1 : 0;
         X.rest_n0 = X.H.n0;
     }
-    if (threadIdx.x < kKT) s_invz[threadIdx.x] = inv_z(*Ap, k0 + threadIdx.x);
+    if (threadIdx.x < kKT) reinterpret_cast<float *>(s_invz)[threadIdx.x] = inv_z(*Ap, k0 + threadIdx.x);
     __syncthreads();
     const LayoutArgs &H = X.H;
     if (p >= H.P) return;  // uniform
@@ -765,7 +765,7 @@ __device__ __forceinline__ void hist_item(const HistArgs *Ap, int p, int cg, int
     // it.  (Prefix tiles from a kernel of their own cost 60 us at 1024 rows x
     // 16384 densities, or five times that beside the contraction, whose
     // operands take the L2 bandwidth; the scan here costs an item 3 us.)
-    const float4 iz4 = ld4(s_invz + 4 * lane);
+    const float4 iz4 = s_invz[lane];
     const int32_t a0 = (int32_t)(nrows * warp / kWarps), a1 = (int32_t)(nrows * (warp + 1) / kWarps);
     PairSum4 t;
     t.clear();
@@ -1101,7 +1101,7 @@ __global__ void __launch_bounds__(hist_warps(MODE) * 32, 1)
     if (hist_stream(A) != hist_stream_of(MODE)) return;  // uniform
     extern __shared__ __align__(128) uint8_t sm[];
     __shared__ ItemCtx X;
-    __shared__ float s_invz[kKT];
+    __shared__ float4 s_invz[kKT / 4];  // (the type: a lane reads four as one 16-byte load)
     __shared__ int abort, next_chunk, s_item, s_G;
     if (threadIdx.x == 0) abort = 0;
     hist_init_mbar(sm, tile_rows, hist_warps(MODE));
@@ -1192,7 +1192,7 @@ __global__ void __launch_bounds__(hist_warps(MODE) * 32, 1) k_hist_batched(const
                                                                      int *__restrict__ next_item) {
     extern __shared__ __align__(128) uint8_t sm[];
     __shared__ ItemCtx X;
-    __shared__ float s_invz[kKT];
+    __shared__ float4 s_invz[kKT / 4];  // (the type: a lane reads four as one 16-byte load)
     __shared__ int abort, next_chunk, s_it;
     if (threadIdx.x == 0) abort = 0;
     hist_init_mbar(sm, tile_rows, hist_warps(MODE));
