@@ -448,6 +448,7 @@ extern "C" vup_status vup_grid_create(int ndim, const int64_t *n, const double *
 extern "C" vup_status vup_grid_destroy(vup_grid g) {
     if (!g) return VUP_ERR_INVALID_ARG;
     cudaDeviceSynchronize();
+    vup_batched_forget(g);
     free_grid(g);
     return VUP_OK;
 }
@@ -471,7 +472,10 @@ static vup_status finish_model(vup_grid g, cudaStream_t s) {
     if (st != VUP_OK) return st;
     // power tables are built on first use by the contraction that needs them
     g->have_model = 1;
-    ++g->model_gen;
+    // one count for all grids: a grid made at the address of a destroyed one never has
+    // its generation, so that nothing kept for a (grid, generation) outlives both
+    static std::atomic<uint64_t> generations{0};
+    g->model_gen = ++generations;
     return VUP_OK;
 }
 

@@ -41,6 +41,7 @@ void free_stages(Stages &S) {
 
 struct Entry {
     std::vector<uint64_t> key;
+    std::vector<vup_grid> grids;
     int device = 0;
     bool bf16 = false;
     int bn_cap = 0;
@@ -206,6 +207,21 @@ void store_tune(const std::string &shape, int cap, const double *ms, const int *
 
 }  // namespace
 
+// (A plan's graph holds the addresses of its grids' arrays, most of which are not in
+// its key.)
+void vup_batched_forget(vup_grid g) {
+    std::lock_guard<std::mutex> lk(g_mu);
+    for (size_t i = 0; i < g_entries.size();) {
+        Entry *e = g_entries[i];
+        if (std::find(e->grids.begin(), e->grids.end(), g) == e->grids.end()) {
+            ++i;
+            continue;
+        }
+        free_entry(e);
+        g_entries.erase(g_entries.begin() + i);
+    }
+}
+
 extern "C" vup_status vup_propagate_batched(int n_inst, const vup_grid *g, const vup_densities *d,
                                             vup_precision precision, double *const *moments_raw,
                                             float *const *hist, vup_stream_t stream) {
@@ -308,6 +324,7 @@ extern "C" vup_status vup_propagate_batched(int n_inst, const vup_grid *g, const
         for (int cap : caps) {
             Entry *c = new Entry();
             c->key = key;
+            c->grids.assign(g, g + n_inst);
             c->device = dev;
             c->bf16 = bf16;
             c->bn_cap = cap;

@@ -254,7 +254,7 @@ struct vup_grid_s {
 
     // model outputs
     int have_model = 0;
-    uint64_t model_gen = 0;        // bumped whenever the model (and its tables) are rebuilt
+    uint64_t model_gen = 0;        // the model's generation, unlike any other grid's (0: none)
     int model_id = 0;              // built-in model of vup_eval_model (0: outputs set by the caller)
     double theta[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     int B = 0, J = 0;
@@ -439,6 +439,8 @@ vup_status vup_weights_path(vup_grid g, int64_t K, const float *W, double *raw, 
                             cudaStream_t s);
 
 int vup_num_sms();
+// Frees the batch plans that a grid about to be destroyed takes part in (no work in flight).
+void vup_batched_forget(vup_grid g);
 // Orientation of the forward tensor-core contraction: the last axis is the
 // reduction (3-D grids apply both rest axes' factors in the epilogue).
 inline int vup_tc_orient(const vup_grid_s *) { return kOrientLast; }

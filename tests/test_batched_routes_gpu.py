@@ -119,3 +119,32 @@ def test_histograms_do_not_depend_on_which_call_came_first():
     for name, hs in results.items():
         for p, a, b in zip(probs, results["alone"], hs):
             np.testing.assert_array_equal(b.cpu().numpy(), a.cpu().numpy(), err_msg=f"{name} {p.name}")
+
+
+@pytest.mark.parametrize("precision", ["fp32", "bf16x3"])
+def test_new_grids_never_replay_the_graph_of_destroyed_ones(precision):
+    """Batches of new grids on the same densities and output buffers, the ones before
+    destroyed: sizes, buffers and (as the allocators go) addresses repeat."""
+    from paper_1908_11246_gb300 import vup
+    probs = I.oscillator_batch(29, n_inst=4, side=(32, 191), kk=(64, 1500), n_bins=67)
+    dds = [vup.densities_to_device(p.dens) for p in probs]
+    grids = _grids(probs)
+    out = vup.batched_outputs(grids, dds)
+    for r in range(10):
+        vup.propagate_batched(grids, dds, precision, out=out)
+        assert vup.vup_batched_report()["source"] != 0, r  # a plan of its own
+        for g in grids:
+            g.sync()
+        if r in (0, 4, 9):
+            for p, raw, h in zip(probs, *out):
+                _check(p, raw, h, precision)
+        vup.propagate_batched(grids, dds, precision, out=out)
+        assert vup.vup_batched_report()["source"] == 0, r  # the same call again replays it
+        for g in grids if r % 2 else reversed(grids):
+            g.close()
+        # other models, so that what a stale graph left behind would show
+        for p in probs:
+            p.theta = (1.0 + 0.7 * (r + 1),)
+        grids = _grids(probs)
+    for g in grids:
+        g.close()
