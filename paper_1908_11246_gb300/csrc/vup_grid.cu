@@ -1696,20 +1696,6 @@ __global__ void k_rec_tables(const int32_t *__restrict__ starts, const int32_t *
 // ---- power tables -----------------------------------------------------------
 // y viewed as a matrix Y[P][S] (flat i = p S + s).  Element (p, s) yields
 // z = (y - c) / s_scale and its powers z^j 2^e, j = 1..4 (FP64, then rounded).
-// mode 0: out[(p*4 + j) * ld + s]      (rows (p, j), cols s)
-// mode 1: out[s * ld + p*4 + j]        (rows s, cols (p, j))
-// mode 2: out[(s*4 + j) * ld + p]      (rows (s, j), cols p)
-// mode 3: out[p * ld + s*4 + j]        (rows p, cols (s, j))
-// A 32 x 32 (p, s) tile goes through shared memory so that both the read of y
-// and the write of the table are coalesced whatever the mode.
-template <typename T>
-struct Store;
-template <>
-struct Store<float> {
-    static __device__ __forceinline__ void put(float *o, float * /*o2*/, int64_t idx, double v) {
-        o[idx] = (float)v;
-    }
-};
 
 // TF32 pair: hi = v rounded to TF32 (10 explicit mantissa bits, stored in a
 // float), lo = the remainder rounded to TF32.
@@ -1718,15 +1704,6 @@ __device__ __forceinline__ float to_tf32(float x) {
     asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
     return __uint_as_float(r);
 }
-struct Tf32Pair {};
-template <>
-struct Store<Tf32Pair> {
-    static __device__ __forceinline__ void put(float *o, float *o2, int64_t idx, double v) {
-        const float h = to_tf32((float)v);
-        o[idx] = h;
-        o2[idx] = to_tf32((float)(v - (double)h));
-    }
-};
 
 // a / s with inv = 1 / s rounded: the quotient estimate corrected once by its
 // exact remainder (P. Markstein, "Computation of elementary functions on the
@@ -1743,10 +1720,14 @@ __device__ __forceinline__ double div_scale(double a, double s, double inv) {
     return fma(fma(-q, s, a), inv, q);
 }
 
-template <typename T, typename O = T>
-__global__ void k_power_table(const double *__restrict__ y, int64_t P, int64_t S,
-                              const double *__restrict__ sc, int mode, int64_t ld,
-                              O *__restrict__ out, O *__restrict__ out2) {
+// TF32 power tables (hi and lo), rows of one (index, power): ROWS_P: out[(p * 4 + j)
+// * ld + s], else out[(s * 4 + j) * ld + p].  A 32 x 32 (p, s) tile goes through
+// shared memory so that both the read of y and the write of the table are
+// coalesced either way.
+template <bool ROWS_P>
+__global__ void k_power_table_tf32(const double *__restrict__ y, int64_t P, int64_t S,
+                                   const double *__restrict__ sc, int64_t ld, float *__restrict__ hi,
+                                   float *__restrict__ lo) {
     __shared__ double tile[32][33];
     const int64_t p0 = (int64_t)blockIdx.y * 32, s0 = (int64_t)blockIdx.x * 32;
     const double scale = sc[kScaleS], shift = sc[kScaleC], pf = sc[kScaleP], inv = 1.0 / scale;
@@ -1760,37 +1741,15 @@ __global__ void k_power_table(const double *__restrict__ y, int64_t P, int64_t S
     // 32 x 32 x 4 values; thread t handles values linear in the output order
     const int tid = threadIdx.y * 32 + threadIdx.x, nthr = 32 * blockDim.y;
     for (int e = tid; e < 32 * 32 * 4; e += nthr) {
-        int a, b, j;  // a = fast output coordinate within the tile
-        int lp, ls;
-        int64_t idx;
-        switch (mode) {
-        case 0: {  // rows (p, j), cols s : fast = s
-            ls = e & 31; j = (e >> 5) & 3; lp = e >> 7;
-            idx = ((p0 + lp) * 4 + j) * ld + (s0 + ls);
-            break;
-        }
-        case 1: {  // rows s, cols (p, j) : fast = (p, j)
-            j = e & 3; lp = (e >> 2) & 31; ls = e >> 7;
-            idx = (s0 + ls) * ld + (p0 + lp) * 4 + j;
-            break;
-        }
-        case 2: {  // rows (s, j), cols p : fast = p
-            lp = e & 31; j = (e >> 5) & 3; ls = e >> 7;
-            idx = ((s0 + ls) * 4 + j) * ld + (p0 + lp);
-            break;
-        }
-        default: {  // rows p, cols (s, j) : fast = (s, j)
-            j = e & 3; ls = (e >> 2) & 31; lp = e >> 7;
-            idx = (p0 + lp) * ld + (s0 + ls) * 4 + j;
-            break;
-        }
-        }
-        (void)a; (void)b;
+        const int j = (e >> 5) & 3, lp = ROWS_P ? e >> 7 : e & 31, ls = ROWS_P ? e & 31 : e >> 7;
         if (p0 + lp >= P || s0 + ls >= S) continue;
+        const int64_t idx = ROWS_P ? ((p0 + lp) * 4 + j) * ld + (s0 + ls) : ((s0 + ls) * 4 + j) * ld + (p0 + lp);
         const double z = tile[lp][ls];
         double v = z * pf;  // (a power of two: exact, whatever the order)
         for (int q = 0; q < j; ++q) v = v * z;
-        Store<T>::put(out, out2, idx, v);
+        const float h = to_tf32((float)v);
+        hi[idx] = h;
+        lo[idx] = to_tf32((float)(v - (double)h));
     }
 }
 
@@ -2408,8 +2367,12 @@ vup_status vup_build_tables(vup_grid g, int orient, int bf16, cudaStream_t s) {
         }
         VUP_CHECK_CUDA(cudaMemsetAsync(g->ztf_hi[orient], 0, bytes, s));
         VUP_CHECK_CUDA(cudaMemsetAsync(g->ztf_lo[orient], 0, bytes, s));
-        k_power_table<Tf32Pair, float><<<grd, blk, 0, s>>>(g->y, P, S, g->ydev_scale, first ? 2 : 0, ld,
-                                                          g->ztf_hi[orient], g->ztf_lo[orient]);
+        if (first)
+            k_power_table_tf32<false><<<grd, blk, 0, s>>>(g->y, P, S, g->ydev_scale, ld, g->ztf_hi[orient],
+                                                          g->ztf_lo[orient]);
+        else
+            k_power_table_tf32<true><<<grd, blk, 0, s>>>(g->y, P, S, g->ydev_scale, ld, g->ztf_hi[orient],
+                                                         g->ztf_lo[orient]);
         VUP_CHECK_LAUNCH();
     } else {
         const int64_t ld = o.R_pad;

@@ -87,8 +87,6 @@ struct HistArgs {
     int C_rec;            // record chunks per part
     int GB;               // record groups per part: ceil(B / kRecBins)
     int points_only;      // 1: point stream whatever the layout choice says
-    int rest_smem;        // 3-D point stream: both rest-axis factor tiles staged in shared memory
-    int64_t rest_n0;      // rows of the first rest axis (3-D)
     float *hist;          // [K][B]
     float *part;          // [P * C][2][K_pad]
     float *direct;        // [P][K][B] (P > 1)
@@ -362,9 +360,7 @@ struct ItemCtx {
     float *direct; // [P * B][K_pad] sums of keys held by one chunk
     int64_t K, K_pad;
     int B, C, C_rec, GB;
-    int mode;      // 0: point stream, tile holds factors; 1: interval stream, tile holds prefix sums
-    int rest_smem;  // (3-D point stream) rest-axis factors [n0][kKT], [n1][kKT] after the staging buffers
-    int64_t rest_n0;
+    int64_t rest_n0;  // (3-D, staged) rows of the first rest axis' factors, before the second's
     int64_t pre_rows;  // rows of a prefix tile (debug build's bound)
     int *dstatus;
 };
@@ -742,10 +738,8 @@ __device__ __forceinline__ void hist_item(const HistArgs *Ap, int p, int cg, int
         X.C = A.C;
         X.C_rec = A.C_rec;
         X.GB = A.GB;
-        X.mode = hist_stream_of(MODE);
         X.pre_rows = X.H.part_rows + 1;
         X.dstatus = A.dstatus;
-        X.rest_smem = hist_staged(MODE) ? 1 : 0;
         X.rest_n0 = X.H.n0;
     }
     if (threadIdx.x < kKT) reinterpret_cast<float *>(s_invz)[threadIdx.x] = inv_z(*Ap, k0 + threadIdx.x);
@@ -1985,8 +1979,7 @@ vup_status vup_hist_fused(vup_grid g, int64_t K, float *hist, cudaStream_t s, co
     const bool in_smem = smem <= kSmemMost && coded;
     // 3-D point stream: both rest-axis factor tiles in shared memory when they fit beside the tile
     const size_t rest_bytes = nd == 3 ? (size_t)(g->n[0] + g->n[1]) * kKT * sizeof(float) : 0;
-    A.rest_n0 = nd == 3 ? g->n[0] : 0;
-    A.rest_smem = in_smem && vup_hist_rest_staged(g);
+    const bool rest_staged = in_smem && vup_hist_rest_staged(g);
     // the global-memory fallback walks points whatever the device chose
     points_only = points_only || !in_smem;
     A.points_only = points_only ? 1 : 0;
@@ -2016,13 +2009,13 @@ vup_status vup_hist_fused(vup_grid g, int64_t K, float *hist, cudaStream_t s, co
                 for (int l = 0; l < g->n_layouts; ++l) rest_rows = std::max(rest_rows, g->N / g->hl[l].n_last);
                 if (nd == 3) rest_rows = g->n[0] + g->n[1];
                 const bool l2_rest = (double)rest_rows * A.K_pad * 4.0 <= 96.0 * 1024 * 1024;
-                if (A.rest_smem) st = launch(k_hist_smem<2, 5>, 5);
+                if (rest_staged) st = launch(k_hist_smem<2, 5>, 5);
                 else if (l2_rest) st = nd == 3 ? launch(k_hist_smem<2, 3>, 3) : launch(k_hist_smem<1, 3>, 3);
                 else st = nd == 3 ? launch(k_hist_smem<2, 2>, 2) : launch(k_hist_smem<1, 2>, 2);
                 if (st != VUP_OK) return st;
             }
             if (keys_ready) VUP_CHECK_CUDA(cudaStreamWaitEvent(s, keys_ready, 0));
-            st = nd == 3 ? (A.rest_smem ? launch(k_hist_smem<2, 4>, 4) : launch(k_hist_smem<2, 0>, 0))
+            st = nd == 3 ? (rest_staged ? launch(k_hist_smem<2, 4>, 4) : launch(k_hist_smem<2, 0>, 0))
                          : launch(k_hist_smem<1, 0>, 0);
             if (st != VUP_OK) return st;
             if (!points_only) {
