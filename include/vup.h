@@ -268,7 +268,7 @@ vup_status vup_propagate_ipsa(vup_grid g, const vup_densities *d, vup_precision 
  *       VUP_ERR_UNSUPPORTED).
  * Every grid must be 2-D with a model (VUP_ERR_STATE otherwise) and each
  * gathered-axis part of its histogram layout must fit one shared-memory tile
- * (704 rows; VUP_ERR_UNSUPPORTED otherwise).
+ * (392 rows; VUP_ERR_UNSUPPORTED otherwise).
  * The first call for a batch (same grids, densities, output pointers and
  * sizes) builds the work lists, chooses the contraction tile width for the
  * batch's shape (VUP_BF16X3: times tile-width caps 256, 128 and 64 once per
@@ -278,7 +278,9 @@ vup_status vup_propagate_ipsa(vup_grid g, const vup_densities *d, vup_precision 
  * graph; later calls replay that graph on `stream`.  The first call is
  * synchronous and allocates; later calls allocate nothing and may be captured
  * into a caller's graph (their stage kernels are then captured directly; a
- * first call made while `stream` is capturing returns VUP_ERR_STATE).  Up to 8 batches are remembered.  Device conditions are
+ * first call made while `stream` is capturing returns VUP_ERR_STATE).  Up to 8
+ * batches are remembered, beside those that a caller's graph was captured from;
+ * destroying a grid forgets its batches.  Device conditions are
  * recorded per grid (VUP_ERR_EMPTY_SUPPORT) and, for an expired wait in the
  * contraction, in g[0]; read them with vup_sync.
  */

@@ -50,6 +50,7 @@ struct Entry {
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     uint64_t used = 0;
+    bool captured = false;  // a caller's graph holds the plan's memory: kept while its grids live
 };
 
 void free_entry(Entry *e) {
@@ -310,10 +311,16 @@ extern "C" vup_status vup_propagate_batched(int n_inst, const vup_grid *g, const
                 source = 2;
             }
         }
-        // evict the least recently used plan (its graph may still be in flight)
-        if (g_entries.size() >= kMaxEntries) {
-            auto lru = std::min_element(g_entries.begin(), g_entries.end(),
-                                        [](const Entry *a, const Entry *b) { return a->used < b->used; });
+        // evict the least recently used plan (its graph may still be in flight), but none
+        // that a caller's graph was captured from
+        auto lru = g_entries.end();
+        size_t n_own = 0;
+        for (auto it = g_entries.begin(); it != g_entries.end(); ++it) {
+            if ((*it)->captured) continue;
+            ++n_own;
+            if (lru == g_entries.end() || (*it)->used < (*lru)->used) lru = it;
+        }
+        if (n_own >= kMaxEntries) {
             VUP_CHECK_CUDA(cudaDeviceSynchronize());
             free_entry(*lru);
             g_entries.erase(lru);
@@ -367,6 +374,7 @@ extern "C" vup_status vup_propagate_batched(int n_inst, const vup_grid *g, const
     t_bn_cap = e->bn_cap;
     // inside a caller's capture the stage kernels join the caller's graph; with
     // profiling on they run one by one so that each stage is timed
+    if (capturing) e->captured = true;
     if (capturing || vup_profiling()) return run_stages(*e, s);
     VUP_CHECK_CUDA(cudaGraphLaunch(e->exec, s));
     return VUP_OK;

@@ -148,3 +148,36 @@ def test_new_grids_never_replay_the_graph_of_destroyed_ones(precision):
         grids = _grids(probs)
     for g in grids:
         g.close()
+
+
+def test_callers_graph_outlives_the_plans_of_other_batches():
+    """A batch captured into a caller's graph, then more other batches than plans are
+    kept for: the graph still replays the batch."""
+    import torch
+    from paper_1908_11246_gb300 import vup
+    probs = I.oscillator_batch(31, n_inst=3, side=(40, 150), kk=(64, 500), n_bins=50)
+    dds = [vup.densities_to_device(p.dens) for p in probs]
+    grids = _grids(probs)
+    out = vup.batched_outputs(grids, dds)
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    vup.propagate_batched(grids, dds, "fp32", out=out, stream=s)
+    s.synchronize()
+    want = [t.clone() for t in out[0] + out[1]]
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=s):
+        vup.propagate_batched(grids, dds, "fp32", out=out, stream=s)
+    others = [vup.batched_outputs(grids, dds) for _ in range(12)]  # 12 batches: other output buffers
+    for _ in range(2):
+        for o in others:
+            vup.propagate_batched(grids, dds, "fp32", out=o)
+    torch.cuda.synchronize()
+    for t in out[0] + out[1]:
+        t.fill_(-1)
+    graph.replay()
+    torch.cuda.synchronize()
+    for a, b in zip(want, out[0] + out[1]):
+        assert torch.equal(a, b)
+    del graph
+    for g in grids:
+        g.close()
