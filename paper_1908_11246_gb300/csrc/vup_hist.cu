@@ -2159,10 +2159,12 @@ vup_status vup_hist_plan(int n, const vup_grid *gs, const int64_t *Ks, float *co
     // SM cycles of an instance's tile fill and of its walk per (part, density
     // tile), from the sizes (its stream and counts are the device's to choose): a
     // walk costs about a cycle per point and 128 densities on smooth models.  An
-    // instance is cut so that no item's walk exceeds a third of an SM's share of
-    // the whole batch, nor falls below its fill: small batches fill the SMs (8
-    // instances of 38 - 170 points a side: 77 -> 69 us), large ones keep one
-    // item per tile.
+    // instance is cut so that no item's walk exceeds an SM's share of the whole
+    // batch, nor falls below its fill: small batches fill the SMs, large ones keep one
+    // item per tile.  32 instances of 32 - 1024 points a side 713 us with items of at
+    // most a third of the share, 694 of the share, 694 of twice that or uncut; 10 of
+    // at most 169: 127, 117, 116, 119; 16 of at most 621: 201, 185, 185, 219; 12 of at
+    // most 202: 116, 116, 132, 157.
     std::vector<int64_t> fill(n), walk(n);
     double share = 0.0;
     for (int i = 0; i < n; ++i) {
@@ -2181,7 +2183,7 @@ vup_status vup_hist_plan(int n, const vup_grid *gs, const int64_t *Ks, float *co
         rows_max = std::max(rows_max, rows);
         const int64_t most = std::max<int64_t>(1, args[i].C_rec / 8);  // at least eight record chunks
         const int G = (int)std::max<int64_t>(
-            1, std::min(most, ceil_div64(walk[i], std::max((int64_t)(share / 3.0), fill[i]))));
+            1, std::min(most, ceil_div64(walk[i], std::max((int64_t)share, fill[i]))));
         args[i].sets = G;
         const int64_t nkt = ceil_div64(Ks[i], kKT);
         const int64_t cost = fill[i] + walk[i] / G;
