@@ -1717,40 +1717,56 @@ __global__ void __launch_bounds__(kHistWarps * 32, 1)
 // H and the posterior means from the walk's sums (parts in order, cut keys from
 // their chunks' partials in chunk order, as the histogram's finish): 128
 // densities x 8 bins per CTA, a warp per bin.
+template <int NO>
 __global__ void __launch_bounds__(256) k_post_finish(const __grid_constant__ PostArgs A) {
-    __shared__ float tile[4][8][128 + 1];
+    __shared__ float tile[NO][8][128 + 1];
     const HistArgs &h = A.h;
     const LayoutArgs &H = h.sel[0] ? h.L1 : h.L0;
-    const int P = h.fold->P[h.sel[0] ? 1 : 0], nd = h.ndim, no = 1 + nd;
+    constexpr int nd = NO - 1;
+    const int P = h.fold->P[h.sel[0] ? 1 : 0];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int b = blockIdx.y * 8 + warp;
     const int64_t k0 = A.k0 + (int64_t)blockIdx.x * 128, k = k0 + 4 * lane;
-    float4 t[4];
+    float4 t[NO];
 #pragma unroll
-    for (int o = 0; o < 4; ++o) t[o] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int o = 0; o < NO; ++o) t[o] = make_float4(0.f, 0.f, 0.f, 0.f);
+    const int64_t kb = A.kb;
+    const float *direct = A.direct + (k - A.k0), *part = A.part + (k - A.k0);
     if (b < h.B)
         for (int p = 0; p < P; ++p) {
             const int32_t key = p * h.B + b;
             const int2 cc = H.key_chunks[key];
             if (cc.x < 0) continue;
             if (cc.x == cc.y) {
-                const float *row = A.direct + (int64_t)key * no * A.kb + (k - A.k0);
+                const float *row = direct + (int64_t)key * NO * kb;
 #pragma unroll
-                for (int o = 0; o < 4; ++o)
-                    if (o < no) add4(t[o], ld4(row + o * A.kb));
+                for (int o = 0; o < NO; ++o) add4(t[o], ld4(row + o * kb));
                 continue;
             }
-            for (int c = cc.x; c <= cc.y; ++c) {
-                if (H.chunk_pt[c] >= H.chunk_pt[c + 1]) continue;
-                const int side = H.chunk_bin[2 * c] == key ? 0 : 1;
-                const float *row = A.part + ((int64_t)c * 2 + side) * no * A.kb + (k - A.k0);
+            // a key cut by many chunks (few bins) is a chain of dependent loads: four
+            // chunks at a time, added in chunk order (an empty chunk's row is not; 1495 x
+            // 1786 points, 20 bins, K = 569: 84 us one at a time, 64 so)
+            for (int c0 = cc.x; c0 <= cc.y; c0 += 4) {
+                float4 v[4][NO];
+                bool live[4];
 #pragma unroll
-                for (int o = 0; o < 4; ++o)
-                    if (o < no) add4(t[o], ld4(row + o * A.kb));
+                for (int u = 0; u < 4; ++u) {
+                    const int c = min(c0 + u, cc.y);
+                    const int side = H.chunk_bin[2 * c] == key ? 0 : 1;
+                    live[u] = c0 + u <= cc.y && H.chunk_pt[c] < H.chunk_pt[c + 1];
+                    const float *row = part + ((int64_t)c * 2 + side) * NO * kb;
+#pragma unroll
+                    for (int o = 0; o < NO; ++o) v[u][o] = ld4(row + o * kb);
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (live[u])
+#pragma unroll
+                        for (int o = 0; o < NO; ++o) add4(t[o], v[u][o]);
             }
         }
 #pragma unroll
-    for (int o = 0; o < 4; ++o) {
+    for (int o = 0; o < NO; ++o) {
         float *q = tile[o][warp] + 4 * lane;
         q[0] = t[o].x;
         q[1] = t[o].y;
@@ -2119,7 +2135,9 @@ vup_status vup_post_fused(vup_grid g, int64_t K, float *hist, float *post, cudaS
             if (st != VUP_OK) return st;
         }
         VUP_PROF("posterior_finish", s, 1);
-        k_post_finish<<<dim3((unsigned)ceil_div64(nk, 128), (unsigned)ceil_div64(g->B, 8)), 256, 0, s>>>(A);
+        const dim3 fin((unsigned)ceil_div64(nk, 128), (unsigned)ceil_div64(g->B, 8));
+        if (nd == 2) k_post_finish<3><<<fin, 256, 0, s>>>(A);
+        else k_post_finish<4><<<fin, 256, 0, s>>>(A);
         VUP_CHECK_LAUNCH();
     }
     return VUP_OK;
